@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "gpe_internal.cuh"
+#include "stencil.cuh"
 
 namespace gpe {
 
@@ -941,41 +942,180 @@ extern "C" int gpe_grid_destroy(gpe_grid *g)
 // ------------------------------------------------------------ Thomas-Fermi mu
 namespace gpe {
 
-// One pass of the Thomas-Fermi solve: over the cells with V < mu, the sum of
-// V and their count (result[0], result[1]).  Blocks take whole x-rows, so a
-// cell's coordinates need no division; dense sources read V directly.
-__global__ void k_tf_pass(VSource src, BoxD box, double mu, double *partials, unsigned int *counter,
-                          double *result)
+// A pass of the Thomas-Fermi solve reads the box once: over the cells with
+// V < mu, the sum of V (FP64) and their count, and over all cells below +inf
+// the largest |V| (its leading 32 bits, as an integer).  Bound by the read of
+// a dense V: 512^3 FP32 takes 0.09 ms (5.9 TB/s).  What keeps FP64 work off
+// that path (an FP64 instruction issues at 1/64 of the FP32 rate here; the
+// former pass compared, added and counted every cell in FP64 and took
+// 1.55 ms): FP32 cells are compared in FP32 against mu rounded up (the same
+// set: a float is below mu exactly if it is below the next float at or above
+// mu), FP64 cells first by their high words, cells are counted in integers,
+// and only selected cells are added in FP64.
+struct TfSum {
+    double sum = 0.0;
+    unsigned long long cnt = 0;
+    uint32_t top = 0;
+};
+
+struct TfLimit {  // mu in the forms the comparisons use
+    double mu;
+    float mu_f;    // smallest float >= mu
+    int32_t hi;    // order-preserving high word of mu
+};
+
+// high word of a double as a signed integer that orders like the double
+__device__ __forceinline__ int32_t ordered_hi(double v)
 {
-    double acc[2] = {0.0, 0.0};
-    const int64_t rows = box.ny * box.nz;
-    for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
-        const int64_t j = r % box.ny, k = r / box.ny;
-        for (int64_t i = threadIdx.x; i < box.nx; i += blockDim.x) {
-            double v0, v1;
-            bool sel;
-            cell_values(src, box, i, j, k, v0, v1, sel);
-            if (v0 < mu) {
-                acc[0] += v0;
-                acc[1] += 1.0;
-            }
-        }
+    const int32_t h = __double2hiint(v);
+    return h < 0 ? h ^ 0x7fffffff : h;
+}
+
+__device__ __forceinline__ void tf_cell(float v, const TfLimit &m, TfSum &a)
+{
+    if (v < INFINITY) a.top = max(a.top, __float_as_uint(fabsf(v)));
+    if (v < m.mu_f) {
+        a.sum += (double)v;
+        ++a.cnt;
     }
-    double tot[2];
+}
+__device__ __forceinline__ void tf_cell(double v, const TfLimit &m, TfSum &a)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(v) & 0x7fffffffu;
+    // below +inf: finite or -inf (NaN and +inf have no place in the sums)
+    const bool below = hi < 0x7ff00000u || (__double2hiint(v) == (int)0xfff00000 && __double2loint(v) == 0);
+    if (!below) return;
+    a.top = max(a.top, hi);
+    if (ordered_hi(v) <= m.hi && v < m.mu) {
+        a.sum += v;
+        ++a.cnt;
+    }
+}
+
+__device__ __forceinline__ void tf_finish(const TfSum &a, double *partials, unsigned int *counter, double *result,
+                                          uint32_t *top)
+{
+    const uint32_t t = __reduce_max_sync(0xffffffffu, a.top);
+    if ((threadIdx.x & 31) == 0 && t > __ldcg(top)) atomicMax(top, t);
+    double acc[2] = {a.sum, (double)a.cnt}, tot[2];
     if (reduce_finish<2>(acc, partials, counter, tot) && threadIdx.x == 0) {
         result[0] = tot[0];
         result[1] = tot[1];
     }
 }
 
+// dense V, n cells; n_vec of them (from the start) by 16-byte loads
+template <typename T>
+__global__ void k_tf_dense(const T *V, int64_t n, int64_t n_vec, TfLimit m, double *partials, unsigned int *counter,
+                           double *result, uint32_t *top)
+{
+    constexpr int W = 16 / (int)sizeof(T);
+    struct alignas(16) Vec {
+        T v[W];
+    };
+    TfSum a;
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    const Vec *src = reinterpret_cast<const Vec *>(V);
+    const int64_t nv = n_vec / W;
+    // four loads in flight a thread
+    int64_t i = t;
+    for (; i + 3 * step < nv; i += 4 * step) {
+        Vec x[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x[k] = src[i + k * step];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int w = 0; w < W; ++w) tf_cell(x[k].v[w], m, a);
+    }
+    for (; i < nv; i += step) {
+        const Vec x = src[i];
+#pragma unroll
+        for (int w = 0; w < W; ++w) tf_cell(x.v[w], m, a);
+    }
+    for (int64_t j = n_vec + t; j < n; j += step) tf_cell(V[j], m, a);
+    tf_finish(a, partials, counter, result, top);
+}
+
+// analytic V: a warp takes 32 cells along x and evaluates them in FP64 unless
+// the FP32 bound rules every one of them out
+__global__ void k_tf_analytic(PotDesc P, BoxD box, TfLimit m, double *partials, unsigned int *counter, double *result,
+                              uint32_t *top)
+{
+    TfSum a;
+    const int lane = threadIdx.x & 31;
+    const int64_t nc = (box.nx + 31) / 32, n = nc * box.ny * box.nz;
+    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t u = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); u < n; u += nw) {
+        const int64_t i0 = u % nc * 32, r = u / nc, j = r % box.ny, k = r / box.ny;
+        const int64_t i1 = min(i0 + 32, box.nx) - 1;
+        const double y = box.y0 + j * box.hy, z = box.z0 + k * box.hz;
+        if (!pot_may_select(P, m.mu, (float)(box.x0 + i0 * box.hx), (float)(box.x0 + i1 * box.hx), (float)y, (float)y,
+                            (float)z, (float)z))
+            continue;
+        if (i0 + lane <= i1) tf_cell(eval_pot(P, box.x0 + (i0 + lane) * box.hx, y, z), m, a);
+    }
+    tf_finish(a, partials, counter, result, top);
+}
+
+// One cell of each of `ns` equal stretches of the box, as float
+constexpr int64_t TF_SAMPLES = 131072;
+__global__ void k_tf_sample(VSource src, BoxD box, int64_t n, int64_t ns, float *out)
+{
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= ns) return;
+    const int64_t lo = i * n / ns, len = (i + 1) * n / ns - lo;
+    const int64_t lin = lo + (int64_t)((uint64_t)i * 2654435761ull % (uint64_t)len);
+    double v0, v1;
+    bool sel;
+    cell_values(src, box, lin % box.nx, lin / box.nx % box.ny, lin / (box.nx * box.ny), v0, v1, sel);
+    out[i] = (float)v0;
+}
+
+// Newton's method on the sample, with the target scaled to it: an estimate
+// that starts the solve over the whole box, so FP32 is enough
+__global__ void k_tf_estimate(const float *v, int n, double target, double *result)
+{
+    __shared__ float s_m;
+    __shared__ int s_stop;
+    float m = INFINITY;
+    double last = -1.0;
+    for (int it = 0; it < 100; ++it) {
+        float sum = 0.0f;
+        int cnt = 0;
+        for (int i = threadIdx.x; i < n; i += blockDim.x)
+            if (v[i] < m) {
+                sum += v[i];
+                ++cnt;
+            }
+        const double tot = block_sum((double)sum);
+        const double c = block_sum((double)cnt);
+        if (threadIdx.x == 0) {
+            const double next = (target + tot) / c;
+            s_stop = !(c > 0.0) || !(next < (double)m) || c == last || !isfinite(next);
+            if (c > 0.0 && isfinite(next) && next < (double)m) s_m = (float)next;
+            else s_m = m;
+            last = c;
+        }
+        __syncthreads();
+        m = s_m;
+        if (s_stop) break;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *result = (double)m;
+}
+
 // Eq. (5): the mu at which the Thomas-Fermi atom number
 //   F(mu) = sum over the box of max(mu - V, 0) / g dV
 // equals N.  F is convex, increasing and piecewise linear in mu, so Newton's
-// method started above the root stays above it and reaches the root exactly
-// once the set {V < mu} stops changing:
-//   mu <- (g N / dV + sum_{V < mu} V) / #{V < mu}.
-// The first pass takes every cell (mu = +inf), whose line lies below F, so
-// its root already bounds the true one from above.
+// method
+//   mu <- (g N / dV + sum_{V < mu} V) / #{V < mu}
+// moves from any start to or above the root (a tangent lies below F), then
+// down to it, and ends exactly once the set {V < mu} stops changing.  It
+// starts from the solution on a sample of the cells, a per cent or so off:
+// three to five passes over the box, where a start at mu = +inf took about
+// eighteen of 1.55 ms (a four-stage 512^3 ramp with FP32 potentials: 148 ms,
+// now 65 ms).
 static int tf_mu_impl(const gpe_box *box, const VSource &src, double g, double N, double *mu, cudaStream_t st)
 {
     if (!(g > 0)) return fail(GPE_ERR_ARG, "g must be > 0 for the Thomas-Fermi estimate");
@@ -983,47 +1123,110 @@ static int tf_mu_impl(const gpe_box *box, const VSource &src, double g, double N
     if (!mu) return fail(GPE_ERR_ARG, "mu is NULL");
     int dev = 0;
     GPE_TRY_CUDA(cudaGetDevice(&dev));
-    const int64_t rows = box->ny * box->nz;
-    const int blocks = (int)std::min<int64_t>(rows, (int64_t)sm_count(dev) * 8);
-    RedScratch r;
-    GPE_TRY(red_alloc(r, blocks));
-    double *res = nullptr, h[2];
-    int rc = dev_alloc_t(&res, 2);
+    const int64_t n = box->nx * box->ny * box->nz;
+    const int64_t ns = std::min(n, TF_SAMPLES);
+    const int blocks = (int)std::min<int64_t>((n + 1023) / 1024, (int64_t)sm_count(dev) * 8);
     const BoxD bd = boxd(*box);
     const double dV = box->hx * box->hy * box->hz;
     const double target = g * N / dV;
+    // one workspace: results (sum, count, estimate), largest |V|, block
+    // counter, block partial sums, sample
+    struct Head {
+        double res[3];
+        uint32_t top;
+        unsigned int counter;
+    };
+    char *ws = nullptr;
+    GPE_TRY(dev_alloc_t(&ws, sizeof(Head) + 16 * (size_t)blocks + 4 * (size_t)ns));
+    Head *head = reinterpret_cast<Head *>(ws), h{};
+    double *partials = reinterpret_cast<double *>(ws + sizeof(Head));
+    float *sample = reinterpret_cast<float *>(partials + 2 * blocks);
     auto pass = [&](double m) -> int {
-        k_tf_pass<<<blocks, 256, 0, st>>>(src, bd, m, r.partials, r.counter, res);
-        GPE_TRY_CUDA(cudaGetLastError());
-        GPE_TRY_CUDA(cudaMemcpyAsync(h, res, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
+        TfLimit lim;
+        lim.mu = m;
+        lim.mu_f = (float)m;
+        if ((double)lim.mu_f < m) lim.mu_f = std::nextafter(lim.mu_f, INFINITY);
+        int64_t bits;
+        memcpy(&bits, &m, 8);
+        lim.hi = (int32_t)(bits >> 32);
+        if (lim.hi < 0) lim.hi ^= 0x7fffffff;
+        if (src.mode != 0) {
+            k_tf_analytic<<<blocks, 256, 0, st>>>(src.p0, bd, lim, partials, &head->counter, head->res, &head->top);
+        } else {
+            const bool aligned = reinterpret_cast<uintptr_t>(src.dense) % 16 == 0;
+            if (src.dtype == GPE_F64)
+                k_tf_dense<double><<<blocks, 256, 0, st>>>((const double *)src.dense, n, aligned ? n / 2 * 2 : 0, lim,
+                                                          partials, &head->counter, head->res, &head->top);
+            else
+                k_tf_dense<float><<<blocks, 256, 0, st>>>((const float *)src.dense, n, aligned ? n / 4 * 4 : 0, lim,
+                                                         partials, &head->counter, head->res, &head->top);
+        }
+        GPE_LAUNCH_CHECK();
+        GPE_TRY_CUDA(cudaMemcpyAsync(&h, head, sizeof h, cudaMemcpyDeviceToHost, st));
         GPE_TRY_CUDA(cudaStreamSynchronize(st));
         return GPE_OK;
     };
-    double m = INFINITY;
-    double count = -1.0;
-    for (int it = 0; it < 200 && rc == GPE_OK; ++it) {
-        rc = pass(m);
-        if (rc != GPE_OK) break;
-        if (!(h[1] > 0.0)) {
-            rc = fail(GPE_ERR_ARG, "Thomas-Fermi solve found no cell below mu (V not finite?)");
-            break;
+    // can the sum over every cell leave the finite range?  (the solve from
+    // mu = +inf refuses such a potential)
+    auto may_overflow = [&]() {
+        double top;
+        if (src.mode != 0) {
+            double c[3] = {std::max(std::fabs(bd.x0), std::fabs(bd.x0 + (bd.nx - 1) * bd.hx)),
+                           std::max(std::fabs(bd.y0), std::fabs(bd.y0 + (bd.ny - 1) * bd.hy)),
+                           std::max(std::fabs(bd.z0), std::fabs(bd.z0 + (bd.nz - 1) * bd.hz))};
+            const double *p = src.p0.p;
+            if (src.p0.kind == GPE_POT_HARMONIC) {
+                top = 0.5 * (p[0] * p[0] * c[0] * c[0] + p[1] * p[1] * c[1] * c[1] + p[2] * p[2] * c[2] * c[2]);
+            } else {
+                const double r = 1.0 + c[0] / p[1] + c[1] / p[2] + c[2] / p[3];
+                top = 0.5 * p[0] * p[0] * r * r;
+            }
+        } else if (src.dtype == GPE_F64) {
+            const uint64_t b = (uint64_t)(h.top + 1u) << 32;
+            memcpy(&top, &b, 8);
+        } else {
+            float f;
+            memcpy(&f, &h.top, 4);
+            top = f;
         }
-        const double next = (target + h[0]) / h[1];
-        const bool same_set = h[1] == count;
-        count = h[1];
-        if (!std::isfinite(next)) {
-            rc = fail(GPE_ERR_ARG, "Thomas-Fermi solve: non-finite mu (V not finite?)");
-            break;
+        return !(top * (double)n < 1e308);
+    };
+    auto solve = [&]() -> int {
+        GPE_TRY_CUDA(cudaMemsetAsync(head, 0, sizeof(Head), st));
+        k_tf_sample<<<(unsigned)((ns + 255) / 256), 256, 0, st>>>(src, bd, n, ns, sample);
+        GPE_LAUNCH_CHECK();
+        k_tf_estimate<<<1, 1024, 0, st>>>(sample, (int)ns, target * ((double)ns / (double)n), &head->res[2]);
+        GPE_LAUNCH_CHECK();
+        GPE_TRY_CUDA(cudaMemcpyAsync(&h, head, sizeof h, cudaMemcpyDeviceToHost, st));
+        GPE_TRY_CUDA(cudaStreamSynchronize(st));
+        double m = std::isfinite(h.res[2]) ? h.res[2] : INFINITY;
+        bool from_any = m < INFINITY;  // the first pass may start below the root
+        double count = -1.0;
+        for (int it = 0; it < 200; ++it) {
+            GPE_TRY(pass(m));
+            const double sum = h.res[0], cnt = h.res[1];
+            if (from_any && (!(cnt > 0.0) || may_overflow())) {  // from the start above every cell
+                m = INFINITY;
+                from_any = false;
+                continue;
+            }
+            if (!(cnt > 0.0)) return fail(GPE_ERR_ARG, "Thomas-Fermi solve found no cell below mu (V not finite?)");
+            const double next = (target + sum) / cnt;
+            const bool same_set = cnt == count;
+            count = cnt;
+            if (!std::isfinite(next)) return fail(GPE_ERR_ARG, "Thomas-Fermi solve: non-finite mu (V not finite?)");
+            if (same_set || (!from_any && !(next < m))) {
+                *mu = std::min(m, next);
+                return GPE_OK;
+            }
+            from_any = false;
+            m = next;
         }
-        if (same_set || !(next < m)) {
-            m = std::min(m, next);
-            break;
-        }
-        m = next;
-    }
-    if (rc == GPE_OK) *mu = m;
-    dev_free(res);
-    red_free(r);
+        *mu = m;
+        return GPE_OK;
+    };
+    const int rc = solve();
+    dev_free(ws);
     return rc;
 }
 
