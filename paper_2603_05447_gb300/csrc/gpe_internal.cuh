@@ -284,6 +284,18 @@ struct RedScratch {
 int red_alloc(RedScratch &r, int max_blocks);
 void red_free(RedScratch &r);
 
+// stored segments a tile, and threads a block of the tile kernels (tiles.cuh)
+constexpr int TILE = 128;
+// neighbour slots and halo lists of a grid's tiles
+struct TileTab {
+    uint2 *d_nbr = nullptr;      // 7-point grids
+    uint4 *d_nbr19 = nullptr;    // 19-point grids
+    uint32_t *d_halo = nullptr;  // [ntiles * stride]
+    uint32_t nseg = 0;
+    int ntiles = 0, stride = 0;
+    int nslot = 0;               // slots of the largest tile: own, zero, halo
+};
+
 }  // namespace gpe
 
 // ------------------------------------------------------------ handles
@@ -309,6 +321,7 @@ struct gpe_grid {
     gpe::BrickRec *d_rec19 = nullptr; // [nb*19] ... and of its 12 edge neighbours (19-point grids)
     int stencil = 7;                  // 7 or 19 points
     int32_t *d_nbr18 = nullptr;       // [nb*18] face then edge neighbour ids (PAIR schedule, built on first use)
+    gpe::TileTab tiles;         // the stencil kernels' tiles
     int32_t *d_bvol = nullptr;  // brick-grid volume nbx*nby*nbz -> brick id or -1
     double *d_V[2] = {nullptr, nullptr};
     float *d_Vf[2] = {nullptr, nullptr};  // float copies, made on first use
@@ -359,6 +372,8 @@ struct gpe_state {
 };
 
 namespace gpe {
+int tiles_build(gpe_grid *g, cudaStream_t st);
+void tiles_free(TileTab &t);
 int ensure_work(gpe_state *st, int n);          // allocate d_work[0..n-1] (zeroed)
 // step drivers of 19-point grids (step19.cu)
 int rk4_run19(gpe_state *st, const gpe_real_params *p, int64_t nsteps, double t0, cudaStream_t s);

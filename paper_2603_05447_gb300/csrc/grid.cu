@@ -484,6 +484,7 @@ static void grid_free(gpe_grid *g)
     dev_free(g->d_rec);
     dev_free(g->d_rec7);
     dev_free(g->d_rec19);
+    tiles_free(g->tiles);
     dev_free(g->d_nbr18);
     dev_free(g->d_chunk_lohi);
     dev_free(g->d_tasks);
@@ -707,6 +708,7 @@ static int build_grid(const gpe_box *box, const VSource &src, const gpe_grid_opt
             BUILD_CUDA(cudaStreamSynchronize(st));
         }
     }
+    BUILD_TRY(tiles_build(g, st));
     for (int sl = 0; sl < g->n_slots; ++sl) {
         BUILD_TRY(dev_alloc_t(&g->d_V[sl], g->n_packed));
         k_pack<<<g->nsm * 8, 256, 0, st>>>(g->n_stored, g->bc, g->d_mask, g->d_rec, tmpV[sl], g->d_V[sl],

@@ -32,6 +32,7 @@
 #include "kernels.cuh"
 #include "itp_pair.cuh"
 #include "pair.cuh"
+#include "tiles.cuh"
 
 namespace gpe {
 
@@ -904,21 +905,20 @@ static int rk4_run(gpe_state *st, const gpe_real_params *p, int64_t nsteps, doub
         }
         return record(s, left);
     }
-    using RS = Rk4Stages<R, BX, BY, BZ>;
-    typename RS::K k[4];
-    int nblk[4];
+    using RT = Rk4Tiles<R, 7>;
+    typename RT::K k[4];
+    const TileLaunch L = tile_launch<CT>(g);
+    unsigned nblk[4];
     for (int stg = 0; stg < 4; ++stg) {
-        k[stg] = RS::get(blend, stg);
-        nblk[stg] = blocks_for_nw(k[stg], g, RS::smem(), RS::NW);
+        k[stg] = RT::get(blend, stg);
+        nblk[stg] = tile_blocks(k[stg], g->nsm, L.T.ntiles, L.smem);
     }
     // steps n0 .. n0+cnt-1 with stage times relative to the device clock
     auto record = [&](cudaStream_t cs, int64_t cnt) -> int {
         for (int64_t n = 0; n < cnt; ++n) {
             a.t_off = (double)n * p->dt;
             for (int stg = 0; stg < 4; ++stg) {
-                // stage 0 follows the scalar kernels of a ramp (no programmatic edge)
-                const bool pdl = st->pdl && !(blend && n == 0 && stg == 0);
-                GPE_TRY_CUDA(launch_stage(k[stg], (unsigned)nblk[stg], RS::THREADS, RS::smem(), cs, pdl, a, G));
+                k[stg]<<<nblk[stg], TILE, L.smem, cs>>>(a, L.T);
                 GPE_LAUNCH_CHECK();
             }
         }

@@ -1,0 +1,350 @@
+// tiles.cuh -- the stencil kernels' unit of work: a tile of TILE consecutive
+// stored segments of the packed layout, one segment a thread, whatever bricks
+// they belong to.  Not part of the ABI.
+//
+// Per tile the grid builder (tiles.cu) keeps the list of the stored segments
+// outside it that its stencils read (its halo) and, per segment, where each
+// neighbour lies in the tile: as one of the tile's own segments (slots
+// 0..TILE-1), as the zero slot (TILE: not stored, psi = 0 there) or as a halo
+// segment (TILE+1 on).  So a kernel looks nothing up: own values come along
+// one contiguous run, the halo by one gather, every lane has a segment.
+//
+// Why this shape.  The former unit, one warp per brick with the neighbours'
+// segment ranks computed from bit masks, spent 330 of its 632 warp
+// instructions a brick on the fill and left a fifth of the lanes idle.  On a
+// thin shell's 8x8x4 bricks a tile of 128 reads 0.88 face segments and 0.29
+// x-halo cells per own segment; 64 would read 1.05 and 0.58, 256 0.80 and
+// 0.14, but neighbour slots of a 256-tile do not fit 10 bits in the worst
+// case (128: 129 + 6 * 128 slots).  The lists cost 12.7 bytes a segment and
+// pass, against 5.3 for the brick records, on 80 to 144 of data.
+#pragma once
+
+#include "stencil.cuh"
+
+
+namespace gpe {
+
+// neighbour fields of a segment: 0-3 its -y +y -z +z segments, 4 and 5 the
+// segments holding its -x and +x cells; with the 19-point stencil also 6-9 the
+// (-y-z) (+y-z) (-y+z) (+y+z) segments, and 10-17 those holding the -x and +x
+// cells of fields 0-3's rows (two each, in that order)
+template <int NP>
+struct TileFields {
+    static constexpr int N = NP == 19 ? 18 : 6;
+    static constexpr int BITS = NP == 19 ? 12 : 10;
+};
+
+struct TileView {
+    const uint2 *nbr;      // per segment: six 10-bit slots, three a word
+    const uint4 *nbr19;    // 19-point grids: two uint4 of 12-bit slots, five a 64-bit word
+    // per tile a row of `stride` entries: its count (whole | single << 16),
+    // then the whole segments, and from the row's end the single cells (bit
+    // 31: the segment's first cell, else its last)
+    const uint32_t *halo;
+    uint32_t nseg;         // stored segments
+    int ntiles, stride;
+    int pstr;              // slots of a 16-byte plane of the shared tile
+};
+
+// Shared tile: UPS planes of 16-byte units (unit k of every slot's segment is
+// contiguous), so that lanes with consecutive slots touch consecutive units
+template <typename CT>
+struct TileMem {
+    static constexpr int UPS = (int)(4 * sizeof(CT) / 16);
+    static constexpr int CPU_ = 4 / UPS;
+    // plane stride with the UPS units of a slot in distinct bank groups
+    static int pstr(int nslot)
+    {
+        const int want = UPS == 1 ? nslot % 8 : (UPS == 2 ? 4 : 2);
+        return nslot + (want - nslot % 8 + 8) % 8;
+    }
+    uint4 *u;
+    int p;
+    __device__ __forceinline__ void get(int s, CT (&v)[4]) const
+    {
+#pragma unroll
+        for (int k = 0; k < UPS; ++k) {
+            const uint4 w = u[k * p + s];
+            const CT *c = reinterpret_cast<const CT *>(&w);
+#pragma unroll
+            for (int i = 0; i < CPU_; ++i) v[k * CPU_ + i] = c[i];
+        }
+    }
+    __device__ __forceinline__ void put(int s, const CT (&v)[4]) const
+    {
+#pragma unroll
+        for (int k = 0; k < UPS; ++k) {
+            uint4 w;
+            CT *c = reinterpret_cast<CT *>(&w);
+#pragma unroll
+            for (int i = 0; i < CPU_; ++i) c[i] = v[k * CPU_ + i];
+            u[k * p + s] = w;
+        }
+    }
+    __device__ __forceinline__ CT *first(int s) const { return reinterpret_cast<CT *>(u + s); }
+    __device__ __forceinline__ CT *last(int s) const
+    {
+        return reinterpret_cast<CT *>(u + (UPS - 1) * p + s) + (CPU_ - 1);
+    }
+};
+
+// shared memory a block may have, less a margin for static arrays
+constexpr size_t TILE_SMEM_MAX = 224 * 1024;
+
+// a segment's neighbour slots
+template <int NP>
+struct TileSlots {
+    uint2 d;
+    __device__ __forceinline__ void load(const TileView &T, uint32_t seg) { d = __ldg(T.nbr + seg); }
+    __device__ __forceinline__ int operator()(int k) const
+    {
+        return (int)(((k < 3 ? d.x : d.y) >> (10 * (k % 3))) & 1023u);
+    }
+};
+template <>
+struct TileSlots<19> {
+    unsigned long long q[4];
+    __device__ __forceinline__ void load(const TileView &T, uint32_t seg)
+    {
+        const uint4 a = __ldg(T.nbr19 + 2 * (size_t)seg), b = __ldg(T.nbr19 + 2 * (size_t)seg + 1);
+        q[0] = a.x | (unsigned long long)a.y << 32;
+        q[1] = a.z | (unsigned long long)a.w << 32;
+        q[2] = b.x | (unsigned long long)b.y << 32;
+        q[3] = b.z | (unsigned long long)b.w << 32;
+    }
+    __device__ __forceinline__ int operator()(int k) const { return (int)((q[k / 5] >> (12 * (k % 5))) & 4095u); }
+};
+
+// The Laplacians L of a segment with values c and neighbour slots f
+template <int NP, typename CT, typename R>
+__device__ __forceinline__ void tile_laplacian(const TileMem<CT> &m, const TileSlots<NP> &f, const CT (&c)[4], R ihx2,
+                                               R ihy2, R ihz2, CT (&L)[4])
+{
+    // opposite neighbours are summed first and the centre term enters once:
+    // L = (x- + x+) / hx^2 + (y- + y+) / hy^2 + (z- + z+) / hz^2 - c6 c
+    const R c6 = (R)2 * (ihx2 + ihy2 + ihz2);
+    CT ym[4], yp[4], zm[4], zp[4];
+    m.get(f(0), ym);
+    m.get(f(1), yp);
+    m.get(f(2), zm);
+    m.get(f(3), zp);
+    const CT xm = *m.last(f(4)), xp = *m.first(f(5));
+    if constexpr (NP != 19) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const CT l = i == 0 ? xm : c[i - 1];
+            const CT rr = i == 3 ? xp : c[i + 1];
+            L[i] = lapv(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], ihx2, ihy2, ihz2, c6);
+        }
+    } else {
+        // App. B: the 7-point part plus w_ab (edges_ab - 2 faces_ab + 4 c) per
+        // plane ab, w_ab = (1/h_a^2 + 1/h_b^2) / 12.  Each face pair lies in
+        // two planes, so the face and centre terms fold into the 7-point form:
+        //   x: 1/hx^2 - 2 (wxy + wxz), y: 1/hy^2 - 2 (wxy + wyz),
+        //   z: 1/hz^2 - 2 (wxz + wyz), centre: c6 - 4 (wxy + wxz + wyz),
+        // and only the three edge sums remain: + wxy exy + wxz exz + wyz eyz.
+        const R wxy = (ihx2 + ihy2) / (R)12, wxz = (ihx2 + ihz2) / (R)12, wyz = (ihy2 + ihz2) / (R)12;
+        const R ax = ihx2 - (R)2 * (wxy + wxz), ay = ihy2 - (R)2 * (wxy + wyz), az = ihz2 - (R)2 * (wxz + wyz);
+        const R c19 = c6 - (R)4 * (wxy + wxz + wyz);
+        CT eyz[4], t4[4];
+        m.get(f(6), eyz);
+#pragma unroll
+        for (int k = 7; k < 10; ++k) {
+            m.get(f(k), t4);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) eyz[i] = vadd(eyz[i], t4[i]);
+        }
+        const CT yml = *m.last(f(10)), ymr = *m.first(f(11)), ypl = *m.last(f(12)), ypr = *m.first(f(13));
+        const CT zml = *m.last(f(14)), zmr = *m.first(f(15)), zpl = *m.last(f(16)), zpr = *m.first(f(17));
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const CT l = i == 0 ? xm : c[i - 1];
+            const CT rr = i == 3 ? xp : c[i + 1];
+            const CT exy = vadd(vadd(i == 0 ? yml : ym[i - 1], i == 3 ? ymr : ym[i + 1]),
+                                vadd(i == 0 ? ypl : yp[i - 1], i == 3 ? ypr : yp[i + 1]));
+            const CT exz = vadd(vadd(i == 0 ? zml : zm[i - 1], i == 3 ? zmr : zm[i + 1]),
+                                vadd(i == 0 ? zpl : zp[i - 1], i == 3 ? zpr : zp[i + 1]));
+            L[i] = edgev(lapv(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], ax, ay, az, c19), exy, exz, eyz[i], wxy, wxz,
+                         wyz);
+        }
+    }
+}
+
+// Bring n bytes (a multiple of 16) from p into L2, by one thread
+__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t n)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(n) : "memory");
+}
+
+// Run body(idx, pre, c, L) over every segment of the tiles blockIdx.x,
+// blockIdx.x + gridDim.x, ...: idx its first cell's packed index, pre what
+// load(idx) returned, c[4] its values and L[4] their Laplacians, from src after
+// xf(value, packed index).  Called once by the whole block of TILE threads.
+// Everything of a tile is in flight before anything is waited for: a thread
+// loads its own segment, its operands, its neighbour slots and its entries of
+// the halo, whose list it holds since the tile before; and one thread has had
+// the tile's runs brought into L2 a tile ahead (prefetch(first cell, cells)
+// adds the operands' runs).  Values go to the shared tile through registers:
+// cp.async into the tile's planes moved 1.3 times the L2 bytes and, with two
+// buffered tiles a block, ran a third slower.
+template <int NP, typename CT, typename R, typename XF, typename PREF, typename LOAD, typename BODY>
+__device__ __forceinline__ void tile_loop(const TileView &T, const CT *src, XF xf, R ihx2, R ihy2, R ihz2,
+                                          PREF prefetch, LOAD load, BODY body)
+{
+    extern __shared__ __align__(16) unsigned char gpe_smem[];
+    using M = TileMem<CT>;
+    constexpr bool PLAIN = std::is_same<XF, Identity>::value;
+    const M m{reinterpret_cast<uint4 *>(gpe_smem), T.pstr};
+    const int tid = threadIdx.x;
+    const uint32_t step = gridDim.x, nt = (uint32_t)T.ntiles;
+    // the list entries of the next tile: two whole segments, one single cell
+    uint32_t cnt = 0, e0 = 0, e1 = 0, es = 0;
+    auto fetch_list = [&](uint32_t tile) {
+        if (tile >= nt) return;
+        const uint32_t *row = T.halo + (size_t)tile * T.stride;
+        cnt = __ldg(row);
+        if (1 + tid < T.stride) {
+            e0 = __ldg(row + 1 + tid);
+            es = __ldg(row + T.stride - 1 - tid);
+        }
+        if (1 + tid + TILE < T.stride) e1 = __ldg(row + 1 + tid + TILE);
+    };
+    auto whole = [&](uint32_t e, CT(&v)[4]) { ld4<false>(src + 4 * (size_t)e, v); };
+    auto put_whole = [&](int t, uint32_t e, CT(&v)[4]) {
+        if constexpr (!PLAIN) xf.seg(v, 4u * e);
+        m.put(TILE + 1 + t, v);
+    };
+    auto cell_of = [](uint32_t e) { return 4u * (e & 0x7fffffffu) + ((e >> 31) ? 0u : 3u); };
+    auto put_cell = [&](int sl, uint32_t e, CT v) {
+        if constexpr (!PLAIN) v = xf(v, cell_of(e));
+        *((e >> 31) ? m.first(sl) : m.last(sl)) = v;
+    };
+    if (tid < M::UPS) m.u[tid * m.p + TILE] = make_uint4(0u, 0u, 0u, 0u);  // the zero slot
+    uint32_t tile = blockIdx.x;
+    fetch_list(tile);
+    for (; tile < nt; tile += step) {
+        const uint32_t seg = tile * TILE + tid, idx = 4u * seg;
+        const bool in = seg < T.nseg;
+        const int nwhole = cnt & 0xffff, nsingle = cnt >> 16;
+        const uint32_t w0 = e0, w1 = e1, s0 = es;
+        CT c[4], h0[4], h1[4], hs = czero<CT>();
+        typename std::decay<decltype(load(0u))>::type pre{};
+        TileSlots<NP> f{};
+        if (in) {
+            ld4<false>(src + idx, c);
+            f.load(T, seg);
+            pre = load(idx);
+        }
+        if (tid < nwhole) whole(w0, h0);
+        if (tid + TILE < nwhole) whole(w1, h1);
+        if (tid < nsingle) hs = src[cell_of(s0)];
+        fetch_list(tile + step);
+        if (tid == 0 && tile + 2 * step < nt) {
+            prefetch_l2(T.halo + (size_t)(tile + 2 * step) * T.stride, T.stride * 4u);
+        }
+        if (tid == 0 && tile + step < nt) {
+            const uint32_t s1 = (tile + step) * TILE, own = min((uint32_t)TILE, T.nseg - s1) & ~1u;
+            if (own > 0) {
+                prefetch_l2(src + 4 * (size_t)s1, own * 4u * (uint32_t)sizeof(CT));
+                if constexpr (NP == 19) prefetch_l2(T.nbr19 + 2 * (size_t)s1, own * 32u);
+                else prefetch_l2(T.nbr + s1, own * 8u);
+                prefetch(4u * s1, own * 4u);
+            }
+        }
+        __syncthreads();  // the previous tile has been read
+        if (in) {
+            if constexpr (!PLAIN) xf.seg(c, idx);
+            m.put(tid, c);
+        }
+        if (tid < nwhole) put_whole(tid, w0, h0);
+        if (tid + TILE < nwhole) put_whole(tid + TILE, w1, h1);
+        if (tid < nsingle) put_cell(TILE + 1 + nwhole + tid, s0, hs);
+        if (nwhole > 2 * TILE || nsingle > TILE) {  // masks with unusually many halo segments
+            const uint32_t *row = T.halo + (size_t)tile * T.stride;
+            for (int t = tid + 2 * TILE; t < nwhole; t += TILE) {
+                const uint32_t e = __ldg(row + 1 + t);
+                whole(e, h0);
+                put_whole(t, e, h0);
+            }
+            for (int t = tid + TILE; t < nsingle; t += TILE) {
+                const uint32_t e = __ldg(row + T.stride - 1 - t);
+                put_cell(TILE + 1 + nwhole + t, e, src[cell_of(e)]);
+            }
+        }
+        __syncthreads();
+        if (in) {
+            CT L[4];
+            tile_laplacian<NP>(m, f, c, ihx2, ihy2, ihz2, L);
+            body(idx, pre, c, L);
+        }
+    }
+}
+
+// ------------------------------------------------------------ launches
+// a grid's tiles for values of type CT, and the shared memory of a block
+struct TileLaunch {
+    TileView T;
+    size_t smem;
+};
+template <typename CT>
+inline TileLaunch tile_launch(const gpe_grid *g)
+{
+    const TileTab &t = g->tiles;
+    const int pstr = TileMem<CT>::pstr(t.nslot);
+    return {TileView{t.d_nbr, t.d_nbr19, t.d_halo, t.nseg, t.ntiles, t.stride, pstr},
+            16 * (size_t)(TileMem<CT>::UPS * pstr)};
+}
+
+// resident blocks an SM of a tile kernel with smem bytes of shared memory;
+// the kernel may use as much as a block can have, so that grids of different
+// halo sizes can launch it from any thread
+int tile_per_sm(const void *kernel, size_t smem);
+// blocks of a launch over n tiles: one a tile, or with `loop` at most the
+// resident ones (kernels that reduce, or that loop over tiles)
+template <typename K>
+inline unsigned tile_blocks(K kernel, int nsm, int n, size_t smem)
+{
+    const int64_t res = (int64_t)nsm * tile_per_sm((const void *)kernel, smem);
+    return (unsigned)(res < n ? res : n);
+}
+
+// blocks an SM: registers of 85 (single) and 168 (double) a thread
+#define GPE_TILE_BOUNDS(R) __launch_bounds__(TILE, sizeof(R) == 4 ? 6 : 3)
+
+// One RK4 stage.  1024^3 shell, 8x8x4 bricks, per step of four: complex64
+// 0.776 -> 0.626 ms (4.0 GB, of which 0.4 GB slots and halo lists: 6.5 TB/s,
+// 0.95 of the copy bandwidth, so bytes bound it now); complex128 8.65 ->
+// 6.75 ms (FP64 issue: full lanes instead of four fifths).  Six blocks an SM
+// (85 registers): 0.626 ms, seven 0.634, eight with spills 0.645; double:
+// three 6.75, four 6.98, five 7.1.  One block a tile instead of looping
+// blocks: 8 % slower (no tile ahead to prefetch).
+template <typename R, bool BLEND, int ST, int NP>
+__global__ void GPE_TILE_BOUNDS(R) k_rk4_tile(const RkArgs<R> a, const TileView T)
+{
+    using CT = typename Cx<R>::T;
+    using B = Rk4Body<R, BLEND, false, ST>;
+    const B body(a, stage_s<R, BLEND>(a, ST));
+    tile_loop<NP>(T, body.yin(), Identity(), a.ihx2, a.ihy2, a.ihz2,
+                  [&](uint32_t idx, uint32_t n) {
+                      prefetch_l2(a.V0 + idx, n * (uint32_t)sizeof(R));
+                      if constexpr (BLEND) prefetch_l2(a.V1 + idx, n * (uint32_t)sizeof(R));
+                      if constexpr (ST > 0) prefetch_l2((ST == 3 ? a.w : a.y0) + idx, n * (uint32_t)sizeof(CT));
+                  },
+                  [&](uint32_t idx) { return body.load(idx); }, body);
+}
+
+// the four stage kernels, static (blend false) or blended
+template <typename R, int NP>
+struct Rk4Tiles {
+    using K = void (*)(RkArgs<R>, TileView);
+    static K get(bool blend, int st)
+    {
+        static const K t[2][4] = {{k_rk4_tile<R, false, 0, NP>, k_rk4_tile<R, false, 1, NP>,
+                                   k_rk4_tile<R, false, 2, NP>, k_rk4_tile<R, false, 3, NP>},
+                                  {k_rk4_tile<R, true, 0, NP>, k_rk4_tile<R, true, 1, NP>,
+                                   k_rk4_tile<R, true, 2, NP>, k_rk4_tile<R, true, 3, NP>}};
+        return t[blend ? 1 : 0][st];
+    }
+};
+
+}  // namespace gpe

@@ -1,0 +1,128 @@
+"""The tiles of the stencil kernels (runs of 128 stored segments with halo
+lists) on masks that the shells do not give: isolated cells, half of all
+cells, stripes whose every neighbour lies in another tile, fewer segments than
+a tile, exactly one tile, one more; every brick shape, both stencils, every
+state type.  Against the FP64 oracle: RK4 and imaginary-time steps and the
+observables at the parity tolerances (1e-12 in FP64; a handful of FP32
+roundings a step: 2e-6)."""
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+from gpu_cases import rel_l2
+from paper_2603_05447_gb300 import gpe, inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+BRICKS = [(8, 8, 8), (8, 8, 4), (8, 4, 4)]
+NPT = {gpe.GPE_C128: np.complex128, gpe.GPE_C64: np.complex64, gpe.GPE_R64: np.float64, gpe.GPE_R32: np.float32}
+
+
+def mask_of(kind):
+    rng = np.random.default_rng(11)
+    if kind == "sparse":
+        return rng.uniform(size=(37, 41, 83)) < 0.02
+    if kind == "half":
+        return rng.uniform(size=(21, 33, 45)) < 0.5
+    if kind == "stripes":       # one segment of every second column, all rows and planes
+        m = np.zeros((40, 48, 64), bool)
+        m[:, :, 1::8] = True
+        m[::3, 1::2, 6::16] = True
+        return m
+    if kind == "few":           # fewer segments than a tile
+        m = np.zeros((9, 10, 21), bool)
+        m[2:5, 3:7, 2:19] = True
+        return m
+    m = np.zeros((8, 8, 24), bool)
+    m[:, :, :8] = True          # 128 segments: one tile of an 8x8x8 brick
+    if kind == "one more":
+        m[3, 4, 8] = True
+    return m
+
+
+MASKS = ["sparse", "half", "stripes", "few", "one tile", "one more"]
+
+
+class Setup:
+    def __init__(self, kind, dtype, brick, stencil):
+        self.m = mask_of(kind)
+        nz, ny, nx = self.m.shape
+        self.h = (0.11, 0.1, 0.12)
+        rng = np.random.default_rng(12)
+        self.V = np.where(self.m, rng.uniform(0.0, 4.0, self.m.shape), 10.0)
+        psi = np.where(self.m, rng.normal(size=self.m.shape) + 1j * rng.normal(size=self.m.shape), 0)
+        if dtype in (gpe.GPE_R64, gpe.GPE_R32):
+            psi = np.abs(psi) + 0j
+        dV = math.prod(self.h)
+        self.psi = inputs.normalise(psi, dV).astype(NPT[dtype] if dtype in (gpe.GPE_C128, gpe.GPE_C64) else complex)
+        self.psi = self.psi.astype(np.complex128)
+        self.og = oracle.Grid(self.m, self.h)
+        self.g, self.dtype, self.stencil = 3.0, dtype, stencil
+        lam = sum(2.0 / h ** 2 for h in self.h) + 10.0
+        self.dt = 0.2 / lam
+        self.grid = gpe.gpe_grid_create_dense(gpe.make_box(nx, ny, nz, *self.h), self.V, 5.0,
+                                              gpe.make_opts(brick, stencil=stencil))
+        self.st = gpe.gpe_state_create(self.grid, dtype)
+        arr = self.psi.real if dtype in (gpe.GPE_R64, gpe.GPE_R32) else self.psi
+        gpe.gpe_state_load(self.st, np.ascontiguousarray(arr.astype(NPT[dtype])), gpe.GPE_LAYOUT_DENSE)
+        self.tol = 1e-12 if dtype in (gpe.GPE_C128, gpe.GPE_R64) else 2e-6
+
+    def __enter__(self):
+        return self
+
+    def __exit__(self, *a):
+        gpe.gpe_state_destroy(self.st)
+        gpe.gpe_grid_destroy(self.grid)
+
+    def dense(self):
+        out = np.zeros(self.m.shape, NPT[self.dtype])
+        gpe.gpe_state_store(self.st, out, gpe.GPE_LAYOUT_DENSE)
+        return out.astype(np.complex128)
+
+
+@pytest.mark.parametrize("stencil", [7, 19])
+@pytest.mark.parametrize("brick", BRICKS)
+@pytest.mark.parametrize("dtype", [gpe.GPE_C128, gpe.GPE_C64])
+@pytest.mark.parametrize("kind", MASKS)
+def test_rk4_on_odd_masks(kind, dtype, brick, stencil):
+    with Setup(kind, dtype, brick, stencil) as S:
+        V = S.og.compact(S.V)
+        y = S.og.compact(S.dense())
+        for _ in range(2):
+            y = oracle.rk_step_np(S.og, V, y, S.g, 0.0, S.dt, stencil=stencil)
+        gpe.gpe_step_real(S.st, gpe.real_params(S.g, S.dt), 2)
+        assert rel_l2(S.og.compact(S.dense()), y) <= S.tol
+
+
+@pytest.mark.parametrize("stencil", [7, 19])
+@pytest.mark.parametrize("brick", BRICKS)
+@pytest.mark.parametrize("dtype", [gpe.GPE_C128, gpe.GPE_C64, gpe.GPE_R64, gpe.GPE_R32])
+@pytest.mark.parametrize("kind", MASKS)
+def test_imaginary_time_and_observables_on_odd_masks(kind, dtype, brick, stencil):
+    with Setup(kind, dtype, brick, stencil) as S:
+        V = S.og.compact(S.V)
+        y = S.og.compact(S.dense())
+        for _ in range(2):
+            y, _ = oracle.itp_step_np(S.og, V, y, S.g, S.dt, stencil=stencil)
+        gpe.gpe_step_imag(S.st, gpe.gpe_imag_params(S.g, S.dt, 1.0), 2)
+        got = S.og.compact(S.dense())
+        assert rel_l2(got, y) <= S.tol
+        o, ref = gpe.gpe_observables(S.st, S.g), oracle.observables_np(S.og, V, S.g, got, stencil=stencil)
+        for k in ("norm", "energy", "mu", "e_kin", "e_pot", "e_int"):
+            assert abs(o[k] - ref[k]) <= S.tol * max(abs(ref[k]), abs(ref["energy"])), k
+
+
+@pytest.mark.parametrize("integrator", ["RKHE3", "RKCK"])
+@pytest.mark.parametrize("dtype", [gpe.GPE_C128, gpe.GPE_C64])
+@pytest.mark.parametrize("kind", ["sparse", "half", "one more"])
+def test_general_integrators_on_odd_masks(kind, dtype, integrator):
+    with Setup(kind, dtype, (8, 8, 4), 7) as S:
+        V = S.og.compact(S.V)
+        y = S.og.compact(S.dense())
+        for _ in range(2):
+            y = oracle.rk_step_np(S.og, V, y, S.g, 0.0, S.dt, method=integrator)
+        gpe.gpe_step_real(S.st, gpe.real_params(S.g, S.dt, integrator=getattr(gpe, "GPE_" + integrator)), 2)
+        assert rel_l2(S.og.compact(S.dense()), y) <= S.tol
