@@ -299,12 +299,6 @@ struct TileTab {
 }  // namespace gpe
 
 // ------------------------------------------------------------ handles
-// launch the staged stage kernels with programmatic dependent launch (off:
-// measured no gain for RK4 and a slower imaginary-time step on GB300)
-#ifndef GPE_PDL
-#define GPE_PDL 0
-#endif
-
 struct gpe_grid {
     int device = 0;
     gpe_box box{};
@@ -364,7 +358,6 @@ struct gpe_state {
     unsigned long long ticket_base = 0, finish_base = 0;
     // CUDA graphs of `graph_steps` staged steps ([0] real time, [1] imaginary)
     int graph_steps = 32;
-    bool pdl = GPE_PDL != 0;  // stage kernels launched with programmatic dependent launch
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};
     unsigned long long gkey[2] = {0, 0};
     int gnodes[2] = {0, 0};

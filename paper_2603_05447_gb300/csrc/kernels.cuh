@@ -4,7 +4,7 @@
 // part of the ABI.
 #pragma once
 
-#include "stencil.cuh"
+#include "tiles.cuh"
 
 namespace gpe {
 
@@ -100,32 +100,114 @@ __device__ __forceinline__ void itp_brick_b(const ItpArgs<R, CT> &a, const GridV
     });
 }
 
-template <typename R, int BX, int BY, int BZ, typename CT = typename Cx<R>::T, int NP = 7>
-__global__ void GPE_BOUNDS_NP(R) k_itp_a(const ItpArgs<R, CT> a, const GridView G)
+// The staged passes, on tiles (tiles.cuh).  A halo segment's propagator is
+// loaded beside its values, an own segment's serves its transform and its
+// update.  1024^3 shell, complex64: 0.382 -> 0.275 ms a step against the
+// former warp-per-brick passes (1.3 GB, 4.7 TB/s); bound by the shared-memory
+// pipe (86 and 80 % busy at 512^3).
+template <typename R, typename CT>
+struct TileDiag {
+    DiagLoad<R, CT> d;
+    struct P4 {
+        R e[4];
+    };
+    using P1 = R;
+    __device__ __forceinline__ P4 load4(uint32_t idx) const
+    {
+        P4 p;
+        ldr4(d.E + idx, p.e);
+        return p;
+    }
+    __device__ __forceinline__ R load1(uint32_t idx) const { return __ldg(d.E + idx); }
+    __device__ __forceinline__ void seg(CT (&v)[4], const P4 &p) const
+    {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = d.apply(v[i], p.e[i]);
+    }
+    __device__ __forceinline__ void own(CT (&v)[4], const typename ELoad<R>::P &p) const
+    {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = d.apply(v[i], p.e[i]);
+    }
+    __device__ __forceinline__ void cell(CT &v, const R &e) const { v = d.apply(v, e); }
+};
+
+// An FP64 sum of many single-precision terms off the FP64 pipe, where an add
+// and a conversion issue at 1/64 of the FP32 rate: the terms are added as an
+// unevaluated pair of floats (hi + lo, each addition's rounding error found
+// exactly by Knuth's two-sum and kept in lo, which itself stays good to
+// 2^-24 of 2^-24), and the pair goes into the FP64 total every FLUSH terms.
+// Double-precision terms are added as they are.
+template <typename R>
+struct Sum64 {
+    double tot = 0.0;
+    __device__ __forceinline__ void add(double x) { tot += x; }
+    __device__ __forceinline__ void flush() {}
+};
+template <>
+struct Sum64<float> {
+    double tot = 0.0;
+    float hi = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ void add(float x)
+    {
+        const float s = __fadd_rn(hi, x), b = __fadd_rn(s, -hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -b)), __fadd_rn(x, -b)));
+        hi = s;
+    }
+    __device__ __forceinline__ void flush()
+    {
+        tot += (double)hi;
+        if (isfinite(lo)) tot += (double)lo;  // an infinite or NaN term shows in hi
+        hi = 0.0f;
+        lo = 0.0f;
+    }
+};
+constexpr int SUM_FLUSH = 16;
+
+template <typename R, typename CT, int NP>
+__global__ void GPE_TILE_BOUNDS(R) k_itp_a(const ItpArgs<R, CT> a, const TileView T)
 {
-    pdl_enter();
-    constexpr int NW = KernelCfg<R>::NW;
-    auto &ws = warp_space<R, BX, BY, BZ, CT, NP>();
-    const int warp = threadIdx.x >> 5;
-    const R sc = (R)a.scalars[0];
-    const int64_t stride = (int64_t)gridDim.x * NW;
-    for (int64_t b = (int64_t)blockIdx.x * NW + warp; b < G.nb; b += stride)
-        itp_brick_a<R, CT, BX, BY, BZ, false, NP>(a, G, b, b + stride < G.nb ? b + stride : -1, ws, sc);
+    const R q4 = a.dt / (R)4;
+    const TileDiag<R, CT> diag{{(R)a.scalars[0], a.g * a.dt / (R)2, a.E}};
+    tile_loop<NP>(T, (const CT *)a.psi, diag, a.ihx2, a.ihy2, a.ihz2,
+                  [&](uint32_t idx, uint32_t n) { prefetch_l2(a.E + idx, n * (uint32_t)sizeof(R)); }, ELoad<R>{a.E},
+                  [&](uint32_t idx, const typename ELoad<R>::P &p, const CT(&c)[4], const CT(&L)[4]) {
+                      CT o[4];
+#pragma unroll
+                      for (int i = 0; i < 4; ++i) {
+                          const bool act = p.e[i] >= (R)0;  // E < 0 marks an inactive cell of a stored segment
+                          o[i] = act ? axpy(c[i], q4, L[i]) : czero<CT>();
+                      }
+                      st4(a.tmp + idx, o);
+                  });
 }
 
-template <typename R, int BX, int BY, int BZ, typename CT = typename Cx<R>::T, int NP = 7>
-__global__ void GPE_BOUNDS_NP(R) k_itp_b(const ItpArgs<R, CT> a, const GridView G, double *partials,
-                                          unsigned int *counter)
+template <typename R, typename CT, int NP>
+__global__ void GPE_TILE_BOUNDS(R) k_itp_b(const ItpArgs<R, CT> a, const TileView T, double *partials,
+                                           unsigned int *counter)
 {
-    pdl_enter();
-    constexpr int NW = KernelCfg<R>::NW;
-    auto &ws = warp_space<R, BX, BY, BZ, CT, NP>();
-    const int warp = threadIdx.x >> 5;
-    double acc[1] = {0.0};
-    const int64_t stride = (int64_t)gridDim.x * NW;
-    for (int64_t b = (int64_t)blockIdx.x * NW + warp; b < G.nb; b += stride)
-        itp_brick_b<R, CT, BX, BY, BZ, false, NP>(a, G, b, b + stride < G.nb ? b + stride : -1, ws, acc[0]);
-    double tot[1];
+    const R hg = a.g * a.dt / (R)2;
+    const R q4 = a.dt / (R)4;
+    Sum64<R> norm;
+    int n = 0;
+    tile_loop<NP>(T, (const CT *)a.tmp, Plain(), a.ihx2, a.ihy2, a.ihz2,
+                  [&](uint32_t idx, uint32_t n) { prefetch_l2(a.E + idx, n * (uint32_t)sizeof(R)); }, ELoad<R>{a.E},
+                  [&](uint32_t idx, const typename ELoad<R>::P &p, const CT(&c)[4], const CT(&L)[4]) {
+                      CT o[4];
+                      R n4 = (R)0;  // the segment's |psi|^2, added to the FP64 sum once
+#pragma unroll
+                      for (int i = 0; i < 4; ++i) {
+                          o[i] = axpy(c[i], q4, L[i]);
+                          const R f = p.e[i] >= (R)0 ? p.e[i] * ((R)1 - hg * norm2(o[i])) : (R)0;
+                          o[i] = scale(o[i], f);
+                          n4 = add_rn(n4, norm2(o[i]));
+                      }
+                      st4(a.psi + idx, o);
+                      norm.add(n4);
+                      if (++n % SUM_FLUSH == 0) norm.flush();
+                  });
+    norm.flush();
+    double acc[1] = {norm.tot}, tot[1];
     if (reduce_finish<1>(acc, partials, counter, tot) && threadIdx.x == 0) {
         const double nrm = tot[0] * a.dV;
         a.scalars[0] = sqrt(a.N / nrm);
@@ -159,40 +241,62 @@ struct ObsArgs {
     gpe_obs *out;
 };
 
-template <typename R, int BX, int BY, int BZ, typename CT = typename Cx<R>::T, int NP = 7>
-__global__ void GPE_BOUNDS_NP(R) k_obs(const ObsArgs<R, CT> a, const GridView G)
-{
-    constexpr int NW = KernelCfg<R>::NW;
-    auto &ws = warp_space<R, BX, BY, BZ, CT, NP>();
-    const int warp = threadIdx.x >> 5;
-    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};  // norm, ekin, epot, eint, nonfinite
-    const int64_t stride = (int64_t)gridDim.x * NW;
-    for (int64_t b = (int64_t)blockIdx.x * NW + warp; b < G.nb; b += stride) {
-        brick_apply<BX, BY, BZ, false>(ws, G, b, b + stride < G.nb ? b + stride : -1, a.psi, Identity(), a.ihx2, a.ihy2, a.ihz2,
-                                       [&](uint32_t idx, const CT(&c)[4], const CT(&L)[4]) {
-            R V0[4], V1[4];
-            ldr4(a.V0 + idx, V0);
-            if (a.V1) ldr4(a.V1 + idx, V1);
-            // the segment's four terms summed in the state precision, then
-            // added to the FP64 sums once (one FP64 add per segment and term)
-            R t[4] = {(R)0, (R)0, (R)0, (R)0};
-            int nf = 0;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                if (!(V0[i] < (R)INFINITY)) continue;
-                const R V = a.V1 ? ((R)1 - a.s) * V0[i] + a.s * V1[i] : V0[i];
-                const R rho = norm2(c[i]);
-                t[0] = add_rn(t[0], rho);
-                t[1] = add_rn(t[1], (R)(-0.5) * dotre(c[i], L[i]));
-                t[2] = add_rn(t[2], V * rho);
-                t[3] = add_rn(t[3], (R)0.5 * a.g * rho * rho);
-                nf += finite_v(c[i]) ? 0 : 1;
-            }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) acc[k] += (double)t[k];
-            acc[4] += (double)nf;
-        });
+// a segment's potential(s), loaded ahead of its terms
+template <typename R>
+struct VLoad {
+    const R *V0, *V1;
+    struct P {
+        R V0[4], V1[4];
+    };
+    __device__ __forceinline__ P operator()(uint32_t idx) const
+    {
+        P p;
+        ldr4(V0 + idx, p.V0);
+        if (V1) ldr4(V1 + idx, p.V1);
+        return p;
     }
+};
+
+template <typename R, typename CT, int NP>
+__global__ void GPE_TILE_BOUNDS(R) k_obs(const ObsArgs<R, CT> a, const TileView T)
+{
+    Sum64<R> sum[4];  // norm, ekin, epot, eint
+    int n = 0, nf = 0;
+    tile_loop<NP>(T, a.psi, Plain(), a.ihx2, a.ihy2, a.ihz2,
+                  [&](uint32_t idx, uint32_t n) {
+                      prefetch_l2(a.V0 + idx, n * (uint32_t)sizeof(R));
+                      if (a.V1) prefetch_l2(a.V1 + idx, n * (uint32_t)sizeof(R));
+                  },
+                  VLoad<R>{a.V0, a.V1},
+                  [&](uint32_t, const typename VLoad<R>::P &p, const CT(&c)[4], const CT(&L)[4]) {
+                      // the segment's four terms summed in the state precision, then
+                      // added to the FP64 sums once
+                      R t[4] = {(R)0, (R)0, (R)0, (R)0};
+#pragma unroll
+                      for (int i = 0; i < 4; ++i) {
+                          if (!(p.V0[i] < (R)INFINITY)) continue;
+                          const R V = a.V1 ? ((R)1 - a.s) * p.V0[i] + a.s * p.V1[i] : p.V0[i];
+                          const R rho = norm2(c[i]);
+                          t[0] = add_rn(t[0], rho);
+                          t[1] = add_rn(t[1], (R)(-0.5) * dotre(c[i], L[i]));
+                          t[2] = add_rn(t[2], V * rho);
+                          t[3] = add_rn(t[3], (R)0.5 * a.g * rho * rho);
+                          nf += finite_v(c[i]) ? 0 : 1;
+                      }
+#pragma unroll
+                      for (int k = 0; k < 4; ++k) sum[k].add(t[k]);
+                      if (++n % SUM_FLUSH == 0) {
+#pragma unroll
+                          for (int k = 0; k < 4; ++k) sum[k].flush();
+                      }
+                  });
+    double acc[5];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        sum[k].flush();
+        acc[k] = sum[k].tot;
+    }
+    acc[4] = (double)nf;
     double tot[5];
     if (reduce_finish<5>(acc, a.partials, a.counter, tot) && threadIdx.x == 0) {
         gpe_obs o;
@@ -205,6 +309,142 @@ __global__ void GPE_BOUNDS_NP(R) k_obs(const ObsArgs<R, CT> a, const GridView G)
         o.nonfinite = tot[4];
         *a.out = o;
     }
+}
+
+// ------------------------------------------------------------ drivers
+__global__ inline void k_set_one(double *p) { *p = 1.0; }
+
+// arguments of the imaginary-time passes of a state; makes the propagator
+// table if dt changed, and sets the pending factor to 1
+template <typename R, typename CT>
+inline int itp_args(gpe_state *st, const gpe_imag_params *p, cudaStream_t s, ItpArgs<R, CT> &a)
+{
+    const gpe_grid *g = st->grid;
+    if (st->E_dt != p->dt) {
+        k_make_E<R><<<g->nsm * 8, 256, 0, s>>>(g->d_V[0], (R *)st->d_E, g->n_packed, p->dt);
+        GPE_LAUNCH_CHECK();
+        st->E_dt = p->dt;
+    }
+    a = ItpArgs<R, CT>{};
+    a.psi = (CT *)st->d_psi;
+    a.tmp = (CT *)st->d_work[0];
+    a.E = (const R *)st->d_E;
+    a.ihx2 = (R)(1.0 / (g->box.hx * g->box.hx));
+    a.ihy2 = (R)(1.0 / (g->box.hy * g->box.hy));
+    a.ihz2 = (R)(1.0 / (g->box.hz * g->box.hz));
+    a.g = (R)p->g;
+    a.dt = (R)p->dt;
+    a.scalars = st->red.scalars;
+    a.N = p->N;
+    a.dV = g->box.hx * g->box.hy * g->box.hz;
+    k_set_one<<<1, 1, 0, s>>>(st->red.scalars);
+    GPE_LAUNCH_CHECK();
+    return GPE_OK;
+}
+
+// cnt imaginary-time steps of two staged passes
+template <typename R, typename CT, int NP>
+inline int itp_steps(gpe_state *st, const ItpArgs<R, CT> &a, int64_t cnt, cudaStream_t s)
+{
+    const gpe_grid *g = st->grid;
+    const TileLaunch L = tile_launch<CT>(g);
+    auto ka = k_itp_a<R, CT, NP>;
+    auto kb = k_itp_b<R, CT, NP>;
+    const unsigned nba = tile_blocks(ka, g->nsm, L.T.ntiles, L.smem), nbb = tile_blocks(kb, g->nsm, L.T.ntiles, L.smem);
+    for (int64_t n = 0; n < cnt; ++n) {
+        ka<<<nba, TILE, L.smem, s>>>(a, L.T);
+        GPE_LAUNCH_CHECK();
+        kb<<<nbb, TILE, L.smem, s>>>(a, L.T, st->red.partials, st->red.counter);
+        GPE_LAUNCH_CHECK();
+    }
+    return GPE_OK;
+}
+
+template <typename CT>
+inline int itp_end(gpe_state *st, cudaStream_t s)
+{
+    const gpe_grid *g = st->grid;
+    k_apply_scale<CT><<<g->nsm * 8, 256, 0, s>>>((CT *)st->d_psi, g->n_packed, st->red.scalars);
+    GPE_LAUNCH_CHECK();
+    return GPE_OK;
+}
+
+template <typename R, typename CT, int NP>
+inline int obs_run(const gpe_state *stc, double gg, double sb, cudaStream_t s)
+{
+    gpe_state *st = const_cast<gpe_state *>(stc);
+    const gpe_grid *g = st->grid;
+    ObsArgs<R, CT> a{};
+    a.psi = (const CT *)st->d_psi;
+    a.V0 = (const R *)potential_ptr(st, 0);
+    a.V1 = (sb != 0.0) ? (const R *)potential_ptr(st, 1) : nullptr;
+    if (sb != 0.0 && !a.V1) return fail(GPE_ERR_ARG, "s_blend != 0 needs potential slot 1");
+    a.s = (R)sb;
+    a.ihx2 = (R)(1.0 / (g->box.hx * g->box.hx));
+    a.ihy2 = (R)(1.0 / (g->box.hy * g->box.hy));
+    a.ihz2 = (R)(1.0 / (g->box.hz * g->box.hz));
+    a.g = (R)gg;
+    a.dV = g->box.hx * g->box.hy * g->box.hz;
+    a.partials = st->red.partials;
+    a.counter = st->red.counter;
+    a.out = (gpe_obs *)(st->red.scalars + 2);
+    const TileLaunch L = tile_launch<CT>(g);
+    auto k = k_obs<R, CT, NP>;
+    k<<<tile_blocks(k, g->nsm, L.T.ntiles, L.smem), TILE, L.smem, s>>>(a, L.T);
+    GPE_LAUNCH_CHECK();
+    return GPE_OK;
+}
+
+// arguments of the RK4 stages of a state (ramps: the clock is set to t0)
+template <typename R>
+inline int rk4_args(gpe_state *st, const gpe_real_params *p, RkArgs<R> &a)
+{
+    using CT = typename Cx<R>::T;
+    const gpe_grid *g = st->grid;
+    const bool blend = p->potential == GPE_V_BLEND;
+    a = RkArgs<R>{};
+    a.V0 = (const R *)potential_ptr(st, 0);
+    a.V1 = blend ? (const R *)potential_ptr(st, 1) : nullptr;
+    if (!a.V0 || (blend && !a.V1)) return fail(GPE_ERR_STATE, "potential slot missing");
+    a.y0 = (CT *)st->d_psi;
+    a.y2 = (CT *)st->d_work[0];
+    a.y3 = (CT *)st->d_work[1];
+    a.y4 = (CT *)st->d_work[0];  // y2 is dead once stage 1 is done
+    a.w = (CT *)st->d_work[2];
+    a.ihx2 = (R)(1.0 / (g->box.hx * g->box.hx));
+    a.ihy2 = (R)(1.0 / (g->box.hy * g->box.hy));
+    a.ihz2 = (R)(1.0 / (g->box.hz * g->box.hz));
+    a.g = (R)p->g;
+    a.dt = (R)p->dt;
+    a.dtd = p->dt;
+    a.ramp.clock = st->d_clock;
+    a.ramp.T = p->T_ramp;
+    a.ramp.n_knots = p->n_knots;
+    for (int k = 0; k < GPE_MAX_KNOTS; ++k) a.ramp.knots[k] = p->knots[k];
+    return GPE_OK;
+}
+
+// cnt RK4 steps of four staged passes, stage times relative to the clock
+template <typename R, int NP>
+inline int rk4_steps(gpe_state *st, RkArgs<R> a, bool blend, int64_t cnt, cudaStream_t s)
+{
+    const gpe_grid *g = st->grid;
+    using RT = Rk4Tiles<R, NP>;
+    const TileLaunch L = tile_launch<typename Cx<R>::T>(g);
+    typename RT::K k[4];
+    unsigned nblk[4];
+    for (int stg = 0; stg < 4; ++stg) {
+        k[stg] = RT::get(blend, stg);
+        nblk[stg] = tile_blocks(k[stg], g->nsm, L.T.ntiles, L.smem);
+    }
+    for (int64_t n = 0; n < cnt; ++n) {
+        a.t_off = (double)n * a.dtd;
+        for (int stg = 0; stg < 4; ++stg) {
+            k[stg]<<<nblk[stg], TILE, L.smem, s>>>(a, L.T);
+            GPE_LAUNCH_CHECK();
+        }
+    }
+    return GPE_OK;
 }
 
 }  // namespace gpe

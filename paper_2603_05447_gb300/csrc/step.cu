@@ -89,26 +89,6 @@ static int blocks_for(K kernel, const gpe_grid *g, size_t smem)
     return blocks_for_nw(kernel, g, smem, KernelCfg<R>::NW);
 }
 
-// Launch a stage kernel; with pdl, with programmatic stream serialisation so
-// that it can become resident during the previous kernel's tail (the kernel
-// itself waits for that grid before reading its output: pdl_enter).
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_stage(void (*k)(KArgs...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s,
-                                bool pdl, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k, args...);
-}
-
 // ------------------------------------------------------------ wavefront sync
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p)
 {
@@ -800,25 +780,8 @@ static int rk4_run(gpe_state *st, const gpe_real_params *p, int64_t nsteps, doub
     using CT = typename Cx<R>::T;
     const gpe_grid *g = st->grid;
     const bool blend = p->potential == GPE_V_BLEND;
-    RkArgs<R> a{};
-    a.V0 = (const R *)potential_ptr(st, 0);
-    a.V1 = blend ? (const R *)potential_ptr(st, 1) : nullptr;
-    if (!a.V0 || (blend && !a.V1)) return fail(GPE_ERR_STATE, "potential slot missing");
-    a.y0 = (CT *)st->d_psi;
-    a.y2 = (CT *)st->d_work[0];
-    a.y3 = (CT *)st->d_work[1];
-    a.y4 = (CT *)st->d_work[0];  // y2 is dead once stage 1 is done
-    a.w = (CT *)st->d_work[2];
-    a.ihx2 = (R)(1.0 / (g->box.hx * g->box.hx));
-    a.ihy2 = (R)(1.0 / (g->box.hy * g->box.hy));
-    a.ihz2 = (R)(1.0 / (g->box.hz * g->box.hz));
-    a.g = (R)p->g;
-    a.dt = (R)p->dt;
-    a.dtd = p->dt;
-    a.ramp.clock = st->d_clock;
-    a.ramp.T = p->T_ramp;
-    a.ramp.n_knots = p->n_knots;
-    for (int k = 0; k < GPE_MAX_KNOTS; ++k) a.ramp.knots[k] = p->knots[k];
+    RkArgs<R> a;
+    GPE_TRY(rk4_args(st, p, a));
     if (blend) {
         k_set_scalar<<<1, 1, 0, s>>>(st->d_clock, t0);
         GPE_LAUNCH_CHECK();
@@ -905,25 +868,8 @@ static int rk4_run(gpe_state *st, const gpe_real_params *p, int64_t nsteps, doub
         }
         return record(s, left);
     }
-    using RT = Rk4Tiles<R, 7>;
-    typename RT::K k[4];
-    const TileLaunch L = tile_launch<CT>(g);
-    unsigned nblk[4];
-    for (int stg = 0; stg < 4; ++stg) {
-        k[stg] = RT::get(blend, stg);
-        nblk[stg] = tile_blocks(k[stg], g->nsm, L.T.ntiles, L.smem);
-    }
     // steps n0 .. n0+cnt-1 with stage times relative to the device clock
-    auto record = [&](cudaStream_t cs, int64_t cnt) -> int {
-        for (int64_t n = 0; n < cnt; ++n) {
-            a.t_off = (double)n * p->dt;
-            for (int stg = 0; stg < 4; ++stg) {
-                k[stg]<<<nblk[stg], TILE, L.smem, cs>>>(a, L.T);
-                GPE_LAUNCH_CHECK();
-            }
-        }
-        return GPE_OK;
-    };
+    auto record = [&](cudaStream_t cs, int64_t cnt) -> int { return rk4_steps<R, 7>(st, a, blend, cnt, cs); };
     int64_t left = nsteps;
     if (use_graph(st, s, nsteps)) {
         const int G_ = st->graph_steps;
@@ -1120,25 +1066,8 @@ template <typename R, int BX, int BY, int BZ, typename CT = typename Cx<R>::T>
 static int itp_run(gpe_state *st, const gpe_imag_params *p, int64_t nsteps, cudaStream_t s)
 {
     const gpe_grid *g = st->grid;
-    if (st->E_dt != p->dt) {
-        k_make_E<R><<<g->nsm * 8, 256, 0, s>>>(g->d_V[0], (R *)st->d_E, g->n_packed, p->dt);
-        GPE_LAUNCH_CHECK();
-        st->E_dt = p->dt;
-    }
-    ItpArgs<R, CT> a{};
-    a.psi = (CT *)st->d_psi;
-    a.tmp = (CT *)st->d_work[0];
-    a.E = (const R *)st->d_E;
-    a.ihx2 = (R)(1.0 / (g->box.hx * g->box.hx));
-    a.ihy2 = (R)(1.0 / (g->box.hy * g->box.hy));
-    a.ihz2 = (R)(1.0 / (g->box.hz * g->box.hz));
-    a.g = (R)p->g;
-    a.dt = (R)p->dt;
-    a.scalars = st->red.scalars;
-    a.N = p->N;
-    a.dV = g->box.hx * g->box.hy * g->box.hz;
-    k_set_scalar<<<1, 1, 0, s>>>(st->red.scalars, 1.0);
-    GPE_LAUNCH_CHECK();
+    ItpArgs<R, CT> a;
+    GPE_TRY(itp_args(st, p, s, a));
     const GridView G = view(g);
     const int th = KernelCfg<R>::THREADS;
     const size_t smem = smem_bytes<R, BX, BY, BZ, CT>();
@@ -1152,9 +1081,7 @@ static int itp_run(gpe_state *st, const gpe_imag_params *p, int64_t nsteps, cuda
             GPE_LAUNCH_CHECK();
             advance_wave(st, 2, nblk, true);
         }
-        k_apply_scale<CT><<<g->nsm * 8, 256, 0, s>>>((CT *)st->d_psi, g->n_packed, st->red.scalars);
-        GPE_LAUNCH_CHECK();
-        return GPE_OK;
+        return itp_end<CT>(st, s);
     }
     if constexpr (is_cplx<CT>()) if (g->sched == GPE_SCHED_PAIR) {
         // one pass per step; the state alternates between the psi buffer and
@@ -1189,24 +1116,10 @@ static int itp_run(gpe_state *st, const gpe_imag_params *p, int64_t nsteps, cuda
             left = nsteps % G_;
         }
         GPE_TRY(record(s, left));
-        k_apply_scale<CT><<<g->nsm * 8, 256, 0, s>>>((CT *)st->d_psi, g->n_packed, st->red.scalars);
-        GPE_LAUNCH_CHECK();
-        return GPE_OK;
+        return itp_end<CT>(st, s);
     }
     {
-        auto ka = k_itp_a<R, BX, BY, BZ, CT>;
-        auto kb = k_itp_b<R, BX, BY, BZ, CT>;
-        const int nba = blocks_for<R>(ka, g, smem), nbb = blocks_for<R>(kb, g, smem);
-        auto record = [&](cudaStream_t cs, int64_t cnt) -> int {
-            for (int64_t n = 0; n < cnt; ++n) {
-                GPE_TRY_CUDA(launch_stage(ka, (unsigned)nba, th, smem, cs, st->pdl && n > 0, a, G));
-                GPE_LAUNCH_CHECK();
-                GPE_TRY_CUDA(launch_stage(kb, (unsigned)nbb, th, smem, cs, st->pdl, a, G, st->red.partials,
-                                          st->red.counter));
-                GPE_LAUNCH_CHECK();
-            }
-            return GPE_OK;
-        };
+        auto record = [&](cudaStream_t cs, int64_t cnt) -> int { return itp_steps<R, CT, 7>(st, a, cnt, cs); };
         int64_t left = nsteps;
         if (use_graph(st, s, nsteps)) {
             const int G_ = st->graph_steps;
@@ -1218,35 +1131,7 @@ static int itp_run(gpe_state *st, const gpe_imag_params *p, int64_t nsteps, cuda
         }
         GPE_TRY(record(s, left));
     }
-    k_apply_scale<CT><<<g->nsm * 8, 256, 0, s>>>((CT *)st->d_psi, g->n_packed, st->red.scalars);
-    GPE_LAUNCH_CHECK();
-    return GPE_OK;
-}
-
-template <typename R, int BX, int BY, int BZ, typename CT = typename Cx<R>::T>
-static int obs_run(const gpe_state *stc, double gg, double sb, cudaStream_t s)
-{
-    gpe_state *st = const_cast<gpe_state *>(stc);
-    const gpe_grid *g = st->grid;
-    ObsArgs<R, CT> a{};
-    a.psi = (const CT *)st->d_psi;
-    a.V0 = (const R *)potential_ptr(st, 0);
-    a.V1 = (sb != 0.0) ? (const R *)potential_ptr(st, 1) : nullptr;
-    if (sb != 0.0 && !a.V1) return fail(GPE_ERR_ARG, "s_blend != 0 needs potential slot 1");
-    a.s = (R)sb;
-    a.ihx2 = (R)(1.0 / (g->box.hx * g->box.hx));
-    a.ihy2 = (R)(1.0 / (g->box.hy * g->box.hy));
-    a.ihz2 = (R)(1.0 / (g->box.hz * g->box.hz));
-    a.g = (R)gg;
-    a.dV = g->box.hx * g->box.hy * g->box.hz;
-    a.partials = st->red.partials;
-    a.counter = st->red.counter;
-    a.out = (gpe_obs *)(st->red.scalars + 2);
-    const size_t smem = smem_bytes<R, BX, BY, BZ, CT>();
-    auto k = k_obs<R, BX, BY, BZ, CT>;
-    k<<<blocks_for<R>(k, g, smem), KernelCfg<R>::THREADS, smem, s>>>(a, view(g));
-    GPE_LAUNCH_CHECK();
-    return GPE_OK;
+    return itp_end<CT>(st, s);
 }
 
 // dense <-> packed copy in the state's value type
@@ -1581,21 +1466,16 @@ extern "C" int gpe_observables(const gpe_state *st, double g, double s_blend, gp
     cudaStream_t s = S(stream);
     const int dt_ = st->dtype;
     int rc = GPE_ERR_STATE;
-#define OBS_CASE(id, X, Y, Z)                                                         \
-    case id:                                                                          \
-        switch (dt_) {                                                                \
-        case GPE_C128: rc = obs_run<double, X, Y, Z>(st, g, s_blend, s); break;       \
-        case GPE_C64: rc = obs_run<float, X, Y, Z>(st, g, s_blend, s); break;         \
-        case GPE_R64: rc = obs_run<double, X, Y, Z, double>(st, g, s_blend, s); break; \
-        default: rc = obs_run<float, X, Y, Z, float>(st, g, s_blend, s); break;       \
-        }                                                                             \
-        break;
     if (st->grid->stencil == 19) {
         rc = obs_run19(st, g, s_blend, s);
     } else {
-        switch (st->grid->shape) { GPE_SHAPES(OBS_CASE) }
+        switch (dt_) {
+        case GPE_C128: rc = obs_run<double, double2, 7>(st, g, s_blend, s); break;
+        case GPE_C64: rc = obs_run<float, float2, 7>(st, g, s_blend, s); break;
+        case GPE_R64: rc = obs_run<double, double, 7>(st, g, s_blend, s); break;
+        default: rc = obs_run<float, float, 7>(st, g, s_blend, s); break;
+        }
     }
-#undef OBS_CASE
     if (rc != GPE_OK) return rc;
     GPE_TRY_CUDA(cudaMemcpyAsync(st->h_obs, st->red.scalars + 2, sizeof(gpe_obs), cudaMemcpyDeviceToHost, s));
     GPE_TRY_CUDA(cudaStreamSynchronize(s));

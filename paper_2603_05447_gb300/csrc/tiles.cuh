@@ -21,7 +21,6 @@
 
 #include "stencil.cuh"
 
-
 namespace gpe {
 
 // neighbour fields of a segment: 0-3 its -y +y -z +z segments, 4 and 5 the
@@ -176,10 +175,23 @@ __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t n)
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(n) : "memory");
 }
 
+// A transform of the values as they are loaded: none, or one whose operands
+// (for a segment or for one cell) are loaded beside the values
+struct Plain {
+    struct P4 {};
+    struct P1 {};
+    __device__ __forceinline__ P4 load4(uint32_t) const { return {}; }
+    __device__ __forceinline__ P1 load1(uint32_t) const { return {}; }
+    template <typename CT>
+    __device__ __forceinline__ void seg(CT (&)[4], const P4 &) const {}
+    template <typename CT>
+    __device__ __forceinline__ void cell(CT &, const P1 &) const {}
+};
+
 // Run body(idx, pre, c, L) over every segment of the tiles blockIdx.x,
 // blockIdx.x + gridDim.x, ...: idx its first cell's packed index, pre what
-// load(idx) returned, c[4] its values and L[4] their Laplacians, from src after
-// xf(value, packed index).  Called once by the whole block of TILE threads.
+// load(idx) returned, c[4] its values and L[4] their Laplacians, of src
+// transformed by xf.  Called once by the whole block of TILE threads.
 // Everything of a tile is in flight before anything is waited for: a thread
 // loads its own segment, its operands, its neighbour slots and its entries of
 // the halo, whose list it holds since the tile before; and one thread has had
@@ -188,12 +200,11 @@ __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t n)
 // cp.async into the tile's planes moved 1.3 times the L2 bytes and, with two
 // buffered tiles a block, ran a third slower.
 template <int NP, typename CT, typename R, typename XF, typename PREF, typename LOAD, typename BODY>
-__device__ __forceinline__ void tile_loop(const TileView &T, const CT *src, XF xf, R ihx2, R ihy2, R ihz2,
-                                          PREF prefetch, LOAD load, BODY body)
+__device__ __forceinline__ void tile_loop(const TileView &T, const CT *src, const XF &xf, const R &ihx2, const R &ihy2,
+                                          const R &ihz2, PREF prefetch, LOAD load, BODY body)
 {
     extern __shared__ __align__(16) unsigned char gpe_smem[];
     using M = TileMem<CT>;
-    constexpr bool PLAIN = std::is_same<XF, Identity>::value;
     const M m{reinterpret_cast<uint4 *>(gpe_smem), T.pstr};
     const int tid = threadIdx.x;
     const uint32_t step = gridDim.x, nt = (uint32_t)T.ntiles;
@@ -209,16 +220,8 @@ __device__ __forceinline__ void tile_loop(const TileView &T, const CT *src, XF x
         }
         if (1 + tid + TILE < T.stride) e1 = __ldg(row + 1 + tid + TILE);
     };
-    auto whole = [&](uint32_t e, CT(&v)[4]) { ld4<false>(src + 4 * (size_t)e, v); };
-    auto put_whole = [&](int t, uint32_t e, CT(&v)[4]) {
-        if constexpr (!PLAIN) xf.seg(v, 4u * e);
-        m.put(TILE + 1 + t, v);
-    };
     auto cell_of = [](uint32_t e) { return 4u * (e & 0x7fffffffu) + ((e >> 31) ? 0u : 3u); };
-    auto put_cell = [&](int sl, uint32_t e, CT v) {
-        if constexpr (!PLAIN) v = xf(v, cell_of(e));
-        *((e >> 31) ? m.first(sl) : m.last(sl)) = v;
-    };
+    auto cell_at = [&](int sl, uint32_t e) -> CT & { return *((e >> 31) ? m.first(sl) : m.last(sl)); };
     if (tid < M::UPS) m.u[tid * m.p + TILE] = make_uint4(0u, 0u, 0u, 0u);  // the zero slot
     uint32_t tile = blockIdx.x;
     fetch_list(tile);
@@ -229,15 +232,26 @@ __device__ __forceinline__ void tile_loop(const TileView &T, const CT *src, XF x
         const uint32_t w0 = e0, w1 = e1, s0 = es;
         CT c[4], h0[4], h1[4], hs = czero<CT>();
         typename std::decay<decltype(load(0u))>::type pre{};
+        typename XF::P4 x0{}, x1{};
+        typename XF::P1 xs{};
         TileSlots<NP> f{};
         if (in) {
             ld4<false>(src + idx, c);
             f.load(T, seg);
             pre = load(idx);
         }
-        if (tid < nwhole) whole(w0, h0);
-        if (tid + TILE < nwhole) whole(w1, h1);
-        if (tid < nsingle) hs = src[cell_of(s0)];
+        if (tid < nwhole) {
+            ld4<false>(src + 4 * (size_t)w0, h0);
+            x0 = xf.load4(4u * w0);
+        }
+        if (tid + TILE < nwhole) {
+            ld4<false>(src + 4 * (size_t)w1, h1);
+            x1 = xf.load4(4u * w1);
+        }
+        if (tid < nsingle) {
+            hs = src[cell_of(s0)];
+            xs = xf.load1(cell_of(s0));
+        }
         fetch_list(tile + step);
         if (tid == 0 && tile + 2 * step < nt) {
             prefetch_l2(T.halo + (size_t)(tile + 2 * step) * T.stride, T.stride * 4u);
@@ -253,22 +267,34 @@ __device__ __forceinline__ void tile_loop(const TileView &T, const CT *src, XF x
         }
         __syncthreads();  // the previous tile has been read
         if (in) {
-            if constexpr (!PLAIN) xf.seg(c, idx);
+            if constexpr (!std::is_same<XF, Plain>::value) xf.own(c, pre);  // the own operands serve the transform
             m.put(tid, c);
         }
-        if (tid < nwhole) put_whole(tid, w0, h0);
-        if (tid + TILE < nwhole) put_whole(tid + TILE, w1, h1);
-        if (tid < nsingle) put_cell(TILE + 1 + nwhole + tid, s0, hs);
+        if (tid < nwhole) {
+            xf.seg(h0, x0);
+            m.put(TILE + 1 + tid, h0);
+        }
+        if (tid + TILE < nwhole) {
+            xf.seg(h1, x1);
+            m.put(2 * TILE + 1 + tid, h1);
+        }
+        if (tid < nsingle) {
+            xf.cell(hs, xs);
+            cell_at(TILE + 1 + nwhole + tid, s0) = hs;
+        }
         if (nwhole > 2 * TILE || nsingle > TILE) {  // masks with unusually many halo segments
             const uint32_t *row = T.halo + (size_t)tile * T.stride;
             for (int t = tid + 2 * TILE; t < nwhole; t += TILE) {
                 const uint32_t e = __ldg(row + 1 + t);
-                whole(e, h0);
-                put_whole(t, e, h0);
+                ld4<false>(src + 4 * (size_t)e, h0);
+                xf.seg(h0, xf.load4(4u * e));
+                m.put(TILE + 1 + t, h0);
             }
             for (int t = tid + TILE; t < nsingle; t += TILE) {
                 const uint32_t e = __ldg(row + T.stride - 1 - t);
-                put_cell(TILE + 1 + nwhole + t, e, src[cell_of(e)]);
+                hs = src[cell_of(e)];
+                xf.cell(hs, xf.load1(cell_of(e)));
+                cell_at(TILE + 1 + nwhole + t, e) = hs;
             }
         }
         __syncthreads();
@@ -324,7 +350,7 @@ __global__ void GPE_TILE_BOUNDS(R) k_rk4_tile(const RkArgs<R> a, const TileView 
     using CT = typename Cx<R>::T;
     using B = Rk4Body<R, BLEND, false, ST>;
     const B body(a, stage_s<R, BLEND>(a, ST));
-    tile_loop<NP>(T, body.yin(), Identity(), a.ihx2, a.ihy2, a.ihz2,
+    tile_loop<NP>(T, body.yin(), Plain(), a.ihx2, a.ihy2, a.ihz2,
                   [&](uint32_t idx, uint32_t n) {
                       prefetch_l2(a.V0 + idx, n * (uint32_t)sizeof(R));
                       if constexpr (BLEND) prefetch_l2(a.V1 + idx, n * (uint32_t)sizeof(R));
