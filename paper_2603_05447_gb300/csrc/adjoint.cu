@@ -27,7 +27,7 @@
 #include <vector>
 
 #include "gpe_internal.cuh"
-#include "stencil.cuh"
+#include "kernels.cuh"
 
 namespace gpe {
 
@@ -45,7 +45,6 @@ struct AdjArgs {
     const R *V1;
     R s;              // schedule value at the stage time
     R cl, cn;
-    int first, last;
     R ihx2, ihy2, ihz2, g;
     double *partials;
     unsigned int *counter;
@@ -54,77 +53,100 @@ struct AdjArgs {
     double w0, w1;    // hat weights of knots k0, k0+1 at the stage time
 };
 
+// mu_i = m_scale lam' at the first stage of the reverse sweep
 template <typename R>
-struct Scale {
+struct TileScale {
     R s;
+    using P4 = Plain::P4;
+    using P1 = Plain::P1;
+    __device__ __forceinline__ P4 load4(uint32_t) const { return {}; }
+    __device__ __forceinline__ P1 load1(uint32_t) const { return {}; }
     template <typename CT>
-    __device__ __forceinline__ CT operator()(CT v, uint32_t) const
+    __device__ __forceinline__ void seg(CT (&v)[4], const P4 &) const
     {
-        v.x *= s;
-        v.y *= s;
-        return v;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = scale(v[i], s);
     }
+    template <typename CT, typename PRE>
+    __device__ __forceinline__ void own(CT (&v)[4], const PRE &) const { seg(v, P4{}); }
+    template <typename CT>
+    __device__ __forceinline__ void cell(CT &v, const P1 &) const { v = scale(v, s); }
 };
 
-template <typename R, int BX, int BY, int BZ, bool BLEND>
-__global__ void GPE_BOUNDS(R) k_adj_stage(const AdjArgs<R> a, const GridView G)
+// POS: 0 the first of the four stages (mu_i is lam' scaled, nothing is
+// accumulated yet), 1 the middle ones, 2 the last (writes lam).  All own-cell
+// operands are loaded with the tile; they were the pass's latency when they
+// were read once the tile was in place.  512^3 ramp, complex64: 70 -> 42, 55
+// and 45 us a stage (5.1 to 5.9 TB/s), bound by bytes in flight: the operands'
+// registers leave five blocks an SM.
+template <typename R, int POS>
+__global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? 5 : 2) k_adj_stage(const AdjArgs<R> a, const TileView T)
 {
     using CT = typename Cx<R>::T;
-    constexpr int NW = KernelCfg<R>::NW;
-    auto &ws = warp_space<R, BX, BY, BZ>();
-    const int warp = threadIdx.x >> 5;
-    double dot[1] = {0.0};
-    const int64_t stride = (int64_t)gridDim.x * NW;
-    for (int64_t b = (int64_t)blockIdx.x * NW + warp; b < G.nb; b += stride) {
-        brick_apply<BX, BY, BZ, false>(ws, G, b, b + stride < G.nb ? b + stride : -1, a.mu_in, Scale<R>{a.m_scale}, a.ihx2, a.ihy2, a.ihz2,
-                                       [&](uint32_t idx, const CT(&M)[4], const CT(&L)[4]) {
-            R V0[4], V1[4];
-            CT Y[4], lam[4], acc[4];
-            ldr4(a.V0 + idx, V0);
-            if (BLEND) ldr4(a.V1 + idx, V1);
-            ld4<false>(a.Y + idx, Y);
-            ld4<false>(a.lam + idx, lam);
-            if (!a.first) ld4<false>(a.acc + idx, acc);
-            CT nacc[4], mo[4];
-            R d4 = (R)0;  // the segment's share of the knot derivative, added in FP64 once
+    using XF = typename std::conditional<POS == 0, TileScale<R>, Plain>::type;
+    struct Pre {
+        R V0[4], V1[4];
+        CT Y[4], lam[4], acc[4];
+    };
+    XF xf{};
+    if constexpr (POS == 0) xf.s = a.m_scale;
+    Sum64<R> dot;
+    int n = 0;
+    tile_loop<7>(T, a.mu_in, xf, a.ihx2, a.ihy2, a.ihz2, EveryTile(),
+                 [&](uint32_t idx, uint32_t m) {
+                     prefetch_l2(a.V0 + idx, m * (uint32_t)sizeof(R));
+                     prefetch_l2(a.V1 + idx, m * (uint32_t)sizeof(R));
+                     prefetch_l2(a.Y + idx, m * (uint32_t)sizeof(CT));
+                     if constexpr (POS != 0) prefetch_l2(a.acc + idx, m * (uint32_t)sizeof(CT));
+                     if constexpr (POS == 1) prefetch_l2(a.lam + idx, m * (uint32_t)sizeof(CT));
+                 },
+                 [&](uint32_t idx) {
+                     Pre p;
+                     ldr4(a.V0 + idx, p.V0);
+                     ldr4(a.V1 + idx, p.V1);
+                     ld4<false>(a.Y + idx, p.Y);
+                     if constexpr (POS != 2) ld4<false>(a.lam + idx, p.lam);
+                     if constexpr (POS != 0) ld4<false>(a.acc + idx, p.acc);
+                     return p;
+                 },
+                 [&](uint32_t idx, const Pre &p, const CT(&M)[4], const CT(&L)[4]) {
+                     CT nacc[4], mo[4];
+                     R d4 = (R)0;  // the segment's share of the knot derivative, added in FP64 once
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                if (!(V0[i] < (R)INFINITY)) {  // inactive cell of a stored segment
-                    nacc[i] = czero<CT>();
-                    mo[i] = czero<CT>();
-                    continue;
-                }
-                const R dV = BLEND ? V1[i] - V0[i] : (R)0;
-                const R Vt = BLEND ? ((R)1 - a.s) * V0[i] + a.s * V1[i] : V0[i];
-                const R rho = Y[i].x * Y[i].x + Y[i].y * Y[i].y;
-                // C = (T + Vt + 2 g rho) M - g Y^2 conj(M);  nu = i C
-                const R w = Vt + (R)2 * a.g * rho;
-                const R y2r = Y[i].x * Y[i].x - Y[i].y * Y[i].y, y2i = (R)2 * Y[i].x * Y[i].y;
-                const R br = y2r * M[i].x + y2i * M[i].y;   // Re(Y^2 conj(M))
-                const R bi = y2i * M[i].x - y2r * M[i].y;   // Im(Y^2 conj(M))
-                const R cr = (R)(-0.5) * L[i].x + w * M[i].x - a.g * br;
-                const R ci = (R)(-0.5) * L[i].y + w * M[i].y - a.g * bi;
-                CT nu;
-                nu.x = -ci;
-                nu.y = cr;
-                if (BLEND) d4 += dV * (M[i].x * Y[i].y - M[i].y * Y[i].x);
-                const CT base = a.first ? lam[i] : acc[i];
-                nacc[i].x = base.x + nu.x;
-                nacc[i].y = base.y + nu.y;
-                mo[i].x = a.cl * lam[i].x + a.cn * nu.x;
-                mo[i].y = a.cl * lam[i].y + a.cn * nu.y;
-            }
-            if (BLEND) dot[0] += (double)d4;
-            if (a.last) {
-                st4(a.lam_out + idx, nacc);
-            } else {
-                st4(a.acc + idx, nacc);
-                st4(a.mu_out + idx, mo);
-            }
-        });
-    }
-    double tot[1];
-    if (reduce_finish<1>(dot, a.partials, a.counter, tot) && threadIdx.x == 0 && BLEND) {
+                     for (int i = 0; i < 4; ++i) {
+                         const bool act = p.V0[i] < (R)INFINITY;  // else an inactive cell of a stored segment
+                         const CT Y = p.Y[i];
+                         const R dV = p.V1[i] - p.V0[i];
+                         const R Vt = ((R)1 - a.s) * p.V0[i] + a.s * p.V1[i];
+                         const R rho = Y.x * Y.x + Y.y * Y.y;
+                         // C = (T + Vt + 2 g rho) M - g Y^2 conj(M);  nu = i C
+                         const R w = Vt + (R)2 * a.g * rho;
+                         const R y2r = Y.x * Y.x - Y.y * Y.y, y2i = (R)2 * Y.x * Y.y;
+                         const R br = y2r * M[i].x + y2i * M[i].y;  // Re(Y^2 conj(M))
+                         const R bi = y2i * M[i].x - y2r * M[i].y;  // Im(Y^2 conj(M))
+                         const R cr = (R)(-0.5) * L[i].x + w * M[i].x - a.g * br;
+                         const R ci = (R)(-0.5) * L[i].y + w * M[i].y - a.g * bi;
+                         const CT nu = act ? cmk<R>(-ci, cr) : czero<CT>();
+                         if (act) d4 += dV * (M[i].x * Y.y - M[i].y * Y.x);
+                         if constexpr (POS == 0) nacc[i] = vadd(p.lam[i], nu);
+                         else nacc[i] = vadd(p.acc[i], nu);
+                         if constexpr (POS != 2) {
+                             mo[i].x = a.cl * p.lam[i].x + a.cn * nu.x;
+                             mo[i].y = a.cl * p.lam[i].y + a.cn * nu.y;
+                         }
+                     }
+                     if constexpr (POS == 2) {
+                         st4(a.lam_out + idx, nacc);
+                     } else {
+                         st4(a.acc + idx, nacc);
+                         st4(a.mu_out + idx, mo);
+                     }
+                     dot.add(d4);
+                     if (++n % SUM_FLUSH == 0) dot.flush();
+                 });
+    dot.flush();
+    double acc[1] = {dot.tot}, tot[1];
+    if (reduce_finish<1>(acc, a.partials, a.counter, tot) && threadIdx.x == 0) {
         a.grad[a.k0] += a.w0 * tot[0];
         a.grad[a.k0 + 1] += a.w1 * tot[0];
     }
@@ -192,7 +214,7 @@ struct gpe_tape {
     double t0 = 0.0;
     int K = 0;
     void *d_ckpt = nullptr;  // [nck * n_packed]
-    void *d_seg = nullptr;   // [K * n_packed]
+    void *d_seg = nullptr;   // [K * n_packed] step-start states of a segment after the first
     void *d_lam = nullptr, *d_mu[2] = {nullptr, nullptr}, *d_acc = nullptr;
     void *d_w[4] = {nullptr, nullptr, nullptr, nullptr};  // Y2, Y3, Y4, RK4 partial sum
     double *d_grad = nullptr;
@@ -277,15 +299,7 @@ extern "C" int gpe_ramp_forward(gpe_state *st, const gpe_real_params *p, int64_t
 
 namespace gpe {
 
-template <typename R, typename K>
-static int adj_blocks(K kernel, const gpe_grid *g, size_t smem, int nw = KernelCfg<R>::NW)
-{
-    const int per = prepare_kernel(kernel, 32 * nw, smem);
-    const int64_t need = (g->nb + nw - 1) / nw;
-    return (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)g->nsm * per, need));
-}
-
-template <typename R, int BX, int BY, int BZ>
+template <typename R>
 static int backward_impl(gpe_tape *t, const gpe_state *target, double *grad, double *loss, cudaStream_t s)
 {
     using CT = typename Cx<R>::T;
@@ -293,7 +307,6 @@ static int backward_impl(gpe_tape *t, const gpe_state *target, double *grad, dou
     const gpe_grid *g = st->grid;
     const gpe_real_params &p = t->p;
     const size_t np = (size_t)g->n_packed;
-    const GridView G = view(g);
     // loss and seed
     double c[2];
     GPE_TRY(gpe_overlap(target, st, c, (gpe_stream)s));
@@ -322,17 +335,17 @@ static int backward_impl(gpe_tape *t, const gpe_state *target, double *grad, dou
     f.ramp.T = p.T_ramp;
     f.ramp.n_knots = p.n_knots;
     for (int k = 0; k < GPE_MAX_KNOTS; ++k) f.ramp.knots[k] = p.knots[k];
-    using RS = Rk4Stages<R, BX, BY, BZ>;
-    typename RS::K kf[4];
-    auto ka = k_adj_stage<R, BX, BY, BZ, true>;
-    const size_t smem = smem_bytes<R, BX, BY, BZ>();
-    const int th = KernelCfg<R>::THREADS;
-    int nbf[4];
-    for (int stg = 0; stg < 4; ++stg) {
-        kf[stg] = RS::get(true, stg);
-        nbf[stg] = adj_blocks<R>(kf[stg], g, RS::smem(), RS::NW);
-    }
-    const int nba = adj_blocks<R>(ka, g, smem);
+    using RT = Rk4Tiles<R, 7>;
+    const TileLaunch tl = tile_launch<CT>(g);
+    auto blocks = [&](auto k) { return tile_blocks(k, g->nsm, tl.T.ntiles, tl.smem); };
+    auto stage = [&](int stg) -> int {
+        const auto k = RT::get(true, stg);
+        k<<<blocks(k), TILE, tl.smem, s>>>(f, tl.T);
+        GPE_LAUNCH_CHECK();
+        return GPE_OK;
+    };
+    using KA = void (*)(AdjArgs<R>, TileView);
+    const KA ka[4] = {k_adj_stage<R, 0>, k_adj_stage<R, 1>, k_adj_stage<R, 1>, k_adj_stage<R, 2>};
     AdjArgs<R> a{};
     a.lam = lam;
     a.lam_out = lam;
@@ -350,25 +363,21 @@ static int backward_impl(gpe_tape *t, const gpe_state *target, double *grad, dou
     CT *seg = (CT *)t->d_seg, *ck = (CT *)t->d_ckpt;
     for (int64_t j = t->nck - 1; j >= 0; --j) {
         const int64_t len = std::min<int64_t>(t->K, t->nsteps - j * t->K);
-        GPE_TRY_CUDA(cudaMemcpyAsync(seg, ck + j * np, np * sizeof(CT), cudaMemcpyDeviceToDevice, s));
-        // step-start states of the segment
+        // step-start states of the segment: the checkpoint, then seg[0], seg[1]
+        // ... (stage 3 reads no y0, so it writes the next one where it stays)
+        auto start = [&](int64_t m) { return m == 0 ? ck + j * np : seg + (m - 1) * np; };
         for (int64_t m = 0; m + 1 < len; ++m) {
-            GPE_TRY_CUDA(cudaMemcpyAsync(seg + (m + 1) * np, seg + m * np, np * sizeof(CT), cudaMemcpyDeviceToDevice, s));
-            f.y0 = seg + (m + 1) * np;
+            f.y0 = start(m);
             f.t_off = t->t0 + (double)(j * t->K + m) * p.dt;
-            for (int stg = 0; stg < 4; ++stg) {
-                kf[stg]<<<nbf[stg], RS::THREADS, RS::smem(), s>>>(f, G);
-                GPE_LAUNCH_CHECK();
-            }
+            for (int stg = 0; stg < 3; ++stg) GPE_TRY(stage(stg));
+            f.y0 = start(m + 1);
+            GPE_TRY(stage(3));
         }
         for (int64_t m = len - 1; m >= 0; --m) {
             const double tm = t->t0 + (double)(j * t->K + m) * p.dt;
-            f.y0 = seg + m * np;
+            f.y0 = start(m);
             f.t_off = tm;
-            for (int stg = 0; stg < 3; ++stg) {  // Y2, Y3, Y4
-                kf[stg]<<<nbf[stg], RS::THREADS, RS::smem(), s>>>(f, G);
-                GPE_LAUNCH_CHECK();
-            }
+            for (int stg = 0; stg < 3; ++stg) GPE_TRY(stage(stg));  // Y2, Y3, Y4
             // stages 4, 3, 2, 1 of the reverse sweep
             const double ts[4] = {tm + p.dt, tm + 0.5 * p.dt, tm + 0.5 * p.dt, tm};
             const CT *Ys[4] = {f.y4, f.y3, f.y2, f.y0};
@@ -383,10 +392,8 @@ static int backward_impl(gpe_tape *t, const gpe_state *target, double *grad, dou
                 a.s = (R)ramp_s_host(p, ts[r]);
                 a.cl = cl[r];
                 a.cn = cn[r];
-                a.first = r == 0;
-                a.last = r == 3;
                 hat(p, ts[r], a.k0, a.w0, a.w1);
-                ka<<<nba, th, smem, s>>>(a, G);
+                ka[r]<<<blocks(ka[r]), TILE, tl.smem, s>>>(a, tl.T);
                 GPE_LAUNCH_CHECK();
             }
         }
@@ -408,9 +415,6 @@ extern "C" int gpe_ramp_backward(gpe_tape *t, const gpe_state *target, double *g
         return fail(GPE_ERR_ARG, "target must share the tape state's grid and dtype");
     const bool c128 = t->st->dtype == GPE_C128;
     cudaStream_t s = S(stream);
-#define ADJ_CASE(id, X, Y, Z) \
-    case id: return c128 ? backward_impl<double, X, Y, Z>(t, target, grad_knots, loss, s) : backward_impl<float, X, Y, Z>(t, target, grad_knots, loss, s);
-    switch (t->st->grid->shape) { GPE_SHAPES(ADJ_CASE) }
-#undef ADJ_CASE
-    return fail(GPE_ERR_STATE, "bad brick shape");
+    return c128 ? backward_impl<double>(t, target, grad_knots, loss, s)
+                : backward_impl<float>(t, target, grad_knots, loss, s);
 }

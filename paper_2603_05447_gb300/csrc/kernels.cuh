@@ -169,7 +169,7 @@ __global__ void GPE_TILE_BOUNDS(R) k_itp_a(const ItpArgs<R, CT> a, const TileVie
 {
     const R q4 = a.dt / (R)4;
     const TileDiag<R, CT> diag{{(R)a.scalars[0], a.g * a.dt / (R)2, a.E}};
-    tile_loop<NP>(T, (const CT *)a.psi, diag, a.ihx2, a.ihy2, a.ihz2,
+    tile_loop<NP>(T, (const CT *)a.psi, diag, a.ihx2, a.ihy2, a.ihz2, EveryTile(),
                   [&](uint32_t idx, uint32_t n) { prefetch_l2(a.E + idx, n * (uint32_t)sizeof(R)); }, ELoad<R>{a.E},
                   [&](uint32_t idx, const typename ELoad<R>::P &p, const CT(&c)[4], const CT(&L)[4]) {
                       CT o[4];
@@ -190,7 +190,7 @@ __global__ void GPE_TILE_BOUNDS(R) k_itp_b(const ItpArgs<R, CT> a, const TileVie
     const R q4 = a.dt / (R)4;
     Sum64<R> norm;
     int n = 0;
-    tile_loop<NP>(T, (const CT *)a.tmp, Plain(), a.ihx2, a.ihy2, a.ihz2,
+    tile_loop<NP>(T, (const CT *)a.tmp, Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
                   [&](uint32_t idx, uint32_t n) { prefetch_l2(a.E + idx, n * (uint32_t)sizeof(R)); }, ELoad<R>{a.E},
                   [&](uint32_t idx, const typename ELoad<R>::P &p, const CT(&c)[4], const CT(&L)[4]) {
                       CT o[4];
@@ -262,7 +262,7 @@ __global__ void GPE_TILE_BOUNDS(R) k_obs(const ObsArgs<R, CT> a, const TileView 
 {
     Sum64<R> sum[4];  // norm, ekin, epot, eint
     int n = 0, nf = 0;
-    tile_loop<NP>(T, a.psi, Plain(), a.ihx2, a.ihy2, a.ihz2,
+    tile_loop<NP>(T, a.psi, Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
                   [&](uint32_t idx, uint32_t n) {
                       prefetch_l2(a.V0 + idx, n * (uint32_t)sizeof(R));
                       if (a.V1) prefetch_l2(a.V1 + idx, n * (uint32_t)sizeof(R));

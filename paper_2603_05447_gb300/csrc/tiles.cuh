@@ -188,6 +188,10 @@ struct Plain {
     __device__ __forceinline__ void cell(CT &, const P1 &) const {}
 };
 
+struct EveryTile {
+    __device__ __forceinline__ bool operator()(uint32_t) const { return true; }
+};
+
 // Run body(idx, pre, c, L) over every segment of the tiles blockIdx.x,
 // blockIdx.x + gridDim.x, ...: idx its first cell's packed index, pre what
 // load(idx) returned, c[4] its values and L[4] their Laplacians, of src
@@ -199,9 +203,12 @@ struct Plain {
 // adds the operands' runs).  Values go to the shared tile through registers:
 // cp.async into the tile's planes moved 1.3 times the L2 bytes and, with two
 // buffered tiles a block, ran a third slower.
-template <int NP, typename CT, typename R, typename XF, typename PREF, typename LOAD, typename BODY>
+//
+// setup(tile), uniform over the block, runs before each tile, may change what
+// xf and the inverse square spacings refer to, and says whether to take it.
+template <int NP, typename CT, typename R, typename XF, typename SETUP, typename PREF, typename LOAD, typename BODY>
 __device__ __forceinline__ void tile_loop(const TileView &T, const CT *src, const XF &xf, const R &ihx2, const R &ihy2,
-                                          const R &ihz2, PREF prefetch, LOAD load, BODY body)
+                                          const R &ihz2, SETUP setup, PREF prefetch, LOAD load, BODY body)
 {
     extern __shared__ __align__(16) unsigned char gpe_smem[];
     using M = TileMem<CT>;
@@ -226,6 +233,10 @@ __device__ __forceinline__ void tile_loop(const TileView &T, const CT *src, cons
     uint32_t tile = blockIdx.x;
     fetch_list(tile);
     for (; tile < nt; tile += step) {
+        if (!setup(tile)) {
+            fetch_list(tile + step);
+            continue;
+        }
         const uint32_t seg = tile * TILE + tid, idx = 4u * seg;
         const bool in = seg < T.nseg;
         const int nwhole = cnt & 0xffff, nsingle = cnt >> 16;
@@ -350,7 +361,7 @@ __global__ void GPE_TILE_BOUNDS(R) k_rk4_tile(const RkArgs<R> a, const TileView 
     using CT = typename Cx<R>::T;
     using B = Rk4Body<R, BLEND, false, ST>;
     const B body(a, stage_s<R, BLEND>(a, ST));
-    tile_loop<NP>(T, body.yin(), Plain(), a.ihx2, a.ihy2, a.ihz2,
+    tile_loop<NP>(T, body.yin(), Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
                   [&](uint32_t idx, uint32_t n) {
                       prefetch_l2(a.V0 + idx, n * (uint32_t)sizeof(R));
                       if constexpr (BLEND) prefetch_l2(a.V1 + idx, n * (uint32_t)sizeof(R));
