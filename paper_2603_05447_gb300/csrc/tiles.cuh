@@ -324,12 +324,17 @@ struct TileLaunch {
     size_t smem;
 };
 template <typename CT>
-inline TileLaunch tile_launch(const gpe_grid *g)
+inline TileLaunch tile_launch(const TileTab &t)
 {
-    const TileTab &t = g->tiles;
     const int pstr = TileMem<CT>::pstr(t.nslot);
     return {TileView{t.d_nbr, t.d_nbr19, t.d_halo, t.nseg, t.ntiles, t.stride, pstr},
             16 * (size_t)(TileMem<CT>::UPS * pstr)};
+}
+
+template <typename CT>
+inline TileLaunch tile_launch(const gpe_grid *g)
+{
+    return tile_launch<CT>(g->tiles);
 }
 
 // resident blocks an SM of a tile kernel with smem bytes of shared memory;
