@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? 5 : 2) k_adj_stage(cons
                      R d4 = (R)0;  // the segment's share of the knot derivative, added in FP64 once
 #pragma unroll
                      for (int i = 0; i < 4; ++i) {
-                         const bool act = p.V0[i] < (R)INFINITY;  // else an inactive cell of a stored segment
+                         const bool act = active_v(p.V0[i]);  // else an inactive cell of a stored segment
                          const CT Y = p.Y[i];
                          const R dV = p.V1[i] - p.V0[i];
                          const R Vt = ((R)1 - a.s) * p.V0[i] + a.s * p.V1[i];

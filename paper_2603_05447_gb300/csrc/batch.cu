@@ -161,7 +161,7 @@ __global__ void GPE_TILE_BOUNDS(R) k_batch_itp(const BatchArgs<R, CT> a, const T
         R n4 = (R)0;  // the segment's |psi|^2, added to the FP64 sum once
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const bool act = E[i] >= (R)0;
+            const bool act = active_e(E[i]);
             o[i] = axpy(c[i], q4, L[i]);
             if (STAGE == 1) {
                 const R f = act ? E[i] * ((R)1 - hg * norm2(o[i])) : (R)0;
@@ -231,7 +231,7 @@ __global__ void GPE_TILE_BOUNDS(R) k_batch_obs(const BatchArgs<R, CT> a, const T
                      R t[4] = {(R)0, (R)0, (R)0, (R)0};  // the segment's terms, added to the FP64 sums once
 #pragma unroll
                      for (int i = 0; i < 4; ++i) {
-                         if (!(p.V0[i] < (R)INFINITY)) continue;
+                         if (!active_v(p.V0[i])) continue;
                          const R rho = norm2(c[i]);
                          t[0] = add_rn(t[0], rho);
                          t[1] = add_rn(t[1], (R)(-0.5) * dotre(c[i], L[i]));

@@ -175,8 +175,8 @@ __global__ void GPE_TILE_BOUNDS(R) k_itp_a(const ItpArgs<R, CT> a, const TileVie
                       CT o[4];
 #pragma unroll
                       for (int i = 0; i < 4; ++i) {
-                          const bool act = p.e[i] >= (R)0;  // E < 0 marks an inactive cell of a stored segment
-                          o[i] = act ? axpy(c[i], q4, L[i]) : czero<CT>();
+                          // E < 0 marks an inactive cell of a stored segment
+                          o[i] = active_e(p.e[i]) ? axpy(c[i], q4, L[i]) : czero<CT>();
                       }
                       st4(a.tmp + idx, o);
                   });
@@ -198,7 +198,7 @@ __global__ void GPE_TILE_BOUNDS(R) k_itp_b(const ItpArgs<R, CT> a, const TileVie
 #pragma unroll
                       for (int i = 0; i < 4; ++i) {
                           o[i] = axpy(c[i], q4, L[i]);
-                          const R f = p.e[i] >= (R)0 ? p.e[i] * ((R)1 - hg * norm2(o[i])) : (R)0;
+                          const R f = active_e(p.e[i]) ? p.e[i] * ((R)1 - hg * norm2(o[i])) : (R)0;
                           o[i] = scale(o[i], f);
                           n4 = add_rn(n4, norm2(o[i]));
                       }
@@ -274,7 +274,7 @@ __global__ void GPE_TILE_BOUNDS(R) k_obs(const ObsArgs<R, CT> a, const TileView 
                       R t[4] = {(R)0, (R)0, (R)0, (R)0};
 #pragma unroll
                       for (int i = 0; i < 4; ++i) {
-                          if (!(p.V0[i] < (R)INFINITY)) continue;
+                          if (!active_v(p.V0[i])) continue;
                           const R V = a.V1 ? ((R)1 - a.s) * p.V0[i] + a.s * p.V1[i] : p.V0[i];
                           const R rho = norm2(c[i]);
                           t[0] = add_rn(t[0], rho);

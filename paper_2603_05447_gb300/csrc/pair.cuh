@@ -29,7 +29,7 @@
 // Stage A runs as three task sets: the brick's stored segments, the stored
 // segments of the one-deep z and y face layers, and the single cells of the
 // one-deep x face layers.  The arithmetic per cell is that of the staged
-// kernels (lapv, Rk4Body::compute), so both schedules give identical bits.
+// kernels (LapRhs, Rk4Body::compute), so both schedules give identical bits.
 #pragma once
 
 #include "stencil.cuh"
@@ -247,7 +247,7 @@ __device__ __forceinline__ void pair_fill(PairSpace<CT, BX, BY, BZ> &ps, const P
 
 // The 7-point Laplacian (Eq. (B1)) of the 4 cells of u slot (hx, y, z); the
 // x neighbours at the row ends come from the row's x halo cells
-template <typename CT, int BX, int BY, int BZ, typename R>
+template <typename LAP = LapFull, typename CT, int BX, int BY, int BZ, typename R>
 __device__ __forceinline__ void pair_lap_u(const PairSpace<CT, BX, BY, BZ> &ps, int hx, int y, int z, CT (&c)[4],
                                            CT (&L)[4], R ihx2, R ihy2, R ihz2, R c6)
 {
@@ -266,12 +266,12 @@ __device__ __forceinline__ void pair_lap_u(const PairSpace<CT, BX, BY, BZ> &ps, 
     for (int i = 0; i < 4; ++i) {
         const CT l = i == 0 ? xm : c[i - 1];
         const CT rr = i == 3 ? xp : c[i + 1];
-        L[i] = lapv(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], ihx2, ihy2, ihz2, c6);
+        L[i] = LAP::of(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], LAP::coef(ihx2), LAP::coef(ihy2), LAP::coef(ihz2), c6);
     }
 }
 
 // The same on the v tile (the brick's own slots only)
-template <typename CT, int BX, int BY, int BZ, typename R>
+template <typename LAP = LapFull, typename CT, int BX, int BY, int BZ, typename R>
 __device__ __forceinline__ void pair_lap_v(const PairSpace<CT, BX, BY, BZ> &ps, int hx, int y, int z, CT (&c)[4],
                                            CT (&L)[4], R ihx2, R ihy2, R ihz2, R c6)
 {
@@ -290,7 +290,7 @@ __device__ __forceinline__ void pair_lap_v(const PairSpace<CT, BX, BY, BZ> &ps, 
     for (int i = 0; i < 4; ++i) {
         const CT l = i == 0 ? xm : c[i - 1];
         const CT rr = i == 3 ? xp : c[i + 1];
-        L[i] = lapv(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], ihx2, ihy2, ihz2, c6);
+        L[i] = LAP::of(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], LAP::coef(ihx2), LAP::coef(ihy2), LAP::coef(ihz2), c6);
     }
 }
 
@@ -320,7 +320,8 @@ __device__ __forceinline__ void pair_brick(PairSpace<typename Cx<R>::T, BX, BY, 
     }
     cp_async_wait_all();
     __syncthreads();
-    const BA bodyA(a, sA);
+    const R c3 = rhs_centre(a.ihx2, a.ihy2, a.ihz2);
+    const BA bodyA(a, sA, c3);
     const int nst = ps.nst;
     const BrickRec &R0 = ps.rec[0];
     // stage A on the stored segments of the brick, then of the one-deep z and
@@ -352,7 +353,7 @@ __device__ __forceinline__ void pair_brick(PairSpace<typename Cx<R>::T, BX, BY, 
         if (!ok) continue;
         const typename BA::P pa = bodyA.load(j);
         CT c[4], L[4], o[4], wv[4];
-        pair_lap_u(ps, hx, y, z, c, L, a.ihx2, a.ihy2, a.ihz2, c6);
+        pair_lap_u<LapRhs>(ps, hx, y, z, c, L, a.ihx2, a.ihy2, a.ihz2, c6);
         bodyA.compute(pa, c, L, o, wv);
         ps.vput(PS::vslot(hx, y, z), o);
     }
@@ -391,7 +392,7 @@ __device__ __forceinline__ void pair_brick(PairSpace<typename Cx<R>::T, BX, BY, 
         if constexpr (BLEND) pa.V1[0] = a.V1[j];
         if constexpr (STA == 2) pa.y[0] = a.y0[j];
         CT c[4] = {c0, czero<CT>(), czero<CT>(), czero<CT>()}, L[4], o[4], wv[4];
-        L[0] = lapv(xp, xm, yp, ym, zp, zm, c0, a.ihx2, a.ihy2, a.ihz2, c6);
+        L[0] = LapRhs::of(xp, xm, yp, ym, zp, zm, c0, LapRhs::coef(a.ihx2), LapRhs::coef(a.ihy2), LapRhs::coef(a.ihz2), c6);
         L[1] = L[2] = L[3] = czero<CT>();
         bodyA.compute(pa, c, L, o, wv);
         (side == 0 ? ps.vxl : ps.vxr)[PS::vrow(y, z)] = o[0];
@@ -400,7 +401,7 @@ __device__ __forceinline__ void pair_brick(PairSpace<typename Cx<R>::T, BX, BY, 
     // stage B on the brick's stored segments
     RkArgs<R> ab = a;
     if constexpr (PASS == 1) ab.y0 = y1out;  // stage 3 writes y1 to the other buffer
-    const BB bodyB(ab, sB);
+    const BB bodyB(ab, sB, c3);
     for (int i = t; i < nst; i += PAIR_THREADS) {
         const int q = ps.list[i];
         const int hx = q % SX, y = (q / SX) % BY, z = q / PL;
@@ -411,7 +412,7 @@ __device__ __forceinline__ void pair_brick(PairSpace<typename Cx<R>::T, BX, BY, 
         if constexpr (STB == 1) ps.uget(PS::slot(hx, y, z), pb.y);  // y0 of the cell (u = y0)
         if constexpr (STB == 3) ld4<false>(a.w + j, pb.y);
         CT c[4], L[4];
-        pair_lap_v(ps, hx, y, z, c, L, a.ihx2, a.ihy2, a.ihz2, c6);
+        pair_lap_v<LapRhs>(ps, hx, y, z, c, L, a.ihx2, a.ihy2, a.ihz2, c6);
         bodyB(j, pb, c, L);
     }
     __syncthreads();  // the tiles are reused for the next brick

@@ -279,6 +279,64 @@ __device__ __forceinline__ CT lapv(const CT &xp, const CT &xm, const CT &yp, con
     }
 }
 
+// What a pass wants of a cell's neighbourhood: its Laplacian (LapFull), or, for
+// the right-hand side of the real-time steps, half of it with the sign of the
+// kinetic term (LapRhs).  In double precision LapRhs leaves out the centre's
+// share, (1/hx^2 + 1/hy^2 + 1/hz^2) c, which the caller adds to the potential
+// for one addition a cell: with the factor -1/2 in the coefficients that saves
+// four of 23 FP64 instructions a cell and stage, and FP64 instructions are
+// what bounds the complex128 steps.  In single precision, bound by bytes, it
+// is the Laplacian as it is.
+// Whether a cell is active, from its potential (+inf, or NaN, marks the inactive
+// cells of stored segments) or its propagator (negative there).  Double values
+// are tested by their high words: an FP64 comparison costs as much as an FP64
+// multiplication.
+__device__ __forceinline__ bool active_v(float V) { return V < INFINITY; }
+__device__ __forceinline__ bool active_v(double V)
+{
+    const int hi = __double2hiint(V);
+    return (hi & 0x7fffffff) < 0x7ff00000 || (hi == (int)0xfff00000 && __double2loint(V) == 0);  // finite or -inf
+}
+__device__ __forceinline__ bool active_e(float E) { return E >= 0.0f; }
+__device__ __forceinline__ bool active_e(double E) { return __double2hiint(E) >= 0; }
+
+struct LapFull {
+    template <typename R>
+    __device__ __forceinline__ static R coef(R a)
+    {
+        return a;
+    }
+    template <typename CT, typename R>
+    __device__ __forceinline__ static CT of(const CT &xp, const CT &xm, const CT &yp, const CT &ym, const CT &zp,
+                                            const CT &zm, const CT &c, R ax, R ay, R az, R c6)
+    {
+        return lapv(xp, xm, yp, ym, zp, zm, c, ax, ay, az, c6);
+    }
+};
+struct LapRhs {
+    __device__ __forceinline__ static float coef(float a) { return a; }
+    __device__ __forceinline__ static double coef(double a) { return -0.5 * a; }
+    __device__ __forceinline__ static float2 of(const float2 &xp, const float2 &xm, const float2 &yp, const float2 &ym,
+                                                const float2 &zp, const float2 &zm, const float2 &c, float ax,
+                                                float ay, float az, float c6)
+    {
+        return lapv(xp, xm, yp, ym, zp, zm, c, ax, ay, az, c6);
+    }
+    // ax, ay, az already through coef()
+    __device__ __forceinline__ static double2 of(const double2 &xp, const double2 &xm, const double2 &yp,
+                                                 const double2 &ym, const double2 &zp, const double2 &zm,
+                                                 const double2 &, double ax, double ay, double az, double)
+    {
+        double2 n;
+        n.x = __fma_rn(az, zp.x + zm.x, __fma_rn(ay, yp.x + ym.x, ax * (xp.x + xm.x)));
+        n.y = __fma_rn(az, zp.y + zm.y, __fma_rn(ay, yp.y + ym.y, ax * (xp.y + xm.y)));
+        return n;
+    }
+};
+// the centre's share that LapRhs leaves to the caller
+__device__ __forceinline__ float rhs_centre(float, float, float) { return 0.0f; }
+__device__ __forceinline__ double rhs_centre(double ihx2, double ihy2, double ihz2) { return ihx2 + ihy2 + ihz2; }
+
 __device__ __forceinline__ float2 shfl_up(float2 v, int d)
 {
     v.x = __shfl_up_sync(0xffffffffu, v.x, d);
@@ -607,7 +665,7 @@ struct NoPre {
 // stores coalesce.  The first 32 segments' operands are loaded while the tile
 // is in flight, the next 32's while a group is computed.  With xf the identity the tile is filled by cp.async;
 // otherwise through registers, where xf is applied.
-template <int BX, int BY, int BZ, bool CG, typename CT, int NP, typename R, typename XF, typename LOAD, typename BODY>
+template <int BX, int BY, int BZ, bool CG, typename LAP = LapFull, typename CT, int NP, typename R, typename XF, typename LOAD, typename BODY>
 __device__ __forceinline__ void brick_apply(WarpSpace<CT, BX, BY, BZ, NP> &ws, const GridView &G, int64_t b,
                                             int64_t next, const CT *src, XF xf, R ihx2, R ihy2, R ihz2, LOAD load,
                                             BODY body)
@@ -793,7 +851,7 @@ __device__ __forceinline__ void brick_apply(WarpSpace<CT, BX, BY, BZ, NP> &ws, c
             for (int i = 0; i < 4; ++i) {
                 const CT l = i == 0 ? xm : c[i - 1];
                 const CT rr = i == 3 ? xp : c[i + 1];
-                L[i] = lapv(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], ihx2, ihy2, ihz2, c6);
+                L[i] = LAP::of(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], LAP::coef(ihx2), LAP::coef(ihy2), LAP::coef(ihz2), c6);
             }
         } else {
             // App. B: the 7-point part plus w_ab (edges_ab - 2 faces_ab + 4 c)
@@ -903,7 +961,7 @@ struct DiagLoad {
     __device__ __forceinline__ CT apply(CT v, R e) const
     {
         v = scale(v, sc);
-        const R f = e >= (R)0 ? e * ((R)1 - hg * norm2(v)) : (R)0;
+        const R f = active_e(e) ? e * ((R)1 - hg * norm2(v)) : (R)0;
         return scale(v, f);
     }
     __device__ __forceinline__ CT operator()(CT v, uint32_t idx) const { return apply(v, __ldg(E + idx)); }
@@ -982,13 +1040,6 @@ __device__ __forceinline__ float div3(float x)
     const float q = __fmul_rn(x, t);
     return __fmaf_rn(__fmaf_rn(-3.0f, q, x), t, q);
 }
-__device__ __forceinline__ double div3(double x)
-{
-    constexpr double t = 1.0 / 3.0;
-    const double q = __dmul_rn(x, t);
-    return __fma_rn(__fma_rn(-3.0, q, x), t, q);
-}
-
 // One RK4 stage (st = 0..3): operand loads and the per-segment update.  The
 // stage is a template argument so that each stage keeps only its own
 // prefetched operands in registers.
@@ -1001,10 +1052,11 @@ struct Rk4Body {
         CT y[4];  // y0 (stages 1, 2) or w (stage 3)
     };
     const RkArgs<R> &a;
-    R s, k;
+    R s, k, c3;
     CT *yout;
-    __device__ __forceinline__ Rk4Body(const RkArgs<R> &a_, R s_)
-        : a(a_), s(s_), k(st == 2 ? a_.dt : (st == 3 ? a_.dt / (R)6 : a_.dt / (R)2)),
+    // c3_: the centre's share of the right-hand side (rhs_centre)
+    __device__ __forceinline__ Rk4Body(const RkArgs<R> &a_, R s_, R c3_)
+        : a(a_), s(s_), k(st == 2 ? a_.dt : (st == 3 ? a_.dt / (R)6 : a_.dt / (R)2)), c3(c3_),
           yout(st == 0 ? a_.y2 : st == 1 ? a_.y3 : st == 2 ? a_.y4 : a_.y0)
     {
     }
@@ -1055,16 +1107,12 @@ struct Rk4Body {
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            if (!(p.V0[i] < (R)INFINITY)) {  // inactive cell of a stored segment
-                o[i] = czero<CT>();
-                wv[i] = czero<CT>();
-                continue;
-            }
             R V = p.V0[i];
             if constexpr (BLEND) V = ((R)1 - s) * p.V0[i] + s * p.V1[i];
-            const R w = V + a.g * (c[i].x * c[i].x + c[i].y * c[i].y);
-            const R hr = (R)(-0.5) * L[i].x + w * c[i].x;
-            const R hi = (R)(-0.5) * L[i].y + w * c[i].y;
+            // L is the neighbours' share of -1/2 lap; the centre's is in w
+            const R w = (V + a.g * (c[i].x * c[i].x + c[i].y * c[i].y)) + c3;
+            const R hr = L[i].x + w * c[i].x;
+            const R hi = L[i].y + w * c[i].y;
             // f = -i (hr + i hi) = hi - i hr
             if constexpr (st == 0) {
                 o[i].x = c[i].x + k * hi;
@@ -1077,8 +1125,17 @@ struct Rk4Body {
                     wv[i].y = -p.y[i].y + c[i].y + (R)2 * o[i].y;
                 }
             } else {
-                o[i].x = div3(p.y[i].x + c[i].x) + k * hi;
-                o[i].y = div3(p.y[i].y + c[i].y) - k * hr;
+                // x/3 + k f with the third in two parts: T + TL is 1/3 to 2^-108,
+                // so the sum is rounded once (a third rounded to T alone would
+                // shrink every step by 2^-54)
+                constexpr double T = 1.0 / 3.0, TL = 1.850371707708594e-17;
+                const R xr = p.y[i].x + c[i].x, xi = p.y[i].y + c[i].y;
+                o[i].x = __fma_rn(T, xr, __fma_rn(k, hi, TL * xr));
+                o[i].y = __fma_rn(T, xi, __fma_rn(-k, hr, TL * xi));
+            }
+            if (!active_v(p.V0[i])) {  // inactive cell of a stored segment
+                o[i] = czero<CT>();
+                if constexpr (st == 1) wv[i] = czero<CT>();
             }
         }
     }
@@ -1097,8 +1154,8 @@ __device__ __forceinline__ void rk4_brick(const RkArgs<R> &a, const GridView &G,
                                           WarpSpace<typename Cx<R>::T, BX, BY, BZ, NP> &ws, R s)
 {
     using B = Rk4Body<R, BLEND, CG, st>;
-    const B body(a, s);
-    brick_apply<BX, BY, BZ, CG>(ws, G, b, next, body.yin(), Identity(), a.ihx2, a.ihy2, a.ihz2,
+    const B body(a, s, rhs_centre(a.ihx2, a.ihy2, a.ihz2));
+    brick_apply<BX, BY, BZ, CG, LapRhs>(ws, G, b, next, body.yin(), Identity(), a.ihx2, a.ihy2, a.ihz2,
                                 [&](uint32_t idx) { return body.load(idx); }, body);
 }
 

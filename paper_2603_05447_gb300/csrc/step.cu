@@ -975,7 +975,9 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? (NS < 3 ? 6 : 5) : (NS 
         CT y[NS > 0 ? NS : 1][4];
     };
     const R s = BLEND ? (R)ramp_s(a.ramp, *a.ramp.clock + a.t_off + a.tc) : (R)0;
-    tile_loop<7>(T, (const CT *)a.y[a.tile], Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
+    const R c3 = rhs_centre(a.ihx2, a.ihy2, a.ihz2);
+    constexpr R HALF = sizeof(R) == 8 ? (R)1 : (R)(-0.5);  // LapRhs leaves the factor in in single precision
+    tile_loop<7, LapRhs>(T, (const CT *)a.y[a.tile], Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
                  [&](uint32_t idx, uint32_t n) {
                      prefetch_l2(a.V0 + idx, n * (uint32_t)sizeof(R));
                      if constexpr (BLEND) prefetch_l2(a.V1 + idx, n * (uint32_t)sizeof(R));
@@ -999,13 +1001,14 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? (NS < 3 ? 6 : 5) : (NS 
                          for (int j = 0; j < NS; ++j) acc = axpy(acc, a.coef[j], p.y[j][i]);
                          R V = p.V0[i];
                          if constexpr (BLEND) V = ((R)1 - s) * p.V0[i] + s * p.V1[i];
-                         const R w = V + a.g * (c[i].x * c[i].x + c[i].y * c[i].y);
-                         const R hr = (R)(-0.5) * L[i].x + w * c[i].x;
-                         const R hi = (R)(-0.5) * L[i].y + w * c[i].y;
+                         R w = V + a.g * (c[i].x * c[i].x + c[i].y * c[i].y);
+                         if constexpr (sizeof(R) == 8) w += c3;
+                         const R hr = HALF * L[i].x + w * c[i].x;
+                         const R hi = HALF * L[i].y + w * c[i].y;
                          // f = -i (hr + i hi) = hi - i hr; +inf marks an inactive cell of a stored segment
                          o[i].x = acc.x + a.kdt * hi;
                          o[i].y = acc.y - a.kdt * hr;
-                         if (!(p.V0[i] < (R)INFINITY)) o[i] = czero<CT>();
+                         if (!active_v(p.V0[i])) o[i] = czero<CT>();
                      }
                      st4(a.y[a.out] + idx, o);
                  });

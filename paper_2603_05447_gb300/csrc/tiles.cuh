@@ -114,8 +114,9 @@ struct TileSlots<19> {
     __device__ __forceinline__ int operator()(int k) const { return (int)((q[k / 5] >> (12 * (k % 5))) & 4095u); }
 };
 
-// The Laplacians L of a segment with values c and neighbour slots f
-template <int NP, typename CT, typename R>
+// L of a segment with values c and neighbour slots f: the Laplacians, or what
+// LAP makes of them
+template <int NP, typename LAP, typename CT, typename R>
 __device__ __forceinline__ void tile_laplacian(const TileMem<CT> &m, const TileSlots<NP> &f, const CT (&c)[4], R ihx2,
                                                R ihy2, R ihz2, CT (&L)[4])
 {
@@ -133,7 +134,7 @@ __device__ __forceinline__ void tile_laplacian(const TileMem<CT> &m, const TileS
         for (int i = 0; i < 4; ++i) {
             const CT l = i == 0 ? xm : c[i - 1];
             const CT rr = i == 3 ? xp : c[i + 1];
-            L[i] = lapv(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], ihx2, ihy2, ihz2, c6);
+            L[i] = LAP::of(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], LAP::coef(ihx2), LAP::coef(ihy2), LAP::coef(ihz2), c6);
         }
     } else {
         // App. B: the 7-point part plus w_ab (edges_ab - 2 faces_ab + 4 c) per
@@ -163,8 +164,8 @@ __device__ __forceinline__ void tile_laplacian(const TileMem<CT> &m, const TileS
                                 vadd(i == 0 ? ypl : yp[i - 1], i == 3 ? ypr : yp[i + 1]));
             const CT exz = vadd(vadd(i == 0 ? zml : zm[i - 1], i == 3 ? zmr : zm[i + 1]),
                                 vadd(i == 0 ? zpl : zp[i - 1], i == 3 ? zpr : zp[i + 1]));
-            L[i] = edgev(lapv(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], ax, ay, az, c19), exy, exz, eyz[i], wxy, wxz,
-                         wyz);
+            L[i] = edgev(LAP::of(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], LAP::coef(ax), LAP::coef(ay), LAP::coef(az), c19),
+                         exy, exz, eyz[i], LAP::coef(wxy), LAP::coef(wxz), LAP::coef(wyz));
         }
     }
 }
@@ -206,7 +207,8 @@ struct EveryTile {
 //
 // setup(tile), uniform over the block, runs before each tile, may change what
 // xf and the inverse square spacings refer to, and says whether to take it.
-template <int NP, typename CT, typename R, typename XF, typename SETUP, typename PREF, typename LOAD, typename BODY>
+template <int NP, typename LAP = LapFull, typename CT, typename R, typename XF, typename SETUP, typename PREF,
+          typename LOAD, typename BODY>
 __device__ __forceinline__ void tile_loop(const TileView &T, const CT *src, const XF &xf, const R &ihx2, const R &ihy2,
                                           const R &ihz2, SETUP setup, PREF prefetch, LOAD load, BODY body)
 {
@@ -311,7 +313,7 @@ __device__ __forceinline__ void tile_loop(const TileView &T, const CT *src, cons
         __syncthreads();
         if (in) {
             CT L[4];
-            tile_laplacian<NP>(m, f, c, ihx2, ihy2, ihz2, L);
+            tile_laplacian<NP, LAP>(m, f, c, ihx2, ihy2, ihz2, L);
             body(idx, pre, c, L);
         }
     }
@@ -353,20 +355,32 @@ inline unsigned tile_blocks(K kernel, int nsm, int n, size_t smem)
 // blocks an SM: registers of 85 (single) and 168 (double) a thread
 #define GPE_TILE_BOUNDS(R) __launch_bounds__(TILE, sizeof(R) == 4 ? 6 : 3)
 
+// the centre's share of the right-hand side with either stencil (App. B's
+// centre weight is c6 - 4 (wxy + wxz + wyz))
+template <int NP, typename R>
+__device__ __forceinline__ R tile_rhs_centre(R ihx2, R ihy2, R ihz2)
+{
+    const R c = rhs_centre(ihx2, ihy2, ihz2);
+    return NP == 19 ? c - c / (R)3 : c;  // 2 (wxy + wxz + wyz) = (1/hx^2 + 1/hy^2 + 1/hz^2) / 3
+}
+
 // One RK4 stage.  1024^3 shell, 8x8x4 bricks, per step of four: complex64
 // 0.776 -> 0.626 ms (4.0 GB, of which 0.4 GB slots and halo lists: 6.5 TB/s,
-// 0.95 of the copy bandwidth, so bytes bound it now); complex128 8.65 ->
-// 6.75 ms (FP64 issue: full lanes instead of four fifths).  Six blocks an SM
-// (85 registers): 0.626 ms, seven 0.634, eight with spills 0.645; double:
-// three 6.75, four 6.98, five 7.1.  One block a tile instead of looping
-// blocks: 8 % slower (no tile ahead to prefetch).
+// 0.95 of the copy bandwidth, so bytes bound it now); complex128 8.65 -> 5.49
+// ms (full lanes instead of four fifths: 6.75; 90 instead of 108 FP64
+// instructions a cell and step, LapRhs, active_v and the split third: 5.49; an
+// FP64 instruction takes 8 to 9.6 ns an SM whatever its lanes do, and they
+// fill the time).  Single precision, six blocks an SM (85 registers): 0.626
+// ms, seven 0.634, eight with spills 0.645; double, registers for two: 5.49,
+// three 5.69, four 5.80.  One block a tile instead of looping blocks: 8 %
+// slower (no tile ahead to prefetch).
 template <typename R, bool BLEND, int ST, int NP>
-__global__ void GPE_TILE_BOUNDS(R) k_rk4_tile(const RkArgs<R> a, const TileView T)
+__global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? 6 : 2) k_rk4_tile(const RkArgs<R> a, const TileView T)
 {
     using CT = typename Cx<R>::T;
     using B = Rk4Body<R, BLEND, false, ST>;
-    const B body(a, stage_s<R, BLEND>(a, ST));
-    tile_loop<NP>(T, body.yin(), Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
+    const B body(a, stage_s<R, BLEND>(a, ST), tile_rhs_centre<NP>(a.ihx2, a.ihy2, a.ihz2));
+    tile_loop<NP, LapRhs>(T, body.yin(), Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
                   [&](uint32_t idx, uint32_t n) {
                       prefetch_l2(a.V0 + idx, n * (uint32_t)sizeof(R));
                       if constexpr (BLEND) prefetch_l2(a.V1 + idx, n * (uint32_t)sizeof(R));
