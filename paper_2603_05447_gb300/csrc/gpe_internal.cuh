@@ -76,15 +76,23 @@ struct BrickRec {
     uint32_t pad[2];
 };
 
+// Brick shapes are powers of two, 8 along x: a lattice cell's brick, local index
+// and position by shifts (64-bit divisions made the builder's and the copies'
+// kernels twice as long)
+struct BrickGeo {
+    int ly, lz;  // log2 of the rows and planes
+    __host__ __device__ int lc() const { return 3 + ly + lz; }  // log2 of the cells
+    __host__ __device__ int64_t brick(int64_t s) const { return s >> lc(); }
+    __host__ __device__ int local(int64_t s) const { return (int)(s & ((1 << lc()) - 1)); }
+    __host__ __device__ int x(int l) const { return l & 7; }
+    __host__ __device__ int y(int l) const { return (l >> 3) & ((1 << ly) - 1); }
+    __host__ __device__ int z(int l) const { return l >> (3 + ly); }
+};
+inline BrickGeo brick_geo(int by, int bz) { return BrickGeo{by == 8 ? 3 : 2, bz == 8 ? 3 : 2}; }
+
 // per brick: its record followed by its six face neighbours' (-x +x -y +y -z
 // +z; empty records for absent neighbours), built on the host
 void build_rec7(const std::vector<BrickRec> &rec, const std::vector<int32_t> &nbr, std::vector<BrickRec> &out);
-// records of each brick, its 6 face and 12 edge neighbours (edge order: xy
-// (-1,-1,0) (+1,-1,0) (-1,+1,0) (+1,+1,0); xz (-1,0,-1) (+1,0,-1) (-1,0,+1)
-// (+1,0,+1); yz (0,-1,-1) (0,+1,-1) (0,-1,+1) (0,+1,+1))
-void build_rec19(const std::vector<BrickRec> &rec, const std::vector<int32_t> &nbr,
-                 const std::vector<int32_t> &nbr_e, std::vector<BrickRec> &out);
-
 // packed index of the first cell of segment q, if stored
 __host__ __device__ __forceinline__ bool seg_index(const BrickRec &r, int q, uint32_t &idx)
 {
@@ -112,109 +120,6 @@ __device__ __forceinline__ typename Cx<R>::T cmk(R x, R y)
     c.x = x;
     c.y = y;
     return c;
-}
-
-// ------------------------------------------------------------ brick tiles
-// A tile holds one brick plus a one-cell face halo (edges/corners unused by
-// the 7-point stencil), (BX+2)(BY+2)(BZ+2) entries, x fastest.
-template <int BX, int BY, int BZ>
-struct Brick {
-    static constexpr int BC = BX * BY * BZ;
-    static constexpr int TX = BX + 2, TY = BY + 2, TZ = BZ + 2;
-    static constexpr int TN = TX * TY * TZ;
-    static constexpr int NXF = BY * BZ, NYF = BX * BZ, NZF = BX * BY;
-    static constexpr int NH = 2 * (NXF + NYF + NZF);
-    __device__ __forceinline__ static int t(int x, int y, int z)
-    {
-        return (x + 1) + TX * ((y + 1) + TY * (z + 1));
-    }
-};
-
-__device__ __forceinline__ bool mask_bit(const uint32_t *__restrict__ mask, int64_t slot)
-{
-    return (__ldg(&mask[slot >> 5]) >> (slot & 31)) & 1u;
-}
-
-// Stage brick b of `src` and its six face halos into shared memory, passing
-// each loaded value through xf(value, slot).  Interior loads are predicated on
-// the active mask (inactive slots are zero in memory; skipping them saves
-// DRAM sectors).  xf(0, slot) must be 0.
-template <int BX, int BY, int BZ, typename CT, typename XF>
-__device__ __forceinline__ void load_tile(CT *tile, const CT *src, int64_t b,
-                                          const int32_t *__restrict__ nbr,
-                                          const uint32_t *__restrict__ mask, XF xf)
-{
-    using B = Brick<BX, BY, BZ>;
-    const int64_t base = b * B::BC;
-    CT zero;
-    zero.x = 0;
-    zero.y = 0;
-    for (int l = threadIdx.x; l < B::BC; l += blockDim.x) {
-        const int64_t s = base + l;
-        CT v = zero;
-        if (mask_bit(mask, s)) v = xf(src[s], s);
-        const int x = l % BX, y = (l / BX) % BY, z = l / (BX * BY);
-        tile[B::t(x, y, z)] = v;
-    }
-    for (int h = threadIdx.x; h < B::NH; h += blockDim.x) {
-        int face, u, lx, ly, lz, tx, ty, tz;
-        if (h < 2 * B::NXF) {
-            face = h / B::NXF;  // 0: -x, 1: +x
-            u = h % B::NXF;
-            ly = u % BY;
-            lz = u / BY;
-            lx = face ? 0 : BX - 1;
-            tx = face ? BX : -1;
-            ty = ly;
-            tz = lz;
-        } else if (h < 2 * (B::NXF + B::NYF)) {
-            const int hh = h - 2 * B::NXF;
-            face = 2 + hh / B::NYF;  // 2: -y, 3: +y
-            u = hh % B::NYF;
-            lx = u % BX;
-            lz = u / BX;
-            ly = (face == 3) ? 0 : BY - 1;
-            tx = lx;
-            ty = (face == 3) ? BY : -1;
-            tz = lz;
-        } else {
-            const int hh = h - 2 * (B::NXF + B::NYF);
-            face = 4 + hh / B::NZF;  // 4: -z, 5: +z
-            u = hh % B::NZF;
-            lx = u % BX;
-            ly = u / BX;
-            lz = (face == 5) ? 0 : BZ - 1;
-            tx = lx;
-            ty = ly;
-            tz = (face == 5) ? BZ : -1;
-        }
-        const int nb = __ldg(&nbr[b * 6 + face]);
-        CT v = zero;
-        if (nb >= 0) {
-            const int64_t s = (int64_t)nb * B::BC + lx + BX * (ly + BY * lz);
-            v = xf(src[s], s);
-        }
-        tile[B::t(tx, ty, tz)] = v;
-    }
-}
-
-// 7-point Laplacian (Eq. (B1)) of tile entry (x, y, z).
-template <int BX, int BY, int BZ, typename R, typename CT>
-__device__ __forceinline__ CT tile_laplacian(const CT *tile, int x, int y, int z,
-                                             R ihx2, R ihy2, R ihz2)
-{
-    using B = Brick<BX, BY, BZ>;
-    const int c = B::t(x, y, z);
-    const CT p = tile[c];
-    const CT xm = tile[c - 1], xp = tile[c + 1];
-    const CT ym = tile[c - B::TX], yp = tile[c + B::TX];
-    const CT zm = tile[c - B::TX * B::TY], zp = tile[c + B::TX * B::TY];
-    CT r;
-    r.x = (xp.x - 2 * p.x + xm.x) * ihx2 + (yp.x - 2 * p.x + ym.x) * ihy2 +
-          (zp.x - 2 * p.x + zm.x) * ihz2;
-    r.y = (xp.y - 2 * p.y + xm.y) * ihx2 + (yp.y - 2 * p.y + ym.y) * ihy2 +
-          (zp.y - 2 * p.y + zm.y) * ihz2;
-    return r;
 }
 
 // ------------------------------------------------------------ reductions
@@ -311,8 +216,7 @@ struct gpe_grid {
     int32_t *d_nbr = nullptr;
     uint32_t *d_mask = nullptr;
     gpe::BrickRec *d_rec = nullptr;
-    gpe::BrickRec *d_rec7 = nullptr;  // [nb*7] record of each brick and of its six face neighbours
-    gpe::BrickRec *d_rec19 = nullptr; // [nb*19] ... and of its 12 edge neighbours (19-point grids)
+    gpe::BrickRec *d_rec7 = nullptr;  // [nb*7] record of each brick and of its six face neighbours (wavefront schedules)
     int stencil = 7;                  // 7 or 19 points
     int32_t *d_nbr18 = nullptr;       // [nb*18] face then edge neighbour ids (PAIR schedule, built on first use)
     gpe::TileTab tiles;         // the stencil kernels' tiles

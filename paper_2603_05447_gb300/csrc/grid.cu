@@ -164,6 +164,181 @@ __global__ void k_occupancy(VSource src, BoxD box, int BX, int BY, int BZ, int64
     }
 }
 
+// A threshold in the forms its comparisons use.  An FP64 comparison issues at
+// 1/64 of the FP32 rate here, so FP32 cells are compared in FP32 against the
+// threshold rounded up (the same set: a float is below t exactly if it is below
+// the next float at or above t), FP64 cells as integers that order like them.
+struct Limit {
+    double t;
+    float f;      // smallest float >= t
+    int64_t ord;  // t as an integer
+};
+constexpr int64_t ORD_MINUS_INF = (int64_t)(0xfff0000000000000ull ^ 0x7fffffffffffffffull);
+
+static Limit limit_of(double t)
+{
+    Limit m;
+    m.t = t;
+    m.f = (float)t;
+    if ((double)m.f < t) m.f = std::nextafter(m.f, INFINITY);
+    int64_t b;
+    memcpy(&b, &t, 8);
+    m.ord = t == 0.0 ? -1 : (b < 0 ? b ^ 0x7fffffffffffffffll : b);  // neither zero is below a zero
+    return m;
+}
+
+// v < t (false for a NaN)
+__device__ __forceinline__ bool below(float v, const Limit &m) { return v < m.f; }
+__device__ __forceinline__ bool below(double v, const Limit &m)
+{
+    const int64_t b = __double_as_longlong(v), o = b < 0 ? b ^ 0x7fffffffffffffffll : b;
+    return o < m.ord && o >= ORD_MINUS_INF;
+}
+
+// (1) for dense potentials: every cell of the box is read once, in rows, a warp
+// a row, and marks its brick.  Bound by that read (512^3 FP32,
+// two potentials in 0.19 ms, 5.8 TB/s); testing brick by brick, a block barrier
+// each and in FP64, took 2.0 ms.  occ is zero before.
+template <typename T>
+__global__ void k_occ_dense(const T *V0, const T *V1, Limit c0, Limit c1, BoxD box, int BY, int BZ, int64_t nbx,
+                            int64_t nby, uint8_t *occ)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t rows = box.ny * box.nz, nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t r = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); r < rows; r += nw) {
+        const int64_t j = r % box.ny, k = r / box.ny;
+        uint8_t *row = occ + nbx * (j / BY + nby * (k / BZ));
+        const T *v0 = V0 + r * box.nx, *v1 = V1 ? V1 + r * box.nx : nullptr;
+        for (int64_t i0 = 0; i0 < box.nx; i0 += 128) {
+            bool sel[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int64_t i = i0 + 32 * q + lane;
+                const T a = i < box.nx ? v0[i] : (T)INFINITY;
+                const T b = v1 && i < box.nx ? v1[i] : (T)INFINITY;
+                sel[q] = i < box.nx && (below(a, c0) | (v1 && below(b, c1)));
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const unsigned any = __ballot_sync(0xffffffffu, sel[q]);
+                if (lane < 4 && ((any >> (8 * lane)) & 0xffu)) row[(i0 + 32 * q) / 8 + lane] = 1;
+            }
+        }
+    }
+}
+
+// (4) for dense potentials: the active bits of the kept bricks, a warp a word
+template <typename T>
+__global__ void k_mask_dense(const T *V0, const T *V1, Limit c0, Limit c1, BoxD box, BrickGeo G, int mask_mode,
+                             const int32_t *org, int64_t nwords, uint32_t *mask,
+                             unsigned long long *n_active)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+    unsigned long long cnt = 0;
+    for (int64_t w = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); w < nwords; w += nw) {
+        const int64_t b = G.brick(32 * w);
+        const int l = G.local(32 * w) + lane;
+        const int64_t i = org[3 * b] + G.x(l), j = org[3 * b + 1] + G.y(l), k = org[3 * b + 2] + G.z(l);
+        bool act = i < box.nx && j < box.ny && k < box.nz;
+        if (act && mask_mode == GPE_MASK_CELL) {
+            const int64_t lin = i + box.nx * (j + box.ny * k);
+            const T a = V0[lin], c = V1 ? V1[lin] : (T)INFINITY;
+            act = below(a, c0) | (V1 && below(c, c1));
+        }
+        const unsigned bits = __ballot_sync(0xffffffffu, act);
+        if (lane == 0) {
+            mask[w] = bits;
+            cnt += __popc(bits);
+        }
+    }
+    if (lane == 0 && cnt) atomicAdd(n_active, cnt);
+}
+
+// |v| as an integer that orders like it, 0 for a NaN
+__device__ __forceinline__ unsigned long long abs_bits(double v)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+    return b <= 0x7ff0000000000000ull ? b : 0ull;
+}
+__device__ __forceinline__ void block_max(unsigned long long v, unsigned long long *out)
+{
+    for (int off = 16; off > 0; off >>= 1) v = max(v, __shfl_down_sync(0xffffffffu, v, off));
+    if ((threadIdx.x & 31) == 0 && v > __ldcg(out)) atomicMax(out, v);
+}
+
+// the packed potentials of a dense source, straight from the box: active cells
+// get their value, inactive cells of stored segments +inf in slot 0 and 0 in
+// slot 1
+template <typename T>
+__global__ void k_fill_dense(const T *S0, const T *S1, BoxD box, BrickGeo G, const int32_t *org, const uint32_t *mask,
+                              const BrickRec *rec, int64_t ns, double *V0, double *V1,
+                             unsigned long long *vmax_bits)
+{
+    unsigned long long vm = 0;
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < ns; s += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t b = G.brick(s);
+        const int l = G.local(s);
+        uint32_t idx;
+        if (!seg_index(rec[b], l >> 2, idx)) continue;
+        idx += l & 3;
+        if ((mask[s >> 5] >> (s & 31)) & 1u) {
+            const int64_t lin = org[3 * b] + G.x(l) +
+                                box.nx * (org[3 * b + 1] + G.y(l) + box.ny * (int64_t)(org[3 * b + 2] + G.z(l)));
+            const double v = (double)S0[lin];
+            V0[idx] = v;
+            vm = max(vm, abs_bits(v));
+            if (V1) {
+                const double w = (double)S1[lin];
+                V1[idx] = w;
+                vm = max(vm, abs_bits(w));
+            }
+        } else {
+            V0[idx] = INFINITY;
+            if (V1) V1[idx] = 0.0;
+        }
+    }
+    block_max(vm, vmax_bits);
+}
+
+// exclusive scan of v[n] in place by one block, total to *tot
+__global__ void k_scan(int64_t *v, int64_t n, int64_t *tot)
+{
+    constexpr int PER = 4;
+    __shared__ int64_t wsum[32];
+    __shared__ int64_t carry;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) carry = 0;
+    __syncthreads();
+    for (int64_t base = 0; base < n; base += (int64_t)blockDim.x * PER) {
+        const int64_t at = base + (int64_t)threadIdx.x * PER;
+        int64_t x[PER], own = 0;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            x[q] = at + q < n ? v[at + q] : 0;
+            own += x[q];
+        }
+        int64_t incl = own;
+        for (int off = 1; off < 32; off <<= 1) {
+            const int64_t y = __shfl_up_sync(0xffffffffu, incl, off);
+            if (lane >= off) incl += y;
+        }
+        if (lane == 31) wsum[warp] = incl;
+        __syncthreads();
+        int64_t pre = carry + incl - own;
+        for (int w = 0; w < warp; ++w) pre += wsum[w];
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            if (at + q < n) v[at + q] = pre;
+            pre += x[q];
+        }
+        __syncthreads();
+        if (threadIdx.x == blockDim.x - 1) carry = pre;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *tot = carry;
+}
+
 __device__ __forceinline__ uint32_t compact3(uint64_t m)
 {
     // keep every third bit of m (bit 3n -> bit n)
@@ -286,15 +461,14 @@ __global__ void k_neighbors(int64_t nb, const int32_t *coords, int64_t nbx, int6
     }
 }
 
-// (4) per-cell potential values and active bits; one block per brick
+// (4) for analytic potentials: per-cell values and active bits; one block per brick
 __global__ void k_cells(VSource src, BoxD box, int BX, int BY, int BZ, int mask_mode,
                         const int32_t *org, double *V0, double *V1, uint32_t *mask,
                         unsigned long long *n_active, unsigned long long *vmax_bits)
 {
     const int64_t id = blockIdx.x;
     const int BC = BX * BY * BZ;
-    unsigned long long cnt = 0;
-    double vm = 0.0;
+    unsigned long long cnt = 0, vm = 0;
     for (int l = threadIdx.x; l < BC; l += blockDim.x) {  // BC % 32 == 0, blockDim % 32 == 0
         int64_t i = org[3 * id] + l % BX, j = org[3 * id + 1] + (l / BX) % BY,
                 k = org[3 * id + 2] + l / (BX * BY);
@@ -310,53 +484,72 @@ __global__ void k_cells(VSource src, BoxD box, int BX, int BY, int BZ, int mask_
         if ((threadIdx.x & 31) == 0) mask[slot >> 5] = bits;
         if (act) {
             ++cnt;
-            vm = fmax(vm, fabs(v0));
-            if (V1) vm = fmax(vm, fabs(v1));
+            vm = max(vm, abs_bits(v0));
+            if (V1) vm = max(vm, abs_bits(v1));
         }
     }
-    for (int off = 16; off > 0; off >>= 1) {
-        cnt += __shfl_down_sync(0xffffffffu, cnt, off);
-        vm = fmax(vm, __shfl_down_sync(0xffffffffu, vm, off));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(n_active, cnt);
-        atomicMax(vmax_bits, (unsigned long long)__double_as_longlong(vm));
-    }
+    for (int off = 16; off > 0; off >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, off);
+    if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(n_active, cnt);
+    block_max(vm, vmax_bits);
 }
 
 // Segment layout: a segment is 4 consecutive cells along x inside a brick
 // (one 32-byte sector of complex64).  A brick stores exactly its segments that
 // hold at least one active cell.  k_seg_records builds each brick's record:
-// the segment bit mask, the number of stored segments before each mask word,
-// and (after the host scan) the packed offset.
-__global__ void k_seg_records(int64_t nb, int BC, const uint32_t *mask, BrickRec *rec, uint32_t *cnt)
+// the segment bit mask, the number of stored segments before each mask word
+// and the packed offset within its block of bricks, whose count goes to
+// bsum[block]; k_seg_offsets adds what precedes the block.
+constexpr int REC_THREADS = 256;
+__global__ void __launch_bounds__(REC_THREADS) k_seg_records(int64_t nb, int BC, const uint32_t *mask, BrickRec *rec,
+                                                             int64_t *bsum)
 {
+    __shared__ uint32_t wsum[REC_THREADS / 32];
     int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (b >= nb) return;
     const int W = BC / 32, nseg = BC / 4;
     BrickRec r{};
     uint32_t c = 0;
-    for (int q = 0; q < nseg; ++q) {
-        // cells 4q..4q+3 of the brick: nibble (q & 7) of mask word q/8
-        const uint32_t word = mask[b * W + (q >> 3)];
-        if ((word >> (4 * (q & 7))) & 0xfu) r.m[q >> 5] |= 1u << (q & 31);
+    if (b < nb) {
+        for (int q0 = 0; q0 < nseg; q0 += 8) {
+            // cells 4q..4q+3 of the brick: nibble (q & 7) of mask word q/8
+            const uint32_t word = mask[b * W + (q0 >> 3)];
+            for (int q = 0; q < 8; ++q)
+                if ((word >> (4 * q)) & 0xfu) r.m[q0 >> 5] |= 1u << ((q0 + q) & 31);
+        }
+        for (int w = 0; w < 4; ++w) {
+            r.pre |= (c & 0xffu) << (8 * w);
+            c += __popc(r.m[w]);
+        }
     }
-    for (int w = 0; w < 4; ++w) {
-        r.pre |= (c & 0xffu) << (8 * w);
-        c += __popc(r.m[w]);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t incl = c;
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += y;
     }
-    rec[b] = r;
-    cnt[b] = c;
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    uint32_t pre = incl - c;
+    for (int w = 0; w < warp; ++w) pre += wsum[w];
+    if (b < nb) {
+        r.off = 4u * pre;
+        rec[b] = r;
+    }
+    if (threadIdx.x == REC_THREADS - 1) bsum[blockIdx.x] = pre + c;
+}
+__global__ void k_seg_offsets(int64_t nb, BrickRec *rec, const int64_t *before)
+{
+    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (b < nb) rec[b].off += (uint32_t)(4 * before[blockIdx.x]);
 }
 
 // scatter stored-lattice values to the packed layout: active cells get their
 // value, inactive cells of stored segments get `fill`
-__global__ void k_pack(int64_t ns, int BC, const uint32_t *mask, const BrickRec *rec, const double *src,
+__global__ void k_pack(int64_t ns, BrickGeo G, const uint32_t *mask, const BrickRec *rec, const double *src,
                        double *dst, double fill)
 {
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < ns; s += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = s / BC;
-        const int l = (int)(s % BC);
+        const int64_t b = G.brick(s);
+        const int l = G.local(s);
         uint32_t idx;
         if (!seg_index(rec[b], l >> 2, idx)) continue;
         const bool act = (mask[s >> 5] >> (s & 31)) & 1u;
@@ -410,37 +603,7 @@ void gpe::build_rec7(const std::vector<BrickRec> &rec, const std::vector<int32_t
     }
 }
 
-void gpe::build_rec19(const std::vector<BrickRec> &rec, const std::vector<int32_t> &nbr,
-                      const std::vector<int32_t> &nbr_e, std::vector<BrickRec> &out)
-{
-    const size_t nb = rec.size();
-    out.assign(nb * 19, BrickRec{});
-    for (size_t b = 0; b < nb; ++b) {
-        out[19 * b] = rec[b];
-        for (int d = 0; d < 6; ++d)
-            if (nbr[6 * b + d] >= 0) out[19 * b + 1 + d] = rec[nbr[6 * b + d]];
-        for (int e = 0; e < 12; ++e)
-            if (nbr_e[12 * b + e] >= 0) out[19 * b + 7 + e] = rec[nbr_e[12 * b + e]];
-    }
-}
-
 namespace gpe {
-
-// the 12 edge neighbours of each brick (order as in build_rec19), -1 if absent
-__global__ void k_edge_neighbors(int64_t nb, const int32_t *coords, int64_t nbx, int64_t nby, int64_t nbz,
-                                 const int32_t *bvol, int32_t *nbr_e)
-{
-    const int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (id >= nb) return;
-    const int8_t d[12][3] = {{-1, -1, 0}, {1, -1, 0}, {-1, 1, 0}, {1, 1, 0}, {-1, 0, -1}, {1, 0, -1},
-                             {-1, 0, 1},  {1, 0, 1},  {0, -1, -1}, {0, 1, -1}, {0, -1, 1}, {0, 1, 1}};
-    for (int e = 0; e < 12; ++e) {
-        const int64_t x = coords[3 * id] + d[e][0], y = coords[3 * id + 1] + d[e][1], z = coords[3 * id + 2] + d[e][2];
-        int32_t r = -1;
-        if (x >= 0 && x < nbx && y >= 0 && y < nby && z >= 0 && z < nbz) r = bvol[x + nbx * (y + nby * z)];
-        nbr_e[12 * id + e] = r;
-    }
-}
 
 static BoxD boxd(const gpe_box &b)
 {
@@ -483,7 +646,6 @@ static void grid_free(gpe_grid *g)
     if (!g) return;
     dev_free(g->d_rec);
     dev_free(g->d_rec7);
-    dev_free(g->d_rec19);
     tiles_free(g->tiles);
     dev_free(g->d_nbr18);
     dev_free(g->d_chunk_lohi);
@@ -545,27 +707,30 @@ static int build_grid(const gpe_box *box, const VSource &src, const gpe_grid_opt
     const int64_t nq = g->nbx * g->nby * g->nbz;
     const BoxD bd = boxd(*box);
 
+    // temporaries: occupancy, block counts and totals, then per-brick data
     uint8_t *occ = nullptr;
     int64_t *bsum = nullptr;
     int32_t *coords = nullptr;
-    unsigned long long *counters = nullptr;
     double *tmpV[2] = {nullptr, nullptr};
-    uint32_t *cnt = nullptr;
+    // read back together: bricks kept; stored segments, active cells, largest |V|
+    struct Totals {
+        int64_t bricks, segs;
+        unsigned long long active, vmax;
+    };
+    Totals *tot = nullptr, ht{};
     int rc = GPE_OK;
     auto cleanup = [&]() {
         dev_free(occ);
         dev_free(bsum);
         dev_free(coords);
-        dev_free(counters);
+        dev_free(tot);
         dev_free(tmpV[0]);
         dev_free(tmpV[1]);
-        dev_free(cnt);
         occ = nullptr;
         bsum = nullptr;
         coords = nullptr;
-        counters = nullptr;
+        tot = nullptr;
         tmpV[0] = tmpV[1] = nullptr;
-        cnt = nullptr;
     };
 #define BUILD_TRY(x)                 \
     do {                             \
@@ -587,8 +752,23 @@ static int build_grid(const gpe_box *box, const VSource &src, const gpe_grid_opt
         }                                                                    \
     } while (0)
 
+    const bool dense = src.mode == 0 || src.mode == 3, two = src.mode == 2 || src.mode == 3;
+    const Limit c0 = limit_of(src.cut0), c1 = limit_of(src.cut1);
+    const BrickGeo geo = brick_geo(o.by, o.bz);
+    BUILD_TRY(dev_alloc_t(&tot, 1));
+    BUILD_CUDA(cudaMemsetAsync(tot, 0, sizeof(Totals), st));
     BUILD_TRY(dev_alloc_t(&occ, nq));
-    {
+    if (dense) {
+        BUILD_CUDA(cudaMemsetAsync(occ, 0, nq, st));
+        const unsigned nblk_rows = (unsigned)std::min<int64_t>((box->ny * box->nz + 7) / 8, (int64_t)g->nsm * 64);
+        if (src.dtype == GPE_F64)
+            k_occ_dense<double><<<nblk_rows, 256, 0, st>>>((const double *)src.dense, (const double *)src.dense1, c0, c1,
+                                                          bd, o.by, o.bz, g->nbx, g->nby, occ);
+        else
+            k_occ_dense<float><<<nblk_rows, 256, 0, st>>>((const float *)src.dense, (const float *)src.dense1, c0, c1,
+                                                         bd, o.by, o.bz, g->nbx, g->nby, occ);
+        BUILD_CUDA(cudaGetLastError());
+    } else {
         const int64_t nblk_occ = (nq + 255) / 256;
         if (nblk_occ > 0x7fffffffLL) BUILD_TRY(fail(GPE_ERR_ARG, "brick grid too large"));
         k_occupancy<<<(unsigned)nblk_occ, 256, 0, st>>>(src, bd, o.bx, o.by, o.bz, g->nbx, g->nby, g->nbz, occ);
@@ -613,21 +793,16 @@ static int build_grid(const gpe_box *box, const VSource &src, const gpe_grid_opt
     BUILD_TRY(dev_alloc_t(&bsum, nblk));
     k_enum_count<<<(unsigned)nblk, ENUM_THREADS, 0, st>>>(E, occ, bsum);
     BUILD_CUDA(cudaGetLastError());
-    std::vector<int64_t> h(nblk);
-    BUILD_CUDA(cudaMemcpyAsync(h.data(), bsum, nblk * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    k_scan<<<1, 1024, 0, st>>>(bsum, nblk, &tot->bricks);
+    BUILD_CUDA(cudaGetLastError());
+    BUILD_CUDA(cudaMemcpyAsync(&ht, tot, sizeof ht, cudaMemcpyDeviceToHost, st));
     BUILD_CUDA(cudaStreamSynchronize(st));
-    int64_t total = 0;
-    for (int64_t i = 0; i < nblk; ++i) {
-        int64_t c = h[i];
-        h[i] = total;
-        total += c;
-    }
+    const int64_t total = ht.bricks;
     if (total == 0) BUILD_TRY(fail(GPE_ERR_ARG, "region of interest is empty (no cell with V < V_cut)"));
     if (total * g->bc > 0x7fffffffLL * 32LL)
         BUILD_TRY(fail(GPE_ERR_ARG, "too many stored cells"));
     g->nb = total;
     g->n_stored = total * g->bc;
-    BUILD_CUDA(cudaMemcpyAsync(bsum, h.data(), nblk * sizeof(int64_t), cudaMemcpyHostToDevice, st));
     BUILD_TRY(dev_alloc_t(&coords, 3 * total));
     k_enum_emit<<<(unsigned)nblk, ENUM_THREADS, 0, st>>>(E, occ, bsum, coords);
     BUILD_CUDA(cudaGetLastError());
@@ -643,79 +818,83 @@ static int build_grid(const gpe_box *box, const VSource &src, const gpe_grid_opt
     BUILD_CUDA(cudaGetLastError());
 
     BUILD_TRY(dev_alloc_t(&g->d_mask, g->n_stored / 32));
-    BUILD_TRY(dev_alloc_t(&tmpV[0], g->n_stored));
-    if (src.mode == 2 || src.mode == 3) {
-        BUILD_TRY(dev_alloc_t(&tmpV[1], g->n_stored));
-        g->n_slots = 2;
-    }
-    BUILD_TRY(dev_alloc_t(&counters, 2));
-    BUILD_CUDA(cudaMemsetAsync(counters, 0, 2 * sizeof(unsigned long long), st));
     if (total > 0x7fffffffLL) BUILD_TRY(fail(GPE_ERR_ARG, "too many bricks"));
-    k_cells<<<(unsigned)total, std::min(g->bc, 256), 0, st>>>(src, bd, o.bx, o.by, o.bz, o.mask_mode,
-                                                            g->d_org, tmpV[0], tmpV[1], g->d_mask,
-                                                            counters, counters + 1);
+    if (two) g->n_slots = 2;
+    if (dense) {
+        const int64_t nwords = g->n_stored / 32;
+        const unsigned nbw = (unsigned)std::min<int64_t>((nwords + 7) / 8, (int64_t)g->nsm * 32);
+        if (src.dtype == GPE_F64)
+            k_mask_dense<double><<<nbw, 256, 0, st>>>((const double *)src.dense, (const double *)src.dense1, c0, c1, bd,
+                                                     geo, o.mask_mode, g->d_org, nwords, g->d_mask,
+                                                     &tot->active);
+        else
+            k_mask_dense<float><<<nbw, 256, 0, st>>>((const float *)src.dense, (const float *)src.dense1, c0, c1, bd,
+                                                    geo, o.mask_mode, g->d_org, nwords, g->d_mask,
+                                                    &tot->active);
+    } else {
+        BUILD_TRY(dev_alloc_t(&tmpV[0], g->n_stored));
+        if (two) BUILD_TRY(dev_alloc_t(&tmpV[1], g->n_stored));
+        k_cells<<<(unsigned)total, std::min(g->bc, 256), 0, st>>>(src, bd, o.bx, o.by, o.bz, o.mask_mode, g->d_org,
+                                                                tmpV[0], tmpV[1], g->d_mask, &tot->active, &tot->vmax);
+    }
     BUILD_CUDA(cudaGetLastError());
-    unsigned long long hc[2];
-    BUILD_CUDA(cudaMemcpyAsync(hc, counters, sizeof hc, cudaMemcpyDeviceToHost, st));
-    BUILD_CUDA(cudaStreamSynchronize(st));
-    g->n_active = (int64_t)hc[0];
-    long long vb = (long long)hc[1];
-    memcpy(&g->v_max, &vb, sizeof(double));
 
     // packed layout: every brick stores its segments (4 cells along x) that
     // hold an active cell, in lattice order, as one run
     BUILD_TRY(dev_alloc_t(&g->d_rec, total));
-    BUILD_TRY(dev_alloc_t(&cnt, total));
-    k_seg_records<<<nbb, 256, 0, st>>>(total, g->bc, g->d_mask, g->d_rec, cnt);
-    BUILD_CUDA(cudaGetLastError());
-    std::vector<uint32_t> hcnt(total);
-    std::vector<BrickRec> hrec(total);
-    BUILD_CUDA(cudaMemcpyAsync(hcnt.data(), cnt, total * sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
-    BUILD_CUDA(cudaMemcpyAsync(hrec.data(), g->d_rec, total * sizeof(BrickRec), cudaMemcpyDeviceToHost, st));
-    BUILD_CUDA(cudaStreamSynchronize(st));
-    uint64_t acc = 0;
-    for (int64_t b = 0; b < total; ++b) {
-        hrec[b].off = (uint32_t)acc;
-        acc += 4ull * hcnt[b];
-        if (acc >= 0xffffffffull) BUILD_TRY(fail(GPE_ERR_ARG, "too many stored cells for 32-bit offsets"));
+    const int64_t nblk_rec = (total + REC_THREADS - 1) / REC_THREADS;
+    if (nblk_rec > nblk) {
+        dev_free(bsum);
+        bsum = nullptr;
+        BUILD_TRY(dev_alloc_t(&bsum, nblk_rec));
     }
-    g->n_packed = (int64_t)acc;
-    BUILD_CUDA(cudaMemcpyAsync(g->d_rec, hrec.data(), total * sizeof(BrickRec), cudaMemcpyHostToDevice, st));
-    {
+    k_seg_records<<<(unsigned)nblk_rec, REC_THREADS, 0, st>>>(total, g->bc, g->d_mask, g->d_rec, bsum);
+    BUILD_CUDA(cudaGetLastError());
+    k_scan<<<1, 1024, 0, st>>>(bsum, nblk_rec, &tot->segs);
+    BUILD_CUDA(cudaGetLastError());
+    k_seg_offsets<<<(unsigned)nblk_rec, REC_THREADS, 0, st>>>(total, g->d_rec, bsum);
+    BUILD_CUDA(cudaGetLastError());
+    BUILD_CUDA(cudaMemcpyAsync(&ht, tot, sizeof ht, cudaMemcpyDeviceToHost, st));
+    BUILD_CUDA(cudaStreamSynchronize(st));
+    g->n_active = (int64_t)ht.active;
+    if (4 * (uint64_t)ht.segs >= 0xffffffffull)
+        BUILD_TRY(fail(GPE_ERR_ARG, "too many stored cells for 32-bit offsets"));
+    g->n_packed = 4 * ht.segs;
+    if (o.sched == GPE_SCHED_WAVE || o.sched == GPE_SCHED_WAVE2) {
+        // the wavefront kernels' record rows
+        std::vector<BrickRec> hrec(total), h7;
         std::vector<int32_t> hnbr(total * 6);
+        BUILD_CUDA(cudaMemcpyAsync(hrec.data(), g->d_rec, total * sizeof(BrickRec), cudaMemcpyDeviceToHost, st));
         BUILD_CUDA(cudaMemcpyAsync(hnbr.data(), g->d_nbr, total * 6 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
         BUILD_CUDA(cudaStreamSynchronize(st));
-        std::vector<BrickRec> h7;
         build_rec7(hrec, hnbr, h7);
         BUILD_TRY(dev_alloc_t(&g->d_rec7, total * 7));
         BUILD_CUDA(cudaMemcpyAsync(g->d_rec7, h7.data(), h7.size() * sizeof(BrickRec), cudaMemcpyHostToDevice, st));
         BUILD_CUDA(cudaStreamSynchronize(st));
-        if (g->stencil == 19) {
-            int32_t *d_e = nullptr;
-            BUILD_TRY(dev_alloc_t(&d_e, total * 12));
-            k_edge_neighbors<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(total, coords, g->nbx, g->nby, g->nbz,
-                                                                            g->d_bvol, d_e);
-            std::vector<int32_t> he(total * 12);
-            cudaError_t e1 = cudaGetLastError();
-            if (e1 == cudaSuccess) e1 = cudaMemcpyAsync(he.data(), d_e, he.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, st);
-            if (e1 == cudaSuccess) e1 = cudaStreamSynchronize(st);
-            dev_free(d_e);
-            BUILD_CUDA(e1);
-            std::vector<BrickRec> h19;
-            build_rec19(hrec, hnbr, he, h19);
-            BUILD_TRY(dev_alloc_t(&g->d_rec19, total * 19));
-            BUILD_CUDA(cudaMemcpyAsync(g->d_rec19, h19.data(), h19.size() * sizeof(BrickRec), cudaMemcpyHostToDevice, st));
-            BUILD_CUDA(cudaStreamSynchronize(st));
-        }
     }
     BUILD_TRY(tiles_build(g, st));
-    for (int sl = 0; sl < g->n_slots; ++sl) {
-        BUILD_TRY(dev_alloc_t(&g->d_V[sl], g->n_packed));
-        k_pack<<<g->nsm * 8, 256, 0, st>>>(g->n_stored, g->bc, g->d_mask, g->d_rec, tmpV[sl], g->d_V[sl],
-                                          sl == 0 ? (double)INFINITY : 0.0);
+    for (int sl = 0; sl < g->n_slots; ++sl) BUILD_TRY(dev_alloc_t(&g->d_V[sl], g->n_packed));
+    if (dense) {
+        const unsigned nbf = (unsigned)g->nsm * 16;
+        if (src.dtype == GPE_F64)
+            k_fill_dense<double><<<nbf, 256, 0, st>>>((const double *)src.dense, (const double *)src.dense1, bd, geo,
+                                                     g->d_org, g->d_mask, g->d_rec, g->n_stored, g->d_V[0],
+                                                     g->d_V[1], &tot->vmax);
+        else
+            k_fill_dense<float><<<nbf, 256, 0, st>>>((const float *)src.dense, (const float *)src.dense1, bd, geo,
+                                                    g->d_org, g->d_mask, g->d_rec, g->n_stored, g->d_V[0],
+                                                    g->d_V[1], &tot->vmax);
         BUILD_CUDA(cudaGetLastError());
+    } else {
+        for (int sl = 0; sl < g->n_slots; ++sl) {
+            k_pack<<<g->nsm * 8, 256, 0, st>>>(g->n_stored, geo, g->d_mask, g->d_rec, tmpV[sl], g->d_V[sl],
+                                              sl == 0 ? (double)INFINITY : 0.0);
+            BUILD_CUDA(cudaGetLastError());
+        }
     }
+    BUILD_CUDA(cudaMemcpyAsync(&ht, tot, sizeof ht, cudaMemcpyDeviceToHost, st));
     BUILD_CUDA(cudaStreamSynchronize(st));
+    memcpy(&g->v_max, &ht.vmax, sizeof(double));
     cleanup();
 #undef BUILD_TRY
 #undef BUILD_CUDA
@@ -946,51 +1125,68 @@ namespace gpe {
 
 // A pass of the Thomas-Fermi solve reads the box once: over the cells with
 // V < mu, the sum of V (FP64) and their count, and over all cells below +inf
-// the largest |V| (its leading 32 bits, as an integer).  Bound by the read of
-// a dense V: 512^3 FP32 takes 0.09 ms (5.9 TB/s).  What keeps FP64 work off
-// that path (an FP64 instruction issues at 1/64 of the FP32 rate here; the
-// former pass compared, added and counted every cell in FP64 and took
-// 1.55 ms): FP32 cells are compared in FP32 against mu rounded up (the same
-// set: a float is below mu exactly if it is below the next float at or above
-// mu), FP64 cells first by their high words, cells are counted in integers,
-// and only selected cells are added in FP64.
+// the largest |V| (its leading 32 bits, as an integer).  512^3 FP32: 0.20 ms,
+// 2.7 TB/s.  FP64 work is kept off that path (an FP64 instruction issues at 1/64 of the FP32 rate, predicated off or
+// not; the first form of the pass compared, added and counted every cell in
+// FP64 and took 1.55 ms): cells are compared as in Limit and counted in
+// integers, and a thread's vector goes into the FP64 sum behind a branch, in a
+// call, so that vectors without a selected cell skip it.
 struct TfSum {
     double sum = 0.0;
     unsigned long long cnt = 0;
     uint32_t top = 0;
 };
 
-struct TfLimit {  // mu in the forms the comparisons use
-    double mu;
-    float mu_f;    // smallest float >= mu
-    int32_t hi;    // order-preserving high word of mu
-};
-
-// high word of a double as a signed integer that orders like the double
-__device__ __forceinline__ int32_t ordered_hi(double v)
+__device__ __forceinline__ uint32_t tf_top(float v) { return v < INFINITY ? __float_as_uint(fabsf(v)) : 0u; }
+__device__ __forceinline__ uint32_t tf_top(double v)
 {
-    const int32_t h = __double2hiint(v);
-    return h < 0 ? h ^ 0x7fffffff : h;
-}
-
-__device__ __forceinline__ void tf_cell(float v, const TfLimit &m, TfSum &a)
-{
-    if (v < INFINITY) a.top = max(a.top, __float_as_uint(fabsf(v)));
-    if (v < m.mu_f) {
-        a.sum += (double)v;
-        ++a.cnt;
-    }
-}
-__device__ __forceinline__ void tf_cell(double v, const TfLimit &m, TfSum &a)
-{
-    const uint32_t hi = (uint32_t)__double2hiint(v) & 0x7fffffffu;
+    const uint32_t hi = (uint32_t)__double2hiint(v), a = hi & 0x7fffffffu;
     // below +inf: finite or -inf (NaN and +inf have no place in the sums)
-    const bool below = hi < 0x7ff00000u || (__double2hiint(v) == (int)0xfff00000 && __double2loint(v) == 0);
-    if (!below) return;
-    a.top = max(a.top, hi);
-    if (ordered_hi(v) <= m.hi && v < m.mu) {
-        a.sum += v;
-        ++a.cnt;
+    return a < 0x7ff00000u || (hi == 0xfff00000u && __double2loint(v) == 0) ? a : 0u;
+}
+
+__device__ __noinline__ double tf_add(double sum, float a, float b, float c, float d, unsigned sel)
+{
+    if (sel & 1u) sum += (double)a;
+    if (sel & 2u) sum += (double)b;
+    if (sel & 4u) sum += (double)c;
+    if (sel & 8u) sum += (double)d;
+    return sum;
+}
+__device__ __noinline__ double tf_add(double sum, double a, double b, unsigned sel)
+{
+    if (sel & 1u) sum += a;
+    if (sel & 2u) sum += b;
+    return sum;
+}
+__device__ __forceinline__ double tf_add(double sum, const float (&v)[4], unsigned sel)
+{
+    return tf_add(sum, v[0], v[1], v[2], v[3], sel);
+}
+__device__ __forceinline__ double tf_add(double sum, const float (&v)[1], unsigned sel)
+{
+    return tf_add(sum, v[0], 0.0f, 0.0f, 0.0f, sel);
+}
+__device__ __forceinline__ double tf_add(double sum, const double (&v)[2], unsigned sel)
+{
+    return tf_add(sum, v[0], v[1], sel);
+}
+__device__ __forceinline__ double tf_add(double sum, const double (&v)[1], unsigned sel)
+{
+    return tf_add(sum, v[0], 0.0, sel);
+}
+template <typename T, int W>
+__device__ __forceinline__ void tf_cells(const T (&v)[W], const Limit &m, TfSum &a)
+{
+    unsigned sel = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        a.top = max(a.top, tf_top(v[w]));
+        sel |= (below(v[w], m) ? 1u : 0u) << w;
+    }
+    if (sel) {
+        a.cnt += __popc(sel);
+        a.sum = tf_add(a.sum, v, sel);
     }
 }
 
@@ -1008,7 +1204,7 @@ __device__ __forceinline__ void tf_finish(const TfSum &a, double *partials, unsi
 
 // dense V, n cells; n_vec of them (from the start) by 16-byte loads
 template <typename T>
-__global__ void k_tf_dense(const T *V, int64_t n, int64_t n_vec, TfLimit m, double *partials, unsigned int *counter,
+__global__ void k_tf_dense(const T *V, int64_t n, int64_t n_vec, Limit m, double *partials, unsigned int *counter,
                            double *result, uint32_t *top)
 {
     constexpr int W = 16 / (int)sizeof(T);
@@ -1026,22 +1222,22 @@ __global__ void k_tf_dense(const T *V, int64_t n, int64_t n_vec, TfLimit m, doub
 #pragma unroll
         for (int k = 0; k < 4; ++k) x[k] = src[i + k * step];
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-#pragma unroll
-            for (int w = 0; w < W; ++w) tf_cell(x[k].v[w], m, a);
+        for (int k = 0; k < 4; ++k) tf_cells<T, W>(x[k].v, m, a);
     }
     for (; i < nv; i += step) {
         const Vec x = src[i];
-#pragma unroll
-        for (int w = 0; w < W; ++w) tf_cell(x.v[w], m, a);
+        tf_cells<T, W>(x.v, m, a);
     }
-    for (int64_t j = n_vec + t; j < n; j += step) tf_cell(V[j], m, a);
+    for (int64_t j = n_vec + t; j < n; j += step) {
+        const T x[1] = {V[j]};
+        tf_cells<T, 1>(x, m, a);
+    }
     tf_finish(a, partials, counter, result, top);
 }
 
 // analytic V: a warp takes 32 cells along x and evaluates them in FP64 unless
 // the FP32 bound rules every one of them out
-__global__ void k_tf_analytic(PotDesc P, BoxD box, TfLimit m, double *partials, unsigned int *counter, double *result,
+__global__ void k_tf_analytic(PotDesc P, BoxD box, Limit m, double *partials, unsigned int *counter, double *result,
                               uint32_t *top)
 {
     TfSum a;
@@ -1052,16 +1248,19 @@ __global__ void k_tf_analytic(PotDesc P, BoxD box, TfLimit m, double *partials, 
         const int64_t i0 = u % nc * 32, r = u / nc, j = r % box.ny, k = r / box.ny;
         const int64_t i1 = min(i0 + 32, box.nx) - 1;
         const double y = box.y0 + j * box.hy, z = box.z0 + k * box.hz;
-        if (!pot_may_select(P, m.mu, (float)(box.x0 + i0 * box.hx), (float)(box.x0 + i1 * box.hx), (float)y, (float)y,
+        if (!pot_may_select(P, m.t, (float)(box.x0 + i0 * box.hx), (float)(box.x0 + i1 * box.hx), (float)y, (float)y,
                             (float)z, (float)z))
             continue;
-        if (i0 + lane <= i1) tf_cell(eval_pot(P, box.x0 + (i0 + lane) * box.hx, y, z), m, a);
+        if (i0 + lane <= i1) {
+            const double x[1] = {eval_pot(P, box.x0 + (i0 + lane) * box.hx, y, z)};
+            tf_cells<double, 1>(x, m, a);
+        }
     }
     tf_finish(a, partials, counter, result, top);
 }
 
 // One cell of each of `ns` equal stretches of the box, as float
-constexpr int64_t TF_SAMPLES = 131072;
+constexpr int64_t TF_SAMPLES = 32768;
 __global__ void k_tf_sample(VSource src, BoxD box, int64_t n, int64_t ns, float *out)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -1075,19 +1274,28 @@ __global__ void k_tf_sample(VSource src, BoxD box, int64_t n, int64_t ns, float 
 }
 
 // Newton's method on the sample, with the target scaled to it: an estimate
-// that starts the solve over the whole box, so FP32 is enough
-__global__ void k_tf_estimate(const float *v, int n, double target, double *result)
+// that starts the solve over the whole box, so FP32 is enough.  One block, the
+// sample in its registers.
+__global__ void __launch_bounds__(1024) k_tf_estimate(const float *v, int n, double target, double *result)
 {
+    constexpr int PER = (int)(TF_SAMPLES / 1024);
     __shared__ float s_m;
     __shared__ int s_stop;
+    float x[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int at = threadIdx.x + 1024 * i;
+        x[i] = at < n ? v[at] : INFINITY;
+    }
     float m = INFINITY;
     double last = -1.0;
     for (int it = 0; it < 100; ++it) {
         float sum = 0.0f;
         int cnt = 0;
-        for (int i = threadIdx.x; i < n; i += blockDim.x)
-            if (v[i] < m) {
-                sum += v[i];
+#pragma unroll
+        for (int i = 0; i < PER; ++i)
+            if (x[i] < m) {
+                sum += x[i];
                 ++cnt;
             }
         const double tot = block_sum((double)sum);
@@ -1116,8 +1324,7 @@ __global__ void k_tf_estimate(const float *v, int n, double target, double *resu
 // down to it, and ends exactly once the set {V < mu} stops changing.  It
 // starts from the solution on a sample of the cells, a per cent or so off:
 // three to five passes over the box, where a start at mu = +inf took about
-// eighteen of 1.55 ms (a four-stage 512^3 ramp with FP32 potentials: 148 ms,
-// now 65 ms).
+// eighteen (512^3 shell, FP32: 28 ms a solve of 1.55 ms passes, now 0.97 ms).
 static int tf_mu_impl(const gpe_box *box, const VSource &src, double g, double N, double *mu, cudaStream_t st)
 {
     if (!(g > 0)) return fail(GPE_ERR_ARG, "g must be > 0 for the Thomas-Fermi estimate");
@@ -1144,14 +1351,7 @@ static int tf_mu_impl(const gpe_box *box, const VSource &src, double g, double N
     double *partials = reinterpret_cast<double *>(ws + sizeof(Head));
     float *sample = reinterpret_cast<float *>(partials + 2 * blocks);
     auto pass = [&](double m) -> int {
-        TfLimit lim;
-        lim.mu = m;
-        lim.mu_f = (float)m;
-        if ((double)lim.mu_f < m) lim.mu_f = std::nextafter(lim.mu_f, INFINITY);
-        int64_t bits;
-        memcpy(&bits, &m, 8);
-        lim.hi = (int32_t)(bits >> 32);
-        if (lim.hi < 0) lim.hi ^= 0x7fffffff;
+        const Limit lim = limit_of(m);
         if (src.mode != 0) {
             k_tf_analytic<<<blocks, 256, 0, st>>>(src.p0, bd, lim, partials, &head->counter, head->res, &head->top);
         } else {

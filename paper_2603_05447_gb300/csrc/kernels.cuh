@@ -60,9 +60,9 @@ struct ELoad {
     }
 };
 
-template <typename R, typename CT, int BX, int BY, int BZ, bool CG, int NP = 7>
+template <typename R, typename CT, int BX, int BY, int BZ, bool CG>
 __device__ __forceinline__ void itp_brick_a(const ItpArgs<R, CT> &a, const GridView &G, int64_t b, int64_t next,
-                                            WarpSpace<CT, BX, BY, BZ, NP> &ws, R sc)
+                                            WarpSpace<CT, BX, BY, BZ> &ws, R sc)
 {
     const R q4 = a.dt / (R)4;
     const DiagLoad<R, CT> diag{sc, a.g * a.dt / (R)2, a.E};
@@ -78,9 +78,9 @@ __device__ __forceinline__ void itp_brick_a(const ItpArgs<R, CT> &a, const GridV
     });
 }
 
-template <typename R, typename CT, int BX, int BY, int BZ, bool CG, int NP = 7>
+template <typename R, typename CT, int BX, int BY, int BZ, bool CG>
 __device__ __forceinline__ void itp_brick_b(const ItpArgs<R, CT> &a, const GridView &G, int64_t b, int64_t next,
-                                            WarpSpace<CT, BX, BY, BZ, NP> &ws, double &acc)
+                                            WarpSpace<CT, BX, BY, BZ> &ws, double &acc)
 {
     const R hg = a.g * a.dt / (R)2;
     const R q4 = a.dt / (R)4;

@@ -40,7 +40,7 @@ constexpr int PAIR_THREADS = 64;  // threads (two warps) per brick
 
 struct PairView {
     const BrickRec *rec;    // per-brick records
-    const int32_t *nbr18;   // per brick: -x +x -y +y -z +z, then the 12 edges (build_rec19 order); -1 = none
+    const int32_t *nbr18;   // per brick: -x +x -y +y -z +z, then the 12 edges (k_nbr18); -1 = none
     int64_t nb;
 };
 

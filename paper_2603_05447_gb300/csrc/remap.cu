@@ -10,7 +10,7 @@ struct RemapSide {
     const BrickRec *rec;
     const uint32_t *mask;  // bc bits per brick
     const int32_t *bvol;   // brick grid -> brick id or -1
-    int bx, by, bz;
+    BrickGeo geo;
     int64_t nbx, nby, nbz;
 };
 
@@ -20,24 +20,21 @@ struct RemapSide {
 template <typename CT>
 __global__ void k_remap(CT *dst, const CT *src, RemapSide D, RemapSide S, int64_t n_lattice)
 {
-    const int dbc = D.bx * D.by * D.bz;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n_lattice;
          t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = t / dbc;
-        const int l = (int)(t % dbc);
+        const int64_t b = D.geo.brick(t);
+        const int l = D.geo.local(t);
         uint32_t jd;
         if (!seg_index(D.rec[b], l >> 2, jd)) continue;
         jd += (uint32_t)(l & 3);
         CT v = czero<CT>();
-        if ((D.mask[b * (dbc / 32) + (l >> 5)] >> (l & 31)) & 1u) {
-            const int64_t i = D.org[3 * b] + l % D.bx;
-            const int64_t j = D.org[3 * b + 1] + (l / D.bx) % D.by;
-            const int64_t k = D.org[3 * b + 2] + l / (D.bx * D.by);
-            const int64_t qx = i / S.bx, qy = j / S.by, qz = k / S.bz;
+        if ((D.mask[t >> 5] >> (t & 31)) & 1u) {
+            const int i = D.org[3 * b] + D.geo.x(l), j = D.org[3 * b + 1] + D.geo.y(l), k = D.org[3 * b + 2] + D.geo.z(l);
+            const int qx = i >> 3, qy = j >> S.geo.ly, qz = k >> S.geo.lz;
             if (qx < S.nbx && qy < S.nby && qz < S.nbz) {
                 const int32_t sb = S.bvol[qx + S.nbx * (qy + S.nby * qz)];
                 if (sb >= 0) {
-                    const int ls = (int)((i - qx * S.bx) + S.bx * ((j - qy * S.by) + S.by * (k - qz * S.bz)));
+                    const int ls = (i & 7) + 8 * ((j - (qy << S.geo.ly)) + ((k - (qz << S.geo.lz)) << S.geo.ly));
                     uint32_t js;
                     if (seg_index(S.rec[sb], ls >> 2, js)) v = src[js + (uint32_t)(ls & 3)];  // 0 where inactive
                 }
@@ -49,7 +46,7 @@ __global__ void k_remap(CT *dst, const CT *src, RemapSide D, RemapSide S, int64_
 
 static RemapSide side(const gpe_grid *g)
 {
-    return RemapSide{g->d_org, g->d_rec, g->d_mask, g->d_bvol, g->bx, g->by, g->bz, g->nbx, g->nby, g->nbz};
+    return RemapSide{g->d_org, g->d_rec, g->d_mask, g->d_bvol, brick_geo(g->by, g->bz), g->nbx, g->nby, g->nbz};
 }
 
 static bool same_box(const gpe_box &a, const gpe_box &b)

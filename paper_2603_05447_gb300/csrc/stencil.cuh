@@ -1,7 +1,7 @@
 // stencil.cuh -- device building blocks shared by the stencil kernels of
-// libgpeshell (steps, batches, adjoint): the packed segment layout, the
-// per-warp brick tile and its 7-point Laplacian (Eq. (B1)), the ramp
-// schedule and small reductions.  Not part of the ABI.
+// libgpeshell (steps, batches, adjoint): the packed segment layout, per-cell
+// arithmetic, the RK4 stages, the ramp schedule and small reductions; and the
+// per-warp brick tile of the wavefront schedules.  Not part of the ABI.
 #pragma once
 
 #include "gpe_internal.cuh"
@@ -10,7 +10,7 @@
 
 namespace gpe {
 
-// Stencil kernels run one brick per warp; a block holds NW warps, each with
+// The wavefront kernels run one brick per warp; a block holds NW warps, each with
 // its own shared-memory workspace (brick tile with face halo, the 7 brick
 // records and the list of stored segments), passed as dynamic shared memory.
 #ifndef GPE_NW_F
@@ -37,12 +37,6 @@ struct KernelCfg {
 #define GPE_MINB_D 3
 #endif
 #define GPE_BOUNDS(R) __launch_bounds__(KernelCfg<R>::THREADS, (min_blocks<R, BX, BY, BZ>()))
-// kernels templated on the stencil NP: the 19-point form needs more
-// registers; in single precision three blocks an SM (80 registers) beat two
-// (about 105) despite a few spilled bytes in some variants
-#define GPE_BOUNDS_NP(R) \
-    __launch_bounds__(KernelCfg<R>::THREADS, (NP == 19 ? (sizeof(R) == 4 ? 3 : 2) : min_blocks<R, BX, BY, BZ>()))
-
 // ------------------------------------------------------------ packed layout
 // supported brick shapes (shape id, BX, BY, BZ)
 #define GPE_SHAPES(M) \
@@ -55,10 +49,9 @@ struct GridView {
     const BrickRec *rec;
     const BrickRec *rec7;   // per brick: its record, then its six face neighbours' (empty if absent)
     int64_t nb;
-    const BrickRec *rec19;  // 19-point grids: the record, 6 face and 12 edge neighbours' records
 };
 
-inline GridView view(const gpe_grid *g) { return GridView{g->d_nbr, g->d_rec, g->d_rec7, g->nb, g->d_rec19}; }
+inline GridView view(const gpe_grid *g) { return GridView{g->d_nbr, g->d_rec, g->d_rec7, g->nb}; }
 
 // segment geometry of a brick shape (BX must be 8: two segments per row)
 template <int BX, int BY, int BZ>
@@ -481,14 +474,11 @@ __device__ __forceinline__ CT ld1(const CT *p)
 // of the brick and its six face neighbours and the brick's stored segments in
 // order, each as its tile slot and x-halo row (slot | h << 8).  The records of the warp's next brick are fetched into nrec while
 // the current brick is processed.
-template <typename CT, int BX, int BY, int BZ, int NP = 7>
+template <typename CT, int BX, int BY, int BZ>
 struct WarpSpace {
     static constexpr int SX = BX / 4, TY = BY + 2, TZ = BZ + 2;
-    // records: own and 6 face neighbours (7-point), and 12 edge neighbours
-    // (19-point); x-halo columns: rows y in [0, BY) x z in [0, BZ), or with
-    // the halo rows y = -1, BY and planes z = -1, BZ for the 19-point stencil
-    static constexpr int NR = NP == 19 ? 19 : 7;
-    static constexpr int XH = NP == 19 ? TY * TZ : BY * BZ;
+    static constexpr int NR = 7;       // records: own and 6 face neighbours
+    static constexpr int XH = BY * BZ;  // x-halo rows
     static constexpr int NSLOT = SX * TY * TZ;                   // segment slots incl. y/z halos
     static constexpr int UPS = (int)(4 * sizeof(CT) / 16);       // 16-byte units per segment
     // plane stride (in units) = 4 (UPS 2) or 2 (UPS 4) mod 8: the UPS units of
@@ -499,10 +489,9 @@ struct WarpSpace {
     static constexpr int NSEG = Seg<BX, BY, BZ>::NSEG;
     static constexpr int ROW = SX, PLANE = SX * TY;              // slot strides in y and z
     __device__ __forceinline__ static int slot(int hx, int y, int z) { return hx + SX * ((y + 1) + TY * (z + 1)); }
-    __device__ __forceinline__ static int h(int y, int z) { return NP == 19 ? (y + 1) + TY * (z + 1) : y + BY * z; }
+    __device__ __forceinline__ static int h(int y, int z) { return y + BY * z; }
     uint4 units[UPS][PSTR];
-    // x halos: per row (for the 19-point stencil also on the halo rows and
-    // planes) the 16-byte unit of the neighbour segment that holds the halo
+    // x halos: per row the 16-byte unit of the neighbour segment that holds the halo
     // cell (cell 3 of the -x brick's last segment of the row, cell 0 of the
     // +x brick's first), filled by cp.async like the tile.
     static constexpr int XW = 16;
@@ -560,10 +549,10 @@ struct WarpSpace {
     }
 };
 
-template <typename R, int BX, int BY, int BZ, typename CT = typename Cx<R>::T, int NP = 7>
+template <typename R, int BX, int BY, int BZ, typename CT = typename Cx<R>::T>
 constexpr size_t smem_bytes()
 {
-    return (size_t)KernelCfg<R>::NW * sizeof(WarpSpace<CT, BX, BY, BZ, NP>);
+    return (size_t)KernelCfg<R>::NW * sizeof(WarpSpace<CT, BX, BY, BZ>);
 }
 
 // the calling warp's workspace (call once per kernel: it resets the
@@ -576,11 +565,11 @@ constexpr int min_blocks()
     return fit < 1 ? 1 : (fit < cap ? fit : cap);
 }
 
-template <typename R, int BX, int BY, int BZ, typename CT = typename Cx<R>::T, int NP = 7>
-__device__ __forceinline__ WarpSpace<CT, BX, BY, BZ, NP> &warp_space()
+template <typename R, int BX, int BY, int BZ, typename CT = typename Cx<R>::T>
+__device__ __forceinline__ WarpSpace<CT, BX, BY, BZ> &warp_space()
 {
     extern __shared__ __align__(16) unsigned char gpe_smem[];
-    auto &ws = reinterpret_cast<WarpSpace<CT, BX, BY, BZ, NP> *>(gpe_smem)[threadIdx.x >> 5];
+    auto &ws = reinterpret_cast<WarpSpace<CT, BX, BY, BZ> *>(gpe_smem)[threadIdx.x >> 5];
 #if GPE_REC_AHEAD
     if ((threadIdx.x & 31) == 0) ws.nrec_b = -1;
     __syncwarp();
@@ -609,10 +598,9 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src, bool vali
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// Records of brick b (slot 0), of its six face neighbours (slots 1..6,
-// order -x +x -y +y -z +z) and, for the 19-point stencil, of its 12 edge
-// neighbours (slots 7..18: xy, xz, yz edges; order as in the grid builder);
-// an absent neighbour has an empty record.  One row (224 or 608 bytes) moved
+// Records of brick b (slot 0) and of its six face neighbours (slots 1..6, order
+// -x +x -y +y -z +z); an absent neighbour has an empty record.  One row (224
+// bytes) moved
 // into ws.rec: from ws.nrec when it was fetched ahead, else from global
 // memory.  Then the row of brick `next` (if >= 0) is fetched ahead into
 // ws.nrec by cp.async; it completes with the tile's copies.
@@ -620,7 +608,7 @@ template <typename WS>
 __device__ __forceinline__ void fetch_recs(WS &ws, const GridView &G, int64_t b, int64_t next)
 {
     constexpr int NU = 2 * WS::NR;  // 16-byte words of one row of records
-    const uint4 *rows = reinterpret_cast<const uint4 *>(WS::NR == 19 ? G.rec19 : G.rec7);
+    const uint4 *rows = reinterpret_cast<const uint4 *>(G.rec7);
     const int lane = threadIdx.x & 31;
     cp_async_wait_all();
     __syncwarp();
@@ -647,12 +635,6 @@ template <typename XF, typename CT>
 struct HasSeg<XF, CT, std::void_t<decltype(std::declval<const XF &>().seg(std::declval<CT (&)[4]>(), 0u))>>
     : std::true_type {};
 
-// no operands to prefetch
-struct NoPre {
-    struct P {};
-    __device__ __forceinline__ P operator()(uint32_t) const { return P{}; }
-};
-
 // Apply body(idx, pre, c, L) to every stored segment of brick b, one warp
 // (next: the brick the warp takes after b, or -1):
 // idx is the packed index of the segment's first cell, pre what load(idx)
@@ -665,13 +647,14 @@ struct NoPre {
 // stores coalesce.  The first 32 segments' operands are loaded while the tile
 // is in flight, the next 32's while a group is computed.  With xf the identity the tile is filled by cp.async;
 // otherwise through registers, where xf is applied.
-template <int BX, int BY, int BZ, bool CG, typename LAP = LapFull, typename CT, int NP, typename R, typename XF, typename LOAD, typename BODY>
-__device__ __forceinline__ void brick_apply(WarpSpace<CT, BX, BY, BZ, NP> &ws, const GridView &G, int64_t b,
+template <int BX, int BY, int BZ, bool CG, typename LAP = LapFull, typename CT, typename R, typename XF, typename LOAD,
+          typename BODY>
+__device__ __forceinline__ void brick_apply(WarpSpace<CT, BX, BY, BZ> &ws, const GridView &G, int64_t b,
                                             int64_t next, const CT *src, XF xf, R ihx2, R ihy2, R ihz2, LOAD load,
                                             BODY body)
 {
     using S = Seg<BX, BY, BZ>;
-    using W = WarpSpace<CT, BX, BY, BZ, NP>;
+    using W = WarpSpace<CT, BX, BY, BZ>;
     constexpr bool ASYNC = std::is_same<XF, Identity>::value;
     const int lane = threadIdx.x & 31;
     fetch_recs(ws, G, b, next);
@@ -751,24 +734,12 @@ __device__ __forceinline__ void brick_apply(WarpSpace<CT, BX, BY, BZ, NP> &ws, c
     // operands of the first 32 stored segments, while the tile is in flight
     typename std::decay<decltype(load(0u))>::type p0{};
     if (lane < nst) p0 = load(R0.off + 4u * (uint32_t)lane);
-    if constexpr (NP == 19) {
-        // y/z edge rows (y = -1 or BY, z = -1 or BZ) from the four yz-edge
-        // neighbours (records 15..18: (0,-1,-1) (0,+1,-1) (0,-1,+1) (0,+1,+1))
-#pragma unroll
-        for (int t = lane; t < 4 * S::SX * LPS; t += 32) {
-            const int v = t / LPS, e = v / S::SX, hx = v % S::SX;
-            const int ys = (e & 1) ? 0 : BY - 1, zs = (e & 2) ? 0 : BZ - 1;
-            seg_to(ws.rec[15 + e], hx + S::SX * ys + S::PLANE * zs,
-                   W::slot(hx, (e & 1) ? BY : -1, (e & 2) ? BZ : -1), t % LPS);
-        }
-    }
     // -x / +x faces, identity transform: per row one 16-byte unit (the one
     // holding cell 3 of the -x brick's segment, or cell 0 of the +x brick's)
-    // by cp.async; absent segments give a zero unit.  For the 19-point
-    // stencil also the halo rows and planes, from the xy-edge (records
-    // 7..10) and xz-edge (11..14) neighbours; the y-z corner rows, read by
-    // no stencil, are zero.
-    if constexpr (NP != 19 && ASYNC) {
+    // by cp.async; absent segments give a zero unit.  Else single cells
+    // through registers, unrolled, so that a lane's loads are all issued
+    // before the first of them is waited for.
+    if constexpr (ASYNC) {
         for (int u = lane; u < 2 * BY * BZ; u += 32) {
             const int face = u / (BY * BZ), v_ = u % (BY * BZ);
             const int y = v_ % BY, z = v_ / BY;
@@ -777,54 +748,16 @@ __device__ __forceinline__ void brick_apply(WarpSpace<CT, BX, BY, BZ, NP> &ws, c
             const char *g = reinterpret_cast<const char *>(src + (ok ? j : 0u)) + (face == 0 ? 16 * (W::UPS - 1) : 0);
             cp_async16((face == 0 ? ws.xlo_ : ws.xhi_) + 16 * W::h(y, z), g, ok);
         }
-    } else if constexpr (ASYNC) {
-        constexpr int HY = BY + 2, HZ = BZ + 2;
-        for (int u = lane; u < 2 * HY * HZ; u += 32) {
-            const int face = u / (HY * HZ), v_ = u % (HY * HZ);
-            const int y = v_ % HY - 1, z = v_ / HY - 1;
-            const bool yin = y >= 0 && y < BY, zin = z >= 0 && z < BZ;
-            int r = 1 + face, ys = y, zs = z;
-            if (!yin) {
-                r = 7 + face + (y == BY ? 2 : 0);
-                ys = y < 0 ? BY - 1 : 0;
-            } else if (!zin) {
-                r = 11 + face + (z == BZ ? 2 : 0);
-                zs = z < 0 ? BZ - 1 : 0;
-            }
-            uint32_t j = 0;
-            const bool ok = (yin || zin) &&
-                            seg_index(ws.rec[r], (face == 0 ? S::SX - 1 : 0) + S::SX * ys + S::PLANE * zs, j);
-            const char *g = reinterpret_cast<const char *>(src + (ok ? j : 0u)) + (face == 0 ? 16 * (W::UPS - 1) : 0);
-            cp_async16((face == 0 ? ws.xlo_ : ws.xhi_) + 16 * W::h(y, z), g, ok);
-        }
-    } else
-    // -x / +x faces: single cells (x = BX-1 of the -x brick, x = 0 of the +x
-    // brick); for the 19-point stencil also on the halo rows and planes,
-    // from the xy-edge (records 7..10) and xz-edge (11..14) neighbours
-    {
-        constexpr int HY = NP == 19 ? BY + 2 : BY, HZ = NP == 19 ? BZ + 2 : BZ, O = NP == 19 ? 1 : 0;
-        // unrolled, so that a lane's loads are all issued before the first
-        // of them is waited for
+    } else {
 #pragma unroll
-        for (int u = lane; u < 2 * HY * HZ; u += 32) {
-            const int face = u / (HY * HZ), v_ = u % (HY * HZ);
-            const int y = v_ % HY - O, z = v_ / HY - O;
-            const bool yin = y >= 0 && y < BY, zin = z >= 0 && z < BZ;
+        for (int u = lane; u < 2 * BY * BZ; u += 32) {
+            const int face = u / (BY * BZ), v_ = u % (BY * BZ);
+            const int y = v_ % BY, z = v_ / BY;
             CT v = czero<CT>();
-            if (yin || zin) {  // the y-z corners are read by no stencil
-                int r = 1 + face, ys = y, zs = z;
-                if (!yin) {
-                    r = 7 + face + (y == BY ? 2 : 0);
-                    ys = y < 0 ? BY - 1 : 0;
-                } else if (!zin) {
-                    r = 11 + face + (z == BZ ? 2 : 0);
-                    zs = z < 0 ? BZ - 1 : 0;
-                }
-                uint32_t j;
-                if (seg_index(ws.rec[r], (face == 0 ? S::SX - 1 : 0) + S::SX * ys + S::PLANE * zs, j)) {
-                    j += face == 0 ? 3 : 0;
-                    v = xf(ld1<CG>(src + j), j);
-                }
+            uint32_t j;
+            if (seg_index(ws.rec[1 + face], (face == 0 ? S::SX - 1 : 0) + S::SX * y + S::PLANE * z, j)) {
+                j += face == 0 ? 3 : 0;
+                v = xf(ld1<CG>(src + j), j);
             }
             *(face == 0 ? ws.xm_slot(W::h(y, z)) : ws.xp_slot(W::h(y, z))) = v;
         }
@@ -846,54 +779,11 @@ __device__ __forceinline__ void brick_apply(WarpSpace<CT, BX, BY, BZ, NP> &ws, c
         ws.get(sl + W::PLANE, zp);
         const CT xm = hx == 0 ? ws.xm_cell(hrow) : ws.last(sl - 1);
         const CT xp = hx == S::SX - 1 ? ws.xp_cell(hrow) : ws.first(sl + 1);
-        if constexpr (NP != 19) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const CT l = i == 0 ? xm : c[i - 1];
-                const CT rr = i == 3 ? xp : c[i + 1];
-                L[i] = LAP::of(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], LAP::coef(ihx2), LAP::coef(ihy2), LAP::coef(ihz2), c6);
-            }
-        } else {
-            // App. B: the 7-point part plus w_ab (edges_ab - 2 faces_ab + 4 c)
-            // per plane ab, w_ab = (h_a^2 + h_b^2) / (12 h_a^2 h_b^2)
-            // = (1/h_a^2 + 1/h_b^2) / 12.  Each face pair lies in two planes,
-            // so the face and centre terms fold into the 7-point form with
-            //   x: 1/hx^2 - 2 (wxy + wxz), y: 1/hy^2 - 2 (wxy + wyz),
-            //   z: 1/hz^2 - 2 (wxz + wyz), centre: c6 - 4 (wxy + wxz + wyz),
-            // and only the three edge sums remain: + wxy exy + wxz exz + wyz eyz.
-            const R wxy = (ihx2 + ihy2) / (R)12, wxz = (ihx2 + ihz2) / (R)12, wyz = (ihy2 + ihz2) / (R)12;
-            const R ax = ihx2 - (R)2 * (wxy + wxz), ay = ihy2 - (R)2 * (wxy + wyz), az = ihz2 - (R)2 * (wxz + wyz);
-            const R c19 = c6 - (R)4 * (wxy + wxz + wyz);
-            const int row = sl / S::SX, y = row % W::TY - 1, z = row / W::TY - 1;
-            auto left = [&](int s2, int yy, int zz) { return hx == 0 ? ws.xm_cell(W::h(yy, zz)) : ws.last(s2 - 1); };
-            auto right = [&](int s2, int yy, int zz) {
-                return hx == S::SX - 1 ? ws.xp_cell(W::h(yy, zz)) : ws.first(s2 + 1);
-            };
-            const CT yml = left(sl - W::ROW, y - 1, z), ymr = right(sl - W::ROW, y - 1, z);
-            const CT ypl = left(sl + W::ROW, y + 1, z), ypr = right(sl + W::ROW, y + 1, z);
-            const CT zml = left(sl - W::PLANE, y, z - 1), zmr = right(sl - W::PLANE, y, z - 1);
-            const CT zpl = left(sl + W::PLANE, y, z + 1), zpr = right(sl + W::PLANE, y, z + 1);
-            CT eyz[4], t4[4];
-            ws.get(sl - W::ROW - W::PLANE, eyz);
-            ws.get(sl + W::ROW - W::PLANE, t4);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) eyz[i] = vadd(eyz[i], t4[i]);
-            ws.get(sl - W::ROW + W::PLANE, t4);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) eyz[i] = vadd(eyz[i], t4[i]);
-            ws.get(sl + W::ROW + W::PLANE, t4);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                eyz[i] = vadd(eyz[i], t4[i]);
-                const CT l = i == 0 ? xm : c[i - 1];
-                const CT rr = i == 3 ? xp : c[i + 1];
-                const CT exy = vadd(vadd(i == 0 ? yml : ym[i - 1], i == 3 ? ymr : ym[i + 1]),
-                                    vadd(i == 0 ? ypl : yp[i - 1], i == 3 ? ypr : yp[i + 1]));
-                const CT exz = vadd(vadd(i == 0 ? zml : zm[i - 1], i == 3 ? zmr : zm[i + 1]),
-                                    vadd(i == 0 ? zpl : zp[i - 1], i == 3 ? zpr : zp[i + 1]));
-                L[i] = edgev(lapv(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], ax, ay, az, c19), exy, exz, eyz[i], wxy,
-                             wxz, wyz);
-            }
+        for (int i = 0; i < 4; ++i) {
+            const CT l = i == 0 ? xm : c[i - 1];
+            const CT rr = i == 3 ? xp : c[i + 1];
+            L[i] = LAP::of(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], LAP::coef(ihx2), LAP::coef(ihy2), LAP::coef(ihz2), c6);
         }
         body(R0.off + 4u * (uint32_t)r, pre, c, L);
     };
@@ -905,17 +795,6 @@ __device__ __forceinline__ void brick_apply(WarpSpace<CT, BX, BY, BZ, NP> &ws, c
         segment(r, cur);
         cur = nxt;
     }
-}
-
-// the same without prefetched operands: body(idx, c, L)
-template <int BX, int BY, int BZ, bool CG, typename CT, int NP, typename R, typename XF, typename BODY>
-__device__ __forceinline__ void brick_apply(WarpSpace<CT, BX, BY, BZ, NP> &ws, const GridView &G, int64_t b,
-                                            int64_t next, const CT *src, XF xf, R ihx2, R ihy2, R ihz2, BODY body)
-{
-    brick_apply<BX, BY, BZ, CG>(ws, G, b, next, src, xf, ihx2, ihy2, ihz2, NoPre(),
-                                [&](uint32_t idx, const NoPre::P &, const CT(&c)[4], const CT(&L)[4]) {
-                                    body(idx, c, L);
-                                });
 }
 
 // one-time launch preparation of a stencil kernel: dynamic shared memory
@@ -1149,59 +1028,14 @@ struct Rk4Body {
 };
 
 // One RK4 stage on brick b, one warp, lane = segment within each group of 32.
-template <typename R, int BX, int BY, int BZ, bool BLEND, bool CG, int st, int NP = 7>
+template <typename R, int BX, int BY, int BZ, bool BLEND, bool CG, int st>
 __device__ __forceinline__ void rk4_brick(const RkArgs<R> &a, const GridView &G, int64_t b, int64_t next,
-                                          WarpSpace<typename Cx<R>::T, BX, BY, BZ, NP> &ws, R s)
+                                          WarpSpace<typename Cx<R>::T, BX, BY, BZ> &ws, R s)
 {
     using B = Rk4Body<R, BLEND, CG, st>;
     const B body(a, s, rhs_centre(a.ihx2, a.ihy2, a.ihz2));
     brick_apply<BX, BY, BZ, CG, LapRhs>(ws, G, b, next, body.yin(), Identity(), a.ihx2, a.ihy2, a.ihz2,
                                 [&](uint32_t idx) { return body.load(idx); }, body);
 }
-
-// Programmatic dependent launch: a stage kernel launched with programmatic
-// stream serialisation may become resident while the previous stage's last
-// blocks still run.  It waits here until that grid has completed and its
-// writes are visible, then lets its own dependent launch in turn (once every
-// block of this grid has passed this point, so at most two grids share the
-// GPU and none waits for a block that cannot become resident).  Without a
-// programmatic dependency both instructions return at once.
-__device__ __forceinline__ void pdl_enter()
-{
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-template <typename R, int BX, int BY, int BZ, bool BLEND, int ST, int NP = 7>
-__global__ void GPE_BOUNDS_NP(R) k_rk4_staged(const RkArgs<R> a, const GridView G)
-{
-    pdl_enter();
-    constexpr int NW = KernelCfg<R>::NW;
-    auto &ws = warp_space<R, BX, BY, BZ, typename Cx<R>::T, NP>();
-    const int warp = threadIdx.x >> 5;
-    const R s = stage_s<R, BLEND>(a, ST);
-    const int64_t stride = (int64_t)gridDim.x * NW;
-    for (int64_t b = (int64_t)blockIdx.x * NW + warp; b < G.nb; b += stride)
-        rk4_brick<R, BX, BY, BZ, BLEND, false, ST, NP>(a, G, b, b + stride < G.nb ? b + stride : -1, ws, s);
-}
-
-// the four stage kernels of one shape, static (BLEND false) or blended, and
-// their launch shape
-template <typename R, int BX, int BY, int BZ, int NP = 7>
-struct Rk4Stages {
-    using K = void (*)(RkArgs<R>, GridView);
-    static constexpr int NW = KernelCfg<R>::NW;
-    static constexpr int THREADS = 32 * NW;
-    static constexpr size_t smem() { return smem_bytes<R, BX, BY, BZ, typename Cx<R>::T, NP>(); }
-    static K get(bool blend, int st)
-    {
-        static const K t[2][4] = {
-            {k_rk4_staged<R, BX, BY, BZ, false, 0, NP>, k_rk4_staged<R, BX, BY, BZ, false, 1, NP>,
-             k_rk4_staged<R, BX, BY, BZ, false, 2, NP>, k_rk4_staged<R, BX, BY, BZ, false, 3, NP>},
-            {k_rk4_staged<R, BX, BY, BZ, true, 0, NP>, k_rk4_staged<R, BX, BY, BZ, true, 1, NP>,
-             k_rk4_staged<R, BX, BY, BZ, true, 2, NP>, k_rk4_staged<R, BX, BY, BZ, true, 3, NP>}};
-        return t[blend ? 1 : 0][st];
-    }
-};
 
 }  // namespace gpe

@@ -390,22 +390,21 @@ __global__ void k_overlap(const CT *a, const CT *b, int64_t n, double dV, double
 // ------------------------------------------------------------ load / store
 struct BoxI {
     int64_t nx, ny, nz;
-    int BX, BY, BZ;
+    BrickGeo geo;
 };
 
 template <typename CT, bool STORE>
 __global__ void k_dense_io(CT *psi, CT *dense, const int32_t *org, const uint32_t *mask, GridView G, int64_t ns,
                            BoxI bi)
 {
-    const int BC = bi.BX * bi.BY * bi.BZ;
+    const BrickGeo geo = bi.geo;
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < ns; s += (int64_t)gridDim.x * blockDim.x) {
         if (!((mask[s >> 5] >> (s & 31)) & 1u)) continue;
-        const int64_t br = s / BC;
-        const int l = (int)(s % BC);
+        const int64_t br = geo.brick(s);
+        const int l = geo.local(s);
         uint32_t idx;
         if (!seg_index(G.rec[br], l >> 2, idx)) continue;  // cannot happen for an active cell
-        const int64_t i = org[3 * br] + l % bi.BX, j = org[3 * br + 1] + (l / bi.BX) % bi.BY,
-                      k = org[3 * br + 2] + l / (bi.BX * bi.BY);
+        const int64_t i = org[3 * br] + geo.x(l), j = org[3 * br + 1] + geo.y(l), k = org[3 * br + 2] + geo.z(l);
         const int64_t lin = i + bi.nx * (j + bi.ny * k);
         if (STORE) dense[lin] = psi[idx + (l & 3)];
         else psi[idx + (l & 3)] = dense[lin];
@@ -1318,7 +1317,7 @@ extern "C" int gpe_state_load(gpe_state *st, const void *psi, int layout, int on
         return GPE_OK;
     }
     if (layout != GPE_LAYOUT_DENSE) return fail(GPE_ERR_ARG, "unknown layout %d", layout);
-    const BoxI bi{g->box.nx, g->box.ny, g->box.nz, g->bx, g->by, g->bz};
+    const BoxI bi{g->box.nx, g->box.ny, g->box.nz, brick_geo(g->by, g->bz)};
     const size_t dbytes = (size_t)g->box.nx * g->box.ny * g->box.nz * st->elem;
     const void *src = psi;
     void *owned = nullptr;
@@ -1359,7 +1358,7 @@ extern "C" int gpe_state_store(const gpe_state *st, void *psi, int layout, int o
         return GPE_OK;
     }
     if (layout != GPE_LAYOUT_DENSE) return fail(GPE_ERR_ARG, "unknown layout %d", layout);
-    const BoxI bi{g->box.nx, g->box.ny, g->box.nz, g->bx, g->by, g->bz};
+    const BoxI bi{g->box.nx, g->box.ny, g->box.nz, brick_geo(g->by, g->bz)};
     const size_t dbytes = (size_t)g->box.nx * g->box.ny * g->box.nz * st->elem;
     void *dst = psi;
     void *owned = nullptr;

@@ -8,6 +8,7 @@
 // memory; its members, sorted (whole segments first, then those of which one
 // cell is read, each by packed position, so that neighbouring lanes gather
 // neighbouring segments), are the halo list.
+#include <algorithm>
 #include <mutex>
 #include <unordered_map>
 
@@ -68,7 +69,9 @@ __device__ __forceinline__ uint32_t seg_at(const TileSrc &S, int64_t sx, int64_t
 // uses of a halo segment
 constexpr uint32_t USE_FIRST = 1, USE_LAST = 2, USE_WHOLE = 4;
 
-template <int NP, bool EMIT>
+// Rows of `stride` entries; a tile with more halo segments than fit leaves its
+// lists out (hmax tells, and the caller builds again with longer rows).
+template <int NP>
 __global__ void __launch_bounds__(TILE) k_tiles(const TileSrc S, int stride, uint2 *nbr, uint4 *nbr19, uint32_t *halo,
                                                 int *hmax)
 {
@@ -80,8 +83,9 @@ __global__ void __launch_bounds__(TILE) k_tiles(const TileSrc S, int stride, uin
                                  {0, -1, -1, 4}, {0, 1, -1, 4}, {0, -1, 1, 4}, {0, 1, 1, 4},  {-1, -1, 0, 2}, {1, -1, 0, 1},
                                  {-1, 1, 0, 2}, {1, 1, 0, 1},  {-1, 0, -1, 2}, {1, 0, -1, 1}, {-1, 0, 1, 2}, {1, 0, 1, 1}};
     __shared__ uint32_t key[HS];
-    __shared__ uint32_t use[HS];  // uses, then the slot
-    __shared__ uint32_t list[EMIT ? HS : 1];
+    __shared__ uint32_t use[HS];   // uses, then the slot
+    __shared__ uint32_t list[NF * TILE];   // the set's members as they sort
+    __shared__ uint16_t where[NF * TILE];  // and their hash slots
     __shared__ int64_t b0;
     __shared__ int n_all, n_whole;
     const int tid = threadIdx.x;
@@ -127,17 +131,17 @@ __global__ void __launch_bounds__(TILE) k_tiles(const TileSrc S, int stride, uin
         const bool wh = whole(use[i]);
         const int at = atomicAdd(&n_all, 1);
         if (wh) atomicAdd(&n_whole, 1);
-        if constexpr (EMIT) list[at] = key[i] | (wh ? 0u : 1u << 31);
+        list[at] = key[i] | (wh ? 0u : 1u << 31);
+        where[at] = (uint16_t)i;
     }
     __syncthreads();
-    if constexpr (!EMIT) {
-        if (tid == 0) atomicMax(hmax, n_all);
-        return;
-    }
     const int n = n_all;
-    for (int i = tid; i < HS; i += TILE) {
-        if (key[i] == NO_SEG) continue;
-        const uint32_t u = use[i], v = key[i] | (whole(u) ? 0u : 1u << 31);
+    if (tid == 0 && n > __ldcg(hmax)) atomicMax(hmax, n);
+    if (n + 1 > stride) return;
+    for (int t = tid; t < n; t += TILE) {
+        const uint32_t v = list[t];
+        const int i = where[t];
+        const uint32_t u = use[i];
         int rank = 0;
         for (int j = 0; j < n; ++j) rank += list[j] < v;
         // whole segments from the front of the tile's entries, single cells from the back
@@ -181,23 +185,59 @@ void tiles_free(TileTab &t)
     t = TileTab{};
 }
 
+// rows of one stride to rows of another, at least as long as every list
+__global__ void k_tile_rows(const uint32_t *from, int sf, uint32_t *to, int st, int ntiles)
+{
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const uint32_t *r = from + (size_t)tile * sf;
+        uint32_t *w = to + (size_t)tile * st;
+        const int whole = r[0] & 0xffff, single = r[0] >> 16;
+        for (int i = threadIdx.x; i <= whole; i += blockDim.x) w[i] = r[i];
+        for (int i = threadIdx.x; i < single; i += blockDim.x) w[st - 1 - i] = r[sf - 1 - i];
+    }
+}
+
 template <int NP>
 static int build(const TileSrc &S, TileTab &t, int *d_hmax, cudaStream_t st)
 {
-    GPE_TRY_CUDA(cudaMemsetAsync(d_hmax, 0, sizeof(int), st));
-    k_tiles<NP, false><<<(unsigned)t.ntiles, TILE, 0, st>>>(S, 0, nullptr, nullptr, nullptr, d_hmax);
-    GPE_LAUNCH_CHECK();
-    int hmax = 0;
-    GPE_TRY_CUDA(cudaMemcpyAsync(&hmax, d_hmax, sizeof hmax, cudaMemcpyDeviceToHost, st));
-    GPE_TRY_CUDA(cudaStreamSynchronize(st));
-    t.stride = (hmax + 8) / 8 * 8;  // and the count; whole sectors
-    t.nslot = TILE + 1 + hmax;
-    GPE_TRY(dev_alloc_t(&t.d_halo, (size_t)t.ntiles * t.stride));
+    // most grids' lists fit rows of 256 (thin shells: at most 208 segments
+    // with the 7-point stencil); the rows kept are as long as the longest list
+    int stride = NP == 19 ? 512 : 256, hmax = 0;
+    uint32_t *rows = nullptr;
     if (NP == 19) GPE_TRY(dev_alloc_t(&t.d_nbr19, 2 * (size_t)t.nseg));
     else GPE_TRY(dev_alloc_t(&t.d_nbr, (size_t)t.nseg));
-    k_tiles<NP, true><<<(unsigned)t.ntiles, TILE, 0, st>>>(S, t.stride, t.d_nbr, t.d_nbr19, t.d_halo, nullptr);
-    GPE_LAUNCH_CHECK();
-    return GPE_OK;
+    int rc = GPE_OK;
+    for (;;) {
+        rc = dev_alloc_t(&rows, (size_t)t.ntiles * stride);
+        if (rc != GPE_OK) return rc;
+        cudaError_t e = cudaMemsetAsync(d_hmax, 0, sizeof(int), st);
+        if (e == cudaSuccess) {
+            k_tiles<NP><<<(unsigned)t.ntiles, TILE, 0, st>>>(S, stride, t.d_nbr, t.d_nbr19, rows, d_hmax);
+            count_launch();
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&hmax, d_hmax, sizeof hmax, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) {
+            dev_free(rows);
+            return cuda_fail(e, "k_tiles", __FILE__, __LINE__);
+        }
+        if (hmax + 1 <= stride) break;
+        dev_free(rows);
+        rows = nullptr;
+        stride = (hmax + 8) / 8 * 8;
+    }
+    t.stride = (hmax + 8) / 8 * 8;  // and the count; whole sectors
+    t.nslot = TILE + 1 + hmax;
+    rc = dev_alloc_t(&t.d_halo, (size_t)t.ntiles * t.stride);
+    if (rc == GPE_OK) {
+        k_tile_rows<<<(unsigned)std::min(t.ntiles, 65536), 128, 0, st>>>(rows, stride, t.d_halo, t.stride, t.ntiles);
+        count_launch();
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) rc = cuda_fail(e, "k_tile_rows", __FILE__, __LINE__);
+    }
+    dev_free(rows);  // waits for the copy
+    return rc;
 }
 
 // the tiles of a grid whose records and brick volume are in place; the work is
