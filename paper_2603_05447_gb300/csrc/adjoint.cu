@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? 5 : 2) k_adj_stage(cons
     };
     XF xf{};
     if constexpr (POS == 0) xf.s = a.m_scale;
-    Sum64<R> dot;
+    Sum64<R> dot[1];
     int n = 0;
     tile_loop<7>(T, a.mu_in, xf, a.ihx2, a.ihy2, a.ihz2, EveryTile(),
                  [&](uint32_t idx, uint32_t m) {
@@ -141,12 +141,12 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? 5 : 2) k_adj_stage(cons
                          st4(a.acc + idx, nacc);
                          st4(a.mu_out + idx, mo);
                      }
-                     dot.add(d4);
-                     if (++n % SUM_FLUSH == 0) dot.flush();
+                     dot[0].add(d4);
+                     if (++n % SUM_FLUSH == 0) dot[0].flush();
                  });
-    dot.flush();
-    double acc[1] = {dot.tot}, tot[1];
-    if (reduce_finish<1>(acc, a.partials, a.counter, tot) && threadIdx.x == 0) {
+    double tot[1];
+    block_totals<1>(dot, T.ntiles >= SUM_FLUSH * (int)gridDim.x, tot);
+    if (launch_totals<1>(tot, a.partials, a.counter) && threadIdx.x == 0) {
         a.grad[a.k0] += a.w0 * tot[0];
         a.grad[a.k0 + 1] += a.w1 * tot[0];
     }

@@ -70,7 +70,7 @@ struct ShellWalk {
     uint32_t cur = 0xffffffffu, next = 0;
     bool live = false;
     R g = 0, dt = 0, ihx2 = 0, ihy2 = 0, ihz2 = 0, scale = 0;
-    Sum64<R> sum[NS > 0 ? NS : 1];
+    Sum64<R> sum[NS > 0 ? NS : 1];  // NS 5: the fifth counts non-finite cells
     int nf = 0, n = 0;
     __device__ __forceinline__ ShellWalk(const BatchArgs<R, CT> &a_, uint32_t nt_) : a(a_), nt(nt_)
     {
@@ -81,19 +81,15 @@ struct ShellWalk {
     {
         if constexpr (NS > 0) {
             if (!live) return;
-            double *p = a.part + 5 * (size_t)part_of(a.tile_base[cur], blockIdx.x, gridDim.x);
+            double *p = a.part + 5 * (size_t)part_of(a.tile_base[cur], blockIdx.x, gridDim.x), tot[NS];
+            if constexpr (NS == 5) sum[4].add((R)nf);
+            block_totals<NS>(sum, nt >= SUM_FLUSH * gridDim.x, tot);
 #pragma unroll
             for (int k = 0; k < NS; ++k) {
-                sum[k].flush();
-                const double x = block_sum(sum[k].tot);
-                if (threadIdx.x == 0) p[k] = x;
+                if (threadIdx.x == 0) p[k] = tot[k];
                 sum[k] = Sum64<R>();
             }
-            if constexpr (NS == 4) {
-                const double x = block_sum((double)nf);
-                if (threadIdx.x == 0) p[4] = x;
-                nf = 0;
-            }
+            nf = 0;
             n = 0;
         }
     }
@@ -120,7 +116,7 @@ struct ShellWalk {
     {
         if (++n % SUM_FLUSH == 0) {
 #pragma unroll
-            for (int k = 0; k < NS; ++k) sum[k].flush();
+            for (int k = 0; k < (NS == 5 ? 4 : NS); ++k) sum[k].flush();
         }
     }
 };
@@ -224,21 +220,13 @@ __global__ void k_batch_reset_scale(ShellParams *sh, int n)
 template <typename R, typename CT>
 __global__ void GPE_TILE_BOUNDS(R) k_batch_obs(const BatchArgs<R, CT> a, const TileView T)
 {
-    ShellWalk<R, CT, 4> w(a, (uint32_t)T.ntiles);
+    ShellWalk<R, CT, 5> w(a, (uint32_t)T.ntiles);
     tile_loop<7>(T, (const CT *)a.psi, Plain(), w.ihx2, w.ihy2, w.ihz2, [&](uint32_t tile) { return w.enter(tile); },
-                 [&](uint32_t idx, uint32_t n) { prefetch_l2(a.V + idx, n * (uint32_t)sizeof(R)); }, VLoad<R>{a.V, nullptr},
-                 [&](uint32_t, const typename VLoad<R>::P &p, const CT(&c)[4], const CT(&L)[4]) {
-                     R t[4] = {(R)0, (R)0, (R)0, (R)0};  // the segment's terms, added to the FP64 sums once
-#pragma unroll
-                     for (int i = 0; i < 4; ++i) {
-                         if (!active_v(p.V0[i])) continue;
-                         const R rho = norm2(c[i]);
-                         t[0] = add_rn(t[0], rho);
-                         t[1] = add_rn(t[1], (R)(-0.5) * dotre(c[i], L[i]));
-                         t[2] = add_rn(t[2], p.V0[i] * rho);
-                         t[3] = add_rn(t[3], (R)0.5 * w.g * rho * rho);
-                         w.nf += finite_v(c[i]) ? 0 : 1;
-                     }
+                 [&](uint32_t idx, uint32_t n) { prefetch_l2(a.V + idx, n * (uint32_t)sizeof(R)); },
+                 VLoad<R, false>{a.V, nullptr},
+                 [&](uint32_t, const typename VLoad<R, false>::P &p, const CT(&c)[4], const CT(&L)[4]) {
+                     R t[4];
+                     obs_terms<false>(p, (R)0, w.g, c, L, t, w.nf);
 #pragma unroll
                      for (int k = 0; k < 4; ++k) w.sum[k].add(t[k]);
                      w.added();

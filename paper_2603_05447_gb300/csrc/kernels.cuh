@@ -132,37 +132,137 @@ struct TileDiag {
     __device__ __forceinline__ void cell(CT &v, const R &e) const { v = d.apply(v, e); }
 };
 
-// An FP64 sum of many single-precision terms off the FP64 pipe, where an add
-// and a conversion issue at 1/64 of the FP32 rate: the terms are added as an
+// An FP64 sum of many single-precision terms off the FP64 pipe, where every
+// add and conversion issues at 1/64 of the FP32 rate: the terms are added as an
 // unevaluated pair of floats (hi + lo, each addition's rounding error found
-// exactly by Knuth's two-sum and kept in lo, which itself stays good to
-// 2^-24 of 2^-24), and the pair goes into the FP64 total every FLUSH terms.
-// Double-precision terms are added as they are.
+// exactly by Knuth's two-sum and kept in lo), and the pair goes into an FP64
+// total every SUM_FLUSH terms.  After n additions the pair is good to about n
+// 2^-48 of the sum, against the 2^-25 of every term.  Double-precision terms
+// are added as they are.
 template <typename R>
 struct Sum64 {
     double tot = 0.0;
     __device__ __forceinline__ void add(double x) { tot += x; }
     __device__ __forceinline__ void flush() {}
 };
+// a call, so that the compiler branches around it: FP64 instructions that are
+// predicated off still take their turn in the pipe
+static __device__ __noinline__ double add_pair(double tot, float hi, float lo)
+{
+    tot += (double)hi;
+    if (isfinite(lo)) tot += (double)lo;  // an infinite or NaN term shows in hi
+    return tot;
+}
 template <>
 struct Sum64<float> {
     double tot = 0.0;
     float hi = 0.0f, lo = 0.0f;
-    __device__ __forceinline__ void add(float x)
+    __device__ __forceinline__ void add(float x) { add(x, 0.0f); }
+    __device__ __forceinline__ void add(float x, float xl)
     {
         const float s = __fadd_rn(hi, x), b = __fadd_rn(s, -hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -b)), __fadd_rn(x, -b)));
+        const float e = __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -b)), __fadd_rn(x, -b));
+        lo = __fadd_rn(lo, __fadd_rn(e, xl));
         hi = s;
     }
     __device__ __forceinline__ void flush()
     {
-        tot += (double)hi;
-        if (isfinite(lo)) tot += (double)lo;  // an infinite or NaN term shows in hi
+        tot = add_pair(tot, hi, lo);
         hi = 0.0f;
         lo = 0.0f;
     }
 };
-constexpr int SUM_FLUSH = 16;
+constexpr int SUM_FLUSH = 64;
+
+// The block's totals of NV sums, to every thread.  Few FP64 instructions, since
+// every warp of an SM queues for the one pipe at a kernel's end: pairs are
+// added across a warp as pairs, and one warp converts; doubles are added
+// across the block by a warp a sum.  flushed: threads may have flushed.
+// Called by the whole block of TILE threads.
+template <int NV>
+__device__ __forceinline__ void block_totals(Sum64<float> (&s)[NV], bool flushed, double (&out)[NV])
+{
+    constexpr int W = TILE / 32;
+    __shared__ float2 sp[NV][W];
+    __shared__ double sd[NV][W], so[NV];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        for (int off = 16; off > 0; off >>= 1)
+            s[k].add(__shfl_down_sync(0xffffffffu, s[k].hi, off), __shfl_down_sync(0xffffffffu, s[k].lo, off));
+        if (lane == 0) sp[k][warp] = make_float2(s[k].hi, s[k].lo);
+        if (flushed) {
+            double x = s[k].tot;
+            for (int off = 16; off > 0; off >>= 1) x += __shfl_down_sync(0xffffffffu, x, off);
+            if (lane == 0) sd[k][warp] = x;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < NV) {
+        double x = 0.0;
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            const float2 p = sp[threadIdx.x][w];
+            x = add_pair(x, p.x, p.y);
+            if (flushed) x += sd[threadIdx.x][w];
+        }
+        so[threadIdx.x] = x;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NV; ++k) out[k] = so[k];
+    __syncthreads();  // the arrays may be used again
+}
+template <int NV>
+__device__ __forceinline__ void block_totals(Sum64<double> (&s)[NV], bool, double (&out)[NV])
+{
+    __shared__ double sm[NV][TILE], so[NV];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) sm[k][threadIdx.x] = s[k].tot;
+    __syncthreads();
+    for (int k = warp; k < NV; k += TILE / 32) {
+        double x = (sm[k][lane] + sm[k][lane + 32]) + (sm[k][lane + 64] + sm[k][lane + 96]);
+        for (int off = 16; off > 0; off >>= 1) x += __shfl_down_sync(0xffffffffu, x, off);
+        if (lane == 0) so[k] = x;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NV; ++k) out[k] = so[k];
+    __syncthreads();
+}
+
+// The launch's totals of the blocks' NV values v (deterministic: the last block
+// to arrive adds the blocks' values in a fixed order).  True in that block,
+// whose threads then hold the totals.
+template <int NV>
+__device__ __forceinline__ bool launch_totals(double (&v)[NV], double *partials, unsigned int *counter)
+{
+    __shared__ bool is_last;
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) partials[(int64_t)blockIdx.x * NV + k] = v[k];
+        __threadfence();
+        is_last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!is_last) return false;
+    __threadfence();
+    Sum64<double> s[NV];
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += 4 * TILE) {
+        double x[4][NV];  // four blocks' values in flight a thread
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int k = 0; k < NV; ++k)
+                x[q][k] = i + q * TILE < (int)gridDim.x ? __ldcg(&partials[(int64_t)(i + q * TILE) * NV + k]) : 0.0;
+#pragma unroll
+        for (int k = 0; k < NV; ++k) s[k].add((x[0][k] + x[1][k]) + (x[2][k] + x[3][k]));
+    }
+    block_totals<NV>(s, false, v);
+    if (threadIdx.x == 0) *counter = 0u;
+    return true;
+}
 
 template <typename R, typename CT, int NP>
 __global__ void GPE_TILE_BOUNDS(R) k_itp_a(const ItpArgs<R, CT> a, const TileView T)
@@ -188,7 +288,7 @@ __global__ void GPE_TILE_BOUNDS(R) k_itp_b(const ItpArgs<R, CT> a, const TileVie
 {
     const R hg = a.g * a.dt / (R)2;
     const R q4 = a.dt / (R)4;
-    Sum64<R> norm;
+    Sum64<R> norm[1];
     int n = 0;
     tile_loop<NP>(T, (const CT *)a.tmp, Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
                   [&](uint32_t idx, uint32_t n) { prefetch_l2(a.E + idx, n * (uint32_t)sizeof(R)); }, ELoad<R>{a.E},
@@ -203,12 +303,12 @@ __global__ void GPE_TILE_BOUNDS(R) k_itp_b(const ItpArgs<R, CT> a, const TileVie
                           n4 = add_rn(n4, norm2(o[i]));
                       }
                       st4(a.psi + idx, o);
-                      norm.add(n4);
-                      if (++n % SUM_FLUSH == 0) norm.flush();
+                      norm[0].add(n4);
+                      if (++n % SUM_FLUSH == 0) norm[0].flush();
                   });
-    norm.flush();
-    double acc[1] = {norm.tot}, tot[1];
-    if (reduce_finish<1>(acc, partials, counter, tot) && threadIdx.x == 0) {
+    double tot[1];
+    block_totals<1>(norm, T.ntiles >= SUM_FLUSH * (int)gridDim.x, tot);
+    if (launch_totals<1>(tot, partials, counter) && threadIdx.x == 0) {
         const double nrm = tot[0] * a.dV;
         a.scalars[0] = sqrt(a.N / nrm);
         a.scalars[1] = nrm;
@@ -242,47 +342,77 @@ struct ObsArgs {
 };
 
 // a segment's potential(s), loaded ahead of its terms
-template <typename R>
+template <typename R, bool BLEND>
 struct VLoad {
     const R *V0, *V1;
     struct P {
-        R V0[4], V1[4];
+        R V0[4], V1[BLEND ? 4 : 1];
     };
     __device__ __forceinline__ P operator()(uint32_t idx) const
     {
         P p;
         ldr4(V0 + idx, p.V0);
-        if (V1) ldr4(V1 + idx, p.V1);
+        if constexpr (BLEND) ldr4(V1 + idx, p.V1);
         return p;
     }
 };
 
-template <typename R, typename CT, int NP>
+__device__ __forceinline__ bool finite1(float v) { return (__float_as_uint(v) & 0x7f800000u) != 0x7f800000u; }
+__device__ __forceinline__ bool finite1(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+template <typename CT>
+__device__ __forceinline__ bool finite_v(const CT &v)
+{
+    if constexpr (is_cplx<CT>())
+        return finite1(v.x) && finite1(v.y);
+    else
+        return finite1(v);
+}
+
+// What a segment adds to the observables: norm, ekin, epot, eint, summed over
+// its four cells in the state precision, then added to the FP64 sums once; and
+// its non-finite cells.
+template <bool BLEND, typename R, typename CT>
+__device__ __forceinline__ void obs_terms(const typename VLoad<R, BLEND>::P &p, R s, R g, const CT (&c)[4],
+                                          const CT (&L)[4], R (&t)[4], int &nf)
+{
+#pragma unroll
+    for (int k = 0; k < 4; ++k) t[k] = (R)0;
+    bool fin = true;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const bool act = active_v(p.V0[i]);
+        R V = p.V0[i];
+        if constexpr (BLEND) V = ((R)1 - s) * p.V0[i] + s * p.V1[i];
+        const R rho = act ? norm2(c[i]) : (R)0;
+        t[0] = add_rn(t[0], rho);
+        t[1] = add_rn(t[1], act ? (R)(-0.5) * dotre(c[i], L[i]) : (R)0);
+        t[2] = add_rn(t[2], act ? V * rho : (R)0);
+        t[3] = add_rn(t[3], (R)0.5 * g * rho * rho);
+        fin = fin && (!act || finite_v(c[i]));
+    }
+    if (!fin) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) nf += active_v(p.V0[i]) && !finite_v(c[i]) ? 1 : 0;
+    }
+}
+
+// 512^3 shell, complex64: 80 us warp by brick with ten FP64 instructions a
+// segment, 66 on tiles with the sums flushed by every warp at its end, 40 now;
+// one pass over psi and V at 3.7 TB/s, the shared-memory pipe 76 % busy.
+template <typename R, typename CT, int NP, bool BLEND>
 __global__ void GPE_TILE_BOUNDS(R) k_obs(const ObsArgs<R, CT> a, const TileView T)
 {
-    Sum64<R> sum[4];  // norm, ekin, epot, eint
+    Sum64<R> sum[5];  // norm, ekin, epot, eint, nonfinite
     int n = 0, nf = 0;
     tile_loop<NP>(T, a.psi, Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
                   [&](uint32_t idx, uint32_t n) {
                       prefetch_l2(a.V0 + idx, n * (uint32_t)sizeof(R));
-                      if (a.V1) prefetch_l2(a.V1 + idx, n * (uint32_t)sizeof(R));
+                      if constexpr (BLEND) prefetch_l2(a.V1 + idx, n * (uint32_t)sizeof(R));
                   },
-                  VLoad<R>{a.V0, a.V1},
-                  [&](uint32_t, const typename VLoad<R>::P &p, const CT(&c)[4], const CT(&L)[4]) {
-                      // the segment's four terms summed in the state precision, then
-                      // added to the FP64 sums once
-                      R t[4] = {(R)0, (R)0, (R)0, (R)0};
-#pragma unroll
-                      for (int i = 0; i < 4; ++i) {
-                          if (!active_v(p.V0[i])) continue;
-                          const R V = a.V1 ? ((R)1 - a.s) * p.V0[i] + a.s * p.V1[i] : p.V0[i];
-                          const R rho = norm2(c[i]);
-                          t[0] = add_rn(t[0], rho);
-                          t[1] = add_rn(t[1], (R)(-0.5) * dotre(c[i], L[i]));
-                          t[2] = add_rn(t[2], V * rho);
-                          t[3] = add_rn(t[3], (R)0.5 * a.g * rho * rho);
-                          nf += finite_v(c[i]) ? 0 : 1;
-                      }
+                  VLoad<R, BLEND>{a.V0, a.V1},
+                  [&](uint32_t, const typename VLoad<R, BLEND>::P &p, const CT(&c)[4], const CT(&L)[4]) {
+                      R t[4];
+                      obs_terms<BLEND>(p, a.s, a.g, c, L, t, nf);
 #pragma unroll
                       for (int k = 0; k < 4; ++k) sum[k].add(t[k]);
                       if (++n % SUM_FLUSH == 0) {
@@ -290,15 +420,10 @@ __global__ void GPE_TILE_BOUNDS(R) k_obs(const ObsArgs<R, CT> a, const TileView 
                           for (int k = 0; k < 4; ++k) sum[k].flush();
                       }
                   });
-    double acc[5];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        sum[k].flush();
-        acc[k] = sum[k].tot;
-    }
-    acc[4] = (double)nf;
+    sum[4].add((R)nf);
     double tot[5];
-    if (reduce_finish<5>(acc, a.partials, a.counter, tot) && threadIdx.x == 0) {
+    block_totals<5>(sum, T.ntiles >= SUM_FLUSH * (int)gridDim.x, tot);
+    if (launch_totals<5>(tot, a.partials, a.counter) && threadIdx.x == 0) {
         gpe_obs o;
         o.norm = tot[0] * a.dV;
         o.e_kin = tot[1] * a.dV;
@@ -389,7 +514,7 @@ inline int obs_run(const gpe_state *stc, double gg, double sb, cudaStream_t s)
     a.counter = st->red.counter;
     a.out = (gpe_obs *)(st->red.scalars + 2);
     const TileLaunch L = tile_launch<CT>(g);
-    auto k = k_obs<R, CT, NP>;
+    auto k = a.V1 ? k_obs<R, CT, NP, true> : k_obs<R, CT, NP, false>;
     k<<<tile_blocks(k, g->nsm, L.T.ntiles, L.smem), TILE, L.smem, s>>>(a, L.T);
     GPE_LAUNCH_CHECK();
     return GPE_OK;

@@ -186,14 +186,6 @@ __device__ __forceinline__ typename RealOf<CT>::T dotre(const CT &a, const CT &b
     else
         return a * b;
 }
-template <typename CT>
-__device__ __forceinline__ bool finite_v(const CT &v)
-{
-    if constexpr (is_cplx<CT>())
-        return isfinite(v.x) && isfinite(v.y);
-    else
-        return isfinite(v);
-}
 __device__ __forceinline__ float2 vadd(const float2 &a, const float2 &b) { return add2(a, b); }
 template <typename CT>
 __device__ __forceinline__ CT vadd(const CT &a, const CT &b)

@@ -87,8 +87,9 @@ struct TileMem {
     }
 };
 
-// shared memory a block may have, less a margin for static arrays
-constexpr size_t TILE_SMEM_MAX = 224 * 1024;
+// shared memory a block may have, less the reductions' static arrays (a tile
+// needs at most 155 KB: 19-point, complex128, 2433 slots)
+constexpr size_t TILE_SMEM_MAX = 208 * 1024;
 
 // a segment's neighbour slots
 template <int NP>
