@@ -251,6 +251,8 @@ struct gpe_state {
     void *d_E = nullptr;    // ITP exp(-V dt/2), state precision
     double E_dt = -1.0;     // dt that d_E was made for
     double *d_clock = nullptr;  // device time base for ramps
+    double *d_stab = nullptr;   // schedule values of the next steps' stages (ramps; made on first use)
+    int stab_cap = 0;           // steps it holds
     gpe::RedScratch red;
     gpe_obs *h_obs = nullptr;   // pinned host landing buffer
     // wavefront bookkeeping: per-chunk completion stamps (monotonic), the
@@ -271,6 +273,7 @@ struct gpe_state {
 namespace gpe {
 int tiles_build(gpe_grid *g, cudaStream_t st);
 void tiles_free(TileTab &t);
+int ensure_stab(gpe_state *st, int steps);      // room for the schedule values of `steps` steps
 int ensure_work(gpe_state *st, int n);          // allocate d_work[0..n-1] (zeroed)
 // step drivers of 19-point grids (step19.cu)
 int rk4_run19(gpe_state *st, const gpe_real_params *p, int64_t nsteps, double t0, cudaStream_t s);

@@ -520,6 +520,25 @@ inline int obs_run(const gpe_state *stc, double gg, double sb, cudaStream_t s)
     return GPE_OK;
 }
 
+// The schedule's values for n steps of nc stages, at *clock + (n0 + m) dt +
+// c[k] dt, then the clock moved on by `advance`: one block.  Every thread of a
+// stage kernel used to evaluate its own (21 FP64 instructions with a division,
+// 24 warps an SM queueing for the FP64 pipe: 4.7 of 39 us of a 512^3 stage).
+struct StageTimes {
+    double c[6];
+};
+static __global__ void k_ramp_table(Ramp r, double *clock, double advance, int64_t n0, int n, int nc, StageTimes c,
+                                    double dt, double *tab)
+{
+    const double t = *clock;
+    __syncthreads();
+    for (int i = threadIdx.x; i < n * nc; i += blockDim.x)
+        tab[i] = ramp_s(r, t + (double)(n0 + i / nc) * dt + c.c[i % nc] * dt);
+    if (threadIdx.x == 0 && advance != 0.0) *clock = t + advance;
+}
+constexpr StageTimes RK4_TIMES = {{0.0, 0.5, 1.0}};
+constexpr int STAB_STEPS = 256;  // steps a table is made for at a time
+
 // arguments of the RK4 stages of a state (ramps: the clock is set to t0)
 template <typename R>
 inline int rk4_args(gpe_state *st, const gpe_real_params *p, RkArgs<R> &a)
@@ -549,9 +568,10 @@ inline int rk4_args(gpe_state *st, const gpe_real_params *p, RkArgs<R> &a)
     return GPE_OK;
 }
 
-// cnt RK4 steps of four staged passes, stage times relative to the clock
+// cnt RK4 steps of four staged passes, stage times relative to the clock, which
+// is then moved on if `advance`; a ramp needs ensure_stab before
 template <typename R, int NP>
-inline int rk4_steps(gpe_state *st, RkArgs<R> a, bool blend, int64_t cnt, cudaStream_t s)
+inline int rk4_steps(gpe_state *st, RkArgs<R> a, bool blend, int64_t cnt, bool advance, cudaStream_t s)
 {
     const gpe_grid *g = st->grid;
     using RT = Rk4Tiles<R, NP>;
@@ -563,8 +583,16 @@ inline int rk4_steps(gpe_state *st, RkArgs<R> a, bool blend, int64_t cnt, cudaSt
         nblk[stg] = tile_blocks(k[stg], g->nsm, L.T.ntiles, L.smem);
     }
     for (int64_t n = 0; n < cnt; ++n) {
-        a.t_off = (double)n * a.dtd;
+        const int m = blend ? (int)(n % st->stab_cap) : 0;
+        if (blend && m == 0) {
+            const int64_t left = cnt - n;
+            const int here = (int)(left < st->stab_cap ? left : st->stab_cap);
+            k_ramp_table<<<1, 256, 0, s>>>(a.ramp, st->d_clock, advance && here == left ? (double)cnt * a.dtd : 0.0, n,
+                                           here, 3, RK4_TIMES, a.dtd, st->d_stab);
+            GPE_LAUNCH_CHECK();
+        }
         for (int stg = 0; stg < 4; ++stg) {
+            a.stab = st->d_stab + 3 * m + (stg + 1) / 2;  // t, t + dt/2 twice, t + dt
             k[stg]<<<nblk[stg], TILE, L.smem, s>>>(a, L.T);
             GPE_LAUNCH_CHECK();
         }

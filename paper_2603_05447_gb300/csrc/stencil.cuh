@@ -888,6 +888,7 @@ struct RkArgs {
     const R *V1;
     R ihx2, ihy2, ihz2, g, dt;
     Ramp ramp;
+    const double *stab;  // tile kernels: this stage's value of the schedule (k_ramp_table)
     double t_off;  // stage-0 time of this step relative to *ramp.clock
     double dtd;    // dt in FP64 for stage times
 };

@@ -456,6 +456,23 @@ static const void *pinned_view(const void *p)
 }
 
 // ------------------------------------------------------------ state helpers
+int ensure_stab(gpe_state *st, int steps)
+{
+    if (st->stab_cap >= steps) return GPE_OK;
+    // a captured graph may hold the old table
+    if (st->gexec[0]) {
+        GPE_TRY_CUDA(cudaDeviceSynchronize());
+        cudaGraphExecDestroy(st->gexec[0]);
+        st->gexec[0] = nullptr;
+    }
+    dev_free(st->d_stab);
+    st->d_stab = nullptr;
+    st->stab_cap = 0;
+    GPE_TRY(dev_alloc_t(&st->d_stab, 6 * (size_t)steps));
+    st->stab_cap = steps;
+    return GPE_OK;
+}
+
 int ensure_work(gpe_state *st, int n)
 {
     for (int i = 0; i < n; ++i) {
@@ -867,8 +884,7 @@ static int rk4_run(gpe_state *st, const gpe_real_params *p, int64_t nsteps, doub
         }
         return record(s, left);
     }
-    // steps n0 .. n0+cnt-1 with stage times relative to the device clock
-    auto record = [&](cudaStream_t cs, int64_t cnt) -> int { return rk4_steps<R, 7>(st, a, blend, cnt, cs); };
+    if (blend) GPE_TRY(ensure_stab(st, std::max(STAB_STEPS, st->graph_steps)));
     int64_t left = nsteps;
     if (use_graph(st, s, nsteps)) {
         const int G_ = st->graph_steps;
@@ -876,18 +892,11 @@ static int rk4_run(gpe_state *st, const gpe_real_params *p, int64_t nsteps, doub
         const void *ptrs[2] = {a.V0, a.V1};
         key = fnv1a(ptrs, sizeof ptrs, key);
         key = fnv1a(&G_, sizeof G_, key);
-        auto rec_block = [&](cudaStream_t cs) -> int {
-            GPE_TRY(record(cs, G_));
-            if (blend) {
-                k_add_scalar<<<1, 1, 0, cs>>>(st->d_clock, (double)G_ * p->dt);
-                GPE_LAUNCH_CHECK();
-            }
-            return GPE_OK;
-        };
+        auto rec_block = [&](cudaStream_t cs) -> int { return rk4_steps<R, 7>(st, a, blend, G_, true, cs); };
         GPE_TRY(replay_graph(st, 0, key, 4 * G_ + (blend ? 1 : 0), nsteps / G_, s, rec_block));
         left = nsteps % G_;
     }
-    return record(s, left);
+    return rk4_steps<R, 7>(st, a, blend, left, false, s);
 }
 
 // ------------------------------------------------------------ general explicit RK (RKHE3, RKCK)
@@ -948,9 +957,7 @@ struct RkGenArgs {
     const R *V0;
     const R *V1;
     R ihx2, ihy2, ihz2, g;
-    Ramp ramp;
-    double t_off;    // step start relative to *ramp.clock
-    double tc;       // c_i dt
+    const double *stab;  // this stage's value of the schedule (k_ramp_table)
     int tile, out;   // y^(i) and the state written (y^(i+1), or y^(1) for y1)
     int nsrc;        // own-cell terms
     int src[5];
@@ -973,7 +980,7 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? (NS < 3 ? 6 : 5) : (NS 
         R V0[4], V1[BLEND ? 4 : 1];
         CT y[NS > 0 ? NS : 1][4];
     };
-    const R s = BLEND ? (R)ramp_s(a.ramp, *a.ramp.clock + a.t_off + a.tc) : (R)0;
+    const R s = BLEND ? (R)__ldg(a.stab) : (R)0;
     const R c3 = rhs_centre(a.ihx2, a.ihy2, a.ihz2);
     constexpr R HALF = sizeof(R) == 8 ? (R)1 : (R)(-0.5);  // LapRhs leaves the factor in in single precision
     tile_loop<7, LapRhs>(T, (const CT *)a.y[a.tile], Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
@@ -1040,23 +1047,32 @@ static int rkgen_run(gpe_state *st, const gpe_real_params *p, int64_t nsteps, do
     a.ihy2 = (R)(1.0 / (g->box.hy * g->box.hy));
     a.ihz2 = (R)(1.0 / (g->box.hz * g->box.hz));
     a.g = (R)p->g;
-    a.ramp.clock = st->d_clock;
-    a.ramp.T = p->T_ramp;
-    a.ramp.n_knots = p->n_knots;
-    for (int k = 0; k < GPE_MAX_KNOTS; ++k) a.ramp.knots[k] = p->knots[k];
+    Ramp ramp{};
+    StageTimes times{};
     if (blend) {
+        ramp.clock = st->d_clock;
+        ramp.T = p->T_ramp;
+        ramp.n_knots = p->n_knots;
+        for (int k = 0; k < GPE_MAX_KNOTS; ++k) ramp.knots[k] = p->knots[k];
+        for (int i = 0; i < T.s; ++i) times.c[i] = T.c[i];
+        GPE_TRY(ensure_stab(st, STAB_STEPS));
         k_set_scalar<<<1, 1, 0, s>>>(st->d_clock, t0);
         GPE_LAUNCH_CHECK();
     }
     const TileLaunch L = tile_launch<CT>(g);
     for (int64_t n = 0; n < nsteps; ++n) {
-        a.t_off = (double)n * p->dt;
+        const int m = blend ? (int)(n % st->stab_cap) : 0;
+        if (blend && m == 0) {
+            k_ramp_table<<<1, 256, 0, s>>>(ramp, st->d_clock, 0.0, n, (int)std::min<int64_t>(nsteps - n, st->stab_cap), T.s,
+                                           times, p->dt, st->d_stab);
+            GPE_LAUNCH_CHECK();
+        }
         for (int i = 0; i < T.s; ++i) {  // stage i + 1 of App. A
             const bool last = i == T.s - 1;
             const double *row = last ? T.b_star : T.a_star[i];
             a.tile = i;
             a.out = last ? 0 : i + 1;
-            a.tc = T.c[i] * p->dt;
+            a.stab = st->d_stab + (size_t)T.s * m + i;
             a.kdt = (R)(T.sub[i] * p->dt);
             a.ctile = (R)row[i];
             a.nsrc = 0;
@@ -1202,6 +1218,7 @@ extern "C" int gpe_state_create(gpe_grid *g, int dtype, gpe_state **out)
     const size_t real_bytes = (dtype == GPE_C128 || dtype == GPE_R64) ? 8 : 4;
     if (rc == GPE_OK) rc = dev_alloc(&st->d_E, g->n_packed * real_bytes);
     if (rc == GPE_OK) rc = dev_alloc_t(&st->d_clock, 1);
+    if (rc == GPE_OK && !is_real_dtype(dtype)) rc = ensure_stab(st, STAB_STEPS);
     if (rc == GPE_OK) rc = red_alloc(st->red, g->nsm * 32);
     if (rc == GPE_OK && cudaMallocHost(&st->h_obs, sizeof(gpe_obs)) != cudaSuccess)
         rc = fail(GPE_ERR_CUDA, "cudaMallocHost failed");
@@ -1209,6 +1226,7 @@ extern "C" int gpe_state_create(gpe_grid *g, int dtype, gpe_state **out)
         dev_free(st->d_psi);
         dev_free(st->d_E);
         dev_free(st->d_clock);
+        dev_free(st->d_stab);
         red_free(st->red);
         if (st->h_obs) cudaFreeHost(st->h_obs);
         delete st;
@@ -1227,6 +1245,7 @@ extern "C" int gpe_state_destroy(gpe_state *st)
     for (int i = 0; i < 6; ++i) dev_free(st->d_work[i]);
     dev_free(st->d_E);
     dev_free(st->d_clock);
+    dev_free(st->d_stab);
     dev_free(st->d_done);
     dev_free(st->d_ctr);
     dev_free(st->d_chunk_norm);
@@ -1269,6 +1288,7 @@ extern "C" int gpe_state_set_graph(gpe_state *st, int steps_per_graph)
 {
     GPE_TRY(check_state(st));
     if (steps_per_graph < 0 || steps_per_graph > 4096) return fail(GPE_ERR_ARG, "steps_per_graph must be in [0, 4096]");
+    if (!is_real_dtype(st->dtype)) GPE_TRY(ensure_stab(st, steps_per_graph));
     st->graph_steps = steps_per_graph;
     return GPE_OK;
 }

@@ -18,10 +18,11 @@ int rk4_19(gpe_state *st, const gpe_real_params *p, int64_t nsteps, double t0, c
     RkArgs<R> a;
     GPE_TRY(rk4_args(st, p, a));
     if (blend) {
+        GPE_TRY(ensure_stab(st, STAB_STEPS));
         k_set_scalar19<<<1, 1, 0, s>>>(st->d_clock, t0);
         GPE_LAUNCH_CHECK();
     }
-    return rk4_steps<R, 19>(st, a, blend, nsteps, s);
+    return rk4_steps<R, 19>(st, a, blend, nsteps, false, s);
 }
 
 template <typename R, typename CT>
