@@ -88,11 +88,12 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? 5 : 2) k_adj_stage(cons
         R V0[4], V1[4];
         CT Y[4], lam[4], acc[4];
     };
+    const TileList list = tile_begin(T);
     XF xf{};
     if constexpr (POS == 0) xf.s = a.m_scale;
     Sum64<R> dot[1];
     int n = 0;
-    tile_loop<7>(T, a.mu_in, xf, a.ihx2, a.ihy2, a.ihz2, EveryTile(),
+    tile_loop<7>(T, list, a.mu_in, xf, a.ihx2, a.ihy2, a.ihz2, EveryTile(),
                  [&](uint32_t idx, uint32_t m) {
                      prefetch_l2(a.V0 + idx, m * (uint32_t)sizeof(R));
                      prefetch_l2(a.V1 + idx, m * (uint32_t)sizeof(R));
@@ -145,7 +146,7 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? 5 : 2) k_adj_stage(cons
                      if (++n % SUM_FLUSH == 0) dot[0].flush();
                  });
     double tot[1];
-    block_totals<1>(dot, T.ntiles >= SUM_FLUSH * (int)gridDim.x, tot);
+    block_totals<1>(dot, sums_flushed((uint32_t)T.ntiles), tot);
     if (launch_totals<1>(tot, a.partials, a.counter) && threadIdx.x == 0) {
         a.grad[a.k0] += a.w0 * tot[0];
         a.grad[a.k0 + 1] += a.w1 * tot[0];
@@ -368,9 +369,7 @@ static int backward_impl(gpe_tape *t, const gpe_state *target, double *grad, dou
             f.y3 = y + np;
             f.y4 = y + 2 * np;
         }
-        k<<<blocks(k), TILE, tl.smem, s>>>(f, tl.T);
-        GPE_LAUNCH_CHECK();
-        return GPE_OK;
+        return tile_run(k, blocks(k), tl, s, f, tl.T);
     };
     using KA = void (*)(AdjArgs<R>, TileView);
     const KA ka[4] = {k_adj_stage<R, 0>, k_adj_stage<R, 1>, k_adj_stage<R, 1>, k_adj_stage<R, 2>};
@@ -428,8 +427,7 @@ static int backward_impl(gpe_tape *t, const gpe_state *target, double *grad, dou
                 a.cl = cl[r];
                 a.cn = cn[r];
                 hat(p, ts[r], a.k0, a.w0, a.w1);
-                ka[r]<<<blocks(ka[r]), TILE, tl.smem, s>>>(a, tl.T);
-                GPE_LAUNCH_CHECK();
+                GPE_TRY(tile_run(ka[r], blocks(ka[r]), tl, s, a, tl.T));
             }
         }
     }

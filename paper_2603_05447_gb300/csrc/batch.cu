@@ -83,7 +83,7 @@ struct ShellWalk {
             if (!live) return;
             double *p = a.part + 5 * (size_t)part_of(a.tile_base[cur], blockIdx.x, gridDim.x), tot[NS];
             if constexpr (NS == 5) sum[4].add((R)nf);
-            block_totals<NS>(sum, nt >= SUM_FLUSH * gridDim.x, tot);
+            block_totals<NS>(sum, sums_flushed(nt), tot);
 #pragma unroll
             for (int k = 0; k < NS; ++k) {
                 if (threadIdx.x == 0) p[k] = tot[k];
@@ -145,6 +145,7 @@ struct WalkDiag {
 template <typename R, typename CT, int STAGE>
 __global__ void GPE_TILE_BOUNDS(R) k_batch_itp(const BatchArgs<R, CT> a, const TileView T)
 {
+    const TileList list = tile_begin(T);
     using W = ShellWalk<R, CT, STAGE>;
     W w(a, (uint32_t)T.ntiles);
     auto enter = [&](uint32_t tile) { return w.enter(tile); };
@@ -174,10 +175,10 @@ __global__ void GPE_TILE_BOUNDS(R) k_batch_itp(const BatchArgs<R, CT> a, const T
         }
     };
     if constexpr (STAGE == 0)
-        tile_loop<7>(T, (const CT *)a.psi, WalkDiag<R, CT, W>{w, a.E}, w.ihx2, w.ihy2, w.ihz2, enter, pref,
+        tile_loop<7>(T, list, (const CT *)a.psi, WalkDiag<R, CT, W>{w, a.E}, w.ihx2, w.ihy2, w.ihz2, enter, pref,
                      ELoad<R>{a.E}, body);
     else
-        tile_loop<7>(T, (const CT *)a.tmp, Plain(), w.ihx2, w.ihy2, w.ihz2, enter, pref, ELoad<R>{a.E}, body);
+        tile_loop<7>(T, list, (const CT *)a.tmp, Plain(), w.ihx2, w.ihy2, w.ihz2, enter, pref, ELoad<R>{a.E}, body);
     w.leave();
 }
 
@@ -220,8 +221,9 @@ __global__ void k_batch_reset_scale(ShellParams *sh, int n)
 template <typename R, typename CT>
 __global__ void GPE_TILE_BOUNDS(R) k_batch_obs(const BatchArgs<R, CT> a, const TileView T)
 {
+    const TileList list = tile_begin(T);
     ShellWalk<R, CT, 5> w(a, (uint32_t)T.ntiles);
-    tile_loop<7>(T, (const CT *)a.psi, Plain(), w.ihx2, w.ihy2, w.ihz2, [&](uint32_t tile) { return w.enter(tile); },
+    tile_loop<7>(T, list, (const CT *)a.psi, Plain(), w.ihx2, w.ihy2, w.ihz2, [&](uint32_t tile) { return w.enter(tile); },
                  [&](uint32_t idx, uint32_t n) { prefetch_l2(a.V + idx, n * (uint32_t)sizeof(R)); },
                  VLoad<R, false>{a.V, nullptr},
                  [&](uint32_t, const typename VLoad<R, false>::P &p, const CT(&c)[4], const CT(&L)[4]) {
@@ -479,10 +481,8 @@ static int batch_record_block(gpe_batch *B, int64_t nsteps, cudaStream_t s)
     const unsigned na = tile_blocks(ka, B->nsm, L.T.ntiles, L.smem), nb = tile_blocks(kb, B->nsm, L.T.ntiles, L.smem),
                    no = tile_blocks(ko, B->nsm, L.T.ntiles, L.smem);
     for (int64_t k = 0; k < nsteps; ++k) {
-        ka<<<na, TILE, L.smem, s>>>(a, L.T);
-        GPE_LAUNCH_CHECK();
-        kb<<<nb, TILE, L.smem, s>>>(a, L.T);
-        GPE_LAUNCH_CHECK();
+        GPE_TRY(tile_run(ka, na, L, s, a, L.T));
+        GPE_TRY(tile_run(kb, nb, L, s, a, L.T));
         k_batch_norm_finish<<<B->n, 256, 0, s>>>(B->d_sh, B->d_part, B->d_tile_base, nb);
         GPE_LAUNCH_CHECK();
     }
@@ -492,8 +492,7 @@ static int batch_record_block(gpe_batch *B, int64_t nsteps, cudaStream_t s)
     GPE_LAUNCH_CHECK();
     k_zero_int<<<1, 1, 0, s>>>(B->d_unconv);
     GPE_LAUNCH_CHECK();
-    ko<<<no, TILE, L.smem, s>>>(a, L.T);
-    GPE_LAUNCH_CHECK();
+    GPE_TRY(tile_run(ko, no, L, s, a, L.T));
     k_batch_obs_finish<<<B->n, 256, 0, s>>>(B->d_sh, B->d_part, B->d_tile_base, no, B->d_unconv);
     GPE_LAUNCH_CHECK();
     return GPE_OK;

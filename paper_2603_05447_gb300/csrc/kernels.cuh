@@ -173,6 +173,9 @@ struct Sum64<float> {
     }
 };
 constexpr int SUM_FLUSH = 64;
+// may a thread have flushed over nt tiles?  (the blocks with the most take
+// ceil(nt / grid) of them)
+__device__ __forceinline__ bool sums_flushed(uint32_t nt) { return nt > (SUM_FLUSH - 1) * gridDim.x; }
 
 // The block's totals of NV sums, to every thread.  Few FP64 instructions, since
 // every warp of an SM queues for the one pipe at a kernel's end: pairs are
@@ -267,9 +270,10 @@ __device__ __forceinline__ bool launch_totals(double (&v)[NV], double *partials,
 template <typename R, typename CT, int NP>
 __global__ void GPE_TILE_BOUNDS(R) k_itp_a(const ItpArgs<R, CT> a, const TileView T)
 {
+    const TileList list = tile_begin(T);
     const R q4 = a.dt / (R)4;
     const TileDiag<R, CT> diag{{(R)a.scalars[0], a.g * a.dt / (R)2, a.E}};
-    tile_loop<NP>(T, (const CT *)a.psi, diag, a.ihx2, a.ihy2, a.ihz2, EveryTile(),
+    tile_loop<NP>(T, list, (const CT *)a.psi, diag, a.ihx2, a.ihy2, a.ihz2, EveryTile(),
                   [&](uint32_t idx, uint32_t n) { prefetch_l2(a.E + idx, n * (uint32_t)sizeof(R)); }, ELoad<R>{a.E},
                   [&](uint32_t idx, const typename ELoad<R>::P &p, const CT(&c)[4], const CT(&L)[4]) {
                       CT o[4];
@@ -286,11 +290,12 @@ template <typename R, typename CT, int NP>
 __global__ void GPE_TILE_BOUNDS(R) k_itp_b(const ItpArgs<R, CT> a, const TileView T, double *partials,
                                            unsigned int *counter)
 {
+    const TileList list = tile_begin(T);
     const R hg = a.g * a.dt / (R)2;
     const R q4 = a.dt / (R)4;
     Sum64<R> norm[1];
     int n = 0;
-    tile_loop<NP>(T, (const CT *)a.tmp, Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
+    tile_loop<NP>(T, list, (const CT *)a.tmp, Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
                   [&](uint32_t idx, uint32_t n) { prefetch_l2(a.E + idx, n * (uint32_t)sizeof(R)); }, ELoad<R>{a.E},
                   [&](uint32_t idx, const typename ELoad<R>::P &p, const CT(&c)[4], const CT(&L)[4]) {
                       CT o[4];
@@ -307,7 +312,7 @@ __global__ void GPE_TILE_BOUNDS(R) k_itp_b(const ItpArgs<R, CT> a, const TileVie
                       if (++n % SUM_FLUSH == 0) norm[0].flush();
                   });
     double tot[1];
-    block_totals<1>(norm, T.ntiles >= SUM_FLUSH * (int)gridDim.x, tot);
+    block_totals<1>(norm, sums_flushed((uint32_t)T.ntiles), tot);
     if (launch_totals<1>(tot, partials, counter) && threadIdx.x == 0) {
         const double nrm = tot[0] * a.dV;
         a.scalars[0] = sqrt(a.N / nrm);
@@ -402,9 +407,10 @@ __device__ __forceinline__ void obs_terms(const typename VLoad<R, BLEND>::P &p, 
 template <typename R, typename CT, int NP, bool BLEND>
 __global__ void GPE_TILE_BOUNDS(R) k_obs(const ObsArgs<R, CT> a, const TileView T)
 {
+    const TileList list = tile_begin(T);
     Sum64<R> sum[5];  // norm, ekin, epot, eint, nonfinite
     int n = 0, nf = 0;
-    tile_loop<NP>(T, a.psi, Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
+    tile_loop<NP>(T, list, a.psi, Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
                   [&](uint32_t idx, uint32_t n) {
                       prefetch_l2(a.V0 + idx, n * (uint32_t)sizeof(R));
                       if constexpr (BLEND) prefetch_l2(a.V1 + idx, n * (uint32_t)sizeof(R));
@@ -422,7 +428,7 @@ __global__ void GPE_TILE_BOUNDS(R) k_obs(const ObsArgs<R, CT> a, const TileView 
                   });
     sum[4].add((R)nf);
     double tot[5];
-    block_totals<5>(sum, T.ntiles >= SUM_FLUSH * (int)gridDim.x, tot);
+    block_totals<5>(sum, sums_flushed((uint32_t)T.ntiles), tot);
     if (launch_totals<5>(tot, a.partials, a.counter) && threadIdx.x == 0) {
         gpe_obs o;
         o.norm = tot[0] * a.dV;
@@ -475,12 +481,10 @@ inline int itp_steps(gpe_state *st, const ItpArgs<R, CT> &a, int64_t cnt, cudaSt
     const TileLaunch L = tile_launch<CT>(g);
     auto ka = k_itp_a<R, CT, NP>;
     auto kb = k_itp_b<R, CT, NP>;
-    const unsigned nba = tile_blocks(ka, g->nsm, L.T.ntiles, L.smem), nbb = tile_blocks(kb, g->nsm, L.T.ntiles, L.smem);
+    const unsigned na = tile_blocks(ka, g->nsm, L.T.ntiles, L.smem), nb = tile_blocks(kb, g->nsm, L.T.ntiles, L.smem);
     for (int64_t n = 0; n < cnt; ++n) {
-        ka<<<nba, TILE, L.smem, s>>>(a, L.T);
-        GPE_LAUNCH_CHECK();
-        kb<<<nbb, TILE, L.smem, s>>>(a, L.T, st->red.partials, st->red.counter);
-        GPE_LAUNCH_CHECK();
+        GPE_TRY(tile_run(ka, na, L, s, a, L.T));
+        GPE_TRY(tile_run(kb, nb, L, s, a, L.T, st->red.partials, st->red.counter));
     }
     return GPE_OK;
 }
@@ -515,9 +519,7 @@ inline int obs_run(const gpe_state *stc, double gg, double sb, cudaStream_t s)
     a.out = (gpe_obs *)(st->red.scalars + 2);
     const TileLaunch L = tile_launch<CT>(g);
     auto k = a.V1 ? k_obs<R, CT, NP, true> : k_obs<R, CT, NP, false>;
-    k<<<tile_blocks(k, g->nsm, L.T.ntiles, L.smem), TILE, L.smem, s>>>(a, L.T);
-    GPE_LAUNCH_CHECK();
-    return GPE_OK;
+    return tile_run(k, tile_blocks(k, g->nsm, L.T.ntiles, L.smem), L, s, a, L.T);
 }
 
 // The schedule's values for n steps of nc stages, at *clock + (n0 + m) dt +
@@ -576,12 +578,8 @@ inline int rk4_steps(gpe_state *st, RkArgs<R> a, bool blend, int64_t cnt, bool a
     const gpe_grid *g = st->grid;
     using RT = Rk4Tiles<R, NP>;
     const TileLaunch L = tile_launch<typename Cx<R>::T>(g);
-    typename RT::K k[4];
-    unsigned nblk[4];
-    for (int stg = 0; stg < 4; ++stg) {
-        k[stg] = RT::get(blend, stg);
-        nblk[stg] = tile_blocks(k[stg], g->nsm, L.T.ntiles, L.smem);
-    }
+    unsigned grid[4];
+    for (int stg = 0; stg < 4; ++stg) grid[stg] = tile_blocks(RT::get(blend, stg), g->nsm, L.T.ntiles, L.smem);
     for (int64_t n = 0; n < cnt; ++n) {
         const int m = blend ? (int)(n % st->stab_cap) : 0;
         if (blend && m == 0) {
@@ -593,8 +591,7 @@ inline int rk4_steps(gpe_state *st, RkArgs<R> a, bool blend, int64_t cnt, bool a
         }
         for (int stg = 0; stg < 4; ++stg) {
             a.stab = st->d_stab + 3 * m + (stg + 1) / 2;  // t, t + dt/2 twice, t + dt
-            k[stg]<<<nblk[stg], TILE, L.smem, s>>>(a, L.T);
-            GPE_LAUNCH_CHECK();
+            GPE_TRY(tile_run(RT::get(blend, stg), grid[stg], L, s, a, L.T));
         }
     }
     return GPE_OK;

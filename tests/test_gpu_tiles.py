@@ -126,3 +126,28 @@ def test_general_integrators_on_odd_masks(kind, dtype, integrator):
             y = oracle.rk_step_np(S.og, V, y, S.g, 0.0, S.dt, method=integrator)
         gpe.gpe_step_real(S.st, gpe.real_params(S.g, S.dt, integrator=getattr(gpe, "GPE_" + integrator)), 2)
         assert rel_l2(S.og.compact(S.dense()), y) <= S.tol
+
+
+# Sums of a block are put into FP64 every 64 tiles.  All-active boxes of bricks
+# of 128 segments (one tile each) around 64 tiles a block on 152 SMs with five
+# to eight blocks an SM, where only some blocks reach the 64th.
+@pytest.mark.parametrize("nb", [(40, 40, 30), (40, 40, 36), (40, 50, 29), (40, 40, 42), (40, 50, 34), (45, 48, 36)])
+@pytest.mark.parametrize("dtype", [gpe.GPE_C64, gpe.GPE_R32])
+def test_sums_over_sixty_odd_tiles_a_block(nb, dtype):
+    h = 0.1
+    box = gpe.make_box(8 * nb[0], 8 * nb[1], 8 * nb[2], h)
+    grid = gpe.gpe_grid_create_analytic(box, gpe.make_potential(gpe.GPE_POT_HARMONIC, 1e-3, 1e-3, 1e-3), 1e9)
+    st = gpe.gpe_state_create(grid, dtype)
+    try:
+        n = 512 * nb[0] * nb[1] * nb[2]
+        gen = torch.Generator(device="cuda").manual_seed(5)
+        re = torch.rand(n, generator=gen, device="cuda") + 0.5
+        psi = re if dtype == gpe.GPE_R32 else torch.complex(re, 0.3 * re)
+        gpe.gpe_state_load(st, psi, gpe.GPE_LAYOUT_COMPACT)
+        want = float(psi.abs().double().square().sum()) * h ** 3
+        assert abs(gpe.gpe_observables(st, 0.1)["norm"] - want) <= 1e-6 * want
+        gpe.gpe_step_imag(st, gpe.gpe_imag_params(0.1, 1e-4, 2.0), 2)
+        assert abs(gpe.gpe_observables(st, 0.1)["norm"] - 2.0) <= 2e-6
+    finally:
+        gpe.gpe_state_destroy(st)
+        gpe.gpe_grid_destroy(grid)
