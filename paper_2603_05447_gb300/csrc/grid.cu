@@ -89,7 +89,8 @@ __device__ __forceinline__ void cell_values(const VSource &src, const BoxD &bx, 
 // potential's minimum directly, and for the ellipsoidal shell the range
 // [rmin, rmax] of the scaled radius, from which the smallest |rho - 1|
 // follows.  Evaluated in FP32 with wide margins: it only has to be
-// conservative, the per-cell FP64 test decides.
+// conservative, the per-cell FP64 test decides.  Where FP32 does not reach (a
+// bound that is not finite, semi-axes far from 1) the answer is yes.
 __device__ __forceinline__ bool pot_may_select(const PotDesc &P, double cut, float xl, float xh, float yl, float yh,
                                                float zl, float zh)
 {
@@ -98,17 +99,20 @@ __device__ __forceinline__ bool pot_may_select(const PotDesc &P, double cut, flo
     if (P.kind == GPE_POT_HARMONIC) {
         const float wx = (float)P.p[0], wy = (float)P.p[1], wz = (float)P.p[2];
         const float vmin = 0.5f * (wx * wx * sqmin(xl, xh) + wy * wy * sqmin(yl, yh) + wz * wz * sqmin(zl, zh));
-        return vmin <= (float)cut * 1.0001f + 1e-30f;
+        return !(vmin > (float)cut * 1.0001f + 1e-30f) || !(vmin < INFINITY);
     }
     if (P.kind == GPE_POT_ELLIPSOID_SHELL) {
         const float w = (float)P.p[0];
         const float ia = 1.f / (float)(P.p[1] * P.p[1]), ib = 1.f / (float)(P.p[2] * P.p[2]),
                     ic = 1.f / (float)(P.p[3] * P.p[3]);
+        const float least = fminf(ia, fminf(ib, ic)), most = fmaxf(ia, fmaxf(ib, ic));
+        if (!(least > 1e-30f && most < 1e30f)) return true;
         const float rmin = sqrtf(sqmin(xl, xh) * ia + sqmin(yl, yh) * ib + sqmin(zl, zh) * ic);
         const float rmax = sqrtf(sqmax(xl, xh) * ia + sqmax(yl, yh) * ib + sqmax(zl, zh) * ic);
         const float d = (rmin <= 1.f && rmax >= 1.f) ? 0.f : fminf(fabsf(rmin - 1.f), fabsf(rmax - 1.f));
         // V = w^2 d^2 / 2 < cut  <=>  |w| d < sqrt(2 cut)
-        return fabsf(w) * d <= sqrtf(2.f * (float)cut) * 1.0001f + 1e-4f * (1.f + rmax) * fabsf(w);
+        const float reach = fabsf(w) * d;
+        return !(reach > sqrtf(2.f * fmaxf((float)cut, 0.f)) * 1.0001f + 1e-4f * (1.f + rmax) * fabsf(w)) || !(reach < INFINITY);
     }
     return true;
 }
@@ -184,6 +188,7 @@ static Limit limit_of(double t)
     int64_t b;
     memcpy(&b, &t, 8);
     m.ord = t == 0.0 ? -1 : (b < 0 ? b ^ 0x7fffffffffffffffll : b);  // neither zero is below a zero
+    if (std::isnan(t)) m.ord = INT64_MIN;                            // nothing is below a NaN
     return m;
 }
 

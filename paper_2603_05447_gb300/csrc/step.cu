@@ -981,7 +981,7 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? (NS < 3 ? 6 : 5) : (NS 
         CT y[NS > 0 ? NS : 1][4];
     };
     const TileList list = tile_begin(T);
-    const R s = BLEND ? (R)__ldg(a.stab) : (R)0;
+    const R s = BLEND ? (R)__ldcg(a.stab) : (R)0;
     const R c3 = rhs_centre(a.ihx2, a.ihy2, a.ihz2);
     constexpr R HALF = sizeof(R) == 8 ? (R)1 : (R)(-0.5);  // LapRhs leaves the factor in in single precision
     tile_loop<7, LapRhs>(T, list, (const CT *)a.y[a.tile], Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),

@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? 6 : 2) k_rk4_tile(const
     using CT = typename Cx<R>::T;
     using B = Rk4Body<R, BLEND, false, ST>;
     const TileList list = tile_begin(T);
-    const B body(a, BLEND ? (R)__ldg(a.stab) : (R)0, tile_rhs_centre<NP>(a.ihx2, a.ihy2, a.ihz2));
+    const B body(a, BLEND ? (R)__ldcg(a.stab) : (R)0, tile_rhs_centre<NP>(a.ihx2, a.ihy2, a.ihz2));
     tile_loop<NP, LapRhs>(T, list, body.yin(), Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
                   [&](uint32_t idx, uint32_t n) {
                       prefetch_l2(a.V0 + idx, n * (uint32_t)sizeof(R));

@@ -71,3 +71,40 @@ def test_tf_mu_sum_that_overflows_is_refused(dtype):
     V[:4] = 1e307
     with pytest.raises(gpe.GpeError):
         gpe.gpe_tf_mu_dense(gpe.make_box(8, 8, 8, 0.1), V, 1.0, 1.0)
+
+
+def test_tf_mu_of_large_fp32_cells_is_the_root():
+    V = potential((33, 34, 35), "shell").astype(np.float32)
+    V[::3] = 2e37  # a thread's float pair would not hold their sum
+    h, target = 0.1, 1e42
+    got = gpe.gpe_tf_mu_dense(gpe.make_box(35, 34, 33, h), V, target * h ** 3, 1.0)
+    want = root(V, target)
+    assert abs(got - want) <= 1e-11 * want
+
+
+@pytest.mark.parametrize("kind", ["harmonic", "shell"])
+def test_tf_mu_analytic_outside_the_range_of_fp32(kind):
+    n, h = 24, 1e-26
+    x = (np.arange(n) - (n - 1) / 2) * h
+    r2 = x[:, None, None] ** 2 + x[:, None] ** 2 + x ** 2
+    if kind == "harmonic":
+        w = 1e26
+        V, pot = 0.5 * w * w * r2, gpe.make_potential(gpe.GPE_POT_HARMONIC, w, w, w)
+    else:
+        w, a = 30.0, 7 * h
+        V, pot = 0.5 * w * w * (np.sqrt(r2 / a ** 2) - 1.0) ** 2, gpe.make_potential(gpe.GPE_POT_ELLIPSOID_SHELL, w, a, a, a)
+    box = gpe.make_box(n, n, n, h, h, h, x[0], x[0], x[0])
+    for target in (3.0, 1e4):
+        got = gpe.gpe_tf_mu_analytic(box, pot, target * h ** 3, 1.0)
+        assert abs(got - root(V, target)) <= 1e-11 * root(V, target)
+
+
+def test_a_cutoff_that_is_not_a_number_selects_nothing():
+    V = potential((17, 18, 19), "shell")
+    box = gpe.make_box(19, 18, 17, 0.1)
+    pot = gpe.make_potential(gpe.GPE_POT_HARMONIC, 1.0, 1.0, 1.0)
+    for make in (lambda: gpe.gpe_grid_create_dense(box, V, np.nan),
+                 lambda: gpe.gpe_grid_create_dense(box, V.astype(np.float32), np.nan),
+                 lambda: gpe.gpe_grid_create_analytic(box, pot, np.nan)):
+        with pytest.raises(gpe.GpeError):
+            make()
