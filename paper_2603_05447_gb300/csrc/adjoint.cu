@@ -357,7 +357,7 @@ static int backward_impl(gpe_tape *t, const gpe_state *target, double *grad, dou
     f.ramp.n_knots = p.n_knots;
     for (int k = 0; k < GPE_MAX_KNOTS; ++k) f.ramp.knots[k] = p.knots[k];
     using RT = Rk4Tiles<R, 7>;
-    const TileLaunch tl = tile_launch<CT>(g);
+    const TileLaunch tl = tile_launch<CT, 7>(g->tiles);
     auto blocks = [&](auto k) { return tile_blocks(k, g->nsm, tl.T.ntiles, tl.smem); };
     // stage stg of step m of the segment, from f.y0
     auto stage = [&](int64_t m, int stg) -> int {

@@ -143,7 +143,7 @@ struct WalkDiag {
 // per brick and one FP64 warp sum per brick; bound by the shared-memory pipe
 // like the single-state passes.
 template <typename R, typename CT, int STAGE>
-__global__ void GPE_TILE_BOUNDS(R) k_batch_itp(const BatchArgs<R, CT> a, const TileView T)
+__global__ void GPE_TILE_BOUNDS(R, 7) k_batch_itp(const BatchArgs<R, CT> a, const TileView T)
 {
     const TileList list = tile_begin(T);
     using W = ShellWalk<R, CT, STAGE>;
@@ -219,7 +219,7 @@ __global__ void k_batch_reset_scale(ShellParams *sh, int n)
 }
 
 template <typename R, typename CT>
-__global__ void GPE_TILE_BOUNDS(R) k_batch_obs(const BatchArgs<R, CT> a, const TileView T)
+__global__ void GPE_TILE_BOUNDS(R, 7) k_batch_obs(const BatchArgs<R, CT> a, const TileView T)
 {
     const TileList list = tile_begin(T);
     ShellWalk<R, CT, 5> w(a, (uint32_t)T.ntiles);
@@ -474,7 +474,7 @@ static int batch_record_block(gpe_batch *B, int64_t nsteps, cudaStream_t s)
     a.tile_shell = B->d_tile_shell;
     a.tile_base = B->d_tile_base;
     a.part = B->d_part;
-    const TileLaunch L = tile_launch<CT>(B->tiles);
+    const TileLaunch L = tile_launch<CT, 7>(B->tiles);
     auto ka = k_batch_itp<R, CT, 0>;
     auto kb = k_batch_itp<R, CT, 1>;
     auto ko = k_batch_obs<R, CT>;

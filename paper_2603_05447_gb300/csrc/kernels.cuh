@@ -268,7 +268,7 @@ __device__ __forceinline__ bool launch_totals(double (&v)[NV], double *partials,
 }
 
 template <typename R, typename CT, int NP>
-__global__ void GPE_TILE_BOUNDS(R) k_itp_a(const ItpArgs<R, CT> a, const TileView T)
+__global__ void GPE_TILE_BOUNDS(R, NP) k_itp_a(const ItpArgs<R, CT> a, const TileView T)
 {
     const TileList list = tile_begin(T);
     const R q4 = a.dt / (R)4;
@@ -287,7 +287,7 @@ __global__ void GPE_TILE_BOUNDS(R) k_itp_a(const ItpArgs<R, CT> a, const TileVie
 }
 
 template <typename R, typename CT, int NP>
-__global__ void GPE_TILE_BOUNDS(R) k_itp_b(const ItpArgs<R, CT> a, const TileView T, double *partials,
+__global__ void GPE_TILE_BOUNDS(R, NP) k_itp_b(const ItpArgs<R, CT> a, const TileView T, double *partials,
                                            unsigned int *counter)
 {
     const TileList list = tile_begin(T);
@@ -405,7 +405,7 @@ __device__ __forceinline__ void obs_terms(const typename VLoad<R, BLEND>::P &p, 
 // segment, 66 on tiles with the sums flushed by every warp at its end, 40 now;
 // one pass over psi and V at 3.7 TB/s, the shared-memory pipe 76 % busy.
 template <typename R, typename CT, int NP, bool BLEND>
-__global__ void GPE_TILE_BOUNDS(R) k_obs(const ObsArgs<R, CT> a, const TileView T)
+__global__ void GPE_TILE_BOUNDS(R, NP) k_obs(const ObsArgs<R, CT> a, const TileView T)
 {
     const TileList list = tile_begin(T);
     Sum64<R> sum[5];  // norm, ekin, epot, eint, nonfinite
@@ -478,7 +478,7 @@ template <typename R, typename CT, int NP>
 inline int itp_steps(gpe_state *st, const ItpArgs<R, CT> &a, int64_t cnt, cudaStream_t s)
 {
     const gpe_grid *g = st->grid;
-    const TileLaunch L = tile_launch<CT>(g);
+    const TileLaunch L = tile_launch<CT, NP>(g->tiles);
     auto ka = k_itp_a<R, CT, NP>;
     auto kb = k_itp_b<R, CT, NP>;
     const unsigned na = tile_blocks(ka, g->nsm, L.T.ntiles, L.smem), nb = tile_blocks(kb, g->nsm, L.T.ntiles, L.smem);
@@ -517,7 +517,7 @@ inline int obs_run(const gpe_state *stc, double gg, double sb, cudaStream_t s)
     a.partials = st->red.partials;
     a.counter = st->red.counter;
     a.out = (gpe_obs *)(st->red.scalars + 2);
-    const TileLaunch L = tile_launch<CT>(g);
+    const TileLaunch L = tile_launch<CT, NP>(g->tiles);
     auto k = a.V1 ? k_obs<R, CT, NP, true> : k_obs<R, CT, NP, false>;
     return tile_run(k, tile_blocks(k, g->nsm, L.T.ntiles, L.smem), L, s, a, L.T);
 }
@@ -577,7 +577,7 @@ inline int rk4_steps(gpe_state *st, RkArgs<R> a, bool blend, int64_t cnt, bool a
 {
     const gpe_grid *g = st->grid;
     using RT = Rk4Tiles<R, NP>;
-    const TileLaunch L = tile_launch<typename Cx<R>::T>(g);
+    const TileLaunch L = tile_launch<typename Cx<R>::T, NP>(g->tiles);
     unsigned grid[4];
     for (int stg = 0; stg < 4; ++stg) grid[stg] = tile_blocks(RT::get(blend, stg), g->nsm, L.T.ntiles, L.smem);
     for (int64_t n = 0; n < cnt; ++n) {

@@ -1060,7 +1060,7 @@ static int rkgen_run(gpe_state *st, const gpe_real_params *p, int64_t nsteps, do
         k_set_scalar<<<1, 1, 0, s>>>(st->d_clock, t0);
         GPE_LAUNCH_CHECK();
     }
-    const TileLaunch L = tile_launch<CT>(g);
+    const TileLaunch L = tile_launch<CT, 7>(g->tiles);
     for (int64_t n = 0; n < nsteps; ++n) {
         const int m = blend ? (int)(n % st->stab_cap) : 0;
         if (blend && m == 0) {

@@ -42,28 +42,33 @@ struct TileView {
     const uint32_t *halo;
     uint32_t nseg;         // stored segments
     int ntiles, stride;
-    int pstr;              // slots of a 16-byte plane of the shared tile
+    int pstr;              // slots of a plane of the shared tile
 };
 
-// Shared tile: UPS planes of 16-byte units (unit k of every slot's segment is
-// contiguous), so that lanes with consecutive slots touch consecutive units
-template <typename CT>
+// Shared tile: planes of units (unit k of every slot's segment is contiguous),
+// so that lanes with consecutive slots touch consecutive units.  Units of 16
+// bytes give the widest loads; with the 19-point stencil, whose ten single end
+// cells a segment would then lie 16 bytes apart and take four wavefronts a
+// load instead of two (complex64), a unit is a cell.  1024^3 shell,
+// complex64, single cells against 16 bytes: 19-point RK4 step 1.189 -> 1.153 ms,
+// 7-point 0.620 -> 0.640 (more loads), real float imaginary time 0.604 -> 0.634.
+template <typename CT, int NP>
 struct TileMem {
-    static constexpr int UPS = (int)(4 * sizeof(CT) / 16);
-    static constexpr int CPU_ = 4 / UPS;
-    // plane stride with the UPS units of a slot in distinct bank groups
+    using U = typename std::conditional<NP == 19 || sizeof(CT) == 16, CT, uint4>::type;
+    static constexpr int UPS = (int)(4 * sizeof(CT) / sizeof(U)), CPU_ = 4 / UPS;
+    // plane stride with the units of a slot in distinct bank groups
     static int pstr(int nslot)
     {
-        const int want = UPS == 1 ? nslot % 8 : (UPS == 2 ? 4 : 2);
-        return nslot + (want - nslot % 8 + 8) % 8;
+        if (UPS == 4) return nslot;
+        return nslot + ((UPS == 1 ? nslot % 8 : 4) - nslot % 8 + 8) % 8;
     }
-    uint4 *u;
+    U *u;
     int p;
     __device__ __forceinline__ void get(int s, CT (&v)[4]) const
     {
 #pragma unroll
         for (int k = 0; k < UPS; ++k) {
-            const uint4 w = u[k * p + s];
+            const U w = u[k * p + s];
             const CT *c = reinterpret_cast<const CT *>(&w);
 #pragma unroll
             for (int i = 0; i < CPU_; ++i) v[k * CPU_ + i] = c[i];
@@ -73,7 +78,7 @@ struct TileMem {
     {
 #pragma unroll
         for (int k = 0; k < UPS; ++k) {
-            uint4 w;
+            U w;
             CT *c = reinterpret_cast<CT *>(&w);
 #pragma unroll
             for (int i = 0; i < CPU_; ++i) c[i] = v[k * CPU_ + i];
@@ -118,7 +123,7 @@ struct TileSlots<19> {
 // L of a segment with values c and neighbour slots f: the Laplacians, or what
 // LAP makes of them
 template <int NP, typename LAP, typename CT, typename R>
-__device__ __forceinline__ void tile_laplacian(const TileMem<CT> &m, const TileSlots<NP> &f, const CT (&c)[4], R ihx2,
+__device__ __forceinline__ void tile_laplacian(const TileMem<CT, NP> &m, const TileSlots<NP> &f, const CT (&c)[4], R ihx2,
                                                R ihy2, R ihz2, CT (&L)[4])
 {
     // opposite neighbours are summed first and the centre term enters once:
@@ -245,13 +250,13 @@ __device__ __forceinline__ void tile_loop(const TileView &T, TileList list, cons
                                           const R &ihy2, const R &ihz2, SETUP setup, PREF prefetch, LOAD load, BODY body)
 {
     extern __shared__ __align__(16) unsigned char gpe_smem[];
-    using M = TileMem<CT>;
-    const M m{reinterpret_cast<uint4 *>(gpe_smem), T.pstr};
+    using M = TileMem<CT, NP>;
+    const M m{reinterpret_cast<typename M::U *>(gpe_smem), T.pstr};
     const int tid = threadIdx.x;
     const uint32_t step = gridDim.x, nt = (uint32_t)T.ntiles;
     auto cell_of = [](uint32_t e) { return 4u * (e & 0x7fffffffu) + ((e >> 31) ? 0u : 3u); };
     auto cell_at = [&](int sl, uint32_t e) -> CT & { return *((e >> 31) ? m.first(sl) : m.last(sl)); };
-    if (tid < M::UPS) m.u[tid * m.p + TILE] = make_uint4(0u, 0u, 0u, 0u);  // the zero slot
+    if (tid < M::UPS) m.u[tid * m.p + TILE] = typename M::U{};  // the zero slot
     for (uint32_t tile = blockIdx.x; tile < nt; tile += step) {
         if (!setup(tile)) {
             list.fetch(T, tile + step);
@@ -343,18 +348,13 @@ struct TileLaunch {
     TileView T;
     size_t smem;
 };
-template <typename CT>
+template <typename CT, int NP>
 inline TileLaunch tile_launch(const TileTab &t)
 {
-    const int pstr = TileMem<CT>::pstr(t.nslot);
+    using M = TileMem<CT, NP>;
+    const int pstr = M::pstr(t.nslot);
     return {TileView{t.d_nbr, t.d_nbr19, t.d_halo, t.nseg, t.ntiles, t.stride, pstr},
-            16 * (size_t)(TileMem<CT>::UPS * pstr)};
-}
-
-template <typename CT>
-inline TileLaunch tile_launch(const gpe_grid *g)
-{
-    return tile_launch<CT>(g->tiles);
+            sizeof(typename M::U) * (size_t)(M::UPS * pstr)};
 }
 
 // resident blocks an SM of a tile kernel with smem bytes of shared memory;
@@ -370,8 +370,11 @@ inline unsigned tile_blocks(K kernel, int nsm, int n, size_t smem)
     return (unsigned)(res < n ? res : n);
 }
 
-// blocks an SM: registers of 85 (single) and 168 (double) a thread
-#define GPE_TILE_BOUNDS(R) __launch_bounds__(TILE, sizeof(R) == 4 ? 6 : 3)
+// blocks an SM: registers of 85 (single; 102 with the 19-point stencil, whose
+// RK4 step spilled at 85: 1.153 -> 1.024 ms on the 1024^3 shell) and 168 (double) a
+// thread
+constexpr int tile_blocks_f(int np) { return np == 19 ? 5 : 6; }
+#define GPE_TILE_BOUNDS(R, NP) __launch_bounds__(TILE, sizeof(R) == 4 ? tile_blocks_f(NP) : 3)
 
 // the centre's share of the right-hand side with either stencil (App. B's
 // centre weight is c6 - 4 (wxy + wxz + wyz))
@@ -393,7 +396,7 @@ __device__ __forceinline__ R tile_rhs_centre(R ihx2, R ihy2, R ihz2)
 // three 5.69, four 5.80.  One block a tile instead of looping blocks: 8 %
 // slower (no tile ahead to prefetch).
 template <typename R, bool BLEND, int ST, int NP>
-__global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? 6 : 2) k_rk4_tile(const RkArgs<R> a, const TileView T)
+__global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? tile_blocks_f(NP) : 2) k_rk4_tile(const RkArgs<R> a, const TileView T)
 {
     using CT = typename Cx<R>::T;
     using B = Rk4Body<R, BLEND, false, ST>;
