@@ -69,7 +69,7 @@ struct ShellWalk {
     uint32_t nt;
     uint32_t cur = 0xffffffffu, next = 0;
     bool live = false;
-    R g = 0, dt = 0, ihx2 = 0, ihy2 = 0, ihz2 = 0, scale = 0;
+    R g = 0, dt = 0, ihx2 = 0, ihy2 = 0, ihz2 = 0, scale = 0;  // spacings: euler_coef of them, but for the observables
     Sum64<R> sum[NS > 0 ? NS : 1];  // NS 5: the fifth counts non-finite cells
     int nf = 0, n = 0;
     __device__ __forceinline__ ShellWalk(const BatchArgs<R, CT> &a_, uint32_t nt_) : a(a_), nt(nt_)
@@ -105,9 +105,10 @@ struct ShellWalk {
             live = !P.converged;
             g = (R)P.g;
             dt = (R)P.dt;
-            ihx2 = (R)P.ihx2;
-            ihy2 = (R)P.ihy2;
-            ihz2 = (R)P.ihz2;
+            const R q = NS == 5 ? (R)1 : dt / (R)4;
+            ihx2 = euler_coef((R)P.ihx2, q);
+            ihy2 = euler_coef((R)P.ihy2, q);
+            ihz2 = euler_coef((R)P.ihz2, q);
             scale = (R)P.scale;
         }
         return live;
@@ -159,7 +160,7 @@ __global__ void GPE_TILE_BOUNDS(R, 7) k_batch_itp(const BatchArgs<R, CT> a, cons
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const bool act = active_e(E[i]);
-            o[i] = axpy(c[i], q4, L[i]);
+            o[i] = euler(c[i], q4, L[i]);
             if (STAGE == 1) {
                 const R f = act ? E[i] * ((R)1 - hg * norm2(o[i])) : (R)0;
                 o[i] = scale(o[i], f);
@@ -175,10 +176,10 @@ __global__ void GPE_TILE_BOUNDS(R, 7) k_batch_itp(const BatchArgs<R, CT> a, cons
         }
     };
     if constexpr (STAGE == 0)
-        tile_loop<7>(T, list, (const CT *)a.psi, WalkDiag<R, CT, W>{w, a.E}, w.ihx2, w.ihy2, w.ihz2, enter, pref,
+        tile_loop<7, LapEuler>(T, list, (const CT *)a.psi, WalkDiag<R, CT, W>{w, a.E}, w.ihx2, w.ihy2, w.ihz2, enter, pref,
                      ELoad<R>{a.E}, body);
     else
-        tile_loop<7>(T, list, (const CT *)a.tmp, Plain(), w.ihx2, w.ihy2, w.ihz2, enter, pref, ELoad<R>{a.E}, body);
+        tile_loop<7, LapEuler>(T, list, (const CT *)a.tmp, Plain(), w.ihx2, w.ihy2, w.ihz2, enter, pref, ELoad<R>{a.E}, body);
     w.leave();
 }
 

@@ -107,8 +107,9 @@ __device__ __forceinline__ void itp_pair_brick(ItpPairSpace<typename Cx<R>::T, B
     constexpr int SX = PS::SX, PL = PS::PLANE_B;
     auto &ps = sp.ps;
     const int t = threadIdx.x;
-    const R c6 = (R)2 * (a.ihx2 + a.ihy2 + a.ihz2);
     const R q4 = a.dt / (R)4, hg = a.g * a.dt / (R)2;
+    const R ax = euler_coef(a.ihx2, q4), ay = euler_coef(a.ihy2, q4), az = euler_coef(a.ihz2, q4);
+    const R c6 = (R)2 * (ax + ay + az);
     pair_fill(ps, P, b, a.psi, EFill<CT, BX, BY, BZ>{&sp, a.E});
     for (int i = t; i < PS::UPS * PS::VPSTR; i += PAIR_THREADS) (&ps.v[0][0])[i] = make_uint4(0, 0, 0, 0);
     for (int i = t; i < BY * BZ; i += PAIR_THREADS) {
@@ -172,10 +173,10 @@ __device__ __forceinline__ void itp_pair_brick(ItpPairSpace<typename Cx<R>::T, B
         if (!ok) continue;
         CT c[4], L[4], o[4];
         R e4[4];
-        pair_lap_u(ps, hx, y, z, c, L, a.ihx2, a.ihy2, a.ihz2, c6);
+        pair_lap_u<LapEuler>(ps, hx, y, z, c, L, ax, ay, az, c6);
         sp.eget(PS::slot(hx, y, z), e4);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) o[k] = e4[k] >= (R)0 ? axpy(c[k], q4, L[k]) : czero<CT>();
+        for (int k = 0; k < 4; ++k) o[k] = e4[k] >= (R)0 ? euler(c[k], q4, L[k]) : czero<CT>();
         ps.vput(PS::vslot(hx, y, z), o);
     }
     // the same on the single cells of the one-deep x face layers
@@ -206,8 +207,8 @@ __device__ __forceinline__ void itp_pair_brick(ItpPairSpace<typename Cx<R>::T, B
             zm = ps.uxr[PS::row(y, z - 1)][0];
             zp = ps.uxr[PS::row(y, z + 1)][0];
         }
-        const CT L = lapv(xp, xm, yp, ym, zp, zm, c0, a.ihx2, a.ihy2, a.ihz2, c6);
-        (side == 0 ? ps.vxl : ps.vxr)[PS::vrow(y, z)] = e >= (R)0 ? axpy(c0, q4, L) : czero<CT>();
+        const CT L = LapEuler::of(xp, xm, yp, ym, zp, zm, c0, ax, ay, az, c6);
+        (side == 0 ? ps.vxl : ps.vxr)[PS::vrow(y, z)] = e >= (R)0 ? euler(c0, q4, L) : czero<CT>();
     }
     __syncthreads();
     // second Euler substep, second half step and the norm on the brick
@@ -217,11 +218,11 @@ __device__ __forceinline__ void itp_pair_brick(ItpPairSpace<typename Cx<R>::T, B
         CT c[4], L[4], o[4];
         R e4[4];
         R n4 = (R)0;  // the segment's |psi|^2, added to the FP64 sum once
-        pair_lap_v(ps, hx, y, z, c, L, a.ihx2, a.ihy2, a.ihz2, c6);
+        pair_lap_v<LapEuler>(ps, hx, y, z, c, L, ax, ay, az, c6);
         sp.eget(PS::slot(hx, y, z), e4);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            o[k] = axpy(c[k], q4, L[k]);
+            o[k] = euler(c[k], q4, L[k]);
             const R f = e4[k] >= (R)0 ? e4[k] * ((R)1 - hg * norm2(o[k])) : (R)0;
             o[k] = scale(o[k], f);
             n4 = add_rn(n4, norm2(o[k]));

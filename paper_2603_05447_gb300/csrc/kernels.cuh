@@ -65,14 +65,15 @@ __device__ __forceinline__ void itp_brick_a(const ItpArgs<R, CT> &a, const GridV
                                             WarpSpace<CT, BX, BY, BZ> &ws, R sc)
 {
     const R q4 = a.dt / (R)4;
+    const R ax = euler_coef(a.ihx2, q4), ay = euler_coef(a.ihy2, q4), az = euler_coef(a.ihz2, q4);
     const DiagLoad<R, CT> diag{sc, a.g * a.dt / (R)2, a.E};
-    brick_apply<BX, BY, BZ, CG>(ws, G, b, next, a.psi, diag, a.ihx2, a.ihy2, a.ihz2, ELoad<R>{a.E},
+    brick_apply<BX, BY, BZ, CG, LapEuler>(ws, G, b, next, a.psi, diag, ax, ay, az, ELoad<R>{a.E},
                                 [&](uint32_t idx, const typename ELoad<R>::P &p, const CT(&c)[4], const CT(&L)[4]) {
         CT o[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const bool act = p.e[i] >= (R)0;  // E < 0 marks an inactive cell of a stored segment
-            o[i] = act ? axpy(c[i], q4, L[i]) : czero<CT>();
+            o[i] = act ? euler(c[i], q4, L[i]) : czero<CT>();
         }
         st4(a.tmp + idx, o);
     });
@@ -84,13 +85,14 @@ __device__ __forceinline__ void itp_brick_b(const ItpArgs<R, CT> &a, const GridV
 {
     const R hg = a.g * a.dt / (R)2;
     const R q4 = a.dt / (R)4;
-    brick_apply<BX, BY, BZ, CG>(ws, G, b, next, a.tmp, Identity(), a.ihx2, a.ihy2, a.ihz2, ELoad<R>{a.E},
+    const R ax = euler_coef(a.ihx2, q4), ay = euler_coef(a.ihy2, q4), az = euler_coef(a.ihz2, q4);
+    brick_apply<BX, BY, BZ, CG, LapEuler>(ws, G, b, next, a.tmp, Identity(), ax, ay, az, ELoad<R>{a.E},
                                 [&](uint32_t idx, const typename ELoad<R>::P &p, const CT(&c)[4], const CT(&L)[4]) {
         CT o[4];
         R n4 = (R)0;  // the segment's |psi|^2, added to the FP64 sum once
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            o[i] = axpy(c[i], q4, L[i]);
+            o[i] = euler(c[i], q4, L[i]);
             const R f = p.e[i] >= (R)0 ? p.e[i] * ((R)1 - hg * norm2(o[i])) : (R)0;
             o[i] = scale(o[i], f);
             n4 = add_rn(n4, norm2(o[i]));
@@ -231,6 +233,7 @@ __device__ __forceinline__ void block_totals(Sum64<double> (&s)[NV], bool, doubl
     }
     __syncthreads();
 #pragma unroll
+    const R ax = euler_coef(a.ihx2, q4), ay = euler_coef(a.ihy2, q4), az = euler_coef(a.ihz2, q4);
     for (int k = 0; k < NV; ++k) out[k] = so[k];
     __syncthreads();
 }
@@ -252,6 +255,7 @@ __device__ __forceinline__ bool launch_totals(double (&v)[NV], double *partials,
     if (!is_last) return false;
     __threadfence();
     Sum64<double> s[NV];
+    const R ax = euler_coef(a.ihx2, q4), ay = euler_coef(a.ihy2, q4), az = euler_coef(a.ihz2, q4);
     for (int i = threadIdx.x; i < (int)gridDim.x; i += 4 * TILE) {
         double x[4][NV];  // four blocks' values in flight a thread
 #pragma unroll
@@ -273,14 +277,14 @@ __global__ void GPE_TILE_BOUNDS(R, NP) k_itp_a(const ItpArgs<R, CT> a, const Til
     const TileList list = tile_begin(T);
     const R q4 = a.dt / (R)4;
     const TileDiag<R, CT> diag{{(R)a.scalars[0], a.g * a.dt / (R)2, a.E}};
-    tile_loop<NP>(T, list, (const CT *)a.psi, diag, a.ihx2, a.ihy2, a.ihz2, EveryTile(),
+    tile_loop<NP, LapEuler>(T, list, (const CT *)a.psi, diag, ax, ay, az, EveryTile(),
                   [&](uint32_t idx, uint32_t n) { prefetch_l2(a.E + idx, n * (uint32_t)sizeof(R)); }, ELoad<R>{a.E},
                   [&](uint32_t idx, const typename ELoad<R>::P &p, const CT(&c)[4], const CT(&L)[4]) {
                       CT o[4];
 #pragma unroll
                       for (int i = 0; i < 4; ++i) {
                           // E < 0 marks an inactive cell of a stored segment
-                          o[i] = active_e(p.e[i]) ? axpy(c[i], q4, L[i]) : czero<CT>();
+                          o[i] = active_e(p.e[i]) ? euler(c[i], q4, L[i]) : czero<CT>();
                       }
                       st4(a.tmp + idx, o);
                   });
@@ -295,14 +299,14 @@ __global__ void GPE_TILE_BOUNDS(R, NP) k_itp_b(const ItpArgs<R, CT> a, const Til
     const R q4 = a.dt / (R)4;
     Sum64<R> norm[1];
     int n = 0;
-    tile_loop<NP>(T, list, (const CT *)a.tmp, Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
+    tile_loop<NP, LapEuler>(T, list, (const CT *)a.tmp, Plain(), ax, ay, az, EveryTile(),
                   [&](uint32_t idx, uint32_t n) { prefetch_l2(a.E + idx, n * (uint32_t)sizeof(R)); }, ELoad<R>{a.E},
                   [&](uint32_t idx, const typename ELoad<R>::P &p, const CT(&c)[4], const CT(&L)[4]) {
                       CT o[4];
                       R n4 = (R)0;  // the segment's |psi|^2, added to the FP64 sum once
 #pragma unroll
                       for (int i = 0; i < 4; ++i) {
-                          o[i] = axpy(c[i], q4, L[i]);
+                          o[i] = euler(c[i], q4, L[i]);
                           const R f = active_e(p.e[i]) ? p.e[i] * ((R)1 - hg * norm2(o[i])) : (R)0;
                           o[i] = scale(o[i], f);
                           n4 = add_rn(n4, norm2(o[i]));
