@@ -221,6 +221,7 @@ struct gpe_tape {
     void *d_stages = nullptr;  // [3 * K * n_packed] the stage states of a segment's steps, where memory allows
     void *d_lam = nullptr, *d_mu[2] = {nullptr, nullptr}, *d_acc = nullptr;
     void *d_w[4] = {nullptr, nullptr, nullptr, nullptr};  // Y2, Y3, Y4, RK4 partial sum
+    void *block = nullptr;     // the allocation that holds every array but the stage states
     double *d_grad = nullptr;
     double *d_clock = nullptr;
     double *d_stab = nullptr;  // [3 * K] schedule values of a segment's stages
@@ -230,18 +231,8 @@ struct gpe_tape {
 static void tape_free(gpe_tape *t)
 {
     if (!t) return;
-    dev_free(t->d_ckpt);
-    dev_free(t->d_seg);
+    dev_free(t->block);
     dev_free(t->d_stages);
-    dev_free(t->d_stab);
-    dev_free(t->d_lam);
-    dev_free(t->d_mu[0]);
-    dev_free(t->d_mu[1]);
-    dev_free(t->d_acc);
-    for (int i = 0; i < 4; ++i) dev_free(t->d_w[i]);
-    dev_free(t->d_grad);
-    dev_free(t->d_clock);
-    red_free(t->red);
     if (t->st) t->st->grid->n_states--;
     delete t;
 }
@@ -271,13 +262,23 @@ extern "C" int gpe_ramp_forward(gpe_state *st, const gpe_real_params *p, int64_t
     t->t0 = t0;
     t->K = (int)std::min<int64_t>(K, nsteps);
     t->nck = (nsteps + t->K - 1) / t->K;
-    int rc = GPE_OK;
-    rc = dev_alloc(&t->d_ckpt, bytes * t->nck);
-    if (rc == GPE_OK) rc = dev_alloc(&t->d_seg, bytes * t->K);
     // every pass writes whole segments before the next one reads them: no zeroing
-    for (void **b : {&t->d_lam, &t->d_mu[0], &t->d_mu[1], &t->d_acc, &t->d_w[0], &t->d_w[1], &t->d_w[2], &t->d_w[3]})
-        if (rc == GPE_OK) rc = dev_alloc(b, bytes);
-    if (rc == GPE_OK) rc = dev_alloc_t(&t->d_stab, 3 * (size_t)t->K);
+    int rc = dev_alloc_parts(&t->block, {{&t->d_ckpt, bytes * t->nck},
+                                         {&t->d_seg, bytes * t->K},
+                                         {&t->d_lam, bytes},
+                                         {&t->d_mu[0], bytes},
+                                         {&t->d_mu[1], bytes},
+                                         {&t->d_acc, bytes},
+                                         {&t->d_w[0], bytes},
+                                         {&t->d_w[1], bytes},
+                                         {&t->d_w[2], bytes},
+                                         {&t->d_w[3], bytes},
+                                         {&t->d_stab, 3 * (size_t)t->K},
+                                         {&t->d_grad, GPE_MAX_KNOTS},
+                                         {&t->d_clock, 1},
+                                         red_partials(t->red, g->nsm),
+                                         red_counter(t->red),
+                                         red_scalars(t->red)});
     // The reverse sweep needs every step's stage states.  Kept from the
     // segment's recomputation they save three of its fifteen passes a step
     // (512^3 ramp, 48 steps, K = 16: 32.5 -> 27.4 ms with the schedule table); they are kept where they take at
@@ -289,9 +290,7 @@ extern "C" int gpe_ramp_forward(gpe_state *st, const gpe_real_params *p, int64_t
             t->d_stages = nullptr;
         cudaGetLastError();
     }
-    if (rc == GPE_OK) rc = dev_alloc_t(&t->d_grad, GPE_MAX_KNOTS);
-    if (rc == GPE_OK) rc = dev_alloc_t(&t->d_clock, 1);
-    if (rc == GPE_OK) rc = red_alloc(t->red, g->nsm * 32);
+    if (rc == GPE_OK) rc = red_zero(t->red);
     if (rc != GPE_OK) {
         tape_free(t);
         return rc;

@@ -46,6 +46,20 @@ int dev_alloc(void **p, size_t bytes)
     return GPE_OK;
 }
 
+int dev_alloc_parts(void **base, std::initializer_list<Part> parts)
+{
+    constexpr size_t ALIGN = 512;
+    size_t total = 0;
+    for (const Part &a : parts) total += (a.bytes + ALIGN - 1) / ALIGN * ALIGN;
+    GPE_TRY(dev_alloc(base, total));
+    char *at = static_cast<char *>(*base);
+    for (const Part &a : parts) {
+        *a.p = at;
+        at += (a.bytes + ALIGN - 1) / ALIGN * ALIGN;
+    }
+    return GPE_OK;
+}
+
 void dev_free(void *p)
 {
     if (p) cudaFree(p);
@@ -78,25 +92,10 @@ int sm_count(int device)
     return n;
 }
 
-int red_alloc(RedScratch &r, int max_blocks)
+int red_zero(const RedScratch &r)
 {
-    if (r.max_blocks >= max_blocks) return GPE_OK;
-    red_free(r);
-    GPE_TRY(dev_alloc_t(&r.partials, (size_t)max_blocks * 8));
-    GPE_TRY(dev_alloc_t(&r.counter, 1));
-    GPE_TRY(dev_alloc_t(&r.scalars, 16));
     GPE_TRY(dev_zero(r.counter, sizeof(unsigned int)));
-    GPE_TRY(dev_zero(r.scalars, 16 * sizeof(double)));
-    r.max_blocks = max_blocks;
-    return GPE_OK;
-}
-
-void red_free(RedScratch &r)
-{
-    dev_free(r.partials);
-    dev_free(r.counter);
-    dev_free(r.scalars);
-    r = RedScratch{};
+    return dev_zero(r.scalars, 16 * sizeof(double));
 }
 
 int launch_blocks(const gpe_grid *g, int threads, int per_sm)

@@ -22,6 +22,7 @@
 
 #include <cstdint>
 #include <cstdio>
+#include <initializer_list>
 #include <vector>
 
 #include "gpe.h"
@@ -59,6 +60,19 @@ inline int dev_alloc_t(T **p, size_t count)
     return dev_alloc(reinterpret_cast<void **>(p), count * sizeof(T));
 }
 void dev_free(void *p);
+// Arrays that live and die together, in one allocation at *base: a cudaMalloc
+// and its cudaFree take 50 to 70 us, and each regrid, state and tape used to
+// make 10 to 17 of them (four regrids and states of a 512^3 ramp: 8 of 34 ms)
+struct Part {
+    void **p;
+    size_t bytes;
+    template <typename T>
+    Part(T **p_, size_t count) : p(reinterpret_cast<void **>(p_)), bytes(count * sizeof(T))
+    {
+    }
+    Part(void **p_, size_t bytes_) : p(p_), bytes(bytes_) {}
+};
+int dev_alloc_parts(void **base, std::initializer_list<Part> parts);
 int dev_zero(void *p, size_t bytes);  // memset 0 and wait (any stream may use it next)
 
 inline cudaStream_t S(gpe_stream s) { return reinterpret_cast<cudaStream_t>(s); }
@@ -184,10 +198,14 @@ struct RedScratch {
     double *partials = nullptr;
     unsigned int *counter = nullptr;
     double *scalars = nullptr;  // [0] ITP scale, [1] last norm, [2..9] observables
-    int max_blocks = 0;
 };
-int red_alloc(RedScratch &r, int max_blocks);
-void red_free(RedScratch &r);
+// the reductions' arrays for up to nsm * RED_PER_SM blocks, as parts of a
+// caller's allocation; red_zero when they are in place
+constexpr int RED_PER_SM = 32;
+inline Part red_partials(RedScratch &r, int nsm) { return Part(&r.partials, (size_t)nsm * RED_PER_SM * 8); }
+inline Part red_counter(RedScratch &r) { return Part(&r.counter, 1); }
+inline Part red_scalars(RedScratch &r) { return Part(&r.scalars, 16); }
+int red_zero(const RedScratch &r);
 
 // stored segments a tile, and threads a block of the tile kernels (tiles.cuh)
 constexpr int TILE = 128;
@@ -219,6 +237,8 @@ struct gpe_grid {
     gpe::BrickRec *d_rec7 = nullptr;  // [nb*7] record of each brick and of its six face neighbours (wavefront schedules)
     int stencil = 7;                  // 7 or 19 points
     int32_t *d_nbr18 = nullptr;       // [nb*18] face then edge neighbour ids (PAIR schedule, built on first use)
+    std::vector<void *> blocks;  // the allocations that hold the arrays above and below, but d_rec7, d_nbr18, d_Vf
+                                 // and the wavefront schedules'
     gpe::TileTab tiles;         // the stencil kernels' tiles
     int32_t *d_bvol = nullptr;  // brick-grid volume nbx*nby*nbz -> brick id or -1
     double *d_V[2] = {nullptr, nullptr};
@@ -247,7 +267,9 @@ struct gpe_state {
     int dtype = GPE_C128;
     size_t elem = 16;       // bytes per complex element
     void *d_psi = nullptr;  // n_packed complex
+    void *block = nullptr;  // the allocation that holds psi, E, the clock and the reductions' arrays
     void *d_work[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};  // RK stage states / ITP tmp
+    std::vector<void *> work_blocks;                                           // the allocations that hold them
     void *d_E = nullptr;    // ITP exp(-V dt/2), state precision
     double E_dt = -1.0;     // dt that d_E was made for
     double *d_clock = nullptr;  // device time base for ramps
@@ -271,7 +293,7 @@ struct gpe_state {
 };
 
 namespace gpe {
-int tiles_build(gpe_grid *g, cudaStream_t st);
+int tiles_build(gpe_grid *g, int *d_hmax, cudaStream_t st);
 void tiles_free(TileTab &t);
 int ensure_stab(gpe_state *st, int steps);      // room for the schedule values of `steps` steps
 int ensure_work(gpe_state *st, int n);          // allocate d_work[0..n-1] (zeroed)

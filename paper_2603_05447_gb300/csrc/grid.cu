@@ -437,25 +437,25 @@ __global__ void k_enum_emit(Enum E, const uint8_t *occ, const int64_t *boff, int
     }
 }
 
-// (3) brick-id volume, origins, neighbour table
-__global__ void k_bricks(int64_t nb, const int32_t *coords, int BX, int BY, int BZ,
-                         int64_t nbx, int64_t nby, int32_t *bvol, int32_t *org)
+// (3) brick-id volume, from the bricks' positions
+__global__ void k_bricks(int64_t nb, const int32_t *coords, int64_t nbx, int64_t nby, int32_t *bvol)
 {
     int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (id >= nb) return;
     int64_t bx = coords[3 * id], by = coords[3 * id + 1], bz = coords[3 * id + 2];
     bvol[bx + nbx * (by + nby * bz)] = (int32_t)id;
-    org[3 * id + 0] = (int32_t)(bx * BX);
-    org[3 * id + 1] = (int32_t)(by * BY);
-    org[3 * id + 2] = (int32_t)(bz * BZ);
 }
 
-__global__ void k_neighbors(int64_t nb, const int32_t *coords, int64_t nbx, int64_t nby,
-                            int64_t nbz, const int32_t *bvol, int32_t *nbr)
+// neighbour table; then the bricks' positions become their origins in cells
+__global__ void k_neighbors(int64_t nb, int32_t *coords, int BX, int BY, int BZ, int64_t nbx, int64_t nby, int64_t nbz,
+                            const int32_t *bvol, int32_t *nbr)
 {
     int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (id >= nb) return;
     const int64_t c[3] = {coords[3 * id], coords[3 * id + 1], coords[3 * id + 2]};
+    coords[3 * id] = (int32_t)(c[0] * BX);
+    coords[3 * id + 1] = (int32_t)(c[1] * BY);
+    coords[3 * id + 2] = (int32_t)(c[2] * BZ);
     const int64_t n[3] = {nbx, nby, nbz};
     for (int d = 0; d < 6; ++d) {
         int64_t q[3] = {c[0], c[1], c[2]};
@@ -649,23 +649,16 @@ static PotDesc potdesc(const gpe_potential &p)
 static void grid_free(gpe_grid *g)
 {
     if (!g) return;
-    dev_free(g->d_rec);
+    for (void *b : g->blocks) dev_free(b);
     dev_free(g->d_rec7);
-    tiles_free(g->tiles);
+    dev_free(g->tiles.d_halo);
     dev_free(g->d_nbr18);
     dev_free(g->d_chunk_lohi);
     dev_free(g->d_tasks);
     dev_free(g->d_dep_off);
     dev_free(g->d_dep_ids);
     dev_free(g->d_tasks_w);
-    dev_free(g->d_org);
-    dev_free(g->d_nbr);
-    dev_free(g->d_mask);
-    dev_free(g->d_bvol);
-    for (int s = 0; s < 2; ++s) {
-        dev_free(g->d_V[s]);
-        dev_free(g->d_Vf[s]);
-    }
+    for (int s = 0; s < 2; ++s) dev_free(g->d_Vf[s]);
     delete g;
 }
 
@@ -712,30 +705,29 @@ static int build_grid(const gpe_box *box, const VSource &src, const gpe_grid_opt
     const int64_t nq = g->nbx * g->nby * g->nbz;
     const BoxD bd = boxd(*box);
 
-    // temporaries: occupancy, block counts and totals, then per-brick data
+    // temporaries: occupancy, block counts and totals, then the analytic
+    // potentials on the lattice
     uint8_t *occ = nullptr;
     int64_t *bsum = nullptr;
-    int32_t *coords = nullptr;
     double *tmpV[2] = {nullptr, nullptr};
     // read back together: bricks kept; stored segments, active cells, largest |V|
     struct Totals {
         int64_t bricks, segs;
         unsigned long long active, vmax;
+        int hmax;  // tiles_build's
     };
     Totals *tot = nullptr, ht{};
+    void *temp[2] = {nullptr, nullptr};
     int rc = GPE_OK;
     auto cleanup = [&]() {
-        dev_free(occ);
-        dev_free(bsum);
-        dev_free(coords);
-        dev_free(tot);
-        dev_free(tmpV[0]);
-        dev_free(tmpV[1]);
-        occ = nullptr;
-        bsum = nullptr;
-        coords = nullptr;
-        tot = nullptr;
-        tmpV[0] = tmpV[1] = nullptr;
+        for (void *b : temp) dev_free(b);
+    };
+    // arrays of the grid, in one allocation
+    auto alloc_own = [&](std::initializer_list<Part> parts) -> int {
+        void *b = nullptr;
+        GPE_TRY(dev_alloc_parts(&b, parts));
+        g->blocks.push_back(b);
+        return GPE_OK;
     };
 #define BUILD_TRY(x)                 \
     do {                             \
@@ -760,25 +752,6 @@ static int build_grid(const gpe_box *box, const VSource &src, const gpe_grid_opt
     const bool dense = src.mode == 0 || src.mode == 3, two = src.mode == 2 || src.mode == 3;
     const Limit c0 = limit_of(src.cut0), c1 = limit_of(src.cut1);
     const BrickGeo geo = brick_geo(o.by, o.bz);
-    BUILD_TRY(dev_alloc_t(&tot, 1));
-    BUILD_CUDA(cudaMemsetAsync(tot, 0, sizeof(Totals), st));
-    BUILD_TRY(dev_alloc_t(&occ, nq));
-    if (dense) {
-        BUILD_CUDA(cudaMemsetAsync(occ, 0, nq, st));
-        const unsigned nblk_rows = (unsigned)std::min<int64_t>((box->ny * box->nz + 7) / 8, (int64_t)g->nsm * 64);
-        if (src.dtype == GPE_F64)
-            k_occ_dense<double><<<nblk_rows, 256, 0, st>>>((const double *)src.dense, (const double *)src.dense1, c0, c1,
-                                                          bd, o.by, o.bz, g->nbx, g->nby, occ);
-        else
-            k_occ_dense<float><<<nblk_rows, 256, 0, st>>>((const float *)src.dense, (const float *)src.dense1, c0, c1,
-                                                         bd, o.by, o.bz, g->nbx, g->nby, occ);
-        BUILD_CUDA(cudaGetLastError());
-    } else {
-        const int64_t nblk_occ = (nq + 255) / 256;
-        if (nblk_occ > 0x7fffffffLL) BUILD_TRY(fail(GPE_ERR_ARG, "brick grid too large"));
-        k_occupancy<<<(unsigned)nblk_occ, 256, 0, st>>>(src, bd, o.bx, o.by, o.bz, g->nbx, g->nby, g->nbz, occ);
-        BUILD_CUDA(cudaGetLastError());
-    }
     Enum E;
     E.order = o.order;
     E.nbx = g->nbx;
@@ -795,7 +768,27 @@ static int build_grid(const gpe_box *box, const VSource &src, const gpe_grid_opt
     }
     const int64_t nblk = (int64_t)((E.nkeys + ENUM_PER_BLOCK - 1) / ENUM_PER_BLOCK);
     if (nblk > 0x7fffffffLL) BUILD_TRY(fail(GPE_ERR_ARG, "brick grid too large"));
-    BUILD_TRY(dev_alloc_t(&bsum, nblk));
+    // block counts: of the enumeration, then of the records (at most nq bricks)
+    BUILD_TRY(dev_alloc_parts(&temp[0], {{&tot, 1},
+                                         {&bsum, (size_t)std::max(nblk, (nq + REC_THREADS - 1) / REC_THREADS)},
+                                         {&occ, (size_t)nq}}));
+    BUILD_CUDA(cudaMemsetAsync(tot, 0, sizeof(Totals), st));
+    if (dense) {
+        BUILD_CUDA(cudaMemsetAsync(occ, 0, nq, st));
+        const unsigned nblk_rows = (unsigned)std::min<int64_t>((box->ny * box->nz + 7) / 8, (int64_t)g->nsm * 64);
+        if (src.dtype == GPE_F64)
+            k_occ_dense<double><<<nblk_rows, 256, 0, st>>>((const double *)src.dense, (const double *)src.dense1, c0, c1,
+                                                          bd, o.by, o.bz, g->nbx, g->nby, occ);
+        else
+            k_occ_dense<float><<<nblk_rows, 256, 0, st>>>((const float *)src.dense, (const float *)src.dense1, c0, c1,
+                                                         bd, o.by, o.bz, g->nbx, g->nby, occ);
+        BUILD_CUDA(cudaGetLastError());
+    } else {
+        const int64_t nblk_occ = (nq + 255) / 256;
+        if (nblk_occ > 0x7fffffffLL) BUILD_TRY(fail(GPE_ERR_ARG, "brick grid too large"));
+        k_occupancy<<<(unsigned)nblk_occ, 256, 0, st>>>(src, bd, o.bx, o.by, o.bz, g->nbx, g->nby, g->nbz, occ);
+        BUILD_CUDA(cudaGetLastError());
+    }
     k_enum_count<<<(unsigned)nblk, ENUM_THREADS, 0, st>>>(E, occ, bsum);
     BUILD_CUDA(cudaGetLastError());
     k_scan<<<1, 1024, 0, st>>>(bsum, nblk, &tot->bricks);
@@ -808,21 +801,20 @@ static int build_grid(const gpe_box *box, const VSource &src, const gpe_grid_opt
         BUILD_TRY(fail(GPE_ERR_ARG, "too many stored cells"));
     g->nb = total;
     g->n_stored = total * g->bc;
-    BUILD_TRY(dev_alloc_t(&coords, 3 * total));
-    k_enum_emit<<<(unsigned)nblk, ENUM_THREADS, 0, st>>>(E, occ, bsum, coords);
+    BUILD_TRY(alloc_own({{&g->d_bvol, (size_t)nq},
+                         {&g->d_org, 3 * (size_t)total},
+                         {&g->d_nbr, 6 * (size_t)total},
+                         {&g->d_mask, (size_t)(g->n_stored / 32)},
+                         {&g->d_rec, (size_t)total}}));
+    k_enum_emit<<<(unsigned)nblk, ENUM_THREADS, 0, st>>>(E, occ, bsum, g->d_org);
     BUILD_CUDA(cudaGetLastError());
-
-    BUILD_TRY(dev_alloc_t(&g->d_bvol, nq));
     BUILD_CUDA(cudaMemsetAsync(g->d_bvol, 0xff, nq * sizeof(int32_t), st));
-    BUILD_TRY(dev_alloc_t(&g->d_org, 3 * total));
-    BUILD_TRY(dev_alloc_t(&g->d_nbr, 6 * total));
     const unsigned nbb = (unsigned)((total + 255) / 256);
-    k_bricks<<<nbb, 256, 0, st>>>(total, coords, o.bx, o.by, o.bz, g->nbx, g->nby, g->d_bvol, g->d_org);
+    k_bricks<<<nbb, 256, 0, st>>>(total, g->d_org, g->nbx, g->nby, g->d_bvol);
     BUILD_CUDA(cudaGetLastError());
-    k_neighbors<<<nbb, 256, 0, st>>>(total, coords, g->nbx, g->nby, g->nbz, g->d_bvol, g->d_nbr);
+    k_neighbors<<<nbb, 256, 0, st>>>(total, g->d_org, o.bx, o.by, o.bz, g->nbx, g->nby, g->nbz, g->d_bvol, g->d_nbr);
     BUILD_CUDA(cudaGetLastError());
 
-    BUILD_TRY(dev_alloc_t(&g->d_mask, g->n_stored / 32));
     if (total > 0x7fffffffLL) BUILD_TRY(fail(GPE_ERR_ARG, "too many bricks"));
     if (two) g->n_slots = 2;
     if (dense) {
@@ -837,8 +829,8 @@ static int build_grid(const gpe_box *box, const VSource &src, const gpe_grid_opt
                                                     geo, o.mask_mode, g->d_org, nwords, g->d_mask,
                                                     &tot->active);
     } else {
-        BUILD_TRY(dev_alloc_t(&tmpV[0], g->n_stored));
-        if (two) BUILD_TRY(dev_alloc_t(&tmpV[1], g->n_stored));
+        BUILD_TRY(dev_alloc_parts(&temp[1], {{&tmpV[0], (size_t)g->n_stored}, {&tmpV[1], two ? (size_t)g->n_stored : 0}}));
+        if (!two) tmpV[1] = nullptr;
         k_cells<<<(unsigned)total, std::min(g->bc, 256), 0, st>>>(src, bd, o.bx, o.by, o.bz, o.mask_mode, g->d_org,
                                                                 tmpV[0], tmpV[1], g->d_mask, &tot->active, &tot->vmax);
     }
@@ -846,13 +838,7 @@ static int build_grid(const gpe_box *box, const VSource &src, const gpe_grid_opt
 
     // packed layout: every brick stores its segments (4 cells along x) that
     // hold an active cell, in lattice order, as one run
-    BUILD_TRY(dev_alloc_t(&g->d_rec, total));
     const int64_t nblk_rec = (total + REC_THREADS - 1) / REC_THREADS;
-    if (nblk_rec > nblk) {
-        dev_free(bsum);
-        bsum = nullptr;
-        BUILD_TRY(dev_alloc_t(&bsum, nblk_rec));
-    }
     k_seg_records<<<(unsigned)nblk_rec, REC_THREADS, 0, st>>>(total, g->bc, g->d_mask, g->d_rec, bsum);
     BUILD_CUDA(cudaGetLastError());
     k_scan<<<1, 1024, 0, st>>>(bsum, nblk_rec, &tot->segs);
@@ -877,8 +863,13 @@ static int build_grid(const gpe_box *box, const VSource &src, const gpe_grid_opt
         BUILD_CUDA(cudaMemcpyAsync(g->d_rec7, h7.data(), h7.size() * sizeof(BrickRec), cudaMemcpyHostToDevice, st));
         BUILD_CUDA(cudaStreamSynchronize(st));
     }
-    BUILD_TRY(tiles_build(g, st));
-    for (int sl = 0; sl < g->n_slots; ++sl) BUILD_TRY(dev_alloc_t(&g->d_V[sl], g->n_packed));
+    const size_t np = (size_t)g->n_packed;
+    BUILD_TRY(alloc_own({{&g->d_V[0], np},
+                         {&g->d_V[1], two ? np : 0},
+                         {&g->tiles.d_nbr, g->stencil == 19 ? 0 : np / 4},
+                         {&g->tiles.d_nbr19, g->stencil == 19 ? np / 2 : 0}}));
+    if (!two) g->d_V[1] = nullptr;
+    BUILD_TRY(tiles_build(g, &tot->hmax, st));
     if (dense) {
         const unsigned nbf = (unsigned)g->nsm * 16;
         if (src.dtype == GPE_F64)
@@ -1042,6 +1033,7 @@ extern "C" int gpe_grid_set_potential(gpe_grid *g, int slot, const void *V, int 
     int rc = GPE_OK;
     if (!g->d_V[slot]) {
         rc = dev_alloc_t(&g->d_V[slot], g->n_packed);
+        if (rc == GPE_OK) g->blocks.push_back(g->d_V[slot]);
         if (rc == GPE_OK) rc = dev_zero(g->d_V[slot], g->n_packed * sizeof(double));
     }
     if (rc == GPE_OK) {

@@ -475,11 +475,19 @@ int ensure_stab(gpe_state *st, int steps)
 
 int ensure_work(gpe_state *st, int n)
 {
-    for (int i = 0; i < n; ++i) {
-        if (st->d_work[i]) continue;
-        GPE_TRY(dev_alloc(&st->d_work[i], st->grid->n_packed * st->elem));
-        GPE_TRY(dev_zero(st->d_work[i], st->grid->n_packed * st->elem));
+    int have = 0;  // they are made in order
+    while (have < n && st->d_work[have]) ++have;
+    if (have == n) return GPE_OK;
+    const size_t bytes = (st->grid->n_packed * st->elem + 511) / 512 * 512;
+    char *b = nullptr;
+    GPE_TRY(dev_alloc_t(&b, bytes * (n - have)));
+    const int rc = dev_zero(b, bytes * (n - have));
+    if (rc != GPE_OK) {
+        dev_free(b);
+        return rc;
     }
+    st->work_blocks.push_back(b);
+    for (int i = have; i < n; ++i) st->d_work[i] = b + bytes * (i - have);
     return GPE_OK;
 }
 
@@ -1119,7 +1127,7 @@ static int itp_run(gpe_state *st, const gpe_imag_params *p, int64_t nsteps, cuda
         auto k = k_itp_fused<R, BX, BY, BZ>;
         const size_t psm = sizeof(ItpPairSpace<CT, BX, BY, BZ>);
         const int64_t res = (int64_t)g->nsm * per_sm_for(k, PAIR_THREADS, psm);
-        const int nbk = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(g->nb, res), st->red.max_blocks));
+        const int nbk = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(g->nb, res), g->nsm * RED_PER_SM));
         CT *bufA = (CT *)st->d_psi, *bufB = (CT *)st->d_work[0];
         // cnt steps from bufA; after an odd count psi is copied back to bufA
         auto record = [&](cudaStream_t cs, int64_t cnt) -> int {
@@ -1212,22 +1220,22 @@ extern "C" int gpe_state_create(gpe_grid *g, int dtype, gpe_state **out)
     st->grid = g;
     st->dtype = dtype;
     st->elem = dtype == GPE_C128 ? 16 : (dtype == GPE_R32 ? 4 : 8);
-    int rc = dev_alloc(&st->d_psi, g->n_packed * st->elem);
-    if (rc == GPE_OK) rc = dev_zero(st->d_psi, g->n_packed * st->elem);
     // E = exp(-V dt/2) in the state's real type (8 bytes for C128 and R64)
     const size_t real_bytes = (dtype == GPE_C128 || dtype == GPE_R64) ? 8 : 4;
-    if (rc == GPE_OK) rc = dev_alloc(&st->d_E, g->n_packed * real_bytes);
-    if (rc == GPE_OK) rc = dev_alloc_t(&st->d_clock, 1);
+    int rc = dev_alloc_parts(&st->block, {{&st->d_psi, g->n_packed * st->elem},
+                                          {&st->d_E, g->n_packed * real_bytes},
+                                          {&st->d_clock, 1},
+                                          red_partials(st->red, g->nsm),
+                                          red_counter(st->red),
+                                          red_scalars(st->red)});
+    if (rc == GPE_OK) rc = dev_zero(st->d_psi, g->n_packed * st->elem);
     if (rc == GPE_OK && !is_real_dtype(dtype)) rc = ensure_stab(st, STAB_STEPS);
-    if (rc == GPE_OK) rc = red_alloc(st->red, g->nsm * 32);
+    if (rc == GPE_OK) rc = red_zero(st->red);
     if (rc == GPE_OK && cudaMallocHost(&st->h_obs, sizeof(gpe_obs)) != cudaSuccess)
         rc = fail(GPE_ERR_CUDA, "cudaMallocHost failed");
     if (rc != GPE_OK) {
-        dev_free(st->d_psi);
-        dev_free(st->d_E);
-        dev_free(st->d_clock);
+        dev_free(st->block);
         dev_free(st->d_stab);
-        red_free(st->red);
         if (st->h_obs) cudaFreeHost(st->h_obs);
         delete st;
         return rc;
@@ -1241,10 +1249,8 @@ extern "C" int gpe_state_destroy(gpe_state *st)
 {
     if (!st) return GPE_OK;
     cudaDeviceSynchronize();
-    dev_free(st->d_psi);
-    for (int i = 0; i < 6; ++i) dev_free(st->d_work[i]);
-    dev_free(st->d_E);
-    dev_free(st->d_clock);
+    dev_free(st->block);
+    for (void *b : st->work_blocks) dev_free(b);
     dev_free(st->d_stab);
     dev_free(st->d_done);
     dev_free(st->d_ctr);
@@ -1252,7 +1258,6 @@ extern "C" int gpe_state_destroy(gpe_state *st)
     for (int i = 0; i < 2; ++i)
         if (st->gexec[i]) cudaGraphExecDestroy(st->gexec[i]);
     if (st->gcap) cudaStreamDestroy(st->gcap);
-    red_free(st->red);
     if (st->h_obs) cudaFreeHost(st->h_obs);
     st->grid->n_states--;
     delete st;

@@ -204,8 +204,6 @@ static int build(const TileSrc &S, TileTab &t, int *d_hmax, cudaStream_t st)
     // with the 7-point stencil); the rows kept are as long as the longest list
     int stride = NP == 19 ? 512 : 256, hmax = 0;
     uint32_t *rows = nullptr;
-    if (NP == 19) GPE_TRY(dev_alloc_t(&t.d_nbr19, 2 * (size_t)t.nseg));
-    else GPE_TRY(dev_alloc_t(&t.d_nbr, (size_t)t.nseg));
     int rc = GPE_OK;
     for (;;) {
         rc = dev_alloc_t(&rows, (size_t)t.ntiles * stride);
@@ -240,19 +238,16 @@ static int build(const TileSrc &S, TileTab &t, int *d_hmax, cudaStream_t st)
     return rc;
 }
 
-// the tiles of a grid whose records and brick volume are in place; the work is
-// on stream st when it returns
-int tiles_build(gpe_grid *g, cudaStream_t st)
+// the tiles of a grid whose records and brick volume are in place, and its
+// neighbour slots (nseg of them) allocated; d_hmax is a word of scratch.  The work is on stream st when it
+// returns.
+int tiles_build(gpe_grid *g, int *d_hmax, cudaStream_t st)
 {
     TileTab &t = g->tiles;
     t.nseg = (uint32_t)(g->n_packed / 4);
     t.ntiles = (int)((t.nseg + TILE - 1) / TILE);
     const TileSrc S{g->d_rec, g->d_org, g->d_bvol, g->nb, g->nbx, g->nby, g->nbz, g->by, g->bz, t.nseg};
-    int *d_hmax = nullptr;
-    GPE_TRY(dev_alloc_t(&d_hmax, 1));
-    const int rc = g->stencil == 19 ? build<19>(S, t, d_hmax, st) : build<7>(S, t, d_hmax, st);
-    dev_free(d_hmax);
-    return rc;
+    return g->stencil == 19 ? build<19>(S, t, d_hmax, st) : build<7>(S, t, d_hmax, st);
 }
 
 int tile_per_sm(const void *kernel, size_t smem)
