@@ -233,7 +233,6 @@ __device__ __forceinline__ void block_totals(Sum64<double> (&s)[NV], bool, doubl
     }
     __syncthreads();
 #pragma unroll
-    const R ax = euler_coef(a.ihx2, q4), ay = euler_coef(a.ihy2, q4), az = euler_coef(a.ihz2, q4);
     for (int k = 0; k < NV; ++k) out[k] = so[k];
     __syncthreads();
 }
@@ -255,7 +254,6 @@ __device__ __forceinline__ bool launch_totals(double (&v)[NV], double *partials,
     if (!is_last) return false;
     __threadfence();
     Sum64<double> s[NV];
-    const R ax = euler_coef(a.ihx2, q4), ay = euler_coef(a.ihy2, q4), az = euler_coef(a.ihz2, q4);
     for (int i = threadIdx.x; i < (int)gridDim.x; i += 4 * TILE) {
         double x[4][NV];  // four blocks' values in flight a thread
 #pragma unroll
@@ -276,6 +274,7 @@ __global__ void GPE_TILE_BOUNDS(R, NP) k_itp_a(const ItpArgs<R, CT> a, const Til
 {
     const TileList list = tile_begin(T);
     const R q4 = a.dt / (R)4;
+    const R ax = euler_coef(a.ihx2, q4), ay = euler_coef(a.ihy2, q4), az = euler_coef(a.ihz2, q4);
     const TileDiag<R, CT> diag{{(R)a.scalars[0], a.g * a.dt / (R)2, a.E}};
     tile_loop<NP, LapEuler>(T, list, (const CT *)a.psi, diag, ax, ay, az, EveryTile(),
                   [&](uint32_t idx, uint32_t n) { prefetch_l2(a.E + idx, n * (uint32_t)sizeof(R)); }, ELoad<R>{a.E},
@@ -297,6 +296,7 @@ __global__ void GPE_TILE_BOUNDS(R, NP) k_itp_b(const ItpArgs<R, CT> a, const Til
     const TileList list = tile_begin(T);
     const R hg = a.g * a.dt / (R)2;
     const R q4 = a.dt / (R)4;
+    const R ax = euler_coef(a.ihx2, q4), ay = euler_coef(a.ihy2, q4), az = euler_coef(a.ihz2, q4);
     Sum64<R> norm[1];
     int n = 0;
     tile_loop<NP, LapEuler>(T, list, (const CT *)a.tmp, Plain(), ax, ay, az, EveryTile(),
