@@ -1122,14 +1122,16 @@ namespace gpe {
 
 // A pass of the Thomas-Fermi solve reads the box once: over the cells with
 // V < mu, the sum of V (FP64) and their count, and over all cells below +inf
-// the largest |V| (its leading 32 bits, as an integer).  512^3 FP32: 0.20 ms,
-// 2.7 TB/s.  FP64 work is kept off that path (an FP64 instruction issues at 1/64 of the FP32 rate, predicated off or
-// not; the first form of the pass compared, added and counted every cell in
-// FP64 and took 1.55 ms): cells are compared as in Limit and counted in
-// integers, and a thread's vector goes into the FP64 sum behind a branch, in a
-// call, so that vectors without a selected cell skip it.
+// the largest |V| (its leading 32 bits, as an integer).  FP64 work is kept off
+// that path (an FP64 instruction issues at 1/64 of the FP32 rate, predicated
+// off or not): cells are compared as in Limit, counted in integers, and FP32
+// cells are added as pairs of floats (Sum64), behind a branch that vectors
+// without a selected cell skip.  512^3 FP32: 1.55 ms compared, added and counted in
+// FP64, 0.19 ms with the selected cells added in FP64 (eight instructions a vector, which
+// filled the FP64 pipe), 0.11 ms so (4.8 TB/s).
+template <typename T>
 struct TfSum {
-    double sum = 0.0;
+    Sum64<T> sum;
     unsigned long long cnt = 0;
     uint32_t top = 0;
 };
@@ -1142,38 +1144,36 @@ __device__ __forceinline__ uint32_t tf_top(double v)
     return a < 0x7ff00000u || (hi == 0xfff00000u && __double2loint(v) == 0) ? a : 0u;
 }
 
-__device__ __noinline__ double tf_add(double sum, float a, float b, float c, float d, unsigned sel)
-{
-    if (sel & 1u) sum += (double)a;
-    if (sel & 2u) sum += (double)b;
-    if (sel & 4u) sum += (double)c;
-    if (sel & 8u) sum += (double)d;
-    return sum;
-}
+// float pairs reach to 3e38, a thread's sum of SUM_FLUSH terms stays below it if
+// the terms do not exceed this; larger ones are added in FP64
+constexpr float TF_PAIR_MAX = 1e30f;
+__device__ __noinline__ double tf_add(double sum, float v) { return sum + (double)v; }
 __device__ __noinline__ double tf_add(double sum, double a, double b, unsigned sel)
 {
     if (sel & 1u) sum += a;
     if (sel & 2u) sum += b;
     return sum;
 }
-__device__ __forceinline__ double tf_add(double sum, const float (&v)[4], unsigned sel)
+template <int W>
+__device__ __forceinline__ void tf_add(Sum64<float> &s, const float (&v)[W], unsigned sel)
 {
-    return tf_add(sum, v[0], v[1], v[2], v[3], sel);
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        const float x = (sel >> w) & 1u ? v[w] : 0.0f;
+        if (fabsf(x) <= TF_PAIR_MAX) s.add(x);
+        else s.tot = tf_add(s.tot, x);
+    }
 }
-__device__ __forceinline__ double tf_add(double sum, const float (&v)[1], unsigned sel)
+__device__ __forceinline__ void tf_add(Sum64<double> &s, const double (&v)[2], unsigned sel)
 {
-    return tf_add(sum, v[0], 0.0f, 0.0f, 0.0f, sel);
+    s.tot = tf_add(s.tot, v[0], v[1], sel);
 }
-__device__ __forceinline__ double tf_add(double sum, const double (&v)[2], unsigned sel)
+__device__ __forceinline__ void tf_add(Sum64<double> &s, const double (&v)[1], unsigned sel)
 {
-    return tf_add(sum, v[0], v[1], sel);
-}
-__device__ __forceinline__ double tf_add(double sum, const double (&v)[1], unsigned sel)
-{
-    return tf_add(sum, v[0], 0.0, sel);
+    s.tot = tf_add(s.tot, v[0], 0.0, sel);
 }
 template <typename T, int W>
-__device__ __forceinline__ void tf_cells(const T (&v)[W], const Limit &m, TfSum &a)
+__device__ __forceinline__ void tf_cells(const T (&v)[W], const Limit &m, TfSum<T> &a)
 {
     unsigned sel = 0;
 #pragma unroll
@@ -1183,16 +1183,18 @@ __device__ __forceinline__ void tf_cells(const T (&v)[W], const Limit &m, TfSum 
     }
     if (sel) {
         a.cnt += __popc(sel);
-        a.sum = tf_add(a.sum, v, sel);
+        tf_add(a.sum, v, sel);
     }
 }
 
-__device__ __forceinline__ void tf_finish(const TfSum &a, double *partials, unsigned int *counter, double *result,
+template <typename T>
+__device__ __forceinline__ void tf_finish(TfSum<T> &a, double *partials, unsigned int *counter, double *result,
                                           uint32_t *top)
 {
     const uint32_t t = __reduce_max_sync(0xffffffffu, a.top);
     if ((threadIdx.x & 31) == 0 && t > __ldcg(top)) atomicMax(top, t);
-    double acc[2] = {a.sum, (double)a.cnt}, tot[2];
+    a.sum.flush();
+    double acc[2] = {a.sum.tot, (double)a.cnt}, tot[2];
     if (reduce_finish<2>(acc, partials, counter, tot) && threadIdx.x == 0) {
         result[0] = tot[0];
         result[1] = tot[1];
@@ -1208,19 +1210,22 @@ __global__ void k_tf_dense(const T *V, int64_t n, int64_t n_vec, Limit m, double
     struct alignas(16) Vec {
         T v[W];
     };
-    TfSum a;
+    TfSum<T> a;
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
     const Vec *src = reinterpret_cast<const Vec *>(V);
     const int64_t nv = n_vec / W;
     // four loads in flight a thread
     int64_t i = t;
+    int n4 = 0;
     for (; i + 3 * step < nv; i += 4 * step) {
+        if (++n4 % (SUM_FLUSH / (4 * W)) == 0) a.sum.flush();
         Vec x[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) x[k] = src[i + k * step];
 #pragma unroll
         for (int k = 0; k < 4; ++k) tf_cells<T, W>(x[k].v, m, a);
     }
+    a.sum.flush();  // at most three vectors are left
     for (; i < nv; i += step) {
         const Vec x = src[i];
         tf_cells<T, W>(x.v, m, a);
@@ -1228,6 +1233,7 @@ __global__ void k_tf_dense(const T *V, int64_t n, int64_t n_vec, Limit m, double
     for (int64_t j = n_vec + t; j < n; j += step) {
         const T x[1] = {V[j]};
         tf_cells<T, 1>(x, m, a);
+        if (++n4 % SUM_FLUSH == 0) a.sum.flush();
     }
     tf_finish(a, partials, counter, result, top);
 }
@@ -1237,7 +1243,7 @@ __global__ void k_tf_dense(const T *V, int64_t n, int64_t n_vec, Limit m, double
 __global__ void k_tf_analytic(PotDesc P, BoxD box, Limit m, double *partials, unsigned int *counter, double *result,
                               uint32_t *top)
 {
-    TfSum a;
+    TfSum<double> a;
     const int lane = threadIdx.x & 31;
     const int64_t nc = (box.nx + 31) / 32, n = nc * box.ny * box.nz;
     const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -1321,7 +1327,7 @@ __global__ void __launch_bounds__(1024) k_tf_estimate(const float *v, int n, dou
 // down to it, and ends exactly once the set {V < mu} stops changing.  It
 // starts from the solution on a sample of the cells, a per cent or so off:
 // three to five passes over the box, where a start at mu = +inf took about
-// eighteen (512^3 shell, FP32: 28 ms a solve of 1.55 ms passes, now 0.97 ms).
+// eighteen (512^3 shell, FP32: 28 ms a solve of 1.55 ms passes, now 0.78 ms).
 static int tf_mu_impl(const gpe_box *box, const VSource &src, double g, double N, double *mu, cudaStream_t st)
 {
     if (!(g > 0)) return fail(GPE_ERR_ARG, "g must be > 0 for the Thomas-Fermi estimate");

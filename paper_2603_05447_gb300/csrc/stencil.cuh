@@ -879,6 +879,48 @@ struct DiagLoad {
     }
 };
 
+// An FP64 sum of many single-precision terms off the FP64 pipe, where every
+// add and conversion issues at 1/64 of the FP32 rate: the terms are added as an
+// unevaluated pair of floats (hi + lo, each addition's rounding error found
+// exactly by Knuth's two-sum and kept in lo), and the pair goes into an FP64
+// total every SUM_FLUSH terms.  After n additions the pair is good to about n
+// 2^-48 of the sum, against the 2^-25 of every term.  Double-precision terms
+// are added as they are.
+template <typename R>
+struct Sum64 {
+    double tot = 0.0;
+    __device__ __forceinline__ void add(double x) { tot += x; }
+    __device__ __forceinline__ void flush() {}
+};
+// a call, so that the compiler branches around it: FP64 instructions that are
+// predicated off still take their turn in the pipe
+static __device__ __noinline__ double add_pair(double tot, float hi, float lo)
+{
+    tot += (double)hi;
+    if (isfinite(lo)) tot += (double)lo;  // an infinite or NaN term shows in hi
+    return tot;
+}
+template <>
+struct Sum64<float> {
+    double tot = 0.0;
+    float hi = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ void add(float x) { add(x, 0.0f); }
+    __device__ __forceinline__ void add(float x, float xl)
+    {
+        const float s = __fadd_rn(hi, x), b = __fadd_rn(s, -hi);
+        const float e = __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -b)), __fadd_rn(x, -b));
+        lo = __fadd_rn(lo, __fadd_rn(e, xl));
+        hi = s;
+    }
+    __device__ __forceinline__ void flush()
+    {
+        tot = add_pair(tot, hi, lo);
+        hi = 0.0f;
+        lo = 0.0f;
+    }
+};
+constexpr int SUM_FLUSH = 64;
+
 // deterministic block sum (result valid in thread 0)
 __device__ __forceinline__ double block_sum(double x)
 {
