@@ -216,6 +216,7 @@ struct gpe_tape {
     int64_t nsteps = 0, nck = 0;
     double t0 = 0.0;
     int K = 0;
+    bool last_kept = false;  // the last segment's states are those that the forward pass left
     void *d_ckpt = nullptr;  // [nck * n_packed]
     void *d_seg = nullptr;   // [K * n_packed] step-start states of a segment after the first
     void *d_stages = nullptr;  // [3 * K * n_packed] the stage states of a segment's steps, where memory allows
@@ -243,6 +244,102 @@ extern "C" int gpe_tape_destroy(gpe_tape *t)
     tape_free(t);
     return GPE_OK;
 }
+
+namespace gpe {
+
+// The RK4 stages of a segment's steps on the tape's buffers.  The step-start
+// states are the segment's checkpoint, then seg[0], seg[1] ... (stage 3 reads
+// no y0, so it writes the next one where it stays); the stage states go to
+// their store where there is one.
+template <typename R>
+struct SegmentSteps {
+    using CT = typename Cx<R>::T;
+    gpe_tape *t;
+    RkArgs<R> f{};
+    TileLaunch L;
+    cudaStream_t s;
+    int init(gpe_tape *t_, cudaStream_t s_)
+    {
+        t = t_;
+        s = s_;
+        gpe_state *st = t->st;
+        const gpe_grid *g = st->grid;
+        const gpe_real_params &p = t->p;
+        f.V0 = (const R *)potential_ptr(st, 0);
+        f.V1 = (const R *)potential_ptr(st, 1);
+        if (!f.V0 || !f.V1) return fail(GPE_ERR_STATE, "ramp needs potential slots 0 and 1");
+        f.y2 = (CT *)t->d_w[0];
+        f.y3 = (CT *)t->d_w[1];
+        f.y4 = (CT *)t->d_w[2];  // kept apart from Y2: the reverse sweep reads all three
+        f.w = (CT *)t->d_w[3];
+        f.ihx2 = (R)(1.0 / (g->box.hx * g->box.hx));
+        f.ihy2 = (R)(1.0 / (g->box.hy * g->box.hy));
+        f.ihz2 = (R)(1.0 / (g->box.hz * g->box.hz));
+        f.g = (R)p.g;
+        f.dt = (R)p.dt;
+        f.dtd = p.dt;
+        f.ramp.clock = t->d_clock;
+        f.ramp.T = p.T_ramp;
+        f.ramp.n_knots = p.n_knots;
+        for (int k = 0; k < GPE_MAX_KNOTS; ++k) f.ramp.knots[k] = p.knots[k];
+        L = tile_launch<CT, 7>(g->tiles);
+        return GPE_OK;
+    }
+    // the schedule's values for len steps from n0 steps after the clock
+    int table(int64_t n0, int64_t len) const
+    {
+        k_ramp_table<<<1, 256, 0, s>>>(f.ramp, t->d_clock, 0.0, n0, (int)len, 3, RK4_TIMES, t->p.dt, t->d_stab);
+        GPE_LAUNCH_CHECK();
+        return GPE_OK;
+    }
+    CT *start(int64_t j, int64_t m) const
+    {
+        const size_t np = (size_t)t->st->grid->n_packed;
+        return m == 0 ? (CT *)t->d_ckpt + j * np : (CT *)t->d_seg + (m - 1) * np;
+    }
+    // stage stg of step m of the segment, from f.y0
+    int stage(int64_t m, int stg)
+    {
+        const auto k = Rk4Tiles<R, 7>::get(true, stg);
+        f.stab = t->d_stab + 3 * m + (stg + 1) / 2;
+        if (t->d_stages) {
+            const size_t np = (size_t)t->st->grid->n_packed;
+            CT *y = (CT *)t->d_stages + 3 * m * np;
+            f.y2 = y;
+            f.y3 = y + np;
+            f.y4 = y + 2 * np;
+        }
+        return tile_run(k, tile_blocks(k, t->st->grid->nsm, L.T.ntiles, L.smem), L, s, f, L.T);
+    }
+    // step m of segment j; its result goes to `end`
+    int step(int64_t j, int64_t m, CT *end)
+    {
+        f.y0 = start(j, m);
+        for (int stg = 0; stg < 3; ++stg) GPE_TRY(stage(m, stg));
+        f.y0 = end;
+        return stage(m, 3);
+    }
+};
+
+// The last segment's steps with every state kept for the reverse sweep, which
+// then does not compute that segment again: 512^3 ramp gradient over 48 steps,
+// K = 16: 25.6 -> 23.5 ms.
+template <typename R>
+static int forward_kept(gpe_tape *t, int64_t n, cudaStream_t s)
+{
+    using CT = typename Cx<R>::T;
+    const int64_t j = t->nck - 1;
+    SegmentSteps<R> run;
+    GPE_TRY(run.init(t, s));
+    k_set_clock<<<1, 1, 0, s>>>(t->d_clock, t->t0 + (double)(j * t->K) * t->p.dt);
+    GPE_LAUNCH_CHECK();
+    GPE_TRY(run.table(0, n));
+    for (int64_t m = 0; m < n; ++m) GPE_TRY(run.step(j, m, m + 1 < n ? run.start(j, m + 1) : (CT *)t->st->d_psi));
+    t->last_kept = true;
+    return GPE_OK;
+}
+
+}  // namespace gpe
 
 extern "C" int gpe_ramp_forward(gpe_state *st, const gpe_real_params *p, int64_t nsteps, double t0, int K,
                                 gpe_tape **out, gpe_stream stream)
@@ -305,7 +402,9 @@ extern "C" int gpe_ramp_forward(gpe_state *st, const gpe_real_params *p, int64_t
             tape_free(t);
             return cuda_fail(e, "checkpoint copy", __FILE__, __LINE__);
         }
-        rc = gpe_step_real(st, p, n, t0 + (double)(j * t->K) * p->dt, stream);
+        const bool keep = j == t->nck - 1 && t->d_stages && g->sched == GPE_SCHED_STAGED;
+        rc = gpe_step_real(st, p, keep ? 0 : n, t0 + (double)(j * t->K) * p->dt, stream);  // no steps: the checks
+        if (rc == GPE_OK && keep) rc = st->dtype == GPE_C128 ? forward_kept<double>(t, n, s) : forward_kept<float>(t, n, s);
         if (rc != GPE_OK) {
             tape_free(t);
             return rc;
@@ -337,39 +436,11 @@ static int backward_impl(gpe_tape *t, const gpe_state *target, double *grad, dou
     // forward stage kernels on tape buffers; times from the tape's start
     k_set_clock<<<1, 1, 0, s>>>(t->d_clock, t->t0);
     GPE_LAUNCH_CHECK();
-    RkArgs<R> f{};
-    f.V0 = (const R *)potential_ptr(st, 0);
-    f.V1 = (const R *)potential_ptr(st, 1);
-    if (!f.V0 || !f.V1) return fail(GPE_ERR_STATE, "ramp needs potential slots 0 and 1");
-    f.y2 = (CT *)t->d_w[0];
-    f.y3 = (CT *)t->d_w[1];
-    f.y4 = (CT *)t->d_w[2];  // kept apart from Y2: the reverse sweep reads all three
-    f.w = (CT *)t->d_w[3];
-    f.ihx2 = (R)(1.0 / (g->box.hx * g->box.hx));
-    f.ihy2 = (R)(1.0 / (g->box.hy * g->box.hy));
-    f.ihz2 = (R)(1.0 / (g->box.hz * g->box.hz));
-    f.g = (R)p.g;
-    f.dt = (R)p.dt;
-    f.dtd = p.dt;
-    f.ramp.clock = t->d_clock;
-    f.ramp.T = p.T_ramp;
-    f.ramp.n_knots = p.n_knots;
-    for (int k = 0; k < GPE_MAX_KNOTS; ++k) f.ramp.knots[k] = p.knots[k];
-    using RT = Rk4Tiles<R, 7>;
-    const TileLaunch tl = tile_launch<CT, 7>(g->tiles);
+    SegmentSteps<R> run;
+    GPE_TRY(run.init(t, s));
+    const RkArgs<R> &f = run.f;
+    const TileLaunch &tl = run.L;
     auto blocks = [&](auto k) { return tile_blocks(k, g->nsm, tl.T.ntiles, tl.smem); };
-    // stage stg of step m of the segment, from f.y0
-    auto stage = [&](int64_t m, int stg) -> int {
-        const auto k = RT::get(true, stg);
-        f.stab = t->d_stab + 3 * m + (stg + 1) / 2;
-        if (t->d_stages) {
-            CT *y = (CT *)t->d_stages + 3 * m * np;
-            f.y2 = y;
-            f.y3 = y + np;
-            f.y4 = y + 2 * np;
-        }
-        return tile_run(k, blocks(k), tl, s, f, tl.T);
-    };
     using KA = void (*)(AdjArgs<R>, TileView);
     const KA ka[4] = {k_adj_stage<R, 0>, k_adj_stage<R, 1>, k_adj_stage<R, 1>, k_adj_stage<R, 2>};
     AdjArgs<R> a{};
@@ -386,25 +457,19 @@ static int backward_impl(gpe_tape *t, const gpe_state *target, double *grad, dou
     a.counter = t->red.counter;
     a.grad = t->d_grad;
     const R dt = (R)p.dt;
-    CT *seg = (CT *)t->d_seg, *ck = (CT *)t->d_ckpt;
     for (int64_t j = t->nck - 1; j >= 0; --j) {
         const int64_t len = std::min<int64_t>(t->K, t->nsteps - j * t->K);
-        // step-start states of the segment: the checkpoint, then seg[0], seg[1]
-        // ... (stage 3 reads no y0, so it writes the next one where it stays)
-        auto start = [&](int64_t m) { return m == 0 ? ck + j * np : seg + (m - 1) * np; };
-        k_ramp_table<<<1, 256, 0, s>>>(f.ramp, t->d_clock, 0.0, j * t->K, (int)len, 3, RK4_TIMES, p.dt, t->d_stab);
-        GPE_LAUNCH_CHECK();
-        for (int64_t m = 0; m + 1 < len; ++m) {
-            f.y0 = start(m);
-            for (int stg = 0; stg < 3; ++stg) GPE_TRY(stage(m, stg));
-            f.y0 = start(m + 1);
-            GPE_TRY(stage(m, 3));
+        const bool kept = t->last_kept && j == t->nck - 1;
+        if (!kept) {
+            GPE_TRY(run.table(j * t->K, len));
+            for (int64_t m = 0; m + 1 < len; ++m) GPE_TRY(run.step(j, m, run.start(j, m + 1)));
         }
+        if (t->nck > 1) t->last_kept = false;  // the other segments take its place
         for (int64_t m = len - 1; m >= 0; --m) {
             const double tm = t->t0 + (double)(j * t->K + m) * p.dt;
-            f.y0 = start(m);
-            if (!t->d_stages || m == len - 1)
-                for (int stg = 0; stg < 3; ++stg) GPE_TRY(stage(m, stg));  // Y2, Y3, Y4
+            run.f.y0 = run.start(j, m);
+            if (!t->d_stages || (m == len - 1 && !kept))
+                for (int stg = 0; stg < 3; ++stg) GPE_TRY(run.stage(m, stg));  // Y2, Y3, Y4
             // stages 4, 3, 2, 1 of the reverse sweep
             const double ts[4] = {tm + p.dt, tm + 0.5 * p.dt, tm + 0.5 * p.dt, tm};
             const CT *Ys[4] = {f.y4, f.y3, f.y2, f.y0};

@@ -188,3 +188,29 @@ def test_autograd_function_gives_the_adjoint_gradient(problem):
     finally:
         prob.close()
         gpe.gpe_grid_destroy(grid)
+
+
+@pytest.mark.parametrize("every", [1, 7, 29, 30, 64])
+def test_gradient_for_any_last_segment_and_asked_for_twice(problem, every):
+    """One step, a remainder, and the whole run in the last segment, whose
+    states the forward pass leaves; the second call finds other segments' in
+    their place.  Tolerances as for one checkpoint interval above."""
+    case, og, loss, grad = problem
+    grid = blend_grid(case)
+    st, tg = (gpe.gpe_state_create(grid, gpe.GPE_C128) for _ in range(2))
+    tape = None
+    try:
+        gpe.gpe_state_load(st, np.ascontiguousarray(case.psi.astype(np.complex128)), gpe.GPE_LAYOUT_DENSE)
+        gpe.gpe_state_load(tg, np.ascontiguousarray(case.target.astype(np.complex128)), gpe.GPE_LAYOUT_DENSE)
+        tape = gpe.gpe_ramp_forward(st, gpe.real_params(case.g, case.dt, gpe.GPE_V_BLEND, case.knots, case.T),
+                                    NSTEPS, 0.0, every)
+        for _ in range(2):
+            l, g = gpe.gpe_ramp_backward(tape, tg, len(case.knots))
+            assert abs(l - loss) <= 1e-12 * abs(loss)
+            assert np.max(np.abs(np.array(g) - grad)) <= 1e-10 * np.max(np.abs(grad))
+    finally:
+        if tape is not None:
+            gpe.gpe_tape_destroy(tape)
+        gpe.gpe_state_destroy(st)
+        gpe.gpe_state_destroy(tg)
+        gpe.gpe_grid_destroy(grid)
