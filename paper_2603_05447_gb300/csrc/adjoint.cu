@@ -88,12 +88,13 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? 5 : 2) k_adj_stage(cons
         R V0[4], V1[4];
         CT Y[4], lam[4], acc[4];
     };
+    const auto co = tile_co<7, LapFull>(a.ihx2, a.ihy2, a.ihz2);  // before the wait
     const TileList list = tile_begin(T);
     XF xf{};
     if constexpr (POS == 0) xf.s = a.m_scale;
     Sum64<R> dot[1];
     int n = 0;
-    tile_loop<7>(T, list, a.mu_in, xf, a.ihx2, a.ihy2, a.ihz2, EveryTile(),
+    tile_loop<7>(T, list, a.mu_in, xf, co, EveryTile(),
                  [&](uint32_t idx, uint32_t m) {
                      prefetch_l2(a.V0 + idx, m * (uint32_t)sizeof(R));
                      prefetch_l2(a.V1 + idx, m * (uint32_t)sizeof(R));

@@ -69,7 +69,8 @@ struct ShellWalk {
     uint32_t nt;
     uint32_t cur = 0xffffffffu, next = 0;
     bool live = false;
-    R g = 0, dt = 0, ihx2 = 0, ihy2 = 0, ihz2 = 0, scale = 0;  // spacings: euler_coef of them, but for the observables
+    R g = 0, dt = 0, scale = 0;
+    TileCo<R> co{};  // of euler_coef of the spacings, but for the observables
     Sum64<R> sum[NS > 0 ? NS : 1];  // NS 5: the fifth counts non-finite cells
     int nf = 0, n = 0;
     __device__ __forceinline__ ShellWalk(const BatchArgs<R, CT> &a_, uint32_t nt_) : a(a_), nt(nt_)
@@ -106,9 +107,7 @@ struct ShellWalk {
             g = (R)P.g;
             dt = (R)P.dt;
             const R q = NS == 5 ? (R)1 : dt / (R)4;
-            ihx2 = euler_coef((R)P.ihx2, q);
-            ihy2 = euler_coef((R)P.ihy2, q);
-            ihz2 = euler_coef((R)P.ihz2, q);
+            co = tile_co<7, LapFull>(euler_coef((R)P.ihx2, q), euler_coef((R)P.ihy2, q), euler_coef((R)P.ihz2, q));
             scale = (R)P.scale;
         }
         return live;
@@ -176,10 +175,10 @@ __global__ void GPE_TILE_BOUNDS(R, 7) k_batch_itp(const BatchArgs<R, CT> a, cons
         }
     };
     if constexpr (STAGE == 0)
-        tile_loop<7, LapEuler>(T, list, (const CT *)a.psi, WalkDiag<R, CT, W>{w, a.E}, w.ihx2, w.ihy2, w.ihz2, enter, pref,
+        tile_loop<7, LapEuler>(T, list, (const CT *)a.psi, WalkDiag<R, CT, W>{w, a.E}, w.co, enter, pref,
                      ELoad<R>{a.E}, body);
     else
-        tile_loop<7, LapEuler>(T, list, (const CT *)a.tmp, Plain(), w.ihx2, w.ihy2, w.ihz2, enter, pref, ELoad<R>{a.E}, body);
+        tile_loop<7, LapEuler>(T, list, (const CT *)a.tmp, Plain(), w.co, enter, pref, ELoad<R>{a.E}, body);
     w.leave();
 }
 
@@ -224,7 +223,7 @@ __global__ void GPE_TILE_BOUNDS(R, 7) k_batch_obs(const BatchArgs<R, CT> a, cons
 {
     const TileList list = tile_begin(T);
     ShellWalk<R, CT, 5> w(a, (uint32_t)T.ntiles);
-    tile_loop<7>(T, list, (const CT *)a.psi, Plain(), w.ihx2, w.ihy2, w.ihz2, [&](uint32_t tile) { return w.enter(tile); },
+    tile_loop<7>(T, list, (const CT *)a.psi, Plain(), w.co, [&](uint32_t tile) { return w.enter(tile); },
                  [&](uint32_t idx, uint32_t n) { prefetch_l2(a.V + idx, n * (uint32_t)sizeof(R)); },
                  VLoad<R, false>{a.V, nullptr},
                  [&](uint32_t, const typename VLoad<R, false>::P &p, const CT(&c)[4], const CT(&L)[4]) {

@@ -109,7 +109,7 @@ __device__ __forceinline__ void itp_pair_brick(ItpPairSpace<typename Cx<R>::T, B
     const int t = threadIdx.x;
     const R q4 = a.dt / (R)4, hg = a.g * a.dt / (R)2;
     const R ax = euler_coef(a.ihx2, q4), ay = euler_coef(a.ihy2, q4), az = euler_coef(a.ihz2, q4);
-    const R c6 = (R)2 * (ax + ay + az);
+    const LapCo<R> co = lap_co<LapEuler>(ax, ay, az);
     pair_fill(ps, P, b, a.psi, EFill<CT, BX, BY, BZ>{&sp, a.E});
     for (int i = t; i < PS::UPS * PS::VPSTR; i += PAIR_THREADS) (&ps.v[0][0])[i] = make_uint4(0, 0, 0, 0);
     for (int i = t; i < BY * BZ; i += PAIR_THREADS) {
@@ -173,7 +173,7 @@ __device__ __forceinline__ void itp_pair_brick(ItpPairSpace<typename Cx<R>::T, B
         if (!ok) continue;
         CT c[4], L[4], o[4];
         R e4[4];
-        pair_lap_u<LapEuler>(ps, hx, y, z, c, L, ax, ay, az, c6);
+        pair_lap_u<LapEuler>(ps, hx, y, z, c, L, co);
         sp.eget(PS::slot(hx, y, z), e4);
 #pragma unroll
         for (int k = 0; k < 4; ++k) o[k] = e4[k] >= (R)0 ? euler(c[k], q4, L[k]) : czero<CT>();
@@ -207,7 +207,7 @@ __device__ __forceinline__ void itp_pair_brick(ItpPairSpace<typename Cx<R>::T, B
             zm = ps.uxr[PS::row(y, z - 1)][0];
             zp = ps.uxr[PS::row(y, z + 1)][0];
         }
-        const CT L = LapEuler::of(xp, xm, yp, ym, zp, zm, c0, ax, ay, az, c6);
+        const CT L = lap_of<LapEuler>(xp, xm, yp, ym, zp, zm, c0, co);
         (side == 0 ? ps.vxl : ps.vxr)[PS::vrow(y, z)] = e >= (R)0 ? euler(c0, q4, L) : czero<CT>();
     }
     __syncthreads();
@@ -218,7 +218,7 @@ __device__ __forceinline__ void itp_pair_brick(ItpPairSpace<typename Cx<R>::T, B
         CT c[4], L[4], o[4];
         R e4[4];
         R n4 = (R)0;  // the segment's |psi|^2, added to the FP64 sum once
-        pair_lap_v<LapEuler>(ps, hx, y, z, c, L, ax, ay, az, c6);
+        pair_lap_v<LapEuler>(ps, hx, y, z, c, L, co);
         sp.eget(PS::slot(hx, y, z), e4);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {

@@ -231,11 +231,11 @@ __device__ __forceinline__ bool launch_totals(double (&v)[NV], double *partials,
 template <typename R, typename CT, int NP>
 __global__ void GPE_TILE_BOUNDS(R, NP) k_itp_a(const ItpArgs<R, CT> a, const TileView T)
 {
-    const TileList list = tile_begin(T);
     const R q4 = a.dt / (R)4;
-    const R ax = euler_coef(a.ihx2, q4), ay = euler_coef(a.ihy2, q4), az = euler_coef(a.ihz2, q4);
+    const auto co = tile_co<NP, LapEuler>(euler_coef(a.ihx2, q4), euler_coef(a.ihy2, q4), euler_coef(a.ihz2, q4));  // before the wait
+    const TileList list = tile_begin(T);
     const TileDiag<R, CT> diag{{(R)a.scalars[0], a.g * a.dt / (R)2, a.E}};
-    tile_loop<NP, LapEuler>(T, list, (const CT *)a.psi, diag, ax, ay, az, EveryTile(),
+    tile_loop<NP, LapEuler>(T, list, (const CT *)a.psi, diag, co, EveryTile(),
                   [&](uint32_t idx, uint32_t n) { prefetch_l2(a.E + idx, n * (uint32_t)sizeof(R)); }, ELoad<R>{a.E},
                   [&](uint32_t idx, const typename ELoad<R>::P &p, const CT(&c)[4], const CT(&L)[4]) {
                       CT o[4];
@@ -252,13 +252,13 @@ template <typename R, typename CT, int NP>
 __global__ void GPE_TILE_BOUNDS(R, NP) k_itp_b(const ItpArgs<R, CT> a, const TileView T, double *partials,
                                            unsigned int *counter)
 {
+    const R q4 = a.dt / (R)4;
+    const auto co = tile_co<NP, LapEuler>(euler_coef(a.ihx2, q4), euler_coef(a.ihy2, q4), euler_coef(a.ihz2, q4));  // before the wait
     const TileList list = tile_begin(T);
     const R hg = a.g * a.dt / (R)2;
-    const R q4 = a.dt / (R)4;
-    const R ax = euler_coef(a.ihx2, q4), ay = euler_coef(a.ihy2, q4), az = euler_coef(a.ihz2, q4);
     Sum64<R> norm[1];
     int n = 0;
-    tile_loop<NP, LapEuler>(T, list, (const CT *)a.tmp, Plain(), ax, ay, az, EveryTile(),
+    tile_loop<NP, LapEuler>(T, list, (const CT *)a.tmp, Plain(), co, EveryTile(),
                   [&](uint32_t idx, uint32_t n) { prefetch_l2(a.E + idx, n * (uint32_t)sizeof(R)); }, ELoad<R>{a.E},
                   [&](uint32_t idx, const typename ELoad<R>::P &p, const CT(&c)[4], const CT(&L)[4]) {
                       CT o[4];
@@ -370,10 +370,11 @@ __device__ __forceinline__ void obs_terms(const typename VLoad<R, BLEND>::P &p, 
 template <typename R, typename CT, int NP, bool BLEND>
 __global__ void GPE_TILE_BOUNDS(R, NP) k_obs(const ObsArgs<R, CT> a, const TileView T)
 {
+    const auto co = tile_co<NP, LapFull>(a.ihx2, a.ihy2, a.ihz2);  // before the wait
     const TileList list = tile_begin(T);
     Sum64<R> sum[5];  // norm, ekin, epot, eint, nonfinite
     int n = 0, nf = 0;
-    tile_loop<NP>(T, list, a.psi, Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
+    tile_loop<NP>(T, list, a.psi, Plain(), co, EveryTile(),
                   [&](uint32_t idx, uint32_t n) {
                       prefetch_l2(a.V0 + idx, n * (uint32_t)sizeof(R));
                       if constexpr (BLEND) prefetch_l2(a.V1 + idx, n * (uint32_t)sizeof(R));

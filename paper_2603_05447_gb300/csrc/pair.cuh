@@ -249,7 +249,7 @@ __device__ __forceinline__ void pair_fill(PairSpace<CT, BX, BY, BZ> &ps, const P
 // x neighbours at the row ends come from the row's x halo cells
 template <typename LAP = LapFull, typename CT, int BX, int BY, int BZ, typename R>
 __device__ __forceinline__ void pair_lap_u(const PairSpace<CT, BX, BY, BZ> &ps, int hx, int y, int z, CT (&c)[4],
-                                           CT (&L)[4], R ihx2, R ihy2, R ihz2, R c6)
+                                           CT (&L)[4], const LapCo<R> &co)
 {
     using PS = PairSpace<CT, BX, BY, BZ>;
     const int s = PS::slot(hx, y, z);
@@ -266,14 +266,14 @@ __device__ __forceinline__ void pair_lap_u(const PairSpace<CT, BX, BY, BZ> &ps, 
     for (int i = 0; i < 4; ++i) {
         const CT l = i == 0 ? xm : c[i - 1];
         const CT rr = i == 3 ? xp : c[i + 1];
-        L[i] = LAP::of(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], LAP::coef(ihx2), LAP::coef(ihy2), LAP::coef(ihz2), c6);
+        L[i] = lap_of<LAP>(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], co);
     }
 }
 
 // The same on the v tile (the brick's own slots only)
 template <typename LAP = LapFull, typename CT, int BX, int BY, int BZ, typename R>
 __device__ __forceinline__ void pair_lap_v(const PairSpace<CT, BX, BY, BZ> &ps, int hx, int y, int z, CT (&c)[4],
-                                           CT (&L)[4], R ihx2, R ihy2, R ihz2, R c6)
+                                           CT (&L)[4], const LapCo<R> &co)
 {
     using PS = PairSpace<CT, BX, BY, BZ>;
     const int s = PS::vslot(hx, y, z);
@@ -290,7 +290,7 @@ __device__ __forceinline__ void pair_lap_v(const PairSpace<CT, BX, BY, BZ> &ps, 
     for (int i = 0; i < 4; ++i) {
         const CT l = i == 0 ? xm : c[i - 1];
         const CT rr = i == 3 ? xp : c[i + 1];
-        L[i] = LAP::of(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], LAP::coef(ihx2), LAP::coef(ihy2), LAP::coef(ihz2), c6);
+        L[i] = lap_of<LAP>(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], co);
     }
 }
 
@@ -309,7 +309,7 @@ __device__ __forceinline__ void pair_brick(PairSpace<typename Cx<R>::T, BX, BY, 
     constexpr int SX = PS::SX, PL = PS::PLANE_B;
     const int t = threadIdx.x;
     const CT *usrc = PASS == 0 ? a.y0 : a.y3;
-    const R c6 = (R)2 * (a.ihx2 + a.ihy2 + a.ihz2);
+    const LapCo<R> co = lap_co<LapRhs>(a.ihx2, a.ihy2, a.ihz2);
     pair_fill(ps, P, b, usrc);
     // v: zero (slots no task writes stay zero: cells outside the region)
     for (int i = t; i < PS::UPS * PS::VPSTR; i += PAIR_THREADS)
@@ -353,7 +353,7 @@ __device__ __forceinline__ void pair_brick(PairSpace<typename Cx<R>::T, BX, BY, 
         if (!ok) continue;
         const typename BA::P pa = bodyA.load(j);
         CT c[4], L[4], o[4], wv[4];
-        pair_lap_u<LapRhs>(ps, hx, y, z, c, L, a.ihx2, a.ihy2, a.ihz2, c6);
+        pair_lap_u<LapRhs>(ps, hx, y, z, c, L, co);
         bodyA.compute(pa, c, L, o, wv);
         ps.vput(PS::vslot(hx, y, z), o);
     }
@@ -392,7 +392,7 @@ __device__ __forceinline__ void pair_brick(PairSpace<typename Cx<R>::T, BX, BY, 
         if constexpr (BLEND) pa.V1[0] = a.V1[j];
         if constexpr (STA == 2) pa.y[0] = a.y0[j];
         CT c[4] = {c0, czero<CT>(), czero<CT>(), czero<CT>()}, L[4], o[4], wv[4];
-        L[0] = LapRhs::of(xp, xm, yp, ym, zp, zm, c0, LapRhs::coef(a.ihx2), LapRhs::coef(a.ihy2), LapRhs::coef(a.ihz2), c6);
+        L[0] = lap_of<LapRhs>(xp, xm, yp, ym, zp, zm, c0, co);
         L[1] = L[2] = L[3] = czero<CT>();
         bodyA.compute(pa, c, L, o, wv);
         (side == 0 ? ps.vxl : ps.vxr)[PS::vrow(y, z)] = o[0];
@@ -412,7 +412,7 @@ __device__ __forceinline__ void pair_brick(PairSpace<typename Cx<R>::T, BX, BY, 
         if constexpr (STB == 1) ps.uget(PS::slot(hx, y, z), pb.y);  // y0 of the cell (u = y0)
         if constexpr (STB == 3) ld4<false>(a.w + j, pb.y);
         CT c[4], L[4];
-        pair_lap_v<LapRhs>(ps, hx, y, z, c, L, a.ihx2, a.ihy2, a.ihz2, c6);
+        pair_lap_v<LapRhs>(ps, hx, y, z, c, L, co);
         bodyB(j, pb, c, L);
     }
     __syncthreads();  // the tiles are reused for the next brick

@@ -285,6 +285,130 @@ __device__ __forceinline__ bool active_v(double V)
 __device__ __forceinline__ bool active_e(float E) { return E >= 0.0f; }
 __device__ __forceinline__ bool active_e(double E) { return __double2hiint(E) >= 0; }
 
+// Coefficients of a cell's neighbour sums, made once a kernel (lap_co)
+template <typename R>
+struct LapCo {
+    R ax, ay, az, c6;
+};
+// Double precision: the sums ax (x- + x+) + ay (y- + y+) + az (z- + z+) of one
+// part of a cell in integers.  An FP64 instruction takes 16 cycles of an SM and the six
+// that a sum needs were half of what bounds the complex128 passes, while
+// the integer pipes stood idle.  The six values become 64-bit fixed point with the
+// largest one's exponent, 59 bits below its leading one, and add without
+// rounding; the coefficients are ref q, q a 64-bit fraction, so that one
+// multiplication by ref remains.  Nothing is lost against FP64 additions: a
+// value is cut at 2^-59 of the largest, an FP64 sum is rounded at 2^-53 of itself,
+// and with q >= 1/8 a sum is never smaller than its cuts make noise.  Spacings more
+// unequal than that, values that are not finite and values far outside any
+// state's range take the FP64 form.  A q of 1 skips its multiplication.
+// RK4 step in complex128: 1024^3 shell 5.44 -> 4.30 ms, 96^3 trap 0.170 -> 0.133;
+// with unequal spacings 0.917 -> 0.738 (200-cell shell).  As a call instead of inline: no gain.
+template <>
+struct LapCo<double> {
+    double ax, ay, az, c6;
+    double ref;                     // the largest coefficient
+    unsigned long long qx, qy, qz;  // 2^64 a / ref; 0: a = ref
+    int lo, hi;                     // exponents (of the largest value) that fixed point serves
+};
+template <typename LAP>
+__device__ __forceinline__ LapCo<float> lap_co(float ihx2, float ihy2, float ihz2)
+{
+    return {LAP::coef(ihx2), LAP::coef(ihy2), LAP::coef(ihz2), 2.0f * (ihx2 + ihy2 + ihz2)};
+}
+template <typename LAP>
+__device__ __forceinline__ LapCo<double> lap_co(double ihx2, double ihy2, double ihz2)
+{
+    LapCo<double> k;
+    k.ax = LAP::coef(ihx2);
+    k.ay = LAP::coef(ihy2);
+    k.az = LAP::coef(ihz2);
+    k.c6 = 2.0 * (ihx2 + ihy2 + ihz2);
+    k.ref = k.ax;
+    k.qx = k.qy = k.qz = 0;
+    bool usual = true;
+    if (ihx2 != ihy2 || ihx2 != ihz2) {
+        k.ref = LAP::coef(fmax(ihx2, fmax(ihy2, ihz2)));
+        const double two64 = 18446744073709551616.0, inv = 1.0 / k.ref;
+        auto frac = [&](double a) -> unsigned long long {
+            const double q = a * inv, rest = __fma_rn(-q, k.ref, a) * inv;
+            usual = usual && q >= 0.125;
+            return a == k.ref ? 0ull : __double2ull_rn(q * two64) + (unsigned long long)__double2ll_rn(rest * two64);
+        };
+        k.qx = frac(k.ax);
+        k.qy = frac(k.ay);
+        k.qz = frac(k.az);
+    }
+    // the result's factor ref 2^(e - 1082) has to be a normal number, and values
+    // 64 binary orders below the largest have to be nothing
+    const int er = (__double2hiint(k.ref) >> 20) & 0x7ff;
+    k.lo = usual && er >= 64 && er <= 1983 ? max(64, 1083 - er) : 0x7fffffff;
+    k.hi = min(2046, 3128 - er);
+    return k;
+}
+
+__device__ __forceinline__ double i64_to_double(long long S)
+{
+    // as __ll2double_rn but for ties, off the FP64 pipe
+    const int sg = (int)(S >> 63);
+    unsigned long long a = (unsigned long long)((S ^ (long long)sg) - (long long)sg);
+    const int z = __clzll((long long)a);
+    a <<= z & 63;
+    const unsigned hi = (unsigned)(a >> 32), lo = (unsigned)a;
+    const unsigned long long m = (unsigned long long)((hi >> 11) + ((unsigned)(1085 - z) << 20)) << 32 |
+                                 __funnelshift_r(lo, hi, 11);
+    const long long r = (long long)(m + ((lo >> 10) & 1u));  // a carry moves the exponent on
+    return S == 0 ? 0.0 : __longlong_as_double(r | (S & (long long)0x8000000000000000ull));
+}
+// S q 2^-64 for a signed S
+__device__ __forceinline__ long long mul_frac(long long S, unsigned long long q)
+{
+    return (long long)(__umul64hi((unsigned long long)S, q) - (S < 0 ? q : 0ull));
+}
+static __device__ __noinline__ double sum6_fp64(double xp, double xm, double yp, double ym, double zp, double zm,
+                                                double ax, double ay, double az)
+{
+    return __fma_rn(az, zp + zm, __fma_rn(ay, yp + ym, ax * (xp + xm)));
+}
+__device__ __forceinline__ double sum6(double xp, double xm, double yp, double ym, double zp, double zm,
+                                       const LapCo<double> &k)
+{
+    const double v[6] = {xp, xm, yp, ym, zp, zm};
+    int e[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) e[i] = (__double2hiint(v[i]) >> 20) & 0x7ff;
+    const int em = max(max(max(e[0], e[1]), max(e[2], e[3])), max(e[4], e[5]));
+    if (em < k.lo || em > k.hi) {
+        long long any = 0;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) any |= __double_as_longlong(v[i]) & 0x7fffffffffffffffll;
+        return any == 0 ? 0.0 : sum6_fp64(xp, xm, yp, ym, zp, zm, k.ax, k.ay, k.az);
+    }
+    long long S[3];
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        S[p] = 0;
+        int neg = 0;
+#pragma unroll
+        for (int i = 2 * p; i < 2 * p + 2; ++i) {
+            const int hi = __double2hiint(v[i]), lo = __double2loint(v[i]);
+            const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+            unsigned long long x;  // the mantissa, its leading one at bit 59 - (em - e); shifts beyond 63 give 0
+            asm("{.reg .b64 t; mov.b64 t, {%1, %2}; shr.u64 %0, t, %3;}"
+                : "=l"(x)
+                : "r"((unsigned)lo << 7), "r"(__funnelshift_l((unsigned)lo, mh, 7)), "r"(em - e[i]));
+            const int sg = hi >> 31;
+            S[p] += (long long)(x ^ (unsigned long long)(long long)sg);  // -x - 1 for a negative value
+            neg += sg;
+        }
+        S[p] -= neg;
+    }
+    if (k.qx) S[0] = mul_frac(S[0], k.qx);
+    if (k.qy) S[1] = mul_frac(S[1], k.qy);
+    if (k.qz) S[2] = mul_frac(S[2], k.qz);
+    const double f = __hiloint2double(__double2hiint(k.ref) + ((em - 1082) << 20), __double2loint(k.ref));
+    return i64_to_double(S[0] + S[1] + S[2]) * f;
+}
+
 struct LapFull {
     template <typename R>
     __device__ __forceinline__ static R coef(R a)
@@ -297,6 +421,7 @@ struct LapFull {
     {
         return lapv(xp, xm, yp, ym, zp, zm, c, ax, ay, az, c6);
     }
+    __device__ __forceinline__ static double with(double c, double s, double c6) { return __fma_rn(-c6, c, s); }
 };
 struct LapRhs {
     __device__ __forceinline__ static float coef(float a) { return a; }
@@ -317,31 +442,47 @@ struct LapRhs {
         n.y = __fma_rn(az, zp.y + zm.y, __fma_rn(ay, yp.y + ym.y, ax * (xp.y + xm.y)));
         return n;
     }
+    __device__ __forceinline__ static double of(double xp, double xm, double yp, double ym, double zp, double zm,
+                                                double, double ax, double ay, double az, double)
+    {
+        return __fma_rn(az, zp + zm, __fma_rn(ay, yp + ym, ax * (xp + xm)));
+    }
+    __device__ __forceinline__ static double with(double, double s, double) { return s; }
 };
 // The Euler kinetic substep c + q lap c of the imaginary-time passes.  In double
 // precision, where FP64 instructions bound them, the spacings carry q
 // (euler_coef) and the centre's two terms are one factor, so that `of` gives
-// the substep's result in 7 instructions a value instead of 9; the rounding of
-// that factor is the same for every cell, so the renormalisation takes it out.
-// In single precision it gives the Laplacian, and euler() adds it.
+// the substep's result; the rounding of that factor is the same for every
+// cell, so the renormalisation takes it out.  In single precision it gives the
+// Laplacian, and euler() adds it.
 struct LapEuler : LapFull {
-    using LapFull::of;
-    __device__ __forceinline__ static double of(double xp, double xm, double yp, double ym, double zp, double zm,
-                                                double c, double ax, double ay, double az, double c6)
-    {
-        const double t = __fma_rn(az, zp + zm, __fma_rn(ay, yp + ym, ax * (xp + xm)));
-        return __fma_rn(1.0 - c6, c, t);
-    }
-    __device__ __forceinline__ static double2 of(const double2 &xp, const double2 &xm, const double2 &yp,
-                                                 const double2 &ym, const double2 &zp, const double2 &zm,
-                                                 const double2 &c, double ax, double ay, double az, double c6)
-    {
-        double2 o;
-        o.x = of(xp.x, xm.x, yp.x, ym.x, zp.x, zm.x, c.x, ax, ay, az, c6);
-        o.y = of(xp.y, xm.y, yp.y, ym.y, zp.y, zm.y, c.y, ax, ay, az, c6);
-        return o;
-    }
+    __device__ __forceinline__ static double with(double c, double s, double c6) { return __fma_rn(1.0 - c6, c, s); }
 };
+// LAP's result from the sum of a cell's neighbours (double precision)
+template <typename LAP>
+__device__ __forceinline__ double with_centre(double c, double s, double c6)
+{
+    return LAP::with(c, s, c6);
+}
+template <typename LAP>
+__device__ __forceinline__ double2 with_centre(const double2 &c, const double2 &s, double c6)
+{
+    return make_double2(LAP::with(c.x, s.x, c6), LAP::with(c.y, s.y, c6));
+}
+// What LAP makes of a cell c and its six neighbours
+template <typename LAP, typename CT, typename R>
+__device__ __forceinline__ CT lap_of(const CT &xp, const CT &xm, const CT &yp, const CT &ym, const CT &zp, const CT &zm,
+                                     const CT &c, const LapCo<R> &k)
+{
+    if constexpr (sizeof(R) == 4) {
+        return LAP::of(xp, xm, yp, ym, zp, zm, c, k.ax, k.ay, k.az, k.c6);
+    } else if constexpr (is_cplx<CT>()) {
+        const CT s = make_double2(sum6(xp.x, xm.x, yp.x, ym.x, zp.x, zm.x, k), sum6(xp.y, xm.y, yp.y, ym.y, zp.y, zm.y, k));
+        return with_centre<LAP>(c, s, k.c6);
+    } else {
+        return LAP::with(c, sum6(xp, xm, yp, ym, zp, zm, k), k.c6);
+    }
+}
 __device__ __forceinline__ float euler_coef(float ih2, float) { return ih2; }
 __device__ __forceinline__ double euler_coef(double ih2, double q) { return ih2 * q; }
 // the substep of value c from what LapEuler gave for it
@@ -792,7 +933,7 @@ __device__ __forceinline__ void brick_apply(WarpSpace<CT, BX, BY, BZ> &ws, const
     // stored segments: Laplacian from the tile, then the body.  Opposite
     // neighbours are summed first and the centre term enters once:
     // L = (x- + x+) / hx^2 + (y- + y+) / hy^2 + (z- + z+) / hz^2 - c6 c.
-    const R c6 = (R)2 * (ihx2 + ihy2 + ihz2);
+    const LapCo<R> co = lap_co<LAP>(ihx2, ihy2, ihz2);
     auto segment = [&](int r, const auto &pre) {
         const int e = ws.list[r];
         const int sl = e & 0xff, hrow = e >> 8, hx = sl % S::SX;
@@ -808,7 +949,7 @@ __device__ __forceinline__ void brick_apply(WarpSpace<CT, BX, BY, BZ> &ws, const
         for (int i = 0; i < 4; ++i) {
             const CT l = i == 0 ? xm : c[i - 1];
             const CT rr = i == 3 ? xp : c[i + 1];
-            L[i] = LAP::of(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], LAP::coef(ihx2), LAP::coef(ihy2), LAP::coef(ihz2), c6);
+            L[i] = lap_of<LAP>(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], co);
         }
         body(R0.off + 4u * (uint32_t)r, pre, c, L);
     };

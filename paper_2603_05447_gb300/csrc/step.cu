@@ -988,11 +988,12 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? (NS < 3 ? 6 : 5) : (NS 
         R V0[4], V1[BLEND ? 4 : 1];
         CT y[NS > 0 ? NS : 1][4];
     };
+    const auto co = tile_co<7, LapRhs>(a.ihx2, a.ihy2, a.ihz2);  // before the wait
     const TileList list = tile_begin(T);
     const R s = BLEND ? (R)__ldcg(a.stab) : (R)0;
     const R c3 = rhs_centre(a.ihx2, a.ihy2, a.ihz2);
     constexpr R HALF = sizeof(R) == 8 ? (R)1 : (R)(-0.5);  // LapRhs leaves the factor in in single precision
-    tile_loop<7, LapRhs>(T, list, (const CT *)a.y[a.tile], Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
+    tile_loop<7, LapRhs>(T, list, (const CT *)a.y[a.tile], Plain(), co, EveryTile(),
                  [&](uint32_t idx, uint32_t n) {
                      prefetch_l2(a.V0 + idx, n * (uint32_t)sizeof(R));
                      if constexpr (BLEND) prefetch_l2(a.V1 + idx, n * (uint32_t)sizeof(R));

@@ -120,15 +120,28 @@ struct TileSlots<19> {
     __device__ __forceinline__ int operator()(int k) const { return (int)((q[k / 5] >> (12 * (k % 5))) & 4095u); }
 };
 
+// a tile kernel's inverse square spacings and what LAP makes of them (7 points)
+template <typename R>
+struct TileCo {
+    R ihx2, ihy2, ihz2;
+    LapCo<R> k;
+};
+template <int NP, typename LAP, typename R>
+__device__ __forceinline__ TileCo<R> tile_co(R ihx2, R ihy2, R ihz2)
+{
+    TileCo<R> co{ihx2, ihy2, ihz2, {}};
+    if constexpr (NP == 7) co.k = lap_co<LAP>(ihx2, ihy2, ihz2);
+    return co;
+}
+
 // L of a segment with values c and neighbour slots f: the Laplacians, or what
 // LAP makes of them
 template <int NP, typename LAP, typename CT, typename R>
-__device__ __forceinline__ void tile_laplacian(const TileMem<CT, NP> &m, const TileSlots<NP> &f, const CT (&c)[4], R ihx2,
-                                               R ihy2, R ihz2, CT (&L)[4])
+__device__ __forceinline__ void tile_laplacian(const TileMem<CT, NP> &m, const TileSlots<NP> &f, const CT (&c)[4],
+                                               const TileCo<R> &co, CT (&L)[4])
 {
     // opposite neighbours are summed first and the centre term enters once:
     // L = (x- + x+) / hx^2 + (y- + y+) / hy^2 + (z- + z+) / hz^2 - c6 c
-    const R c6 = (R)2 * (ihx2 + ihy2 + ihz2);
     CT ym[4], yp[4], zm[4], zp[4];
     m.get(f(0), ym);
     m.get(f(1), yp);
@@ -140,7 +153,7 @@ __device__ __forceinline__ void tile_laplacian(const TileMem<CT, NP> &m, const T
         for (int i = 0; i < 4; ++i) {
             const CT l = i == 0 ? xm : c[i - 1];
             const CT rr = i == 3 ? xp : c[i + 1];
-            L[i] = LAP::of(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], LAP::coef(ihx2), LAP::coef(ihy2), LAP::coef(ihz2), c6);
+            L[i] = lap_of<LAP>(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], co.k);
         }
     } else {
         // App. B: the 7-point part plus w_ab (edges_ab - 2 faces_ab + 4 c) per
@@ -149,6 +162,7 @@ __device__ __forceinline__ void tile_laplacian(const TileMem<CT, NP> &m, const T
         //   x: 1/hx^2 - 2 (wxy + wxz), y: 1/hy^2 - 2 (wxy + wyz),
         //   z: 1/hz^2 - 2 (wxz + wyz), centre: c6 - 4 (wxy + wxz + wyz),
         // and only the three edge sums remain: + wxy exy + wxz exz + wyz eyz.
+        const R ihx2 = co.ihx2, ihy2 = co.ihy2, ihz2 = co.ihz2, c6 = (R)2 * (ihx2 + ihy2 + ihz2);
         const R wxy = (ihx2 + ihy2) / (R)12, wxz = (ihx2 + ihz2) / (R)12, wyz = (ihy2 + ihz2) / (R)12;
         const R ax = ihx2 - (R)2 * (wxy + wxz), ay = ihy2 - (R)2 * (wxy + wyz), az = ihz2 - (R)2 * (wxz + wyz);
         const R c19 = c6 - (R)4 * (wxy + wxz + wyz);
@@ -170,8 +184,14 @@ __device__ __forceinline__ void tile_laplacian(const TileMem<CT, NP> &m, const T
                                 vadd(i == 0 ? ypl : yp[i - 1], i == 3 ? ypr : yp[i + 1]));
             const CT exz = vadd(vadd(i == 0 ? zml : zm[i - 1], i == 3 ? zmr : zm[i + 1]),
                                 vadd(i == 0 ? zpl : zp[i - 1], i == 3 ? zpr : zp[i + 1]));
-            L[i] = edgev(LAP::of(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], LAP::coef(ax), LAP::coef(ay), LAP::coef(az), c19),
-                         exy, exz, eyz[i], LAP::coef(wxy), LAP::coef(wxz), LAP::coef(wyz));
+            if constexpr (sizeof(R) == 8 && std::is_same<LAP, LapEuler>::value) {
+                // the centre comes last, so that only its addition rounds at the result's size
+                const CT faces = LapRhs::of(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], ax, ay, az, c19);
+                L[i] = with_centre<LAP>(c[i], edgev(faces, exy, exz, eyz[i], wxy, wxz, wyz), c19);
+            } else {
+                L[i] = edgev(LAP::of(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], LAP::coef(ax), LAP::coef(ay), LAP::coef(az), c19),
+                             exy, exz, eyz[i], LAP::coef(wxy), LAP::coef(wxz), LAP::coef(wyz));
+            }
         }
     }
 }
@@ -243,11 +263,11 @@ struct EveryTile {
 // buffered tiles a block, ran a third slower.
 //
 // setup(tile), uniform over the block, runs before each tile, may change what
-// xf and the inverse square spacings refer to, and says whether to take it.
+// xf and co refer to, and says whether to take it.
 template <int NP, typename LAP = LapFull, typename CT, typename R, typename XF, typename SETUP, typename PREF,
           typename LOAD, typename BODY>
-__device__ __forceinline__ void tile_loop(const TileView &T, TileList list, const CT *src, const XF &xf, const R &ihx2,
-                                          const R &ihy2, const R &ihz2, SETUP setup, PREF prefetch, LOAD load, BODY body)
+__device__ __forceinline__ void tile_loop(const TileView &T, TileList list, const CT *src, const XF &xf,
+                                          const TileCo<R> &co, SETUP setup, PREF prefetch, LOAD load, BODY body)
 {
     extern __shared__ __align__(16) unsigned char gpe_smem[];
     using M = TileMem<CT, NP>;
@@ -336,7 +356,7 @@ __device__ __forceinline__ void tile_loop(const TileView &T, TileList list, cons
         __syncthreads();
         if (in) {
             CT L[4];
-            tile_laplacian<NP, LAP>(m, f, c, ihx2, ihy2, ihz2, L);
+            tile_laplacian<NP, LAP>(m, f, c, co, L);
             body(idx, pre, c, L);
         }
     }
@@ -386,23 +406,24 @@ __device__ __forceinline__ R tile_rhs_centre(R ihx2, R ihy2, R ihz2)
 }
 
 // One RK4 stage.  1024^3 shell, 8x8x4 bricks, per step of four: complex64
-// 0.776 -> 0.626 ms (4.0 GB, of which 0.4 GB slots and halo lists: 6.5 TB/s,
-// 0.95 of the copy bandwidth, so bytes bound it now); complex128 8.65 -> 5.49
+// 0.776 -> 0.622 ms (4.0 GB, of which 0.4 GB slots and halo lists: 6.5 TB/s,
+// 0.95 of the copy bandwidth, so bytes bound it now); complex128 8.65 -> 4.30
 // ms (full lanes instead of four fifths: 6.75; 90 instead of 108 FP64
-// instructions a cell and step, LapRhs, active_v and the split third: 5.49; an
-// FP64 instruction takes 8 to 9.6 ns an SM whatever its lanes do, and they
-// fill the time).  Single precision, six blocks an SM (85 registers): 0.626
-// ms, seven 0.634, eight with spills 0.645; double, registers for two: 5.49,
-// three 5.69, four 5.80.  One block a tile instead of looping blocks: 8 %
-// slower (no tile ahead to prefetch).
+// instructions a cell and step, LapRhs, active_v and the split third: 5.44;
+// the neighbour sums in integers, sum6: 4.30; an FP64 instruction takes 16
+// cycles of an SM whatever its lanes do).  Single precision, six blocks an SM
+// (85 registers): 0.626 ms, seven 0.634, eight with spills 0.645; double, three
+// blocks (168 registers) 4.30, two 4.37; blended two, which three lose 1 % to.
+// One block a tile instead of looping blocks: 8 % slower (no tile ahead to prefetch).
 template <typename R, bool BLEND, int ST, int NP>
-__global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? tile_blocks_f(NP) : 2) k_rk4_tile(const RkArgs<R> a, const TileView T)
+__global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? tile_blocks_f(NP) : (BLEND || NP == 19 ? 2 : 3)) k_rk4_tile(const RkArgs<R> a, const TileView T)
 {
     using CT = typename Cx<R>::T;
     using B = Rk4Body<R, BLEND, false, ST>;
+    const auto co = tile_co<NP, LapRhs>(a.ihx2, a.ihy2, a.ihz2);  // before the wait
     const TileList list = tile_begin(T);
     const B body(a, BLEND ? (R)__ldcg(a.stab) : (R)0, tile_rhs_centre<NP>(a.ihx2, a.ihy2, a.ihz2));
-    tile_loop<NP, LapRhs>(T, list, body.yin(), Plain(), a.ihx2, a.ihy2, a.ihz2, EveryTile(),
+    tile_loop<NP, LapRhs>(T, list, body.yin(), Plain(), co, EveryTile(),
                   [&](uint32_t idx, uint32_t n) {
                       prefetch_l2(a.V0 + idx, n * (uint32_t)sizeof(R));
                       if constexpr (BLEND) prefetch_l2(a.V1 + idx, n * (uint32_t)sizeof(R));
