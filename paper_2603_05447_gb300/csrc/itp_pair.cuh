@@ -207,7 +207,7 @@ __device__ __forceinline__ void itp_pair_brick(ItpPairSpace<typename Cx<R>::T, B
             zm = ps.uxr[PS::row(y, z - 1)][0];
             zp = ps.uxr[PS::row(y, z + 1)][0];
         }
-        const CT L = lap_of<LapEuler>(xp, xm, yp, ym, zp, zm, c0, co);
+        const CT L = lap_of<LapEuler, true>(xp, xm, yp, ym, zp, zm, c0, co);
         (side == 0 ? ps.vxl : ps.vxr)[PS::vrow(y, z)] = e >= (R)0 ? euler(c0, q4, L) : czero<CT>();
     }
     __syncthreads();

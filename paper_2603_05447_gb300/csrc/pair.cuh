@@ -266,7 +266,7 @@ __device__ __forceinline__ void pair_lap_u(const PairSpace<CT, BX, BY, BZ> &ps, 
     for (int i = 0; i < 4; ++i) {
         const CT l = i == 0 ? xm : c[i - 1];
         const CT rr = i == 3 ? xp : c[i + 1];
-        L[i] = lap_of<LAP>(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], co);
+        L[i] = lap_of<LAP, true>(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], co);
     }
 }
 
@@ -290,7 +290,7 @@ __device__ __forceinline__ void pair_lap_v(const PairSpace<CT, BX, BY, BZ> &ps, 
     for (int i = 0; i < 4; ++i) {
         const CT l = i == 0 ? xm : c[i - 1];
         const CT rr = i == 3 ? xp : c[i + 1];
-        L[i] = lap_of<LAP>(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], co);
+        L[i] = lap_of<LAP, true>(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], co);
     }
 }
 
@@ -320,8 +320,7 @@ __device__ __forceinline__ void pair_brick(PairSpace<typename Cx<R>::T, BX, BY, 
     }
     cp_async_wait_all();
     __syncthreads();
-    const R c3 = rhs_centre(a.ihx2, a.ihy2, a.ihz2);
-    const BA bodyA(a, sA, c3);
+    const BA bodyA(a, sA);
     const int nst = ps.nst;
     const BrickRec &R0 = ps.rec[0];
     // stage A on the stored segments of the brick, then of the one-deep z and
@@ -392,7 +391,7 @@ __device__ __forceinline__ void pair_brick(PairSpace<typename Cx<R>::T, BX, BY, 
         if constexpr (BLEND) pa.V1[0] = a.V1[j];
         if constexpr (STA == 2) pa.y[0] = a.y0[j];
         CT c[4] = {c0, czero<CT>(), czero<CT>(), czero<CT>()}, L[4], o[4], wv[4];
-        L[0] = lap_of<LapRhs>(xp, xm, yp, ym, zp, zm, c0, co);
+        L[0] = lap_of<LapRhs, true>(xp, xm, yp, ym, zp, zm, c0, co);
         L[1] = L[2] = L[3] = czero<CT>();
         bodyA.compute(pa, c, L, o, wv);
         (side == 0 ? ps.vxl : ps.vxr)[PS::vrow(y, z)] = o[0];
@@ -401,7 +400,7 @@ __device__ __forceinline__ void pair_brick(PairSpace<typename Cx<R>::T, BX, BY, 
     // stage B on the brick's stored segments
     RkArgs<R> ab = a;
     if constexpr (PASS == 1) ab.y0 = y1out;  // stage 3 writes y1 to the other buffer
-    const BB bodyB(ab, sB, c3);
+    const BB bodyB(ab, sB);
     for (int i = t; i < nst; i += PAIR_THREADS) {
         const int q = ps.list[i];
         const int hx = q % SX, y = (q / SX) % BY, z = q / PL;

@@ -265,13 +265,12 @@ __device__ __forceinline__ CT lapv(const CT &xp, const CT &xm, const CT &yp, con
 }
 
 // What a pass wants of a cell's neighbourhood: its Laplacian (LapFull), or, for
-// the right-hand side of the real-time steps, half of it with the sign of the
-// kinetic term (LapRhs).  In double precision LapRhs leaves out the centre's
-// share, (1/hx^2 + 1/hy^2 + 1/hz^2) c, which the caller adds to the potential
-// for one addition a cell: with the factor -1/2 in the coefficients that saves
-// four of 23 FP64 instructions a cell and stage, and FP64 instructions are
-// what bounds the complex128 steps.  In single precision, bound by bytes, it
-// is the Laplacian as it is.
+// the right-hand side of the real-time steps in double precision, half of it with
+// the sign of the kinetic term (LapRhs): FP64 instructions bound the complex128
+// steps, and the factor -1/2 costs none in the coefficients.  (The centre's
+// share in the potential would save one more of about fourteen a cell and stage,
+// 3 % of a step, but rounds the potential at the size of 1/h^2: 19-point errors
+// 2 % larger.)  In single precision, bound by bytes, it is the Laplacian as it is.
 // Whether a cell is active, from its potential (+inf, or NaN, marks the inactive
 // cells of stored segments) or its propagator (negative there).  Double values
 // are tested by their high words: an FP64 comparison costs as much as an FP64
@@ -301,8 +300,8 @@ struct LapCo {
 // and with q >= 1/8 a sum is never smaller than its cuts make noise.  Spacings more
 // unequal than that, values that are not finite and values far outside any
 // state's range take the FP64 form.  A q of 1 skips its multiplication.
-// RK4 step in complex128: 1024^3 shell 5.44 -> 4.30 ms, 96^3 trap 0.170 -> 0.133;
-// with unequal spacings 0.917 -> 0.738 (200-cell shell).  As a call instead of inline: no gain.
+// RK4 step in complex128: 1024^3 shell 5.44 -> 4.45 ms, 96^3 trap 0.170 -> 0.138;
+// with unequal spacings 0.917 -> 0.764 (200-cell shell).  As a call instead of inline: no gain.
 template <>
 struct LapCo<double> {
     double ax, ay, az, c6;
@@ -447,16 +446,16 @@ struct LapRhs {
     {
         return __fma_rn(az, zp + zm, __fma_rn(ay, yp + ym, ax * (xp + xm)));
     }
-    __device__ __forceinline__ static double with(double, double s, double) { return s; }
+    __device__ __forceinline__ static double with(double c, double s, double c6) { return __fma_rn(0.5 * c6, c, s); }
 };
 // The Euler kinetic substep c + q lap c of the imaginary-time passes.  In double
 // precision, where FP64 instructions bound them, the spacings carry q
-// (euler_coef) and the centre's two terms are one factor, so that `of` gives
-// the substep's result; the rounding of that factor is the same for every
-// cell, so the renormalisation takes it out.  In single precision it gives the
-// Laplacian, and euler() adds it.
+// (euler_coef) and lap_of gives the substep's result, c + (sums - c6 c).  (One factor
+// 1 - c6 for the centre's two terms would save an instruction; its rounding
+// made the errors 11 % larger.)  In single precision it gives the Laplacian,
+// and euler() adds it.
 struct LapEuler : LapFull {
-    __device__ __forceinline__ static double with(double c, double s, double c6) { return __fma_rn(1.0 - c6, c, s); }
+    __device__ __forceinline__ static double with(double c, double s, double c6) { return c + __fma_rn(-c6, c, s); }
 };
 // LAP's result from the sum of a cell's neighbours (double precision)
 template <typename LAP>
@@ -469,18 +468,31 @@ __device__ __forceinline__ double2 with_centre(const double2 &c, const double2 &
 {
     return make_double2(LAP::with(c.x, s.x, c6), LAP::with(c.y, s.y, c6));
 }
-// What LAP makes of a cell c and its six neighbours
-template <typename LAP, typename CT, typename R>
+// sum6 as a call, for the kernels that hold several stages' code: inline, its eight
+// copies a stage no longer fit the instruction cache and the registers
+// (120-cell shell, WAVE schedule, eight RK4 steps: 6.8 ms inline, 3.9 so, 3.85
+// in FP64)
+static __device__ __noinline__ double sum6_call(double xp, double xm, double yp, double ym, double zp, double zm,
+                                                const LapCo<double> *k)
+{
+    return sum6(xp, xm, yp, ym, zp, zm, *k);
+}
+
+// What LAP makes of a cell c and its six neighbours; CALL: by sum6_call
+template <typename LAP, bool CALL = false, typename CT, typename R>
 __device__ __forceinline__ CT lap_of(const CT &xp, const CT &xm, const CT &yp, const CT &ym, const CT &zp, const CT &zm,
                                      const CT &c, const LapCo<R> &k)
 {
     if constexpr (sizeof(R) == 4) {
         return LAP::of(xp, xm, yp, ym, zp, zm, c, k.ax, k.ay, k.az, k.c6);
-    } else if constexpr (is_cplx<CT>()) {
-        const CT s = make_double2(sum6(xp.x, xm.x, yp.x, ym.x, zp.x, zm.x, k), sum6(xp.y, xm.y, yp.y, ym.y, zp.y, zm.y, k));
-        return with_centre<LAP>(c, s, k.c6);
     } else {
-        return LAP::with(c, sum6(xp, xm, yp, ym, zp, zm, k), k.c6);
+        auto sum = [&](double a, double b, double e, double f, double g, double h) {
+            return CALL ? sum6_call(a, b, e, f, g, h, &k) : sum6(a, b, e, f, g, h, k);
+        };
+        if constexpr (is_cplx<CT>())
+            return with_centre<LAP>(c, make_double2(sum(xp.x, xm.x, yp.x, ym.x, zp.x, zm.x), sum(xp.y, xm.y, yp.y, ym.y, zp.y, zm.y)), k.c6);
+        else
+            return with_centre<LAP>(c, sum(xp, xm, yp, ym, zp, zm), k.c6);
     }
 }
 __device__ __forceinline__ float euler_coef(float ih2, float) { return ih2; }
@@ -492,9 +504,6 @@ __device__ __forceinline__ CT euler(const CT &c, R q, const CT &L)
     if constexpr (sizeof(R) == 8) return L;
     else return axpy(c, q, L);
 }
-// the centre's share that LapRhs leaves to the caller
-__device__ __forceinline__ float rhs_centre(float, float, float) { return 0.0f; }
-__device__ __forceinline__ double rhs_centre(double ihx2, double ihy2, double ihz2) { return ihx2 + ihy2 + ihz2; }
 
 __device__ __forceinline__ float2 shfl_up(float2 v, int d)
 {
@@ -949,7 +958,7 @@ __device__ __forceinline__ void brick_apply(WarpSpace<CT, BX, BY, BZ> &ws, const
         for (int i = 0; i < 4; ++i) {
             const CT l = i == 0 ? xm : c[i - 1];
             const CT rr = i == 3 ? xp : c[i + 1];
-            L[i] = lap_of<LAP>(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], co);
+            L[i] = lap_of<LAP, true>(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], co);
         }
         body(R0.off + 4u * (uint32_t)r, pre, c, L);
     };
@@ -1140,11 +1149,10 @@ struct Rk4Body {
         CT y[4];  // y0 (stages 1, 2) or w (stage 3)
     };
     const RkArgs<R> &a;
-    R s, k, c3;
+    R s, k;
     CT *yout;
-    // c3_: the centre's share of the right-hand side (rhs_centre)
-    __device__ __forceinline__ Rk4Body(const RkArgs<R> &a_, R s_, R c3_)
-        : a(a_), s(s_), k(st == 2 ? a_.dt : (st == 3 ? a_.dt / (R)6 : a_.dt / (R)2)), c3(c3_),
+    __device__ __forceinline__ Rk4Body(const RkArgs<R> &a_, R s_)
+        : a(a_), s(s_), k(st == 2 ? a_.dt : (st == 3 ? a_.dt / (R)6 : a_.dt / (R)2)),
           yout(st == 0 ? a_.y2 : st == 1 ? a_.y3 : st == 2 ? a_.y4 : a_.y0)
     {
     }
@@ -1197,8 +1205,8 @@ struct Rk4Body {
         for (int i = 0; i < 4; ++i) {
             R V = p.V0[i];
             if constexpr (BLEND) V = ((R)1 - s) * p.V0[i] + s * p.V1[i];
-            // L is the neighbours' share of -1/2 lap; the centre's is in w
-            const R w = (V + a.g * (c[i].x * c[i].x + c[i].y * c[i].y)) + c3;
+            // L is -1/2 lap
+            const R w = V + a.g * (c[i].x * c[i].x + c[i].y * c[i].y);
             const R hr = L[i].x + w * c[i].x;
             const R hi = L[i].y + w * c[i].y;
             // f = -i (hr + i hi) = hi - i hr
@@ -1242,7 +1250,7 @@ __device__ __forceinline__ void rk4_brick(const RkArgs<R> &a, const GridView &G,
                                           WarpSpace<typename Cx<R>::T, BX, BY, BZ> &ws, R s)
 {
     using B = Rk4Body<R, BLEND, CG, st>;
-    const B body(a, s, rhs_centre(a.ihx2, a.ihy2, a.ihz2));
+    const B body(a, s);
     brick_apply<BX, BY, BZ, CG, LapRhs>(ws, G, b, next, body.yin(), Identity(), a.ihx2, a.ihy2, a.ihz2,
                                 [&](uint32_t idx) { return body.load(idx); }, body);
 }

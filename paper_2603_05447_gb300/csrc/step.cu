@@ -991,7 +991,6 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? (NS < 3 ? 6 : 5) : (NS 
     const auto co = tile_co<7, LapRhs>(a.ihx2, a.ihy2, a.ihz2);  // before the wait
     const TileList list = tile_begin(T);
     const R s = BLEND ? (R)__ldcg(a.stab) : (R)0;
-    const R c3 = rhs_centre(a.ihx2, a.ihy2, a.ihz2);
     constexpr R HALF = sizeof(R) == 8 ? (R)1 : (R)(-0.5);  // LapRhs leaves the factor in in single precision
     tile_loop<7, LapRhs>(T, list, (const CT *)a.y[a.tile], Plain(), co, EveryTile(),
                  [&](uint32_t idx, uint32_t n) {
@@ -1017,8 +1016,7 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? (NS < 3 ? 6 : 5) : (NS 
                          for (int j = 0; j < NS; ++j) acc = axpy(acc, a.coef[j], p.y[j][i]);
                          R V = p.V0[i];
                          if constexpr (BLEND) V = ((R)1 - s) * p.V0[i] + s * p.V1[i];
-                         R w = V + a.g * (c[i].x * c[i].x + c[i].y * c[i].y);
-                         if constexpr (sizeof(R) == 8) w += c3;
+                         const R w = V + a.g * (c[i].x * c[i].x + c[i].y * c[i].y);
                          const R hr = HALF * L[i].x + w * c[i].x;
                          const R hi = HALF * L[i].y + w * c[i].y;
                          // f = -i (hr + i hi) = hi - i hr; +inf marks an inactive cell of a stored segment

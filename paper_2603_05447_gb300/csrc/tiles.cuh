@@ -184,10 +184,10 @@ __device__ __forceinline__ void tile_laplacian(const TileMem<CT, NP> &m, const T
                                 vadd(i == 0 ? ypl : yp[i - 1], i == 3 ? ypr : yp[i + 1]));
             const CT exz = vadd(vadd(i == 0 ? zml : zm[i - 1], i == 3 ? zmr : zm[i + 1]),
                                 vadd(i == 0 ? zpl : zp[i - 1], i == 3 ? zpr : zp[i + 1]));
-            if constexpr (sizeof(R) == 8 && std::is_same<LAP, LapEuler>::value) {
+            if constexpr (sizeof(R) == 8 && !std::is_same<LAP, LapFull>::value) {
                 // the centre comes last, so that only its addition rounds at the result's size
-                const CT faces = LapRhs::of(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], ax, ay, az, c19);
-                L[i] = with_centre<LAP>(c[i], edgev(faces, exy, exz, eyz[i], wxy, wxz, wyz), c19);
+                const CT faces = LapRhs::of(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], LAP::coef(ax), LAP::coef(ay), LAP::coef(az), c19);
+                L[i] = with_centre<LAP>(c[i], edgev(faces, exy, exz, eyz[i], LAP::coef(wxy), LAP::coef(wxz), LAP::coef(wyz)), c19);
             } else {
                 L[i] = edgev(LAP::of(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], LAP::coef(ax), LAP::coef(ay), LAP::coef(az), c19),
                              exy, exz, eyz[i], LAP::coef(wxy), LAP::coef(wxz), LAP::coef(wyz));
@@ -396,24 +396,15 @@ inline unsigned tile_blocks(K kernel, int nsm, int n, size_t smem)
 constexpr int tile_blocks_f(int np) { return np == 19 ? 5 : 6; }
 #define GPE_TILE_BOUNDS(R, NP) __launch_bounds__(TILE, sizeof(R) == 4 ? tile_blocks_f(NP) : 3)
 
-// the centre's share of the right-hand side with either stencil (App. B's
-// centre weight is c6 - 4 (wxy + wxz + wyz))
-template <int NP, typename R>
-__device__ __forceinline__ R tile_rhs_centre(R ihx2, R ihy2, R ihz2)
-{
-    const R c = rhs_centre(ihx2, ihy2, ihz2);
-    return NP == 19 ? c - c / (R)3 : c;  // 2 (wxy + wxz + wyz) = (1/hx^2 + 1/hy^2 + 1/hz^2) / 3
-}
-
 // One RK4 stage.  1024^3 shell, 8x8x4 bricks, per step of four: complex64
 // 0.776 -> 0.622 ms (4.0 GB, of which 0.4 GB slots and halo lists: 6.5 TB/s,
-// 0.95 of the copy bandwidth, so bytes bound it now); complex128 8.65 -> 4.30
+// 0.95 of the copy bandwidth, so bytes bound it now); complex128 8.65 -> 4.45
 // ms (full lanes instead of four fifths: 6.75; 90 instead of 108 FP64
 // instructions a cell and step, LapRhs, active_v and the split third: 5.44;
-// the neighbour sums in integers, sum6: 4.30; an FP64 instruction takes 16
+// the neighbour sums in integers, sum6: 4.45; an FP64 instruction takes 16
 // cycles of an SM whatever its lanes do).  Single precision, six blocks an SM
 // (85 registers): 0.626 ms, seven 0.634, eight with spills 0.645; double, three
-// blocks (168 registers) 4.30, two 4.37; blended two, which three lose 1 % to.
+// blocks (168 registers) are 1.5 % ahead of two; blended two, which three lose 1 % to.
 // One block a tile instead of looping blocks: 8 % slower (no tile ahead to prefetch).
 template <typename R, bool BLEND, int ST, int NP>
 __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? tile_blocks_f(NP) : (BLEND || NP == 19 ? 2 : 3)) k_rk4_tile(const RkArgs<R> a, const TileView T)
@@ -422,7 +413,7 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? tile_blocks_f(NP) : (BL
     using B = Rk4Body<R, BLEND, false, ST>;
     const auto co = tile_co<NP, LapRhs>(a.ihx2, a.ihy2, a.ihz2);  // before the wait
     const TileList list = tile_begin(T);
-    const B body(a, BLEND ? (R)__ldcg(a.stab) : (R)0, tile_rhs_centre<NP>(a.ihx2, a.ihy2, a.ihz2));
+    const B body(a, BLEND ? (R)__ldcg(a.stab) : (R)0);
     tile_loop<NP, LapRhs>(T, list, body.yin(), Plain(), co, EveryTile(),
                   [&](uint32_t idx, uint32_t n) {
                       prefetch_l2(a.V0 + idx, n * (uint32_t)sizeof(R));
