@@ -44,7 +44,7 @@ def kernel_source_hash():
     launch code, device code and shared internals)."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2603_05447_gb300", "csrc")
-    for f in ("gpe_internal.cuh", "stencil.cuh", "step.cu"):
+    for f in ("gpe_internal.cuh", "stencil.cuh", "tiles.cuh", "kernels.cuh", "step.cu"):
         h.update(open(os.path.join(csrc, f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -508,7 +508,7 @@ def _run_ours(args, torch, world, rank, local):
                    "parallelism": f"replicas x{world}"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
-                     "kernel": {0: "RK4 step (k_rk4_staged, four launches per step)",
+                     "kernel": {0: "RK4 step (k_rk4_tile, four launches per step)",
                                 1: "RK4 step (k_rk4_wave, one launch per step)",
                                 2: "RK4 step (k_rk4_wave, two launches of two stages per step)",
                                 3: "RK4 step (k_rk4_fused, two launches of two fused stages per step)"}[args.sched],
