@@ -144,10 +144,10 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? 5 : 2) k_adj_stage(cons
                          st4(a.mu_out + idx, mo);
                      }
                      dot[0].add(d4);
-                     if (++n % SUM_FLUSH == 0) dot[0].flush();
+                     keep<1>(dot, ++n);
                  });
     double tot[1];
-    block_totals<1>(dot, sums_flushed((uint32_t)T.ntiles), tot);
+    block_totals<1>(dot, tot);
     if (launch_totals<1>(tot, a.partials, a.counter) && threadIdx.x == 0) {
         a.grad[a.k0] += a.w0 * tot[0];
         a.grad[a.k0 + 1] += a.w1 * tot[0];

@@ -84,7 +84,7 @@ struct ShellWalk {
             if (!live) return;
             double *p = a.part + 5 * (size_t)part_of(a.tile_base[cur], blockIdx.x, gridDim.x), tot[NS];
             if constexpr (NS == 5) sum[4].add((R)nf);
-            block_totals<NS>(sum, sums_flushed(nt), tot);
+            block_totals<NS>(sum, tot);
 #pragma unroll
             for (int k = 0; k < NS; ++k) {
                 if (threadIdx.x == 0) p[k] = tot[k];
@@ -112,13 +112,7 @@ struct ShellWalk {
         }
         return live;
     }
-    __device__ __forceinline__ void added()
-    {
-        if (++n % SUM_FLUSH == 0) {
-#pragma unroll
-            for (int k = 0; k < (NS == 5 ? 4 : NS); ++k) sum[k].flush();
-        }
-    }
+    __device__ __forceinline__ void added() { keep<(NS == 5 ? 4 : NS)>(sum, ++n); }
 };
 
 // the diagonal half step at the load, with the current shell's parameters

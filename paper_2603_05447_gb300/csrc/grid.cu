@@ -1144,9 +1144,8 @@ __device__ __forceinline__ uint32_t tf_top(double v)
     return a < 0x7ff00000u || (hi == 0xfff00000u && __double2loint(v) == 0) ? a : 0u;
 }
 
-// float pairs reach to 3e38, a thread's sum of SUM_FLUSH terms stays below it if
-// the terms do not exceed this; larger ones are added in FP64
-constexpr float TF_PAIR_MAX = 1e30f;
+// a thread's sum of SUM_FLUSH terms stays within a float pair if none exceeds
+// PAIR_MAX; larger ones are added in FP64
 __device__ __noinline__ double tf_add(double sum, float v) { return sum + (double)v; }
 __device__ __noinline__ double tf_add(double sum, double a, double b, unsigned sel)
 {
@@ -1160,7 +1159,7 @@ __device__ __forceinline__ void tf_add(Sum64<float> &s, const float (&v)[W], uns
 #pragma unroll
     for (int w = 0; w < W; ++w) {
         const float x = (sel >> w) & 1u ? v[w] : 0.0f;
-        if (fabsf(x) <= TF_PAIR_MAX) s.add(x);
+        if (fabsf(x) <= PAIR_MAX) s.add(x);
         else s.tot = tf_add(s.tot, x);
     }
 }

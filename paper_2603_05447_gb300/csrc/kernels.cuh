@@ -134,41 +134,44 @@ struct TileDiag {
     __device__ __forceinline__ void cell(CT &v, const R &e) const { v = d.apply(v, e); }
 };
 
-// may a thread have flushed over nt tiles?  (the blocks with the most take
-// ceil(nt / grid) of them)
-__device__ __forceinline__ bool sums_flushed(uint32_t nt) { return nt > (SUM_FLUSH - 1) * gridDim.x; }
-
 // The block's totals of NV sums, to every thread.  Few FP64 instructions, since
 // every warp of an SM queues for the one pipe at a kernel's end: pairs are
 // added across a warp as pairs, and one warp converts; doubles are added
-// across the block by a warp a sum.  flushed: threads may have flushed.
+// across the block by a warp a sum.  The threads' FP64 totals (flushed pairs) are
+// added only in blocks that have any.
 // Called by the whole block of TILE threads.
 template <int NV>
-__device__ __forceinline__ void block_totals(Sum64<float> (&s)[NV], bool flushed, double (&out)[NV])
+__device__ __forceinline__ void block_totals(Sum64<float> (&s)[NV], double (&out)[NV])
 {
     constexpr int W = TILE / 32;
     __shared__ float2 sp[NV][W];
     __shared__ double sd[NV][W], so[NV];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    bool own = false;
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
         for (int off = 16; off > 0; off >>= 1)
             s[k].add(__shfl_down_sync(0xffffffffu, s[k].hi, off), __shfl_down_sync(0xffffffffu, s[k].lo, off));
         if (lane == 0) sp[k][warp] = make_float2(s[k].hi, s[k].lo);
-        if (flushed) {
+        own |= __double_as_longlong(s[k].tot) != 0;
+    }
+    const bool any = __syncthreads_or(own);
+    if (any) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
             double x = s[k].tot;
             for (int off = 16; off > 0; off >>= 1) x += __shfl_down_sync(0xffffffffu, x, off);
             if (lane == 0) sd[k][warp] = x;
         }
+        __syncthreads();
     }
-    __syncthreads();
     if (threadIdx.x < NV) {
         double x = 0.0;
 #pragma unroll
         for (int w = 0; w < W; ++w) {
             const float2 p = sp[threadIdx.x][w];
             x = add_pair(x, p.x, p.y);
-            if (flushed) x += sd[threadIdx.x][w];
+            if (any) x += sd[threadIdx.x][w];
         }
         so[threadIdx.x] = x;
     }
@@ -178,7 +181,7 @@ __device__ __forceinline__ void block_totals(Sum64<float> (&s)[NV], bool flushed
     __syncthreads();  // the arrays may be used again
 }
 template <int NV>
-__device__ __forceinline__ void block_totals(Sum64<double> (&s)[NV], bool, double (&out)[NV])
+__device__ __forceinline__ void block_totals(Sum64<double> (&s)[NV], double (&out)[NV])
 {
     __shared__ double sm[NV][TILE], so[NV];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -223,7 +226,7 @@ __device__ __forceinline__ bool launch_totals(double (&v)[NV], double *partials,
 #pragma unroll
         for (int k = 0; k < NV; ++k) s[k].add((x[0][k] + x[1][k]) + (x[2][k] + x[3][k]));
     }
-    block_totals<NV>(s, false, v);
+    block_totals<NV>(s, v);
     if (threadIdx.x == 0) *counter = 0u;
     return true;
 }
@@ -272,10 +275,10 @@ __global__ void GPE_TILE_BOUNDS(R, NP) k_itp_b(const ItpArgs<R, CT> a, const Til
                       }
                       st4(a.psi + idx, o);
                       norm[0].add(n4);
-                      if (++n % SUM_FLUSH == 0) norm[0].flush();
+                      keep<1>(norm, ++n);
                   });
     double tot[1];
-    block_totals<1>(norm, sums_flushed((uint32_t)T.ntiles), tot);
+    block_totals<1>(norm, tot);
     if (launch_totals<1>(tot, partials, counter) && threadIdx.x == 0) {
         const double nrm = tot[0] * a.dV;
         a.scalars[0] = sqrt(a.N / nrm);
@@ -385,14 +388,11 @@ __global__ void GPE_TILE_BOUNDS(R, NP) k_obs(const ObsArgs<R, CT> a, const TileV
                       obs_terms<BLEND>(p, a.s, a.g, c, L, t, nf);
 #pragma unroll
                       for (int k = 0; k < 4; ++k) sum[k].add(t[k]);
-                      if (++n % SUM_FLUSH == 0) {
-#pragma unroll
-                          for (int k = 0; k < 4; ++k) sum[k].flush();
-                      }
+                      keep<4>(sum, ++n);
                   });
     sum[4].add((R)nf);
     double tot[5];
-    block_totals<5>(sum, sums_flushed((uint32_t)T.ntiles), tot);
+    block_totals<5>(sum, tot);
     if (launch_totals<5>(tot, a.partials, a.counter) && threadIdx.x == 0) {
         gpe_obs o;
         o.norm = tot[0] * a.dV;

@@ -1036,11 +1036,17 @@ struct DiagLoad {
 // total every SUM_FLUSH terms.  After n additions the pair is good to about n
 // 2^-48 of the sum, against the 2^-25 of every term.  Double-precision terms
 // are added as they are.
+// A pair holds up to 3e38: one that has grown beyond PAIR_MAX (or is NaN) goes
+// into the FP64 total at once (keep), so that neither the next term nor a
+// warp's lanes (block_totals) can take it out of range.
+constexpr int SUM_FLUSH = 64;
+constexpr float PAIR_MAX = 1e30f;
 template <typename R>
 struct Sum64 {
     double tot = 0.0;
     __device__ __forceinline__ void add(double x) { tot += x; }
     __device__ __forceinline__ void flush() {}
+    __device__ __forceinline__ bool large() const { return false; }
 };
 // a call, so that the compiler branches around it: FP64 instructions that are
 // predicated off still take their turn in the pipe
@@ -1068,8 +1074,20 @@ struct Sum64<float> {
         hi = 0.0f;
         lo = 0.0f;
     }
+    __device__ __forceinline__ bool large() const { return !(fabsf(hi) <= PAIR_MAX); }
 };
-constexpr int SUM_FLUSH = 64;
+// after the n-th term of each of the first K of some sums: flushes them when due
+template <int K, typename R, int NV>
+__device__ __forceinline__ void keep(Sum64<R> (&s)[NV], int n)
+{
+    bool due = n % SUM_FLUSH == 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) due |= s[k].large();
+    if (due) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) s[k].flush();
+    }
+}
 
 // deterministic block sum (result valid in thread 0)
 __device__ __forceinline__ double block_sum(double x)
