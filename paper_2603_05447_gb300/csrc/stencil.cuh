@@ -358,10 +358,12 @@ __device__ __forceinline__ double i64_to_double(long long S)
     const long long r = (long long)(m + ((lo >> 10) & 1u));  // a carry moves the exponent on
     return S == 0 ? 0.0 : __longlong_as_double(r | (S & (long long)0x8000000000000000ull));
 }
-// S q 2^-64 for a signed S
+// S q 2^-64, cut towards zero: of opposite values the results are opposite, as
+// FP64's are (an odd state stays exactly odd)
 __device__ __forceinline__ long long mul_frac(long long S, unsigned long long q)
 {
-    return (long long)(__umul64hi((unsigned long long)S, q) - (S < 0 ? q : 0ull));
+    const long long sg = S >> 63;
+    return ((long long)__umul64hi((unsigned long long)((S ^ sg) - sg), q) ^ sg) - sg;
 }
 static __device__ __noinline__ double sum6_fp64(double xp, double xm, double yp, double ym, double zp, double zm,
                                                 double ax, double ay, double az)
