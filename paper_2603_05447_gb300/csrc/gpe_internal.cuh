@@ -257,6 +257,7 @@ struct gpe_grid {
     int32_t *d_tasks_w = nullptr;     // [2*n_chunks]
     int sched = -1;                   // GPE_SCHED_* used by the step calls
     int n_slots = 1;
+    unsigned long long v0_version = 0;  // how often slot 0 has been replaced: tables made from it hold the count
     double v_max = 0.0;
     int nsm = 0;
     int n_states = 0;
@@ -271,7 +272,8 @@ struct gpe_state {
     void *d_work[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};  // RK stage states / ITP tmp
     std::vector<void *> work_blocks;                                           // the allocations that hold them
     void *d_E = nullptr;    // ITP exp(-V dt/2), state precision
-    double E_dt = -1.0;     // dt that d_E was made for
+    double E_dt = -1.0;     // dt and
+    unsigned long long E_version = 0;  // potential (gpe_grid::v0_version) that d_E was made for
     double *d_clock = nullptr;  // device time base for ramps
     double *d_stab = nullptr;   // schedule values of the next steps' stages (ramps; made on first use)
     int stab_cap = 0;           // steps it holds

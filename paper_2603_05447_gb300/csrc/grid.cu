@@ -1043,6 +1043,7 @@ extern "C" int gpe_grid_set_potential(gpe_grid *g, int slot, const void *V, int 
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) rc = cuda_fail(e, "k_set_potential", __FILE__, __LINE__);
     }
+    if (rc == GPE_OK && slot == 0) ++g->v0_version;
     if (rc == GPE_OK && slot == 1) g->n_slots = 2;
     unsigned long long *vb = nullptr;
     if (rc == GPE_OK) rc = dev_alloc_t(&vb, 1);

@@ -410,15 +410,16 @@ __global__ void GPE_TILE_BOUNDS(R, NP) k_obs(const ObsArgs<R, CT> a, const TileV
 __global__ inline void k_set_one(double *p) { *p = 1.0; }
 
 // arguments of the imaginary-time passes of a state; makes the propagator
-// table if dt changed, and sets the pending factor to 1
+// table if dt or the potential changed, and sets the pending factor to 1
 template <typename R, typename CT>
 inline int itp_args(gpe_state *st, const gpe_imag_params *p, cudaStream_t s, ItpArgs<R, CT> &a)
 {
     const gpe_grid *g = st->grid;
-    if (st->E_dt != p->dt) {
+    if (st->E_dt != p->dt || st->E_version != g->v0_version) {
         k_make_E<R><<<g->nsm * 8, 256, 0, s>>>(g->d_V[0], (R *)st->d_E, g->n_packed, p->dt);
         GPE_LAUNCH_CHECK();
         st->E_dt = p->dt;
+        st->E_version = g->v0_version;
     }
     a = ItpArgs<R, CT>{};
     a.psi = (CT *)st->d_psi;
