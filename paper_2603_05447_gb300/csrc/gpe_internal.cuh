@@ -81,6 +81,9 @@ inline cudaStream_t S(gpe_stream s) { return reinterpret_cast<cudaStream_t>(s); 
 int shape_id(int bx, int by, int bz);  // 0: 8x8x8, 1: 8x8x4, 2: 8x4x4
 
 int sm_count(int device);
+// resident blocks an SM of a kernel with smem bytes of dynamic shared memory on
+// the current device; the kernel is allowed smem_max bytes there (occupancy.h)
+int blocks_per_sm(const void *kernel, int threads, size_t smem, size_t smem_max);
 
 // per-brick record of the packed layout (32 bytes)
 struct BrickRec {

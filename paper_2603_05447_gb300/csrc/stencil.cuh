@@ -974,21 +974,6 @@ __device__ __forceinline__ void brick_apply(WarpSpace<CT, BX, BY, BZ> &ws, const
     }
 }
 
-// one-time launch preparation of a stencil kernel: dynamic shared memory
-// beyond 48 KiB needs an opt-in; returns resident blocks per SM
-template <typename K>
-inline int prepare_kernel(K kernel, int threads, size_t smem)
-{
-    static_assert(sizeof(K) > 0, "");
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int per = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem) != cudaSuccess || per < 1) {
-        cudaGetLastError();
-        per = 1;
-    }
-    return per;
-}
-
 // ------------------------------------------------------------ ramp schedule
 struct Ramp {
     const double *clock;  // device time base

@@ -24,8 +24,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
-#include <mutex>
-#include <unordered_map>
 #include <vector>
 
 #include "gpe_internal.cuh"
@@ -54,23 +52,11 @@ int convert_to_float(const double *src, float *dst, int64_t n)
 __global__ void k_set_scalar(double *p, double v) { *p = v; }
 
 // ------------------------------------------------------------ launch helper
-static std::mutex g_occ_mu;
-static std::unordered_map<const void *, int> g_occ;
-
-// resident blocks per SM of a stencil kernel (prepared once: dynamic shared
-// memory opt-in and occupancy query)
+// resident blocks per SM of a stencil kernel
 template <typename K>
 static int per_sm_for(K kernel, int threads, size_t smem)
 {
-    {
-        std::lock_guard<std::mutex> lk(g_occ_mu);
-        auto it = g_occ.find((const void *)kernel);
-        if (it != g_occ.end()) return it->second;
-    }
-    const int per = prepare_kernel(kernel, threads, smem);
-    std::lock_guard<std::mutex> lk(g_occ_mu);
-    g_occ[(const void *)kernel] = per;
-    return per;
+    return blocks_per_sm((const void *)kernel, threads, smem, smem);
 }
 
 // a grid of resident blocks of nw warps, no more than one warp per brick

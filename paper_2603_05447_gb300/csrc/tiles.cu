@@ -9,9 +9,8 @@
 // cell is read, each by packed position, so that neighbouring lanes gather
 // neighbouring segments), are the halo list.
 #include <algorithm>
-#include <mutex>
-#include <unordered_map>
 
+#include "occupancy.h"
 #include "tiles.cuh"
 
 namespace gpe {
@@ -250,25 +249,30 @@ int tiles_build(gpe_grid *g, int *d_hmax, cudaStream_t st)
     return g->stencil == 19 ? build<19>(S, t, d_hmax, st) : build<7>(S, t, d_hmax, st);
 }
 
-int tile_per_sm(const void *kernel, size_t smem)
+int blocks_per_sm(const void *kernel, int threads, size_t smem, size_t smem_max)
 {
-    static std::mutex mu;
-    static std::unordered_map<const void *, std::unordered_map<size_t, int>> known;
-    std::lock_guard<std::mutex> lk(mu);
-    auto &of = known[kernel];
-    auto it = of.find(smem);
-    if (it != of.end()) return it->second;
-    if (of.empty()) {
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM_MAX);
+    static Occupancy known;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();
+        return 1;
     }
-    int per = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, TILE, smem) != cudaSuccess || per < 1) {
-        cudaGetLastError();
-        per = 1;
-    }
-    if (of.size() < 256) of[smem] = per;
-    return per;
+    return known.blocks(
+        dev, kernel, smem,
+        [&] {
+            const bool ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)smem_max) == cudaSuccess;
+            if (!ok) cudaGetLastError();
+            return ok;
+        },
+        [&] {
+            int per = 0;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem) != cudaSuccess) {
+                cudaGetLastError();
+                per = 0;
+            }
+            return per;
+        });
 }
 
 }  // namespace gpe

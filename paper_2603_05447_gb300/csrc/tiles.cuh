@@ -377,16 +377,13 @@ inline TileLaunch tile_launch(const TileTab &t)
             sizeof(typename M::U) * (size_t)(M::UPS * pstr)};
 }
 
-// resident blocks an SM of a tile kernel with smem bytes of shared memory;
-// the kernel may use as much as a block can have, so that grids of different
-// halo sizes can launch it from any thread
-int tile_per_sm(const void *kernel, size_t smem);
-// blocks of a launch over n tiles: one a tile, or with `loop` at most the
-// resident ones (kernels that reduce, or that loop over tiles)
+// blocks of a launch over n tiles: one a tile, at most the resident ones.  A
+// tile kernel may use as much shared memory as a block can have, so that grids
+// of different halo sizes can launch it from any thread.
 template <typename K>
 inline unsigned tile_blocks(K kernel, int nsm, int n, size_t smem)
 {
-    const int64_t res = (int64_t)nsm * tile_per_sm((const void *)kernel, smem);
+    const int64_t res = (int64_t)nsm * blocks_per_sm((const void *)kernel, TILE, smem, TILE_SMEM_MAX);
     return (unsigned)(res < n ? res : n);
 }
 
