@@ -362,8 +362,8 @@ __device__ __forceinline__ double i64_to_double(long long S)
 // FP64's are (an odd state stays exactly odd)
 __device__ __forceinline__ long long mul_frac(long long S, unsigned long long q)
 {
-    const long long sg = S >> 63;
-    return ((long long)__umul64hi((unsigned long long)((S ^ sg) - sg), q) ^ sg) - sg;
+    const long long m = (long long)__umul64hi((unsigned long long)llabs(S), q);
+    return S < 0 ? -m : m;
 }
 static __device__ __noinline__ double sum6_fp64(double xp, double xm, double yp, double ym, double zp, double zm,
                                                 double ax, double ay, double az)
@@ -403,9 +403,11 @@ __device__ __forceinline__ double sum6(double xp, double xm, double yp, double y
         }
         S[p] -= neg;
     }
-    if (k.qx) S[0] = mul_frac(S[0], k.qx);
-    if (k.qy) S[1] = mul_frac(S[1], k.qy);
-    if (k.qz) S[2] = mul_frac(S[2], k.qz);
+    if (k.qx | k.qy | k.qz) {  // one branch: three in a row were predicated (64^3 ground state 1.93 ms for 1.87)
+        if (k.qx) S[0] = mul_frac(S[0], k.qx);
+        if (k.qy) S[1] = mul_frac(S[1], k.qy);
+        if (k.qz) S[2] = mul_frac(S[2], k.qz);
+    }
     const double f = __hiloint2double(__double2hiint(k.ref) + ((em - 1082) << 20), __double2loint(k.ref));
     return i64_to_double(S[0] + S[1] + S[2]) * f;
 }
