@@ -301,7 +301,7 @@ struct SegmentSteps {
     // stage stg of step m of the segment, from f.y0
     int stage(int64_t m, int stg)
     {
-        const auto k = Rk4Tiles<R, 7>::get(true, stg);
+        const auto k = Rk4Tiles<R, 7>::get(true, stg, fixed_spacings(t->st->grid->box));
         f.stab = t->d_stab + 3 * m + (stg + 1) / 2;
         if (t->d_stages) {
             const size_t np = (size_t)t->st->grid->n_packed;

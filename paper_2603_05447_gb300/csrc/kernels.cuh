@@ -231,14 +231,15 @@ __device__ __forceinline__ bool launch_totals(double (&v)[NV], double *partials,
     return true;
 }
 
-template <typename R, typename CT, int NP>
+template <typename R, typename CT, int NP, bool FX = true>
 __global__ void GPE_TILE_BOUNDS(R, NP) k_itp_a(const ItpArgs<R, CT> a, const TileView T)
 {
     const R q4 = a.dt / (R)4;
-    const auto co = tile_co<NP, LapEuler>(euler_coef(a.ihx2, q4), euler_coef(a.ihy2, q4), euler_coef(a.ihz2, q4));  // before the wait
+    using LAP = LapIn<LapEuler, FX>;
+    const auto co = tile_co<NP, LAP>(euler_coef(a.ihx2, q4), euler_coef(a.ihy2, q4), euler_coef(a.ihz2, q4));  // before the wait
     const TileList list = tile_begin(T);
     const TileDiag<R, CT> diag{{(R)a.scalars[0], a.g * a.dt / (R)2, a.E}};
-    tile_loop<NP, LapEuler>(T, list, (const CT *)a.psi, diag, co, EveryTile(),
+    tile_loop<NP, LAP>(T, list, (const CT *)a.psi, diag, co, EveryTile(),
                   [&](uint32_t idx, uint32_t n) { prefetch_l2(a.E + idx, n * (uint32_t)sizeof(R)); }, ELoad<R>{a.E},
                   [&](uint32_t idx, const typename ELoad<R>::P &p, const CT(&c)[4], const CT(&L)[4]) {
                       CT o[4];
@@ -251,17 +252,18 @@ __global__ void GPE_TILE_BOUNDS(R, NP) k_itp_a(const ItpArgs<R, CT> a, const Til
                   });
 }
 
-template <typename R, typename CT, int NP>
+template <typename R, typename CT, int NP, bool FX = true>
 __global__ void GPE_TILE_BOUNDS(R, NP) k_itp_b(const ItpArgs<R, CT> a, const TileView T, double *partials,
                                            unsigned int *counter)
 {
     const R q4 = a.dt / (R)4;
-    const auto co = tile_co<NP, LapEuler>(euler_coef(a.ihx2, q4), euler_coef(a.ihy2, q4), euler_coef(a.ihz2, q4));  // before the wait
+    using LAP = LapIn<LapEuler, FX>;
+    const auto co = tile_co<NP, LAP>(euler_coef(a.ihx2, q4), euler_coef(a.ihy2, q4), euler_coef(a.ihz2, q4));  // before the wait
     const TileList list = tile_begin(T);
     const R hg = a.g * a.dt / (R)2;
     Sum64<R> norm[1];
     int n = 0;
-    tile_loop<NP, LapEuler>(T, list, (const CT *)a.tmp, Plain(), co, EveryTile(),
+    tile_loop<NP, LAP>(T, list, (const CT *)a.tmp, Plain(), co, EveryTile(),
                   [&](uint32_t idx, uint32_t n) { prefetch_l2(a.E + idx, n * (uint32_t)sizeof(R)); }, ELoad<R>{a.E},
                   [&](uint32_t idx, const typename ELoad<R>::P &p, const CT(&c)[4], const CT(&L)[4]) {
                       CT o[4];
@@ -444,8 +446,10 @@ inline int itp_steps(gpe_state *st, const ItpArgs<R, CT> &a, int64_t cnt, cudaSt
 {
     const gpe_grid *g = st->grid;
     const TileLaunch L = tile_launch<CT, NP>(g->tiles);
-    auto ka = k_itp_a<R, CT, NP>;
-    auto kb = k_itp_b<R, CT, NP>;
+    constexpr bool F = !two_forms<R, NP>();
+    const bool fixed = fixed_spacings(g->box);
+    auto ka = fixed ? k_itp_a<R, CT, NP> : k_itp_a<R, CT, NP, F>;
+    auto kb = fixed ? k_itp_b<R, CT, NP> : k_itp_b<R, CT, NP, F>;
     const unsigned na = tile_blocks(ka, g->nsm, L.T.ntiles, L.smem), nb = tile_blocks(kb, g->nsm, L.T.ntiles, L.smem);
     for (int64_t n = 0; n < cnt; ++n) {
         GPE_TRY(tile_run(ka, na, L, s, a, L.T));
@@ -543,8 +547,9 @@ inline int rk4_steps(gpe_state *st, RkArgs<R> a, bool blend, int64_t cnt, bool a
     const gpe_grid *g = st->grid;
     using RT = Rk4Tiles<R, NP>;
     const TileLaunch L = tile_launch<typename Cx<R>::T, NP>(g->tiles);
+    const bool fixed = fixed_spacings(g->box);
     unsigned grid[4];
-    for (int stg = 0; stg < 4; ++stg) grid[stg] = tile_blocks(RT::get(blend, stg), g->nsm, L.T.ntiles, L.smem);
+    for (int stg = 0; stg < 4; ++stg) grid[stg] = tile_blocks(RT::get(blend, stg, fixed), g->nsm, L.T.ntiles, L.smem);
     for (int64_t n = 0; n < cnt; ++n) {
         const int m = blend ? (int)(n % st->stab_cap) : 0;
         if (blend && m == 0) {
@@ -556,7 +561,7 @@ inline int rk4_steps(gpe_state *st, RkArgs<R> a, bool blend, int64_t cnt, bool a
         }
         for (int stg = 0; stg < 4; ++stg) {
             a.stab = st->d_stab + 3 * m + (stg + 1) / 2;  // t, t + dt/2 twice, t + dt
-            GPE_TRY(tile_run(RT::get(blend, stg), grid[stg], L, s, a, L.T));
+            GPE_TRY(tile_run(RT::get(blend, stg, fixed), grid[stg], L, s, a, L.T));
         }
     }
     return GPE_OK;

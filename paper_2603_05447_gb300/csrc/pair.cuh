@@ -262,12 +262,7 @@ __device__ __forceinline__ void pair_lap_u(const PairSpace<CT, BX, BY, BZ> &ps, 
     const int h = PS::row(y, z);
     const CT xm = hx == 0 ? ps.uxl[h][1] : ps.ucell(s - 1, 3);
     const CT xp = hx == PS::SX - 1 ? ps.uxr[h][0] : ps.ucell(s + 1, 0);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const CT l = i == 0 ? xm : c[i - 1];
-        const CT rr = i == 3 ? xp : c[i + 1];
-        L[i] = lap_of<LAP, true>(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], co);
-    }
+    lap4<LAP, true, true>(xm, xp, ym, yp, zm, zp, c, co, L);
 }
 
 // The same on the v tile (the brick's own slots only)
@@ -286,12 +281,7 @@ __device__ __forceinline__ void pair_lap_v(const PairSpace<CT, BX, BY, BZ> &ps, 
     const int h = PS::vrow(y, z);
     const CT xm = hx == 0 ? ps.vxl[h] : ps.vcell(s - 1, 3);
     const CT xp = hx == PS::SX - 1 ? ps.vxr[h] : ps.vcell(s + 1, 0);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const CT l = i == 0 ? xm : c[i - 1];
-        const CT rr = i == 3 ? xp : c[i + 1];
-        L[i] = lap_of<LAP, true>(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], co);
-    }
+    lap4<LAP, true, true>(xm, xp, ym, yp, zm, zp, c, co, L);
 }
 
 // Two RK4 stages of one brick.  PASS 0: stages 0 and 1 (u = y0); PASS 1:

@@ -308,6 +308,7 @@ struct LapCo<double> {
     double ref;                     // the largest coefficient
     unsigned long long qx, qy, qz;  // 2^64 a / ref; 0: a = ref
     int lo, hi;                     // exponents (of the largest value) that fixed point serves
+    __device__ __forceinline__ bool fixed() const { return lo <= hi; }
 };
 template <typename LAP>
 __device__ __forceinline__ LapCo<float> lap_co(float ihx2, float ihy2, float ihz2)
@@ -317,11 +318,12 @@ __device__ __forceinline__ LapCo<float> lap_co(float ihx2, float ihy2, float ihz
 template <typename LAP>
 __device__ __forceinline__ LapCo<double> lap_co(double ihx2, double ihy2, double ihz2)
 {
-    LapCo<double> k;
+    LapCo<double> k{};
     k.ax = LAP::coef(ihx2);
     k.ay = LAP::coef(ihy2);
     k.az = LAP::coef(ihz2);
     k.c6 = 2.0 * (ihx2 + ihy2 + ihz2);
+    if constexpr (!LAP::FIXED) return k;
     k.ref = k.ax;
     k.qx = k.qy = k.qz = 0;
     bool usual = true;
@@ -413,6 +415,7 @@ __device__ __forceinline__ double sum6(double xp, double xm, double yp, double y
 }
 
 struct LapFull {
+    static constexpr bool FIXED = true;  // double precision: sums in fixed point where the spacings allow
     template <typename R>
     __device__ __forceinline__ static R coef(R a)
     {
@@ -427,6 +430,7 @@ struct LapFull {
     __device__ __forceinline__ static double with(double c, double s, double c6) { return __fma_rn(-c6, c, s); }
 };
 struct LapRhs {
+    static constexpr bool FIXED = true;
     __device__ __forceinline__ static float coef(float a) { return a; }
     __device__ __forceinline__ static double coef(double a) { return -0.5 * a; }
     __device__ __forceinline__ static float2 of(const float2 &xp, const float2 &xm, const float2 &yp, const float2 &ym,
@@ -461,6 +465,13 @@ struct LapRhs {
 struct LapEuler : LapFull {
     __device__ __forceinline__ static double with(double c, double s, double c6) { return c + __fma_rn(-c6, c, s); }
 };
+// LAP with the sums in FP64, for grids whose spacings fixed point does not serve
+template <typename LAP>
+struct InFp64 : LAP {
+    static constexpr bool FIXED = false;
+};
+template <typename LAP, bool FX>
+using LapIn = typename std::conditional<FX, LAP, InFp64<LAP>>::type;
 // LAP's result from the sum of a cell's neighbours (double precision)
 template <typename LAP>
 __device__ __forceinline__ double with_centre(double c, double s, double c6)
@@ -475,7 +486,7 @@ __device__ __forceinline__ double2 with_centre(const double2 &c, const double2 &
 // sum6 as a call, for the kernels that hold several stages' code: inline, its eight
 // copies a stage no longer fit the instruction cache and the registers
 // (120-cell shell, WAVE schedule, eight RK4 steps: 6.8 ms inline, 3.9 so, 3.85
-// in FP64)
+// in FP64).
 static __device__ __noinline__ double sum6_call(double xp, double xm, double yp, double ym, double zp, double zm,
                                                 const LapCo<double> *k)
 {
@@ -489,6 +500,8 @@ __device__ __forceinline__ CT lap_of(const CT &xp, const CT &xm, const CT &yp, c
 {
     if constexpr (sizeof(R) == 4) {
         return LAP::of(xp, xm, yp, ym, zp, zm, c, k.ax, k.ay, k.az, k.c6);
+    } else if constexpr (!LAP::FIXED) {
+        return with_centre<LAP>(c, LapRhs::of(xp, xm, yp, ym, zp, zm, c, k.ax, k.ay, k.az, k.c6), k.c6);
     } else {
         auto sum = [&](double a, double b, double e, double f, double g, double h) {
             return CALL ? sum6_call(a, b, e, f, g, h, &k) : sum6(a, b, e, f, g, h, k);
@@ -498,6 +511,40 @@ __device__ __forceinline__ CT lap_of(const CT &xp, const CT &xm, const CT &yp, c
         else
             return with_centre<LAP>(c, sum(xp, xm, yp, ym, zp, zm), k.c6);
     }
+}
+// not 0 unless v is 0 (or -0: bit 63)
+__device__ __forceinline__ long long bits_of(double v) { return __double_as_longlong(v); }
+__device__ __forceinline__ long long bits_of(const double2 &v) { return __double_as_longlong(v.x) | __double_as_longlong(v.y); }
+// The same of a segment's four cells c: xm and xp its end cells' neighbours.
+// ASK: whether fixed point serves the spacings is asked here, once, and not by
+// every sum.  Fused pairs, complex128, 64 x 64 x 21 trap with spacings 1 : 1 : 3,
+// four RK4 steps: 287 -> 238 us (the wavefront kernels, which spill registers,
+// lost 3 % on equal spacings and go on asking at every sum).
+template <typename LAP, bool CALL = false, bool ASK = false, typename CT, typename R>
+__device__ __forceinline__ void lap4(const CT &xm, const CT &xp, const CT (&ym)[4], const CT (&yp)[4], const CT (&zm)[4],
+                                     const CT (&zp)[4], const CT (&c)[4], const LapCo<R> &k, CT (&L)[4])
+{
+    auto each = [&](auto lap) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            L[i] = lap_of<decltype(lap), CALL>(i == 3 ? xp : c[i + 1], i == 0 ? xm : c[i - 1], yp[i], ym[i], zp[i], zm[i], c[i], k);
+    };
+    if constexpr (ASK && sizeof(R) == 8) {
+        if (!k.fixed()) return each(InFp64<LAP>{});
+    }
+    if constexpr (sizeof(R) == 8 && !LAP::FIXED) {
+        // no FP64 instructions where the state is zero (a ramp's shell before the
+        // core has reached it): 100-cell ramp, spacings 1 : 1 : 3, 918 -> 589 us
+        long long any = bits_of(xm) | bits_of(xp);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) any |= bits_of(c[i]) | bits_of(ym[i]) | bits_of(yp[i]) | bits_of(zm[i]) | bits_of(zp[i]);
+        if ((any << 1) == 0) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) L[i] = czero<CT>();
+            return;
+        }
+    }
+    each(LAP{});
 }
 __device__ __forceinline__ float euler_coef(float ih2, float) { return ih2; }
 __device__ __forceinline__ double euler_coef(double ih2, double q) { return ih2 * q; }
@@ -958,12 +1005,7 @@ __device__ __forceinline__ void brick_apply(WarpSpace<CT, BX, BY, BZ> &ws, const
         ws.get(sl + W::PLANE, zp);
         const CT xm = hx == 0 ? ws.xm_cell(hrow) : ws.last(sl - 1);
         const CT xp = hx == S::SX - 1 ? ws.xp_cell(hrow) : ws.first(sl + 1);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const CT l = i == 0 ? xm : c[i - 1];
-            const CT rr = i == 3 ? xp : c[i + 1];
-            L[i] = lap_of<LAP, true>(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], co);
-        }
+        lap4<LAP, true>(xm, xp, ym, yp, zm, zp, c, co, L);
         body(R0.off + 4u * (uint32_t)r, pre, c, L);
     };
     // each iteration loads the operands of the next before computing its own

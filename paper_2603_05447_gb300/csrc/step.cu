@@ -965,7 +965,7 @@ struct RkGenArgs {
 // registers, so fewer blocks share an SM.  512^3 shell, complex64, RKCK: 0.47 ->
 // 0.32 ms a step; stages 35 to 72 us, 4.4 to 6.7 TB/s, the shared-memory pipe
 // 86 % busy with no extra term and DRAM the bound with five.
-template <typename R, bool BLEND, int NS>
+template <typename R, bool BLEND, int NS, bool FX = true>
 __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? (NS < 3 ? 6 : 5) : (NS < 3 ? 3 : 2))
     k_rk_stage(const RkGenArgs<R> a, const TileView T)
 {
@@ -974,11 +974,12 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? (NS < 3 ? 6 : 5) : (NS 
         R V0[4], V1[BLEND ? 4 : 1];
         CT y[NS > 0 ? NS : 1][4];
     };
-    const auto co = tile_co<7, LapRhs>(a.ihx2, a.ihy2, a.ihz2);  // before the wait
+    using LAP = LapIn<LapRhs, FX>;
+    const auto co = tile_co<7, LAP>(a.ihx2, a.ihy2, a.ihz2);  // before the wait
     const TileList list = tile_begin(T);
     const R s = BLEND ? (R)__ldcg(a.stab) : (R)0;
     constexpr R HALF = sizeof(R) == 8 ? (R)1 : (R)(-0.5);  // LapRhs leaves the factor in in single precision
-    tile_loop<7, LapRhs>(T, list, (const CT *)a.y[a.tile], Plain(), co, EveryTile(),
+    tile_loop<7, LAP>(T, list, (const CT *)a.y[a.tile], Plain(), co, EveryTile(),
                  [&](uint32_t idx, uint32_t n) {
                      prefetch_l2(a.V0 + idx, n * (uint32_t)sizeof(R));
                      if constexpr (BLEND) prefetch_l2(a.V1 + idx, n * (uint32_t)sizeof(R));
@@ -1016,12 +1017,20 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? (NS < 3 ? 6 : 5) : (NS 
 
 template <typename R>
 using RkStageKernel = void (*)(RkGenArgs<R>, TileView);
-template <typename R, bool BLEND>
+template <typename R, bool BLEND, bool FX>
 static RkStageKernel<R> rk_stage_kernel(int ns)
 {
-    static const RkStageKernel<R> k[6] = {k_rk_stage<R, BLEND, 0>, k_rk_stage<R, BLEND, 1>, k_rk_stage<R, BLEND, 2>,
-                                          k_rk_stage<R, BLEND, 3>, k_rk_stage<R, BLEND, 4>, k_rk_stage<R, BLEND, 5>};
+    static const RkStageKernel<R> k[6] = {k_rk_stage<R, BLEND, 0, FX>, k_rk_stage<R, BLEND, 1, FX>,
+                                          k_rk_stage<R, BLEND, 2, FX>, k_rk_stage<R, BLEND, 3, FX>,
+                                          k_rk_stage<R, BLEND, 4, FX>, k_rk_stage<R, BLEND, 5, FX>};
     return k[ns];
+}
+template <typename R>
+static RkStageKernel<R> rk_stage_kernel(int ns, bool blend, bool fixed)
+{
+    constexpr bool F = !two_forms<R, 7>();
+    if (fixed) return blend ? rk_stage_kernel<R, true, true>(ns) : rk_stage_kernel<R, false, true>(ns);
+    return blend ? rk_stage_kernel<R, true, F>(ns) : rk_stage_kernel<R, false, F>(ns);
 }
 
 template <typename R>
@@ -1054,6 +1063,7 @@ static int rkgen_run(gpe_state *st, const gpe_real_params *p, int64_t nsteps, do
         GPE_LAUNCH_CHECK();
     }
     const TileLaunch L = tile_launch<CT, 7>(g->tiles);
+    const bool fixed = fixed_spacings(g->box);
     for (int64_t n = 0; n < nsteps; ++n) {
         const int m = blend ? (int)(n % st->stab_cap) : 0;
         if (blend && m == 0) {
@@ -1076,7 +1086,7 @@ static int rkgen_run(gpe_state *st, const gpe_real_params *p, int64_t nsteps, do
                     a.coef[a.nsrc] = (R)row[j];
                     ++a.nsrc;
                 }
-            const auto k = blend ? rk_stage_kernel<R, true>(a.nsrc) : rk_stage_kernel<R, false>(a.nsrc);
+            const auto k = rk_stage_kernel<R>(a.nsrc, blend, fixed);
             GPE_TRY(tile_run(k, tile_blocks(k, g->nsm, L.T.ntiles, L.smem), L, s, a, L.T));
         }
     }

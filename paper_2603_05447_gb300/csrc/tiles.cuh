@@ -19,6 +19,8 @@
 // pass, against 5.3 for the brick records, on 80 to 144 of data.
 #pragma once
 
+#include <algorithm>
+
 #include "stencil.cuh"
 
 namespace gpe {
@@ -149,12 +151,7 @@ __device__ __forceinline__ void tile_laplacian(const TileMem<CT, NP> &m, const T
     m.get(f(3), zp);
     const CT xm = *m.last(f(4)), xp = *m.first(f(5));
     if constexpr (NP != 19) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const CT l = i == 0 ? xm : c[i - 1];
-            const CT rr = i == 3 ? xp : c[i + 1];
-            L[i] = lap_of<LAP>(rr, l, yp[i], ym[i], zp[i], zm[i], c[i], co.k);
-        }
+        lap4<LAP>(xm, xp, ym, yp, zm, zp, c, co.k, L);
     } else {
         // App. B: the 7-point part plus w_ab (edges_ab - 2 faces_ab + 4 c) per
         // plane ab, w_ab = (1/h_a^2 + 1/h_b^2) / 12.  Each face pair lies in
@@ -403,15 +400,16 @@ constexpr int tile_blocks_f(int np) { return np == 19 ? 5 : 6; }
 // (85 registers): 0.626 ms, seven 0.634, eight with spills 0.645; double, three
 // blocks (168 registers) are 1.5 % ahead of two; blended two, which three lose 1 % to.
 // One block a tile instead of looping blocks: 8 % slower (no tile ahead to prefetch).
-template <typename R, bool BLEND, int ST, int NP>
+template <typename R, bool BLEND, int ST, int NP, bool FX = true>
 __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? tile_blocks_f(NP) : (BLEND || NP == 19 ? 2 : 3)) k_rk4_tile(const RkArgs<R> a, const TileView T)
 {
     using CT = typename Cx<R>::T;
     using B = Rk4Body<R, BLEND, false, ST>;
-    const auto co = tile_co<NP, LapRhs>(a.ihx2, a.ihy2, a.ihz2);  // before the wait
+    using LAP = LapIn<LapRhs, FX>;
+    const auto co = tile_co<NP, LAP>(a.ihx2, a.ihy2, a.ihz2);  // before the wait
     const TileList list = tile_begin(T);
     const B body(a, BLEND ? (R)__ldcg(a.stab) : (R)0);
-    tile_loop<NP, LapRhs>(T, list, body.yin(), Plain(), co, EveryTile(),
+    tile_loop<NP, LAP>(T, list, body.yin(), Plain(), co, EveryTile(),
                   [&](uint32_t idx, uint32_t n) {
                       prefetch_l2(a.V0 + idx, n * (uint32_t)sizeof(R));
                       if constexpr (BLEND) prefetch_l2(a.V1 + idx, n * (uint32_t)sizeof(R));
@@ -447,17 +445,41 @@ inline int tile_run(void (*k)(KArgs...), unsigned grid, const TileLaunch &L, cud
     return GPE_OK;
 }
 
+// Does fixed point serve a grid's sums?  (lap_co's rule for the spacings' ratio.)
+// If not, the double-precision 7-point passes of single states take the FP64
+// form as an instance of their own.  Eight steps of a 96 x 96 x 32 trap with
+// spacings 1 : 1 : 3, complex128: RK4 804 us with sums that look at their values
+// before they turn to it, 652 so; imaginary time 484 and 414.  Both forms behind a
+// branch in one kernel: equal spacings 1 to 7 % slower (registers).
+inline bool fixed_spacings(const gpe_box &b)
+{
+    const double x = 1.0 / (b.hx * b.hx), y = 1.0 / (b.hy * b.hy), z = 1.0 / (b.hz * b.hz);
+    const double inv = 1.0 / std::max(x, std::max(y, z));
+    return x * inv >= 0.125 && y * inv >= 0.125 && z * inv >= 0.125;
+}
+// are there two instances of a kernel?
+template <typename R, int NP>
+constexpr bool two_forms()
+{
+    return sizeof(R) == 8 && NP == 7;
+}
+
 // the four stage kernels, static (blend false) or blended
 template <typename R, int NP>
 struct Rk4Tiles {
     using K = void (*)(RkArgs<R>, TileView);
-    static K get(bool blend, int st)
+    static K get(bool blend, int st, bool fixed)
     {
-        static const K t[2][4] = {{k_rk4_tile<R, false, 0, NP>, k_rk4_tile<R, false, 1, NP>,
-                                   k_rk4_tile<R, false, 2, NP>, k_rk4_tile<R, false, 3, NP>},
-                                  {k_rk4_tile<R, true, 0, NP>, k_rk4_tile<R, true, 1, NP>,
-                                   k_rk4_tile<R, true, 2, NP>, k_rk4_tile<R, true, 3, NP>}};
-        return t[blend ? 1 : 0][st];
+        constexpr bool F = !two_forms<R, NP>();
+        static const K t[2][2][4] = {{{k_rk4_tile<R, false, 0, NP, F>, k_rk4_tile<R, false, 1, NP, F>,
+                                       k_rk4_tile<R, false, 2, NP, F>, k_rk4_tile<R, false, 3, NP, F>},
+                                      {k_rk4_tile<R, true, 0, NP, F>, k_rk4_tile<R, true, 1, NP, F>,
+                                       k_rk4_tile<R, true, 2, NP, F>, k_rk4_tile<R, true, 3, NP, F>}},
+                                     {{k_rk4_tile<R, false, 0, NP>, k_rk4_tile<R, false, 1, NP>,
+                                       k_rk4_tile<R, false, 2, NP>, k_rk4_tile<R, false, 3, NP>},
+                                      {k_rk4_tile<R, true, 0, NP>, k_rk4_tile<R, true, 1, NP>,
+                                       k_rk4_tile<R, true, 2, NP>, k_rk4_tile<R, true, 3, NP>}}};
+        return t[fixed ? 1 : 0][blend ? 1 : 0][st];
     }
 };
 
