@@ -90,15 +90,22 @@ __device__ __forceinline__ void cell_values(const VSource &src, const BoxD &bx, 
 // [rmin, rmax] of the scaled radius, from which the smallest |rho - 1|
 // follows.  Evaluated in FP32 with wide margins: it only has to be
 // conservative, the per-cell FP64 test decides.  Where FP32 does not reach (a
-// bound that is not finite, semi-axes far from 1) the answer is yes.
+// bound that is not finite, semi-axes far from 1, a stiffness so small that
+// its bound and the cutoff lose bits) the answer is yes.
 __device__ __forceinline__ bool pot_may_select(const PotDesc &P, double cut, float xl, float xh, float yl, float yh,
                                                float zl, float zh)
 {
     auto sqmin = [](float l, float h) { return (l <= 0.f && h >= 0.f) ? 0.f : fminf(l * l, h * h); };
     auto sqmax = [](float l, float h) { return fmaxf(l * l, h * h); };
     if (P.kind == GPE_POT_HARMONIC) {
-        const float wx = (float)P.p[0], wy = (float)P.p[1], wz = (float)P.p[2];
-        const float vmin = 0.5f * (wx * wx * sqmin(xl, xh) + wy * wy * sqmin(yl, yh) + wz * wz * sqmin(zl, zh));
+        // |w| times the least |coordinate|, squared as a product, since either
+        // square may underflow; factors without their full bits count as 0
+        auto least = [](double w, float l, float h) {
+            const float a = fabsf((float)w), d = (l <= 0.f && h >= 0.f) ? 0.f : fminf(fabsf(l), fabsf(h));
+            return a < 1e-37f || d < 1e-37f ? 0.f : a * d;
+        };
+        const float tx = least(P.p[0], xl, xh), ty = least(P.p[1], yl, yh), tz = least(P.p[2], zl, zh);
+        const float vmin = 0.5f * (tx * tx + ty * ty + tz * tz);
         return !(vmin > (float)cut * 1.0001f + 1e-30f) || !(vmin < INFINITY);
     }
     if (P.kind == GPE_POT_ELLIPSOID_SHELL) {
@@ -106,7 +113,7 @@ __device__ __forceinline__ bool pot_may_select(const PotDesc &P, double cut, flo
         const float ia = 1.f / (float)(P.p[1] * P.p[1]), ib = 1.f / (float)(P.p[2] * P.p[2]),
                     ic = 1.f / (float)(P.p[3] * P.p[3]);
         const float least = fminf(ia, fminf(ib, ic)), most = fmaxf(ia, fmaxf(ib, ic));
-        if (!(least > 1e-30f && most < 1e30f)) return true;
+        if (!(least > 1e-30f && most < 1e30f && fabsf(w) >= 1e-15f)) return true;
         const float rmin = sqrtf(sqmin(xl, xh) * ia + sqmin(yl, yh) * ib + sqmin(zl, zh) * ic);
         const float rmax = sqrtf(sqmax(xl, xh) * ia + sqmax(yl, yh) * ib + sqmax(zl, zh) * ic);
         const float d = (rmin <= 1.f && rmax >= 1.f) ? 0.f : fminf(fabsf(rmin - 1.f), fabsf(rmax - 1.f));
