@@ -107,9 +107,6 @@ struct BrickGeo {
 };
 inline BrickGeo brick_geo(int by, int bz) { return BrickGeo{by == 8 ? 3 : 2, bz == 8 ? 3 : 2}; }
 
-// per brick: its record followed by its six face neighbours' (-x +x -y +y -z
-// +z; empty records for absent neighbours), built on the host
-void build_rec7(const std::vector<BrickRec> &rec, const std::vector<int32_t> &nbr, std::vector<BrickRec> &out);
 // packed index of the first cell of segment q, if stored
 __host__ __device__ __forceinline__ bool seg_index(const BrickRec &r, int q, uint32_t &idx)
 {

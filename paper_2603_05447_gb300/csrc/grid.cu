@@ -602,18 +602,19 @@ __global__ void k_vmax(int64_t np, const double *V0, const double *V1, unsigned 
     if ((threadIdx.x & 31) == 0) atomicMax(vmax_bits, (unsigned long long)__double_as_longlong(vm));
 }
 
-}  // namespace gpe
-
-void gpe::build_rec7(const std::vector<BrickRec> &rec, const std::vector<int32_t> &nbr, std::vector<BrickRec> &out)
+// per brick: its record followed by its six face neighbours' (-x +x -y +y -z
+// +z; empty records for absent neighbours), a thread a record.  The wavefront
+// grids' rows used to be made on the host: 256^3 shell grid 1.40 -> 1.22 ms.
+__global__ void k_rec7(int64_t nb, const BrickRec *rec, const int32_t *nbr, BrickRec *out)
 {
-    const size_t nb = rec.size();
-    out.assign(nb * 7, BrickRec{});
-    for (size_t b = 0; b < nb; ++b) {
-        out[7 * b] = rec[b];
-        for (int d = 0; d < 6; ++d)
-            if (nbr[6 * b + d] >= 0) out[7 * b + 1 + d] = rec[nbr[6 * b + d]];
-    }
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, b = i / 7;
+    if (b >= nb) return;
+    const int d = (int)(i - 7 * b);
+    const int64_t from = d == 0 ? b : nbr[6 * b + d - 1];
+    out[i] = from >= 0 ? rec[from] : BrickRec{};
 }
+
+}  // namespace gpe
 
 namespace gpe {
 
@@ -860,15 +861,9 @@ static int build_grid(const gpe_box *box, const VSource &src, const gpe_grid_opt
     g->n_packed = 4 * ht.segs;
     if (o.sched == GPE_SCHED_WAVE || o.sched == GPE_SCHED_WAVE2) {
         // the wavefront kernels' record rows
-        std::vector<BrickRec> hrec(total), h7;
-        std::vector<int32_t> hnbr(total * 6);
-        BUILD_CUDA(cudaMemcpyAsync(hrec.data(), g->d_rec, total * sizeof(BrickRec), cudaMemcpyDeviceToHost, st));
-        BUILD_CUDA(cudaMemcpyAsync(hnbr.data(), g->d_nbr, total * 6 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        BUILD_CUDA(cudaStreamSynchronize(st));
-        build_rec7(hrec, hnbr, h7);
         BUILD_TRY(dev_alloc_t(&g->d_rec7, total * 7));
-        BUILD_CUDA(cudaMemcpyAsync(g->d_rec7, h7.data(), h7.size() * sizeof(BrickRec), cudaMemcpyHostToDevice, st));
-        BUILD_CUDA(cudaStreamSynchronize(st));
+        k_rec7<<<(unsigned)((7 * total + 255) / 256), 256, 0, st>>>(total, g->d_rec, g->d_nbr, g->d_rec7);
+        BUILD_CUDA(cudaGetLastError());
     }
     const size_t np = (size_t)g->n_packed;
     BUILD_TRY(alloc_own({{&g->d_V[0], np},
