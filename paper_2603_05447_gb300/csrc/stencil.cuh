@@ -295,13 +295,21 @@ struct LapCo {
 // the integer pipes stood idle.  The six values become 64-bit fixed point with the
 // largest one's exponent, 59 bits below its leading one, and add without
 // rounding; the coefficients are ref q, q a 64-bit fraction, so that one
-// multiplication by ref remains.  Nothing is lost against FP64 additions: a
-// value is cut at 2^-59 of the largest, an FP64 sum is rounded at 2^-53 of itself,
-// and with q >= 1/8 a sum is never smaller than its cuts make noise.  Spacings more
-// unequal than that, values that are not finite and values far outside any
-// state's range take the FP64 form.  A q of 1 skips its multiplication.
-// RK4 step in complex128: 1024^3 shell 5.44 -> 4.45 ms, 96^3 trap 0.170 -> 0.138;
-// with unequal spacings 0.917 -> 0.764 (200-cell shell).  As a call instead of inline: no gain.
+// multiplication by ref remains.  The error is absolute: each of the six cuts (and
+// of the products with q) loses less than 2^-59 of the largest neighbour, so a sum
+// is good to 9 2^-59 of that times ref, and to a few 2^-53 of itself.  FP64
+// additions round at 2^-53 of the sums they meet, 64 times as much for neighbours
+// of one sign; but where opposite neighbours cancel exactly they would keep
+// smaller ones whole, of which nothing is left here below 2^-59 of the largest.
+// With q >= 1/8 the largest neighbour's own share of the sum is at least 2^-3 of
+// it, so its cut stays below an FP64 rounding of that share; spacings more unequal
+// than that, values that are not finite and values far outside any state's
+// range take the FP64 form.  Errors against extended precision (80 bits), FP64
+// sums and these: 40 RK4 steps of the 64^3 trap 6.75e-16 and 6.0e-16 (spacings
+// 1 : 1.05 : 0.97: 6.9e-16 and 6.0e-16), 50 imaginary-time steps 1.454e-15 and
+// 1.458e-15, where seeds differ by 2 %.
+// RK4 step in complex128, FP64 sums and these: 1024^3 shell 5.44 -> 4.23 ms, 96^3
+// trap 0.170 -> 0.137; with unequal spacings 0.917 -> 0.764 (200-cell shell).
 template <>
 struct LapCo<double> {
     double ax, ay, az, c6;
