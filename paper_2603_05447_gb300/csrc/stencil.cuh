@@ -1183,17 +1183,6 @@ __device__ __forceinline__ R stage_s(const RkArgs<R> &a, int st)
     return (R)ramp_s(a.ramp, *a.ramp.clock + a.t_off + c * a.dtd);
 }
 
-// x / 3, correctly rounded, without a division: q = RN(x * RN(1/3)) is within
-// one ulp of x/3, the residual r = x - 3q is exact with a fused multiply-add,
-// and RN(q + r * RN(1/3)) is the correctly rounded quotient (Markstein's
-// theorem on division with a fused multiply-add; Muller et al., Handbook of
-// Floating-Point Arithmetic, the section on Newton-Raphson-based division).
-__device__ __forceinline__ float div3(float x)
-{
-    constexpr float t = 1.0f / 3.0f;
-    const float q = __fmul_rn(x, t);
-    return __fmaf_rn(__fmaf_rn(-3.0f, q, x), t, q);
-}
 // One RK4 stage (st = 0..3): operand loads and the per-segment update.  The
 // stage is a template argument so that each stage keeps only its own
 // prefetched operands in registers.
@@ -1250,10 +1239,16 @@ struct Rk4Body {
                     o[i] = fma2(kk, hs, p.y[i]);
                     if constexpr (st == 1) wv[i] = fma2(dup2(2.0f), o[i], sub2(c[i], p.y[i]));
                 } else {
+                    // x / 3, correctly rounded, without a division: q = RN(x RN(1/3)) is
+                    // within one ulp of x/3, the residual x - 3q is exact with a fused
+                    // multiply-add, and RN(q + (x - 3q) RN(1/3)) is the correctly rounded
+                    // quotient (Markstein's theorem on division with a fused
+                    // multiply-add; Muller et al., Handbook of Floating-Point
+                    // Arithmetic, the section on Newton-Raphson-based division)
                     const float2 x = add2(p.y[i], c[i]);
                     const float2 t3 = dup2(1.0f / 3.0f);
                     const float2 q = mul2(x, t3);
-                    o[i] = fma2(kk, hs, fma2(fma2(dup2(-3.0f), q, x), t3, q));  // div3 of both parts
+                    o[i] = fma2(kk, hs, fma2(fma2(dup2(-3.0f), q, x), t3, q));
                 }
             }
             return;
@@ -1279,8 +1274,8 @@ struct Rk4Body {
                 }
             } else {
                 // x/3 + k f with the third in two parts: T + TL is 1/3 to 2^-108,
-                // so the sum is rounded once (a third rounded to T alone would
-                // shrink every step by 2^-54)
+                // so the sum is rounded once, and x/3 alone correctly (a third
+                // rounded to T alone would shrink every step by 2^-54)
                 constexpr double T = 1.0 / 3.0, TL = 1.850371707708594e-17;
                 const R xr = p.y[i].x + c[i].x, xi = p.y[i].y + c[i].y;
                 o[i].x = __fma_rn(T, xr, __fma_rn(k, hi, TL * xr));
