@@ -98,15 +98,6 @@ int red_zero(const RedScratch &r)
     return dev_zero(r.scalars, 16 * sizeof(double));
 }
 
-int launch_blocks(const gpe_grid *g, int threads, int per_sm)
-{
-    (void)threads;
-    int64_t want = (int64_t)g->nsm * per_sm;
-    if (want > g->nb) want = g->nb;
-    if (want < 1) want = 1;
-    return (int)want;
-}
-
 }  // namespace gpe
 
 extern "C" int gpe_version(void) { return 100; }

@@ -305,5 +305,4 @@ int itp_run19(gpe_state *st, const gpe_imag_params *p, int64_t nsteps, cudaStrea
 int obs_run19(const gpe_state *st, double g, double s_blend, cudaStream_t s);
 int ensure_vf(gpe_grid *g, int slot);           // float copy of a potential slot
 const void *potential_ptr(gpe_state *st, int slot);  // V slot in state precision
-int launch_blocks(const gpe_grid *g, int threads, int per_sm);
 }  // namespace gpe

@@ -564,43 +564,6 @@ __device__ __forceinline__ CT euler(const CT &c, R q, const CT &L)
     else return axpy(c, q, L);
 }
 
-__device__ __forceinline__ float2 shfl_up(float2 v, int d)
-{
-    v.x = __shfl_up_sync(0xffffffffu, v.x, d);
-    v.y = __shfl_up_sync(0xffffffffu, v.y, d);
-    return v;
-}
-__device__ __forceinline__ double2 shfl_up(double2 v, int d)
-{
-    v.x = __shfl_up_sync(0xffffffffu, v.x, d);
-    v.y = __shfl_up_sync(0xffffffffu, v.y, d);
-    return v;
-}
-__device__ __forceinline__ float2 shfl_down(float2 v, int d)
-{
-    v.x = __shfl_down_sync(0xffffffffu, v.x, d);
-    v.y = __shfl_down_sync(0xffffffffu, v.y, d);
-    return v;
-}
-__device__ __forceinline__ double2 shfl_down(double2 v, int d)
-{
-    v.x = __shfl_down_sync(0xffffffffu, v.x, d);
-    v.y = __shfl_down_sync(0xffffffffu, v.y, d);
-    return v;
-}
-__device__ __forceinline__ float2 shfl_xor(float2 v, int d)
-{
-    v.x = __shfl_xor_sync(0xffffffffu, v.x, d);
-    v.y = __shfl_xor_sync(0xffffffffu, v.y, d);
-    return v;
-}
-__device__ __forceinline__ double2 shfl_xor(double2 v, int d)
-{
-    v.x = __shfl_xor_sync(0xffffffffu, v.x, d);
-    v.y = __shfl_xor_sync(0xffffffffu, v.y, d);
-    return v;
-}
-
 // 4 consecutive complex values (one segment, 32-byte aligned) with 256-bit
 // accesses, so that each lane moves whole 32-byte sectors; CG: read through
 // L2 only (data written by other blocks of the same launch)
@@ -809,15 +772,6 @@ __device__ __forceinline__ WarpSpace<CT, BX, BY, BZ> &warp_space()
     __syncwarp();
 #endif
     return ws;
-}
-
-template <typename CT>
-__device__ __forceinline__ void put4(CT *t, const CT (&v)[4])
-{
-    t[0] = v[0];
-    t[1] = v[1];
-    t[2] = v[2];
-    t[3] = v[3];
 }
 
 // 16-byte asynchronous global -> shared copies (cp.async, L2 only): the tile

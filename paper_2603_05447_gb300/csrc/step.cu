@@ -59,22 +59,6 @@ static int per_sm_for(K kernel, int threads, size_t smem)
     return blocks_per_sm((const void *)kernel, threads, smem, smem);
 }
 
-// a grid of resident blocks of nw warps, no more than one warp per brick
-template <typename K>
-static int blocks_for_nw(K kernel, const gpe_grid *g, size_t smem, int nw)
-{
-    int64_t b = (int64_t)g->nsm * per_sm_for(kernel, 32 * nw, smem);
-    const int64_t need = (g->nb + nw - 1) / nw;
-    if (b > need) b = need;
-    if (b < 1) b = 1;
-    return (int)b;
-}
-template <typename R, typename K>
-static int blocks_for(K kernel, const gpe_grid *g, size_t smem)
-{
-    return blocks_for_nw(kernel, g, smem, KernelCfg<R>::NW);
-}
-
 // ------------------------------------------------------------ wavefront sync
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p)
 {

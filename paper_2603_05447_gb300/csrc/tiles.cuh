@@ -32,7 +32,6 @@ namespace gpe {
 template <int NP>
 struct TileFields {
     static constexpr int N = NP == 19 ? 18 : 6;
-    static constexpr int BITS = NP == 19 ? 12 : 10;
 };
 
 struct TileView {
