@@ -155,16 +155,18 @@ __global__ void __launch_bounds__(TILE, sizeof(R) == 4 ? 5 : 2) k_adj_stage(cons
 }
 
 // seed of the reverse sweep: lam = dL/dpsi(T) = -2 dV c psi_t for
-// L = 1 - |c|^2, c = <psi_t|psi(T)>
-template <typename CT>
-__global__ void k_seed(CT *lam, const CT *tgt, int64_t n, double cr, double ci, double dV)
+// L = 1 - |c|^2, c = <psi_t|psi(T)>.  Nothing at inactive cells, where psi(T) is 0
+// whatever the target holds (a cell of the region may have V0 = +inf, a wall):
+// the stages keep lam there as it is.
+template <typename R, typename CT>
+__global__ void k_seed(CT *lam, const CT *tgt, const R *V0, int64_t n, double cr, double ci, double dV)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const CT t = tgt[i];
         CT o;
         o.x = (-2.0 * dV) * (cr * t.x - ci * t.y);
         o.y = (-2.0 * dV) * (cr * t.y + ci * t.x);
-        lam[i] = o;
+        lam[i] = active_v(V0[i]) ? o : czero<CT>();
     }
 }
 
@@ -431,8 +433,6 @@ static int backward_impl(gpe_tape *t, const gpe_state *target, double *grad, dou
     *loss = 1.0 - (c[0] * c[0] + c[1] * c[1]);
     const double dV = g->box.hx * g->box.hy * g->box.hz;
     CT *lam = (CT *)t->d_lam;
-    k_seed<CT><<<g->nsm * 8, 256, 0, s>>>(lam, (const CT *)target->d_psi, (int64_t)np, c[0], c[1], dV);
-    GPE_LAUNCH_CHECK();
     GPE_TRY_CUDA(cudaMemsetAsync(t->d_grad, 0, GPE_MAX_KNOTS * sizeof(double), s));
     // forward stage kernels on tape buffers; times from the tape's start
     k_set_clock<<<1, 1, 0, s>>>(t->d_clock, t->t0);
@@ -440,6 +440,8 @@ static int backward_impl(gpe_tape *t, const gpe_state *target, double *grad, dou
     SegmentSteps<R> run;
     GPE_TRY(run.init(t, s));
     const RkArgs<R> &f = run.f;
+    k_seed<R, CT><<<g->nsm * 8, 256, 0, s>>>(lam, (const CT *)target->d_psi, f.V0, (int64_t)np, c[0], c[1], dV);
+    GPE_LAUNCH_CHECK();
     const TileLaunch &tl = run.L;
     auto blocks = [&](auto k) { return tile_blocks(k, g->nsm, tl.T.ntiles, tl.smem); };
     using KA = void (*)(AdjArgs<R>, TileView);
