@@ -270,12 +270,12 @@ struct gpe_state {
     void *d_psi = nullptr;  // n_packed complex
     void *block = nullptr;  // the allocation that holds psi, E, the clock and the reductions' arrays
     void *d_work[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};  // RK stage states / ITP tmp
-    std::vector<void *> work_blocks;                                           // the allocations that hold them
+    std::vector<void *> work_blocks;  // the allocations that hold them and the schedule tables
     void *d_E = nullptr;    // ITP exp(-V dt/2), state precision
     double E_dt = -1.0;     // dt and
     unsigned long long E_version = 0;  // potential (gpe_grid::v0_version) that d_E was made for
     double *d_clock = nullptr;  // device time base for ramps
-    double *d_stab = nullptr;   // schedule values of the next steps' stages (ramps; made on first use)
+    double *d_stab = nullptr;   // schedule values of the next steps' stages (ramps)
     int stab_cap = 0;           // steps it holds
     gpe::RedScratch red;
     gpe_obs *h_obs = nullptr;   // pinned host landing buffer

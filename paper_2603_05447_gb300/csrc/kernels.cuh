@@ -509,6 +509,7 @@ static __global__ void k_ramp_table(Ramp r, double *clock, double advance, int64
 }
 constexpr StageTimes RK4_TIMES = {{0.0, 0.5, 1.0}};
 constexpr int STAB_STEPS = 256;  // steps a table is made for at a time
+constexpr int GRAPH_STEPS_MAX = 4096;  // steps of a graph at most, and then a table's
 
 // arguments of the RK4 stages of a state (ramps: the clock is set to t0)
 template <typename R>

@@ -426,20 +426,17 @@ static const void *pinned_view(const void *p)
 }
 
 // ------------------------------------------------------------ state helpers
+// Two sizes at most, and both stay until the state is destroyed: a graph, the
+// state's own or one that a caller captured, may hold the smaller one.
 int ensure_stab(gpe_state *st, int steps)
 {
     if (st->stab_cap >= steps) return GPE_OK;
-    // a captured graph may hold the old table
-    if (st->gexec[0]) {
-        GPE_TRY_CUDA(cudaDeviceSynchronize());
-        cudaGraphExecDestroy(st->gexec[0]);
-        st->gexec[0] = nullptr;
-    }
-    dev_free(st->d_stab);
-    st->d_stab = nullptr;
-    st->stab_cap = 0;
-    GPE_TRY(dev_alloc_t(&st->d_stab, 6 * (size_t)steps));
-    st->stab_cap = steps;
+    const int cap = steps <= STAB_STEPS ? STAB_STEPS : GRAPH_STEPS_MAX;
+    double *t = nullptr;
+    GPE_TRY(dev_alloc_t(&t, 6 * (size_t)cap));
+    st->work_blocks.push_back(t);
+    st->d_stab = t;
+    st->stab_cap = cap;
     return GPE_OK;
 }
 
@@ -1214,7 +1211,7 @@ extern "C" int gpe_state_create(gpe_grid *g, int dtype, gpe_state **out)
         rc = fail(GPE_ERR_CUDA, "cudaMallocHost failed");
     if (rc != GPE_OK) {
         dev_free(st->block);
-        dev_free(st->d_stab);
+        for (void *b : st->work_blocks) dev_free(b);
         if (st->h_obs) cudaFreeHost(st->h_obs);
         delete st;
         return rc;
@@ -1230,7 +1227,6 @@ extern "C" int gpe_state_destroy(gpe_state *st)
     cudaDeviceSynchronize();
     dev_free(st->block);
     for (void *b : st->work_blocks) dev_free(b);
-    dev_free(st->d_stab);
     dev_free(st->d_done);
     dev_free(st->d_ctr);
     dev_free(st->d_chunk_norm);
@@ -1271,7 +1267,8 @@ extern "C" int gpe_wait_selftest(double limit_s, int *timed_out, double *waited_
 extern "C" int gpe_state_set_graph(gpe_state *st, int steps_per_graph)
 {
     GPE_TRY(check_state(st));
-    if (steps_per_graph < 0 || steps_per_graph > 4096) return fail(GPE_ERR_ARG, "steps_per_graph must be in [0, 4096]");
+    if (steps_per_graph < 0 || steps_per_graph > GRAPH_STEPS_MAX)
+        return fail(GPE_ERR_ARG, "steps_per_graph must be in [0, %d]", GRAPH_STEPS_MAX);
     if (!is_real_dtype(st->dtype)) GPE_TRY(ensure_stab(st, steps_per_graph));
     st->graph_steps = steps_per_graph;
     return GPE_OK;
