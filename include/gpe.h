@@ -351,9 +351,12 @@ int gpe_step_real(gpe_state *st, const gpe_real_params *p, int64_t nsteps,
                   double t0, gpe_stream stream);
 
 /* ------------------------------------------------------------------ observables */
-/* FP64 reductions over the active cells (products in the state's precision,
- * each 4-cell segment's terms summed in that precision, the segment sums
- * accumulated in FP64 in a fixed order):
+/* Reductions over the active cells, in a fixed order: products in the state's
+ * precision, each 4-cell segment's terms summed in that precision, the segment
+ * sums accumulated in FP64 (states of 64-bit reals), or as unevaluated pairs of
+ * floats that are good to about 2^-47 and go into FP64 at the latest after 64
+ * terms of a thread, 32 threads and whenever they grow beyond 1e30 (states of
+ * 32-bit reals).  From there on FP64:
  *   norm   = sum |psi|^2 dV                           (Eq. (3))
  *   e_kin  = sum Re(conj(psi) T psi) dV
  *   e_pot  = sum V |psi|^2 dV,  V = (1 - s_blend) V0 + s_blend V1
@@ -513,15 +516,19 @@ int gpe_ramp_stages(const gpe_state *psi0, const gpe_ramp_pot *pots,
  *
  * gpe_ramp_forward runs nsteps real-time RK4 steps of a GPE_V_BLEND ramp from
  * the state's psi (as gpe_step_real, from time t0) and records a tape: a
- * checkpoint of psi every K steps, kept in device memory (ceil(nsteps/K)
- * copies of the state plus K more for the backward pass).  The state ends at
- * psi(T).  Asynchronous for the steps; returns the tape.
+ * checkpoint of psi every K steps, kept in device memory: ceil(nsteps/K)
+ * copies of the state, K + 8 more for the backward pass, and, where they take at
+ * most an eighth of the memory that is free at the call, another 3 K for the
+ * stage states of a segment (the backward pass then computes no stage twice; the
+ * results are the same without them).  The tape's destruction frees all of it.
+ * The state ends at psi(T).  Asynchronous for the steps; returns the tape.
  *
  * gpe_ramp_backward computes L = 1 - |<target|psi(T)>|^2 (target: a state on
  * the same grid and type, e.g. the ground state of the final potential) and
  * dL/d knots[k] for k < n_knots, by recomputing each K-step segment from its
- * checkpoint and applying the transposed RK4 step in reverse (bulk in the
- * state's precision, gradient accumulated in FP64).  The tape can be reused
+ * checkpoint (but for the last one, whose states are still in place when all
+ * were kept) and applying the transposed RK4 step in reverse: bulk in the state's
+ * precision, the gradient accumulated like the observables.  The tape can be reused
  * with other targets while the state still holds psi(T).  Synchronous. */
 int gpe_ramp_forward(gpe_state *st, const gpe_real_params *p, int64_t nsteps,
                      double t0, int K, gpe_tape **out, gpe_stream stream);

@@ -6,10 +6,12 @@
 // grid in Morton or z-major key order with an order-preserving compaction (two
 // passes: per-block counts, then emission at scanned offsets); (3) a dense
 // brick-id volume and the 6-entry face-neighbour table; (4) per-cell potential
-// values and the active-cell bit mask.  The paper's GPU variant keeps a
-// 488-entry halo index list per 8^3 block (Sec. II B); here six neighbour ids
-// per brick are enough because the halo is gathered from neighbour bricks at
-// fixed offsets inside the step kernels.
+// values and the active-cell bit mask; (5) the packed layout's records; (6) the
+// stencil kernels' tiles (tiles.cu).  The paper's GPU variant keeps a 488-entry
+// halo index list per 8^3 block (Sec. II B, 3.8 bytes a cell); here a tile of 128
+// stored segments has neighbour slots and a list of the segments outside it,
+// 3.2 bytes a stored cell, and the wavefront and fused schedules gather a brick's
+// halo at fixed offsets from its neighbours.
 #include <algorithm>
 #include <cmath>
 #include <vector>

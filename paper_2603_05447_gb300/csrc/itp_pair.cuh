@@ -20,7 +20,7 @@
 // other bricks, so the result goes to a second buffer and the state
 // alternates between two buffers from step to step.
 //
-// The per-cell arithmetic is the staged kernels' (DiagLoad::apply, lapv,
+// The per-cell arithmetic is the staged kernels' (DiagLoad::apply, lap4,
 // axpy), so before the final factor the two schedules agree bit for bit;
 // the norm is summed in another order, so the factor can differ in its last
 // bit.  Complex states only (a real float segment is a single 16-byte unit,

@@ -23,7 +23,7 @@
 //    row the two cells on either side in x (x = -2, -1 and BX, BX+1, from the
 //    x-face and the xy/xz-edge neighbours); filled by cp.async;
 //  * v: stage A on the brick and its one-deep face halo (the layout of the
-//    staged kernels' tile), written by the block's threads;
+//    wavefront kernels' tile), written by the block's threads;
 //  * the records of the brick, its 6 face and 12 edge neighbours, looked up
 //    through the per-brick neighbour ids (the 32-byte records stay in L2).
 // Stage A runs as three task sets: the brick's stored segments, the stored

@@ -264,13 +264,6 @@ __device__ __forceinline__ CT lapv(const CT &xp, const CT &xm, const CT &yp, con
     }
 }
 
-// What a pass wants of a cell's neighbourhood: its Laplacian (LapFull), or, for
-// the right-hand side of the real-time steps in double precision, half of it with
-// the sign of the kinetic term (LapRhs): FP64 instructions bound the complex128
-// steps, and the factor -1/2 costs none in the coefficients.  (The centre's
-// share in the potential would save one more of about fourteen a cell and stage,
-// 3 % of a step, but rounds the potential at the size of 1/h^2: 19-point errors
-// 2 % larger.)  In single precision, bound by bytes, it is the Laplacian as it is.
 // Whether a cell is active, from its potential (+inf, or NaN, marks the inactive
 // cells of stored segments) or its propagator (negative there).  Double values
 // are tested by their high words: an FP64 comparison costs as much as an FP64
@@ -422,6 +415,13 @@ __device__ __forceinline__ double sum6(double xp, double xm, double yp, double y
     return i64_to_double(S[0] + S[1] + S[2]) * f;
 }
 
+// What a pass wants of a cell's neighbourhood: its Laplacian (LapFull), or, for
+// the right-hand side of the real-time steps in double precision, half of it with
+// the sign of the kinetic term (LapRhs): FP64 instructions bound the complex128
+// steps, and the factor -1/2 costs none in the coefficients.  (The centre's
+// share in the potential would save one more of about fourteen a cell and stage,
+// 3 % of a step, but rounds the potential at the size of 1/h^2: 19-point errors
+// 2 % larger.)  In single precision, bound by bytes, it is the Laplacian as it is.
 struct LapFull {
     static constexpr bool FIXED = true;  // double precision: sums in fixed point where the spacings allow
     template <typename R>

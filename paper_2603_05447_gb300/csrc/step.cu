@@ -1,17 +1,16 @@
 // step.cu -- wavefunction states, the real-time RK4 step, the imaginary-time
 // split step with renormalisation, and the FP64 observables of libgpeshell.
 //
-// Every stencil kernel stages one brick plus its face halo in shared memory
-// (the paper's per-block tile of Sec. II B, gathered here from the six face
-// neighbours through the brick-neighbour table and the packed-layout ranks),
-// evaluates the 7-point Laplacian of Eq. (B1) from the tile, applies the
-// pointwise terms of the equation and writes the active cells.
-//
-// Two schedules run the same per-brick arithmetic:
-//  * STAGED: one launch per stage; blocks walk the brick list with a fixed
-//    stride, so per-block partial sums (and every FP64 reduction) are
-//    deterministic.
-//  * WAVE: one persistent launch per time step.  The work is split into
+// Schedules of the step:
+//  * STAGED: one launch per stage, on tiles of consecutive stored segments with
+//    halo lists (tiles.cuh).  A block takes tiles at a fixed stride, so the
+//    partial sums (and every FP64 reduction) are deterministic.
+//  * PAIR: the stages fused in pairs, a block a brick (pair.cuh, itp_pair.cuh).
+//  * WAVE, WAVE2: one persistent launch per time step, or two of stage pairs, on
+//    bricks: a warp stages its brick plus the face halo in shared memory (the
+//    paper's per-block tile of Sec. II B, gathered from the six face neighbours
+//    through the brick-neighbour table and the packed-layout ranks) and
+//    evaluates the 7-point Laplacian of Eq. (B1) from it.  The work is split into
 //    (stage, chunk) tasks, a chunk being `cb` consecutive bricks.  Tasks are
 //    handed out from an atomic ticket counter in an order where every
 //    dependency of a task has a smaller ticket (stage s of chunk c needs stage

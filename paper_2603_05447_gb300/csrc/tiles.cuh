@@ -391,10 +391,10 @@ constexpr int tile_blocks_f(int np) { return np == 19 ? 5 : 6; }
 
 // One RK4 stage.  1024^3 shell, 8x8x4 bricks, per step of four: complex64
 // 0.776 -> 0.622 ms (4.0 GB, of which 0.4 GB slots and halo lists: 6.5 TB/s,
-// 0.95 of the copy bandwidth, so bytes bound it now); complex128 8.65 -> 4.45
+// 0.95 of the copy bandwidth, so bytes bound it now); complex128 8.65 -> 4.23
 // ms (full lanes instead of four fifths: 6.75; 90 instead of 108 FP64
 // instructions a cell and step, LapRhs, active_v and the split third: 5.44;
-// the neighbour sums in integers, sum6: 4.45; an FP64 instruction takes 16
+// the neighbour sums in integers, sum6: 4.45, their products behind a branch 4.23; an FP64 instruction takes 16
 // cycles of an SM whatever its lanes do).  Single precision, six blocks an SM
 // (85 registers): 0.626 ms, seven 0.634, eight with spills 0.645; double, three
 // blocks (168 registers) are 1.5 % ahead of two; blended two, which three lose 1 % to.
