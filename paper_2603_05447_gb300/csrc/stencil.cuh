@@ -28,15 +28,18 @@ struct KernelCfg {
 
 // Minimum resident blocks per SM requested from the register allocator:
 // as many as the shared-memory workspaces allow (228 KiB per SM, 1 KiB
-// reserved per block), at most GPE_MINB_F (single precision) / GPE_MINB_D
-// (double precision, whose kernels need more registers).
+// reserved per block), at most GPE_MINB_F (single precision) or a kernel's own
+// number in double precision, whose forms need more registers: three, but two for
+// the blended steps of WAVE2, which at three spill 272 bytes a thread around their
+// calls of sum6.  Eight such steps, FP64 sums, sum6 at three blocks and at two: 48-cell
+// ramp with spacings 1 : 1.2 : 1.08 2062, 2514 and 2009 us, 160-cell ramp with equal
+// ones 8830, 7553 and 7106.  (WAVE: 1717 -> 1267 and 7668 -> 8116 us, static 6356 ->
+// 7492: not taken.)
 #ifndef GPE_MINB_F
 #define GPE_MINB_F 4
 #endif
-#ifndef GPE_MINB_D
-#define GPE_MINB_D 3
-#endif
-#define GPE_BOUNDS(R) __launch_bounds__(KernelCfg<R>::THREADS, (min_blocks<R, BX, BY, BZ>()))
+// (D: blocks of the double-precision form)
+#define GPE_BOUNDS(R, D) __launch_bounds__(KernelCfg<R>::THREADS, (min_blocks<R, BX, BY, BZ>(D)))
 // ------------------------------------------------------------ packed layout
 // supported brick shapes (shape id, BX, BY, BZ)
 #define GPE_SHAPES(M) \
@@ -755,9 +758,9 @@ constexpr size_t smem_bytes()
 // the calling warp's workspace (call once per kernel: it resets the
 // next-record tag)
 template <typename R, int BX, int BY, int BZ>
-constexpr int min_blocks()
+constexpr int min_blocks(int in_double)
 {
-    const int cap = sizeof(R) == 4 ? GPE_MINB_F : GPE_MINB_D;
+    const int cap = sizeof(R) == 4 ? GPE_MINB_F : in_double;
     const int fit = (int)((228u * 1024u) / (smem_bytes<R, BX, BY, BZ>() + 1024u));
     return fit < 1 ? 1 : (fit < cap ? fit : cap);
 }

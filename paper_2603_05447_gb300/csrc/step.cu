@@ -212,7 +212,7 @@ __device__ bool wait_deps(const WaveW &w, int c, uint32_t target)
 
 // RK4 stages first and first + 1 (first = 0 or 2) of one step, warp tasks
 template <typename R, int BX, int BY, int BZ, bool BLEND>
-__global__ void GPE_BOUNDS(R) k_rk4_pair(const RkArgs<R> a, const GridView G, const WaveW w, int first)
+__global__ void GPE_BOUNDS(R, (BLEND ? 2 : 3)) k_rk4_pair(const RkArgs<R> a, const GridView G, const WaveW w, int first)
 {
     auto &ws = warp_space<R, BX, BY, BZ>();
     const int lane = threadIdx.x & 31;
@@ -249,7 +249,7 @@ __global__ void GPE_BOUNDS(R) k_rk4_pair(const RkArgs<R> a, const GridView G, co
 // persistent launch: first = 0 with the 4-stage task list (WAVE), or 0 and
 // then 2 with the 2-stage list (WAVE2).
 template <typename R, int BX, int BY, int BZ, bool BLEND>
-__global__ void GPE_BOUNDS(R) k_rk4_wave(const RkArgs<R> a, const GridView G, const Wave w, int first)
+__global__ void GPE_BOUNDS(R, 3) k_rk4_wave(const RkArgs<R> a, const GridView G, const Wave w, int first)
 {
     using CT = typename Cx<R>::T;
     constexpr int NW = KernelCfg<R>::NW;
@@ -289,7 +289,7 @@ __global__ void GPE_BOUNDS(R) k_rk4_wave(const RkArgs<R> a, const GridView G, co
 
 
 template <typename R, int BX, int BY, int BZ>
-__global__ void GPE_BOUNDS(R) k_itp_wave(const ItpArgs<R> a, const GridView G, const Wave w, double *chunk_norm)
+__global__ void GPE_BOUNDS(R, 3) k_itp_wave(const ItpArgs<R> a, const GridView G, const Wave w, double *chunk_norm)
 {
     constexpr int NW = KernelCfg<R>::NW;
     auto &ws = warp_space<R, BX, BY, BZ>();
